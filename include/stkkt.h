@@ -207,9 +207,12 @@ kkt_status ras_setup(kkt_problem* p, const int nsub[4], int overlap, int local, 
  *   (a tuning and testing hook; the paper has no counterpart).  The shape
  *   decides how the solve kernel runs, not what it computes: every compiled
  *   shape applies the same ILU(0) factors.
- *   shape[0]  points per chunk of a wavefront (FP64: 34, 26, 18; FP32: 52, 36,
- *             20; BF16: 72, 40, 8)
- *   shape[1]  buffers of the factor-copy ring, 2..4
+ *   shape[0]  size class of a box's CTA, by names from when it was a number of
+ *             points (FP64: 34, 26, 18; FP32: 52, 36, 20; BF16: 72, 40, 8): 16,
+ *             8 or 4 warps, each taking 8 points of a wavefront at a time
+ *   shape[1]  2..4: groups of 8 points whose factor values a warp holds, the one
+ *             in use included (one less are buffers in shared memory; FP64 reads
+ *             its factors from global memory and takes the field as given)
  *   shape[2]  lanes per point: 4 (the one compiled)
  *   shape[3]  1 = local vectors in shared memory, 2 = in global memory
  *   A 0 in a field leaves that choice to the library (as ras_setup does).
@@ -236,10 +239,10 @@ kkt_status ras_setup_batch(kkt_problem* const* probs, int nprob, const int nsub[
 
 /*
  * ras_autotune -- choose the subdomain solve's shape by measurement: every
- *   compiled chunk size with 2 and 3 copy buffers is set up on these problems
+ *   compiled size class with 2 and 3 groups held is set up on these problems
  *   (split as in ras_setup_batch, ILU(0), factor_prec) and timed over `reps`
- *   applies with CUDA events; shape_out gets the fastest {chunk points, ring
- *   buffers, 4, 0} and *best_ms (may be NULL) its time per apply.  With a
+ *   applies with CUDA events; shape_out gets the fastest {size class, groups
+ *   held, 4, 0} and *best_ms (may be NULL) its time per apply.  With a
  *   cache_path (may be NULL) an earlier result for the same problem sizes,
  *   split, precision and device is read from that text file instead, and a
  *   new one is appended.  Synchronous; a tuning aid with no counterpart in the
@@ -258,9 +261,9 @@ kkt_status ras_info(const ras_precond* m, int* nbox, long long* points, long lon
 
 /*
  * ras_solve_shape -- how the subdomain solve of a preconditioner runs (chosen
- *   at ras_setup from the boxes' sizes and the device's occupancy): points per
- *   chunk of a wavefront, buffers of its factor-copy ring, lanes per point,
- *   and 1 if the local vectors live in shared memory.  Any output may be
+ *   at ras_setup from the boxes' sizes and the device's occupancy): size class
+ *   of the CTA and groups held (ras_setup_shape), lanes per point, and 1 if the
+ *   local vectors live in shared memory.  Any output may be
  *   NULL.  Reporting only; the paper has no counterpart.
  */
 kkt_status ras_solve_shape(const ras_precond* m, int* chunk_points, int* stages, int* lanes, int* smem_vectors);
@@ -269,8 +272,8 @@ kkt_status ras_solve_shape(const ras_precond* m, int* chunk_points, int* stages,
  * ras_status -- the preconditioner's device status word, read on `stream`
  *   (synchronises that stream): 0 = fine; 1 = the last factorisation met a
  *   zero or non-finite pivot (returns ZERO_PIVOT); 2 = a subdomain solve gave
- *   up waiting for a factor copy after its 2 s limit and left z unwritten
- *   (returns ERR_CUDA).  ras_apply and ras_apply_static never synchronise, so
+ *   up waiting for a factor copy or an earlier wavefront after its 2 s limit
+ *   and left z unwritten (returns ERR_CUDA).  ras_apply and ras_apply_static never synchronise, so
  *   a caller that does not go through gmres_solve reads the outcome of its
  *   applies here.  The word is cleared by ras_refactor.
  */

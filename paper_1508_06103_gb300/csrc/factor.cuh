@@ -32,6 +32,12 @@ constexpr int kGatherThreads = 256;
 template <typename T>
 constexpr int factor_threads = sizeof(T) == 4 ? 192 : 128;
 
+// offset of the column of group place q in the box's factor values
+template <typename T>
+__device__ __forceinline__ int group_column(int q) {
+  return q / kGroup * group_vals(8 * sizeof(T)) + q % kGroup;
+}
+
 // One thread per point (wavefront order, so the threads of a chunk write
 // consecutive addresses); all threads of a warp on the same slot.  Entries are
 // formed in the factor precision, with the arithmetic of slot_value, but one
@@ -43,28 +49,28 @@ constexpr int factor_threads = sizeof(T) == 4 ? 192 : 128;
 template <typename T>
 __global__ void __launch_bounds__(kGatherThreads) gather_chunks(const DevProblem* __restrict__ probs,
                                                                 const BoxDesc* __restrict__ boxes,
-                                                                const int* __restrict__ perm,
-                                                                const int2* __restrict__ ptab, T* __restrict__ F) {
+                                                                const int* __restrict__ gptr,
+                                                                const int* __restrict__ perm, T* __restrict__ F) {
   const BoxDesc bx = boxes[blockIdx.y];
   const DevProblem p = probs[bx.prob];
   T* Fb = F + bx.foff;
   if (blockIdx.x == 0)
     for (int s = threadIdx.x; s < kSlots; s += blockDim.x)
-      Fb[bx.unit + c_gen_rank[s]] = (s == kDiagC || s == kDiagG || s == kDiagF) ? (T)1 : (T)0;
-  const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (q >= bx.P) return;
+      Fb[bx.unit + c_gen_rank[s] * kGroup] = (s == kDiagC || s == kDiagG || s == kDiagF) ? (T)1 : (T)0;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= kGroup * gptr[bx.loff + bx.nlev]) return;
+  const int lex = perm[kGroup * bx.goff + q];
+  if (lex < 0) return;
   const Coefs<T> cf = coefs<T>(p);
-  const PointRow<T> pr = point_row<T>(p, bx, perm[bx.poff + q]);
-  const int2 pt = ptab[bx.poff + q];
-  T* dst = Fb + pt.x;
-  const long long st = pt.y;
+  const PointRow<T> pr = point_row<T>(p, bx, lex);
+  T* dst = Fb + group_column<T>(q);
   const T tau = (T)p.tau, th = (T)p.theta, th1 = (T)(1.0 - p.theta), b1 = (T)p.beta1, b2 = (T)p.beta2;
   const T mt1 = tau / (T)6, lt1 = -(T)1 / tau;
   const bool idC = pr.n == 0 || pr.dirj, idG = pr.n == p.M || pr.dirj;   // identity rows
   const bool tm = pr.kt > 0, tp = pr.kt + 1 < bx.lt;                      // levels n-1, n+1 in the box
   const T z = (T)0;
   // slot (row type c, level offset dt, spatial offset d, column component cc)
-#define PUT(c, dt, d, cc, v) dst[(long long)c_gen_rank_of[c][(dt) + 1][d][cc] * st] = (v)
+#define PUT(c, dt, d, cc, v) dst[c_gen_rank_of[c][(dt) + 1][d][cc] * kGroup] = (v)
 #pragma unroll
   for (int d = 0; d < kStencil; ++d) {
     const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
@@ -108,52 +114,50 @@ __device__ __forceinline__ void check_pivot(double d, int* status) {
 
 template <typename T>
 __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDesc* __restrict__ boxes,
-                                                                    const int* __restrict__ iperm,
+                                                                    const int* __restrict__ gptr,
                                                                     const int* __restrict__ perm,
-                                                                    const int* __restrict__ lptr,
-                                                                    const int2* __restrict__ ptab,
+                                                                    const int* __restrict__ ptab,
                                                                     T* __restrict__ F, int* __restrict__ status) {
-  // per thread and pivot point: {offset of its column in Fb, row stride of its block}
+  // per thread and pivot point: offset of its column in Fb
   constexpr int NS = factor_threads<T>;
-  __shared__ int2 nbs[kGenNbrs * NS];
+  __shared__ int nbs[kGenNbrs * NS];
   const BoxDesc bx = boxes[blockIdx.x];
   T* Fb = F + bx.foff;
-  const int* lp = lptr + bx.loff;
-  const int* ip = iperm + bx.poff;
-  const int2* pb = ptab + bx.poff;
-  int2* nb = nbs + threadIdx.x;
+  const int* gp = gptr + bx.loff;
+  const int* pm = perm + kGroup * bx.goff;
+  const int* pb = ptab + bx.poff;
+  int* nb = nbs + threadIdx.x;
   const int unit = (int)bx.unit;
   for (int w = 0; w < bx.nlev; ++w) {
-    const int npts = lp[w + 1] - lp[w];
-    for (int j = threadIdx.x; j < npts; j += blockDim.x) {
-      const int q = lp[w] + j;
-      const int lex = perm[bx.poff + q];
+    const int q1 = kGroup * gp[w + 1];
+    for (int q = kGroup * gp[w] + threadIdx.x; q < q1; q += blockDim.x) {
+      const int lex = pm[q];
+      if (lex < 0) continue;
       const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
       const int kt = lex / (bx.lx * bx.ly * bx.lz);
 #pragma unroll 1
       for (int i = 0; i < kGenNbrs; ++i) {
         const int dt = c_gen_nbr[i][0], dz = c_gen_nbr[i][1], dy = c_gen_nbr[i][2], dx = c_gen_nbr[i][3];
         const int ax = kx + dx, ay = ky + dy, az = kz + dz, at = kt + dt;
-        int2 e = make_int2(unit, 1);
+        int e = unit;
         if (ax >= 0 && ax < bx.lx && ay >= 0 && ay < bx.ly && az >= 0 && az < bx.lz && at >= 0 && at < bx.lt)
-          e = pb[ip[ax + bx.lx * (ay + bx.ly * (az + bx.lz * at))]];
+          e = pb[ax + bx.lx * (ay + bx.ly * (az + bx.lz * at))];
         nb[i * NS] = e;
       }
-      const int2 pt = pb[q];
-      T* own = Fb + pt.x;
+      T* own = Fb + group_column<T>(q);
       // the G and f rows read the U parts of this point's C and G rows
       if constexpr (sizeof(T) == 4) {
-        check_pivot((double)ilu_row0_32<T, NS>(own, pt.y, Fb, nb), status);
+        check_pivot((double)ilu_row0_32<T, NS>(own, Fb, nb), status);
         asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row1_32<T, NS>(own, pt.y, Fb, nb), status);
+        check_pivot((double)ilu_row1_32<T, NS>(own, Fb, nb), status);
         asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row2_32<T, NS>(own, pt.y, Fb, nb), status);
+        check_pivot((double)ilu_row2_32<T, NS>(own, Fb, nb), status);
       } else {
-        check_pivot((double)ilu_row0_64<T, NS>(own, pt.y, Fb, nb), status);
+        check_pivot((double)ilu_row0_64<T, NS>(own, Fb, nb), status);
         asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row1_64<T, NS>(own, pt.y, Fb, nb), status);
+        check_pivot((double)ilu_row1_64<T, NS>(own, Fb, nb), status);
         asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row2_64<T, NS>(own, pt.y, Fb, nb), status);
+        check_pivot((double)ilu_row2_64<T, NS>(own, Fb, nb), status);
       }
     }
     __syncthreads();
@@ -163,15 +167,13 @@ __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDes
 // gather, then factor, in place on F (chunk layout); both on stream s
 template <typename T>
 kkt_status factor_launch(ras_precond* m, T* F, cudaStream_t s) {
-  long long pmax = 0;
-  for (const BoxDesc& b : m->boxes_h) pmax = std::max(pmax, b.P);
-  const dim3 g((unsigned)((pmax + kGatherThreads - 1) / kGatherThreads), m->nbox);
-  gather_chunks<T><<<g, kGatherThreads, 0, s>>>(m->dprobs, m->boxes, m->perm, m->ptab, F);
+  const dim3 g((unsigned)((kGroup * (long long)m->max_groups + kGatherThreads - 1) / kGatherThreads), m->nbox);
+  gather_chunks<T><<<g, kGatherThreads, 0, s>>>(m->dprobs, m->boxes, m->gptr, m->perm, F);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   {
     TimedScope timed(&m->factor_timing, s);
-    ilu0_factor<T><<<m->nbox, factor_threads<T>, 0, s>>>(m->boxes, m->iperm, m->perm, m->lptr, m->ptab, F,
+    ilu0_factor<T><<<m->nbox, factor_threads<T>, 0, s>>>(m->boxes, m->gptr, m->perm, m->ptab, F,
                                                       m->status);
   }
   KKT_COUNT(1);

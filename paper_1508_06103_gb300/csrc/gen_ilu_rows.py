@@ -1,6 +1,6 @@
 """Generate ilu_rows.inc: straight-line ILU(0) elimination of one KKT row per thread.
 
-(and ilu_slots.inc: the slot list's checksum and each slot's row in a chunk block,
+(and ilu_slots.inc: the slot list's checksum and each slot's row in a group,
 also indexed by the slot's offsets for the value gather)
 
 Every row of the space-time KKT matrix is one of three types (C, G, f) with
@@ -66,8 +66,8 @@ def slot_tables():
 
 
 def slot_rank(s, base, diag, count):
-    """Row of slot s in a chunk block: the L-slots of C, G, f, then the diagonal
-    and U-slots of C, G, f (the order the subdomain solve streams them in)."""
+    """Row of slot s in a group: the L-slots of C, G, f, then the diagonal
+    and U-slots of C, G, f (the order the sweeps use them in)."""
     nl = [diag[c] - base[c] for c in range(3)]
     nu = [count[c] - nl[c] for c in range(3)]
     for c in range(3):
@@ -100,24 +100,23 @@ def row_function(c, prec, group, nl, cnt, base, slots, diag, rank, nbrs, contrib
     registers for the rest of the row.
     """
     o = [
-        "// own: the point's column in its chunk block (row stride ost); F + nb[i * NS].x: pivot point i's",
-        "// column (the unit row outside the box), nb[i * NS].y: its row stride.  Stores 1/pivot in the",
-        "// diagonal slot and returns the pivot.",
+        "// own: the point's column in its group; F + nb[i * NS]: pivot point i's column (the unit row",
+        "// outside the box).  Stores 1/pivot in the diagonal slot and returns the pivot.",
         "template <typename T, int NS>",
-        f"__device__ __forceinline__ T ilu_row{c}_{prec}(T* __restrict__ own, const int ost, "
-        "const T* __restrict__ F, const int2* __restrict__ nb) {",
+        f"__device__ __forceinline__ T ilu_row{c}_{prec}(T* __restrict__ own, const T* __restrict__ F, "
+        "const int* __restrict__ nb) {",
         f"  T l[{nl}], u[{group}], d;",
     ]
 
     def accumulate(x, dst):
         o.append("  {")
-        o.append(f"    T acc = own[{rank[base + x]} * ost];")
+        o.append(f"    T acc = own[{rank[base + x]} * 8];")
         for (s, i, t) in contrib[x]:
-            o.append(f"    {{ const int2 q = nb[{i} * NS]; acc -= l[{s}] * F[q.x + {rank[t]} * q.y]; }}")
+            o.append(f"    acc -= l[{s}] * F[nb[{i} * NS] + {rank[t]} * 8];")
         if x < nl:
             dt, dz, dy, dx, ck = slots[base + x]
             i = nbrs.index((dt, dz, dy, dx))
-            o.append(f"    {{ const int2 q = nb[{i} * NS]; l[{x}] = acc * F[q.x + {rank[diag[ck]]} * q.y]; }}")
+            o.append(f"    l[{x}] = acc * F[nb[{i} * NS] + {rank[diag[ck]]} * 8];")
         else:
             o.append(f"    {dst} = acc;")
         o.append("  }")
@@ -133,7 +132,7 @@ def row_function(c, prec, group, nl, cnt, base, slots, diag, rank, nbrs, contrib
             o.append("  u[0] = (T)1 / u[0];")
         for x in range(g0, g1):
             val = f"l[{x}]" if x < nl else f"u[{x - g0}]"
-            o.append(f"  own[{rank[base + x]} * ost] = {val};")
+            o.append(f"  own[{rank[base + x]} * 8] = {val};")
     o.append("  return d;")
     o.append("}")
     o.append("")
@@ -156,13 +155,13 @@ def generate() -> str:
     rank = [slot_rank(s, base, diag, count) for s in range(len(slots))]
     hdr = [
         "// Generated by gen_ilu_rows.py from the KKT row stencils -- do not edit by hand.",
-        "// Slot list of the three row types (C, G, f) and their rows in a chunk block.",
+        "// Slot list of the three row types (C, G, f) and their rows in a group.",
         "#pragma once",
         "",
         f"constexpr long long kGenSlotChecksum = {checksum(slots)}LL;",
         f"constexpr int kGenSlots = {len(slots)};",
         f"constexpr int kGenRowSlots0 = {count[0]}, kGenRowSlots1 = {count[1]}, kGenRowSlots2 = {count[2]};",
-        "// rank of each slot in a chunk block",
+        "// rank of each slot in a group",
         "constexpr short kGenRank[%d] = {" % len(slots),
     ]
     for a in range(0, len(slots), 20):
@@ -174,7 +173,7 @@ def generate() -> str:
     for a in range(0, len(slots), 8):
         hdr.append("    " + ", ".join("{%d, %d, %d, %d, %d}" % sl for sl in slots[a:a + 8]) + ",")
     hdr.append("};")
-    hdr.append("// rank of each slot in a chunk block (device copy of kGenRank)")
+    hdr.append("// rank of each slot in a group (device copy of kGenRank)")
     hdr.append("__constant__ short c_gen_rank[%d] = {" % len(slots))
     for a in range(0, len(slots), 20):
         hdr.append("    " + ", ".join(str(r) for r in rank[a:a + 20]) + ",")
@@ -200,7 +199,7 @@ def generate() -> str:
     out = [
         "// Generated by gen_ilu_rows.py from the KKT row stencils -- do not edit by hand.",
         "// ILU(0) elimination of one row of each type (C, G, f), one target entry at a time,",
-        "// on the chunk layout (slot s of a point at offset kGenRank[s] * stride).",
+        "// in place on groups of 8 points (slot s of a point at offset 8 kGenRank[s]).",
         "#pragma once",
         "",
         f"constexpr int kGenNbrs = {len(nbrs)};",

@@ -17,13 +17,12 @@
 // outside the box hold 0, which is the same as leaving them out of the
 // pattern.
 //
-// Layout in HBM.  The points of each wavefront are cut into chunks of at most
-// CH points (56 in FP32, 28 in FP64).  A chunk's values form one contiguous
-// block [slot rank][point of the chunk] with a row stride cp >= the chunk's
-// point count chosen so that the shared-memory reads of the solve are free of
-// bank conflicts; the L-slots of the three rows come first (175 ranks), then
-// the diagonal and U-slots (151 ranks).  The forward sweep therefore streams
-// one contiguous L block per chunk and the backward sweep one U block.
+// Layout in HBM.  The points of each wavefront are stored in groups of 8, one
+// after the other; the values of a group form one block, the L-slots first,
+// then the diagonals and U-slots, so the forward sweep streams the lower
+// halves of the groups in order and the backward sweep the upper halves.  In
+// FP32 and BF16 a half is ordered by the lanes of the solve (lane_place, ras.cuh),
+// in FP64 by slot rank ([rank][8 points]).
 //
 // Ordering and parallelism.  Points are processed in the natural
 // (lexicographic) order of the box; with this stencil every lower-triangular
@@ -40,14 +39,10 @@
 // slot of a factored row stores 1/u_kk, so both the factorisation and the
 // backward sweep multiply instead of divide.
 //
-// Solve.  One CTA per box runs a two-stage pipeline over its chunks: thread 0
-// issues a TMA bulk copy (cp.async.bulk, completion on an mbarrier) of the
-// next chunk's L (or U) block into one of two shared-memory buffers while the
-// CTA computes the current chunk from the other.  The local vector of each box
-// has a ghost layer of zeros one point wide in every direction, so the
-// triangular sweeps need no bounds tests: a slot whose column leaves the box
-// reads 0 and has factor value 0.  Small boxes keep the local vector in shared
-// memory as well.
+// Solve.  One CTA per box; a warp takes a group of 8 points of the wavefront.
+// The local vector of each box has a ghost layer of zeros one point wide in
+// every direction, so the triangular sweeps need no bounds tests: a slot whose
+// column leaves the box reads 0 and has factor value 0.
 
 #include <algorithm>
 #include <array>
@@ -107,7 +102,7 @@ const SlotTables& tables() {
   return T;
 }
 
-// Checksum of the slot list and chunk block rank of every slot, as the
+// Checksum of the slot list and group rank of every slot, as the
 // generated factorisation code (factor32.cu, factor64.cu) assumes them.
 #include "ilu_slots.inc"
 
@@ -120,7 +115,7 @@ constexpr int kUnitRowSpan = (kSlots + 3) / 4 * 4;
 constexpr int kLRanks = 175;        // L-slots of the three rows
 constexpr int kURanks = 151;        // diagonals and U-slots of the three rows
 
-// rank of slot s in a chunk block: L-slots of C, G, f, then diag+U of C, G, f
+// rank of slot s in a group: L-slots of C, G, f, then diag+U of C, G, f
 int slot_rank(int s) {
   if (s < kCDiag) return s;
   if (s >= kGBase && s < kGDiag) return 80 + (s - kGBase);
@@ -130,34 +125,19 @@ int slot_rank(int s) {
   return kLRanks + 70 + (s - kFDiag);
 }
 
-// Chunk configurations of the subdomain solve, per stored type S: candidate
-// chunk sizes (points) and the row-stride rule cp = R (mod Q) of a chunk
-// block.  In a step the 4 lanes of a point take the stencil neighbours
-// q = lane + 4 i; the factor entries of neighbour q in the C and f rows sit
-// in block rows a + 2q (+1), so the 4 lanes of a point read rows 2 apart and
-// the 8 points of a warp read 8 consecutive columns: with 2 cp = 8 (mod 32)
-// 4-byte words the 32 reads of a warp fall in 32 different banks (for 8-byte
-// values every half warp does; for 2-byte values, two per word).  cp is also
-// a multiple of 16 bytes' worth of values over the 175 and 151 block rows,
-// so every bulk copy starts and ends on 16-byte boundaries.
+// Size classes of the solve's CTA, per stored type S: the first field of a
+// shape (its names are fixed by the interface) and the warps it stands for.
 template <typename S>
-struct ChunkCfg;
-// The chunk sizes are strides the rule allows, so a full chunk carries no
-// padding columns.
-template <>
-struct ChunkCfg<float> {
-  static constexpr int CH = 52, CH2 = 36, CH3 = 20;
-  static constexpr int Q = 16, R = 4;                  // cp = 4 (mod 16)
+struct SizeClasses {   // FP32
+  static constexpr int name[3] = {52, 36, 20}, warps[3] = {16, 8, 4};
 };
 template <>
-struct ChunkCfg<double> {
-  static constexpr int CH = 34, CH2 = 26, CH3 = 18;
-  static constexpr int Q = 8, R = 2;                   // cp = 2 (mod 8)
+struct SizeClasses<double> {
+  static constexpr int name[3] = {34, 26, 18}, warps[3] = {16, 8, 4};
 };
 template <>
-struct ChunkCfg<__nv_bfloat16> {                      // FP32 factors stored as BF16
-  static constexpr int CH = 72, CH2 = 40, CH3 = 8;
-  static constexpr int Q = 32, R = 8;                  // cp = 8 (mod 32): two values per bank word
+struct SizeClasses<__nv_bfloat16> {   // FP32 factors stored as BF16
+  static constexpr int name[3] = {72, 40, 8}, warps[3] = {16, 8, 4};
 };
 constexpr int kLanes = 4;   // lanes per point of the subdomain solve
 // arithmetic type of the solve for a storage type (BF16 factors: FP32)
@@ -169,42 +149,8 @@ template <>
 struct SolveArith<__nv_bfloat16> {
   using type = float;
 };
-template <typename T, typename S>
-__device__ __forceinline__ T arith(S v) {
-  return static_cast<T>(v);
-}
-template <>
-__device__ __forceinline__ float arith<float, __nv_bfloat16>(__nv_bfloat16 v) {
-  return __bfloat162float(v);
-}
-
-template <typename S>
-int chunk_stride(int n) {
-  const int Q = ChunkCfg<S>::Q, R = ChunkCfg<S>::R;
-  return n <= R ? R : R + ((n - R + Q - 1) / Q) * Q;
-}
-template <typename S>
-__host__ __device__ constexpr int chunk_stride_dev(int n) {
-  return n <= ChunkCfg<S>::R ? ChunkCfg<S>::R
-                             : ChunkCfg<S>::R + ((n - ChunkCfg<S>::R + ChunkCfg<S>::Q - 1) / ChunkCfg<S>::Q) *
-                                                    ChunkCfg<S>::Q;
-}
-static_assert(chunk_stride_dev<float>(ChunkCfg<float>::CH) == ChunkCfg<float>::CH, "full FP32 chunk unpadded");
-static_assert(chunk_stride_dev<double>(ChunkCfg<double>::CH) == ChunkCfg<double>::CH, "full FP64 chunk unpadded");
-static_assert(chunk_stride_dev<__nv_bfloat16>(ChunkCfg<__nv_bfloat16>::CH) == ChunkCfg<__nv_bfloat16>::CH,
-              "full BF16 chunk unpadded");
-int chunk_stride_of(int prec, int n) {
-  if (prec == 64) return chunk_stride<double>(n);
-  if (prec == 16) return chunk_stride<__nv_bfloat16>(n);
-  return chunk_stride<float>(n);
-}
-
 // ---------------------------------------------------------------------------
-// kernels
-// ---------------------------------------------------------------------------
-
-// ---------------------------------------------------------------------------
-// TMA bulk copies and mbarriers (inline PTX)
+// TMA bulk copies, mbarriers and counters (inline PTX)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));
@@ -227,6 +173,14 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
+__device__ __forceinline__ int ld_acquire_cta(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void add_release_cta(int* p, int v) {
+  asm volatile("red.release.cta.shared::cta.add.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
   unsigned done;
   asm volatile(
@@ -243,7 +197,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 // Bounded wait on phase `parity` of an mbarrier: gives up after limit_ns
 // nanoseconds of polling, records status 2 in *failed and returns false.
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s: a block copy takes microseconds
+constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s: copies and wavefronts take microseconds
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, int* failed,
                                           unsigned long long limit_ns = kWaitLimitNs) {
   // the timer is read only every 64 polls, so a copy that lands within the
@@ -277,25 +231,30 @@ __global__ void wait_selftest(int* status, unsigned long long limit_ns) {
 
 // ---------------------------------------------------------------------------
 // Subdomain solve z = sum_boxes (R^0)^T M^{-1} R^delta r: one CTA per box,
-// 4 lanes per point, one chunk of points per step.
+// 4 lanes per point, one group of 8 points per warp at a time.
 //
 // The box's padded local vector holds 4 values per point (C, G, f and a zero),
 // so one 16-byte load fetches a neighbour's three unknowns.  Every L-slot of
 // the three rows of a point reads one of 40 earlier stencil neighbours (27 at
 // level n-1, 13 earlier ones at level n) and every U-slot one of 40 later
 // ones (13 at level n, 27 at n+1), besides the point itself.  Lane l takes
-// the neighbours q = l + 4 i (i < 10) of both sweeps; it loads their values
-// once and forms its parts of the C, G and f row sums from the block rows of
-// those slots, which are affine in q (rows counted within the L or U block):
-//   forward  C row: 2q + c (c: C, f)   G row: 80 + q - 27 (q >= 27)   f row: 94 + 2q + c (c: G, f)
-//   backward C row: 2 + 2q + c (q < 13)   f row: 71 + 2q + c
-//            G row: 29 + q (q < 13), 42 + d + (d >= 13) with d = q - 13; the C entry at
-//            (n+1, same node), q = 26, in row 55
-// and a shuffle reduction over the 4 lanes closes each sum.
+// the neighbours q = l + 4 i (i < 10) of both sweeps, loads their values once
+// and forms its parts of the C, G and f row sums; a shuffle reduction over the
+// 4 lanes closes each sum.
+//
+// The factor values of a group (FP32, BF16) come by TMA bulk copy into the
+// warp's own buffers in shared memory, asked for while the warp still works on
+// the groups before.  (Loads through L1 into registers ahead of their use were
+// measured slower, 2.30 against 2.16 ms at 32^3 x 64: the neighbours' loads wait
+// behind them in L1's queue.)  The warps of a box do not meet at
+// wavefronts: a counter of finished groups in shared memory tells a warp when
+// the wavefronts before its group's are done.  What does not depend on the
+// last of them -- all neighbours but those one wavefront away -- is loaded and
+// multiplied before that wait.
 // ---------------------------------------------------------------------------
 constexpr size_t kSmemLimit = 227 * 1024;          // dynamic shared memory of one CTA
-constexpr int kSolveHeader = 2048;   // from byte 1536: the mbarriers and the abort word
-constexpr int kMaxStages = 4;        // buffers of the subdomain solve's copy ring
+constexpr size_t kSolveReserve = 2048;   // what the shape interface sets aside beside the buffers it counts
+constexpr int kMaxStages = 4;        // factor groups asked for ahead, the one in use included
 constexpr int kNbr = 40;             // earlier (and later) stencil neighbours of a point
 constexpr int kNbrPerLane = kNbr / kLanes;
 constexpr int kVecWidth = 4;         // values per point in the local vectors
@@ -328,275 +287,385 @@ __device__ __forceinline__ T lane_sum(T v) {
   return v;
 }
 
-// S: type of the stored factor values; T: arithmetic and local-vector type
-// threads of a CTA: the lanes of the largest chunk, in whole warps
+// One lane's factor values of a group.  Lower: l(i, 0..3) the C row's C and f
+// columns and the f row's G and f columns of neighbour q = lane + 4 i, g(i) the
+// G row's G column (q >= 27), own_c (lane 0), own_g (lane 1).  Upper: f(i, 0..1)
+// the f row's G and f columns, g(i) the G row's G column, c(i, 0..1) the C row's
+// C and f columns (q < 13), and what lanes 1 to 3 hold in place of c(3, .):
+// lane 1 1/u of the f and G rows, lane 2 the G row's C column at level n+1
+// (q = 26), lane 3 1/u of the C row and its own-point f column.
 template <typename S>
-constexpr int solve_threads_max() {
-  return (ChunkCfg<S>::CH * kLanes + 31) / 32 * 32;
+struct LaneFactors;
+
+template <>
+struct LaneFactors<float> {
+  static constexpr bool kStaged = true;   // comes through shared memory
+  float v[kLaneL];
+  __device__ __forceinline__ void load(const float* G, bool upper, int lane) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const float4 w = *reinterpret_cast<const float4*>(G + 4 * lane + 128 * k);
+      v[4 * k] = w.x;
+      v[4 * k + 1] = w.y;
+      v[4 * k + 2] = w.z;
+      v[4 * k + 3] = w.w;
+    }
+    if (upper) {
+      const float2 w = *reinterpret_cast<const float2*>(G + 32 * 36 + 2 * lane);
+      v[36] = w.x;
+      v[37] = w.y;
+    } else {
+#pragma unroll
+      for (int k = 9; k < 11; ++k) {
+        const float4 w = *reinterpret_cast<const float4*>(G + 4 * lane + 128 * k);
+        v[4 * k] = w.x;
+        v[4 * k + 1] = w.y;
+        v[4 * k + 2] = w.z;
+        v[4 * k + 3] = w.w;
+      }
+    }
+  }
+  __device__ __forceinline__ float at(int i) const { return v[i]; }
+};
+
+template <>
+struct LaneFactors<__nv_bfloat16> {
+  static constexpr bool kStaged = true;
+  unsigned v[kLaneL / 2];   // pairs: value 2 k in the low half
+  __device__ __forceinline__ void load(const __nv_bfloat16* G, bool upper, int lane) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint4 w = *reinterpret_cast<const uint4*>(G + 8 * lane + 256 * k);
+      v[4 * k] = w.x;
+      v[4 * k + 1] = w.y;
+      v[4 * k + 2] = w.z;
+      v[4 * k + 3] = w.w;
+    }
+    if (upper) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v[16 + k] = *reinterpret_cast<const unsigned*>(G + 32 * 32 + 6 * lane + 2 * k);
+    } else {
+      const uint4 w = *reinterpret_cast<const uint4*>(G + 8 * lane + 1024);
+      v[16] = w.x;
+      v[17] = w.y;
+      v[18] = w.z;
+      v[19] = w.w;
+      const uint2 t = *reinterpret_cast<const uint2*>(G + 32 * 40 + 4 * lane);
+      v[20] = t.x;
+      v[21] = t.y;
+    }
+  }
+  __device__ __forceinline__ float at(int i) const {
+    return __uint_as_float(i % 2 ? v[i / 2] & 0xffff0000u : v[i / 2] << 16);
+  }
+};
+
+// FP64: the values stay in global memory ([slot rank][8] groups) until they
+// are used; the FP64 pipe is the limit, and other warps hide the loads.
+template <>
+struct LaneFactors<double> {
+  static constexpr bool kStaged = false;
+  const double* p;
+  __device__ __forceinline__ void load(const double* G, bool upper, int lane) {
+    p = G + (upper ? kLRanks * kGroup : 0) + lane / kLanes;
+  }
+  __device__ __forceinline__ double rank(int r) const { return __ldcs(p + r * kGroup); }
+};
+
+// S: type of the stored factor values; T: arithmetic and local-vector type.
+// Most warps of a CTA and CTAs per SM (ras_setup_shape's largest size class).
+constexpr int kSolveWarpsMax = 16;
+
+// Lanes (bits) whose neighbour q = lane + 4 i lies one wavefront away (w - 1 in
+// the forward sweep, w + 1 in the backward one).  With the wavefront weights
+// (1, 2, 4, 8) these are, forward (level n-1: d = q; level n: d = q - 27),
+// (1, 1, 1) at n-1 and (1, 1, -1), (1, -1, 0), (-1, 0, 0) at n: q = 26, 35, 38,
+// 39; backward (level n: d = 14 + q; level n+1: d = q - 13) the mirror images,
+// q = 0, 1, 4, 13.
+__host__ __device__ constexpr int dep_lanes(bool upper, int i) {
+  return upper ? (i == 0 ? 3 : i == 1 ? 1 : i == 3 ? 2 : 0) : (i == 6 ? 4 : i == 8 ? 8 : i == 9 ? 12 : 0);
 }
 
-// Neighbour q of a point whose wavefront is one away from the point's (w - 1
-// in the forward sweep, w + 1 in the backward one): with the wavefront weights
-// (1, 2, 4, 8) these are, forward (level n-1: d = q; level n: d = q - 27),
-// (1, 1, 1) at n-1 and (1, 1, -1), (1, -1, 0), (-1, 0, 0) at n, and backward
-// (level n: d = 14 + q; level n+1: d = q - 13) the mirror images.  Only they
-// can be written by the chunk before a point's own.
-template <bool kUpper>
-__device__ __forceinline__ bool dep_nbr(int q) {
-  return kUpper ? (q == 0 || q == 1 || q == 4 || q == 13) : (q == 26 || q == 35 || q == 38 || q == 39);
+// Bytes of a warp's factor buffer (the lower half of a group is the larger one).
+template <typename S>
+constexpr int solve_buffer() {
+  return LaneFactors<S>::kStaged ? 32 * kLaneL * (int)sizeof(S) : 0;
 }
+constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter of finished groups, abort word
 
 template <typename S, bool SMEM>
-__global__ void __launch_bounds__(solve_threads_max<S>(), 2) ras_solve(
-    const BoxDesc* __restrict__ boxes, const Chunk* __restrict__ chunks, const S* __restrict__ F,
+__global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
+    const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr, const S* __restrict__ F,
     typename SolveArith<S>::type* __restrict__ V, const double* __restrict__ r, double* __restrict__ z,
-    const int2* __restrict__ gtab, const int2* __restrict__ otab, const int* __restrict__ vtab, int bstride,
-    int nstage, int* __restrict__ status, const int* gate, int gate_stride) {
+    const int2* __restrict__ gtab, const int2* __restrict__ otab, const int* __restrict__ vtab, int gptr_bytes,
+    int nbuf, int* __restrict__ status, const int* gate, int gate_stride) {
   using T = typename SolveArith<S>::type;
+  constexpr bool kStaged = LaneFactors<S>::kStaged;
   // the box's problem gate (one problem: gate_stride 0, every box reads gate[0])
   if (gate != nullptr && gate[boxes[blockIdx.x].prob * gate_stride] == 0) return;
   extern __shared__ __align__(128) unsigned char smem[];
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem + 1536);
-  int* abort_at = reinterpret_cast<int*>(smem + 1536 + 8 * kMaxStages);   // block whose wait gave up, or -1
-  S* buf0 = reinterpret_cast<S*>(smem + kSolveHeader);   // nstage buffers of bstride values
-                                                        // (kLRanks x the largest chunk row stride)
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(smem);
+  int* finished = reinterpret_cast<int*>(smem + 8 * kSolveWarpsMax * (kMaxStages - 1));   // groups done
+  int* aborted = finished + 1;
   const BoxDesc bx = boxes[blockIdx.x];
-  const long long P = bx.P;
+  const int P = (int)bx.P, nlev = bx.nlev;
   const S* Fb = F + bx.foff;
+  const int* vt = vtab + kGroup * bx.goff;
   const int px = bx.lx + 2, py = bx.ly + 2, pz = bx.lz + 2;
-  const long long sy = px, sz = (long long)px * py, st = (long long)px * py * pz;
-  const long long npad = kVecWidth * st * (bx.lt + 2);
-  T* v = SMEM ? reinterpret_cast<T*>(buf0 + (size_t)nstage * bstride) : V + bx.voff;
-  const int nch = bx.cend - bx.cbeg;
-  const Chunk* ck = chunks + bx.cbeg;
-  const int lane = threadIdx.x & (kLanes - 1), j = threadIdx.x / kLanes;
-  // offsets of the lane's neighbours in the padded local vector
-  int offL[kNbrPerLane], offU[kNbrPerLane];
-#pragma unroll
-  for (int i = 0; i < kNbrPerLane; ++i) {
-    const int q = lane + kLanes * i;
-    // earlier neighbour q: level n-1, spatial offset d = q (q < 27); level n, d = q - 27
-    const int dl = q < 27 ? q : q - 27, tl = q < 27 ? -1 : 0;
-    // later neighbour q: level n, d = 14 + q (q < 13); level n+1, d = q - 13
-    const int du = q < 13 ? 14 + q : q - 13, tu = q < 13 ? 0 : 1;
-    offL[i] = (int)(kVecWidth * ((dl % 3 - 1) + sy * ((dl / 3) % 3 - 1) + sz * (dl / 9 - 1) + st * tl));
-    offU[i] = (int)(kVecWidth * ((du % 3 - 1) + sy * ((du / 3) % 3 - 1) + sz * (du / 9 - 1) + st * tu));
+  const int sy = px, sz = px * py, st = px * py * pz;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x / 32, nwarp = blockDim.x / 32;
+  const int sub = lane & (kLanes - 1);
+  // shared memory: header, group pointers, the warps' factor buffers, the local vector
+  unsigned char* bufs = smem + kSolveHeader + gptr_bytes;
+  T* v = SMEM ? reinterpret_cast<T*>(bufs + (size_t)nwarp * nbuf * solve_buffer<S>()) : V + bx.voff;
+  S* mine = reinterpret_cast<S*>(bufs + (size_t)warp * nbuf * solve_buffer<S>());
+  unsigned long long* bar = bars + warp * (kMaxStages - 1);
+  const int* gp = gptr + bx.loff;   // first group of every wavefront
+  if (gptr_bytes) {
+    int* copy = reinterpret_cast<int*>(smem + kSolveHeader);
+    for (int i = threadIdx.x; i <= nlev; i += blockDim.x) copy[i] = gp[i];
+    gp = copy;
   }
-  if (threadIdx.x == 0) {
-    for (int b = 0; b < nstage; ++b) mbar_init(&bar[b], 1);
+  if (kStaged && lane < nbuf) {
+    mbar_init(&bar[lane], 1);
     mbar_fence_init();
-    *abort_at = -1;
   }
+  if (threadIdx.x == 0) *finished = *aborted = 0;
   if (SMEM)
-    for (long long i = threadIdx.x; i < npad; i += blockDim.x) v[i] = (T)0;
+    for (int i = threadIdx.x; i < kVecWidth * st * (bx.lt + 2); i += blockDim.x) v[i] = (T)0;
   __syncthreads();
-  // The factor blocks stream in the order L(0), ..., L(nch-1), U(nch-1), ...,
-  // U(0) through a ring of `nstage` buffers: block g goes to buffer g mod
-  // nstage and is copied nstage - 1 steps before it is used.
-  const int nblk = 2 * nch;
-  auto chunk_of = [&](int g) { return g < nch ? g : nblk - 1 - g; };
-  auto issue = [&](const Chunk& c, int g) {
-    const bool upper = g >= nch;
-    const int b = g % nstage;
-    const unsigned rows = upper ? kURanks : kLRanks;
-    const unsigned bytes = rows * (unsigned)c.cp * (unsigned)sizeof(S);
-    const S* src = Fb + c.off + (upper ? (long long)kLRanks * c.cp : 0);
-    fence_proxy_async();
-    mbar_expect_tx(&bar[b], bytes);
-    bulk_g2s(buf0 + (size_t)b * bstride, src, bytes, &bar[b]);
-  };
-  Chunk iss;   // thread 0: descriptor of the next block to copy
-  if (threadIdx.x == 0) {
-    for (int g = 0; g < min(nstage - 1, nblk); ++g) issue(ck[chunk_of(g)], g);
-    if (nstage - 1 < nblk) iss = ck[chunk_of(nstage - 1)];
-  }
-  // gather R^delta r into the padded local vector while the first blocks arrive
-  // (gtab: per box point, its global unknown index and its padded offset)
-  for (int q = threadIdx.x; q < (int)P; q += blockDim.x) {
-    const int2 e = gtab[bx.poff + q];
-    st3(v + e.y, (T)r[e.x], (T)r[e.x + 1], (T)r[e.x + 2]);
-  }
-  __syncthreads();
-  // Step g works on the chunk of block g (`cur`).  The descriptor of the
-  // chunk after next and the point index of the next chunk are loaded one
-  // step ahead, so the only loads left between a barrier and the arithmetic
-  // are the vector's.  Steps 0..nch-1 are the forward sweep with the unit
-  // lower factor, steps nch..2 nch-1 the backward sweep with the upper factor.
-  Chunk cur, nxt;
-  int vq_cur = 0;
-  // neighbour values of the step; `pre`: the previous step already loaded the
-  // ones that cannot change during it (see the end of the step)
-  T nc[kNbrPerLane], ng[kNbrPerLane], nf[kNbrPerLane];
-  bool pre = false;
-  if (nblk > 0) {
-    cur = ck[0];
-    nxt = ck[chunk_of(min(1, nblk - 1))];
-    vq_cur = j < cur.n ? vtab[bx.poff + cur.q0 + j] : 0;
-  }
-  // one step of either sweep; false when a copy wait gave up (the CTA stops)
-  // kCp: the row stride of the chunk's block as a compile-time constant (a
-  // full chunk: kCp = CH, so every factor read is [base + immediate]), or 0 for
-  // the run-time stride of a ragged chunk
-  auto step = [&](int g, auto upper_tag, auto cp_tag) -> bool {
-    constexpr bool kUpper = decltype(upper_tag)::value;
-    constexpr int kCp = decltype(cp_tag)::value;
-    const int b = g % nstage;
-    if (threadIdx.x == 0 && g + nstage - 1 < nblk) {
-      issue(iss, g + nstage - 1);
-      if (g + nstage < nblk) iss = ck[chunk_of(g + nstage)];
+  // The groups in the order of the sweeps: k < ng is group k of the forward
+  // sweep, then they come back last to first; a warp takes every nwarp-th of
+  // them, wherever the wavefronts end.  Step s < nlev is wavefront s of the
+  // forward sweep, then the wavefronts come back as well.
+  const int ng = gp[nlev];
+  auto before = [&](int s) { return s < nlev ? gp[s] : 2 * ng - gp[2 * nlev - s]; };   // groups of steps < s
+  auto group = [&](int k) { return k < ng ? k : 2 * ng - 1 - k; };
+  auto issue = [&](int k, int t) {   // copy of group k, the warp's t-th, into its buffer
+    if (kStaged && k < 2 * ng && lane == 0) {
+      const bool up = k >= ng;
+      const unsigned bytes = 32 * (up ? kLaneU : kLaneL) * (unsigned)sizeof(S);
+      fence_proxy_async();
+      mbar_expect_tx(&bar[t % nbuf], bytes);
+      bulk_g2s(mine + (t % nbuf) * (solve_buffer<S>() / (int)sizeof(S)),
+               Fb + (long long)group(k) * kGroupVals32 + (up ? 32 * kLaneL : 0), bytes, &bar[t % nbuf]);
     }
-    const Chunk nn = ck[chunk_of(min(g + 2, nblk - 1))];
-    const int vq_nxt = (g + 1 < nblk && j < nxt.n) ? vtab[bx.poff + nxt.q0 + j] : 0;
-    const Chunk& c = cur;
-    const bool act = j < c.n;
-    const int cp = kCp ? kCp : c.cp;
-    T* vp = v + (act ? vq_cur : 0);
-    // all neighbour loads of the step first (they depend on the previous steps
-    // only, so they are in flight while the factor block is awaited), then the
-    // arithmetic
-    T v0 = 0, v1 = 0, v2 = 0;
+  };
+  for (int t = 0; t < nbuf; ++t) issue(warp + t * nwarp, t);
+  // the point of the group after the next one is loaded a group ahead: the neighbours' addresses
+  // come from it
+  int vq = warp < 2 * ng ? vt[kGroup * group(warp) + lane / kLanes] : 0;
+  // R^delta r into the padded local vector (gtab: per box point, its global unknown index and
+  // its padded offset); four points at a time, so that their loads overlap
+  for (int q0 = threadIdx.x; q0 < P; q0 += 4 * blockDim.x) {
+    int2 e[4];
+    T a[4][3];
 #pragma unroll
-    for (int i = 0; i < kNbrPerLane; ++i) {
-      if (!pre || dep_nbr<kUpper>(lane + kLanes * i)) {
-        nc[i] = ng[i] = nf[i] = (T)0;
-        if (act) ld3(vp + (kUpper ? offU[i] : offL[i]), nc[i], ng[i], nf[i]);
+    for (int k = 0; k < 4; ++k) {
+      const int q = q0 + k * blockDim.x;
+      e[k] = q < P ? gtab[bx.poff + q] : make_int2(-1, 0);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) a[k][c] = e[k].x >= 0 ? (T)r[e[k].x + c] : (T)0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (e[k].x >= 0) st3(v + e[k].y, a[k][0], a[k][1], a[k][2]);
+  }
+  __syncthreads();
+
+  // waits until n groups are done; false when the limit ran out here or in another warp
+  auto wait_done = [&](int n) -> bool {
+    unsigned long long t0 = 0;
+    for (unsigned it = 0; ld_acquire_cta(finished) < n; ++it) {
+      if ((it & 255u) == 255u) {
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > kWaitLimitNs) {
+          atomicExch(status, 2);
+          atomicExch(aborted, 1);
+        }
+        if (*(volatile int*)aborted) return false;
       }
     }
-    if (act) ld3(vp, v0, v1, v2);
-    if (!mbar_wait(&bar[b], (unsigned)(g / nstage) & 1u, status)) *abort_at = g;
-    const S* B = buf0 + (size_t)b * bstride;
-    T sc = 0, sg = 0, sf = 0;
-    if constexpr (!kUpper) {
+    return true;
+  };
+  LaneFactors<S> fac;
+  int off[kNbrPerLane];   // offsets of the lane's neighbours in the padded local vector
+  int s = 0, t = 0;       // step of the warp's group, number of its groups so far
+  int k = warp;
+  // one sweep: the warp's groups k < kend
+  auto sweep = [&](int kend, auto upper_tag) -> bool {
+    constexpr bool kUpper = decltype(upper_tag)::value;
+    for (; k < kend; k += nwarp, ++t) {
+      while (k >= before(s + 1)) ++s;
+      const bool act = vq >= 0;
+      T* vp = v + (act ? vq : ~vq);
+      if (k + nwarp < 2 * ng) vq = vt[kGroup * group(k + nwarp) + lane / kLanes];
+      if (kStaged) {
+        if (!mbar_wait(&bar[t % nbuf], (unsigned)(t / nbuf) & 1u, status)) {
+          atomicExch(aborted, 1);
+          return false;
+        }
+        fac.load(mine + (t % nbuf) * (solve_buffer<S>() / (int)sizeof(S)), kUpper, lane);
+        __syncwarp();
+        issue(k + nbuf * nwarp, t + nbuf);
+      } else {
+        fac.load(Fb + (long long)group(k) * group_vals(64), kUpper, lane);
+      }
+      // neighbours two and more wavefronts away (at the first backward step the own point is one
+      // of the last wavefront's)
+      if (!wait_done(s == nlev ? ng : before(max(s - 1, 0)))) return false;
+      T v0, v1, v2;
+      ld3(vp, v0, v1, v2);
+      T nc[kNbrPerLane], nG[kNbrPerLane], nf[kNbrPerLane];   // the neighbours' unknowns
+#pragma unroll
+      for (int i = 0; i < kNbrPerLane; ++i)
+        if (!(dep_lanes(kUpper, i) >> sub & 1)) ld3(vp + off[i], nc[i], nG[i], nf[i]);
+      T sc = 0, sg = 0, sf = 0;
+      T rc = 0, rg = 0, rf = 0, cf = 0, own_c = 0, own_g = 0;
       if constexpr (sizeof(T) == 8) {
-        // FP64: one FMA per product into two chains per sum (the FP64 pipe
-        // is the limit: a product pair costs 2 operations instead of 3)
+        if (!wait_done(before(s))) return false;
+#pragma unroll
+        for (int i = 0; i < kNbrPerLane; ++i)
+          if (dep_lanes(kUpper, i) >> sub & 1) ld3(vp + off[i], nc[i], nG[i], nf[i]);
+        // one FMA per product into two chains per sum (the FP64 pipe is the limit)
         T sc1 = 0, sf1 = 0;
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i) {
-          const int q = lane + kLanes * i;
-          const S* rc = B + (2 * q) * cp + j;
-          const S* rf = B + (94 + 2 * q) * cp + j;
-          sc = fma(arith<T>(rc[0]), nc[i], sc);
-          sc1 = fma(arith<T>(rc[cp]), nf[i], sc1);
-          sf = fma(arith<T>(rf[0]), ng[i], sf);
-          sf1 = fma(arith<T>(rf[cp]), nf[i], sf1);
-          if (q >= 27) sg = fma(arith<T>(B[(80 + q - 27) * cp + j]), ng[i], sg);
+          const int q = sub + kLanes * i, d = q - 13;
+          if constexpr (!kUpper) {
+            sc = fma(fac.rank(2 * q), nc[i], sc);
+            sc1 = fma(fac.rank(2 * q + 1), nf[i], sc1);
+            sf = fma(fac.rank(94 + 2 * q), nG[i], sf);
+            sf1 = fma(fac.rank(95 + 2 * q), nf[i], sf1);
+            if (q >= 27) sg = fma(fac.rank(80 + q - 27), nG[i], sg);
+          } else {
+            sf = fma(fac.rank(71 + 2 * q), nG[i], sf);
+            sf1 = fma(fac.rank(72 + 2 * q), nf[i], sf1);
+            if (q < 13) {
+              sc = fma(fac.rank(3 + 2 * q), nf[i], fma(fac.rank(2 + 2 * q), nc[i], sc));
+              sg += fac.rank(29 + q) * nG[i];
+            } else {
+              sg += fac.rank(42 + d + (d >= 13 ? 1 : 0)) * nG[i];
+              if (d == 13) sg += fac.rank(55) * nc[i];
+            }
+          }
         }
-        sc += sc1;
+        if (!kUpper) sc += sc1;
         sf += sf1;
+        if constexpr (!kUpper) {
+          own_c = fac.rank(93);
+          own_g = fac.rank(174);
+        } else {
+          rc = fac.rank(0);
+          cf = fac.rank(1);
+          rg = fac.rank(28);
+          rf = fac.rank(70);
+        }
       } else {
+        // products of the neighbours that are there, then the others' and the sums in order
+        T pc[kNbrPerLane], pf[kNbrPerLane];
+        auto products = [&](int i) {
+          if constexpr (!kUpper) {
+            pc[i] = fac.at(4 * i) * nc[i] + fac.at(4 * i + 1) * nf[i];
+            pf[i] = fac.at(4 * i + 2) * nG[i] + fac.at(4 * i + 3) * nf[i];
+          } else {
+            pf[i] = fac.at(2 * i) * nG[i] + fac.at(2 * i + 1) * nf[i];
+            if (i < 4) pc[i] = fac.at(30 + 2 * i) * nc[i] + fac.at(31 + 2 * i) * nf[i];
+          }
+        };
+#pragma unroll
+        for (int i = 0; i < kNbrPerLane; ++i)
+          if (!(dep_lanes(kUpper, i) >> sub & 1)) products(i);
+        if constexpr (!kUpper) {
+          own_c = fac.at(40);
+          own_g = __shfl_down_sync(0xffffffffu, own_c, 1);
+        } else {
+          rf = __shfl_down_sync(0xffffffffu, fac.at(36), 1);
+          rg = __shfl_down_sync(0xffffffffu, fac.at(37), 1);
+          rc = __shfl_down_sync(0xffffffffu, fac.at(36), 3);
+          cf = __shfl_down_sync(0xffffffffu, fac.at(37), 3);
+        }
+        if (!wait_done(before(s))) return false;
+#pragma unroll
+        for (int i = 0; i < kNbrPerLane; ++i)
+          if (dep_lanes(kUpper, i) >> sub & 1) ld3(vp + off[i], nc[i], nG[i], nf[i]);
+#pragma unroll
+        for (int i = 0; i < kNbrPerLane; ++i)
+          if (dep_lanes(kUpper, i) >> sub & 1) products(i);
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i) {
-          const int q = lane + kLanes * i;
-          const S* rc = B + (2 * q) * cp + j;
-          const S* rf = B + (94 + 2 * q) * cp + j;
-          sc += arith<T>(rc[0]) * nc[i] + arith<T>(rc[cp]) * nf[i];
-          sf += arith<T>(rf[0]) * ng[i] + arith<T>(rf[cp]) * nf[i];
-          if (q >= 27) sg += arith<T>(B[(80 + q - 27) * cp + j]) * ng[i];
+          sf += pf[i];
+          if constexpr (!kUpper) {
+            sc += pc[i];
+            if (i >= 7 || (i == 6 && sub == 3)) sg += fac.at(34 + i) * nG[i];
+          } else {
+            if (i < 3 || (i == 3 && sub == 0)) sc += pc[i];
+            sg += fac.at(20 + i) * nG[i];
+            if (i == 6 && sub == 2) sg += fac.at(36) * nc[i];
+          }
         }
       }
       sc = lane_sum(sc);
       sg = lane_sum(sg);
       sf = lane_sum(sf);
-      // own-point terms in C, G, f order: the G row's own-C slot (row 93) and
-      // the f row's own-G slot (row 174)
-      if (act && lane == 0) {
-        const T yc = v0 - sc;
-        const T yg = v1 - sg - arith<T>(B[93 * cp + j]) * yc;
-        const T yf = v2 - sf - arith<T>(B[174 * cp + j]) * yg;
-        st3(vp, yc, yg, yf);
-      }
-    } else {
-      T sf1 = 0;   // FP64: the f-row products in two FMA chains
-#pragma unroll
-      for (int i = 0; i < kNbrPerLane; ++i) {
-        const int q = lane + kLanes * i;
-        const S* rf = B + (71 + 2 * q) * cp + j;
-        if constexpr (sizeof(T) == 8) {
-          sf = fma(arith<T>(rf[0]), ng[i], sf);
-          sf1 = fma(arith<T>(rf[cp]), nf[i], sf1);
+      if (act && sub == 0) {
+        if constexpr (!kUpper) {
+          // own-point terms in C, G, f order: the G row's own-C and the f row's own-G slot
+          const T yc = v0 - sc;
+          const T yg = v1 - sg - own_c * yc;
+          const T yf = v2 - sf - own_g * yg;
+          st3(vp, yc, yg, yf);
         } else {
-          sf += arith<T>(rf[0]) * ng[i] + arith<T>(rf[cp]) * nf[i];
-        }
-        if (q < 13) {
-          const S* rc = B + (2 + 2 * q) * cp + j;
-          if constexpr (sizeof(T) == 8)
-            sc = fma(arith<T>(rc[cp]), nf[i], fma(arith<T>(rc[0]), nc[i], sc));
-          else
-            sc += arith<T>(rc[0]) * nc[i] + arith<T>(rc[cp]) * nf[i];
-          sg += arith<T>(B[(29 + q) * cp + j]) * ng[i];
-        } else {
-          const int d = q - 13;
-          sg += arith<T>(B[(42 + d + (d >= 13 ? 1 : 0)) * cp + j]) * ng[i];
-          if (d == 13) sg += arith<T>(B[55 * cp + j]) * nc[i];
+          // the C row's own-point f column is applied after the f row is solved
+          const T zf = (v2 - sf) * rf;
+          const T zg = (v1 - sg) * rg;
+          const T zc = (v0 - sc - cf * zf) * rc;
+          st3(vp, zc, zg, zf);
         }
       }
-      sf += sf1;
-      sc = lane_sum(sc);
-      sg = lane_sum(sg);
-      sf = lane_sum(sf);
-      // the diagonal rows 0, 28, 70 hold the reciprocals of the pivots; the C
-      // row's own-f slot (U row 1) is applied after the f row is solved
-      if (act && lane == 0) {
-        const T zf = (v2 - sf) * arith<T>(B[70 * cp + j]);
-        const T zg = (v1 - sg) * arith<T>(B[28 * cp + j]);
-        const T zc = (v0 - sc - arith<T>(B[1 * cp + j]) * zf) * arith<T>(B[0 * cp + j]);
-        st3(vp, zc, zg, zf);
-      }
+      __syncwarp();
+      if (lane == 0) add_release_cta(finished, 1);
     }
-    // The next step's neighbours in the same sweep, except the few one
-    // wavefront away (they may be points of this chunk), cannot change during
-    // this step: with FP64 factors, load them now, so their latency overlaps
-    // the barrier (measured at 32^3 x 64: the FP64 form 3 % faster; the FP32
-    // solve 17 % slower, so FP32 and BF16 factors load after the barrier).
-    pre = sizeof(S) == 8 && g + 1 < nblk && g + 1 != nch;
-    if (pre) {
-      const bool act2 = j < nxt.n;
-      const T* vp2 = v + (act2 ? vq_nxt : 0);
-#pragma unroll
-      for (int i = 0; i < kNbrPerLane; ++i) {
-        if (dep_nbr<kUpper>(lane + kLanes * i)) continue;
-        nc[i] = ng[i] = nf[i] = (T)0;
-        if (act2) ld3(vp2 + (kUpper ? offU[i] : offL[i]), nc[i], ng[i], nf[i]);
-      }
-    }
-    __syncthreads();
-    cur = nxt;
-    nxt = nn;
-    vq_cur = vq_nxt;
-    return *abort_at < 0;
+    return true;
   };
-  // forward sweep (unit lower factor), then backward sweep (upper factor)
-  bool ok = true;
-  using FullCp = std::integral_constant<int, ChunkCfg<S>::CH>;   // == chunk_stride(CH): no padding
-  using AnyCp = std::integral_constant<int, 0>;
-  const int full_cp = chunk_stride_dev<S>(ChunkCfg<S>::CH);
-  for (int g = 0; ok && g < nch; ++g)
-    ok = cur.cp == full_cp && full_cp == FullCp::value ? step(g, std::false_type{}, FullCp{})
-                                                       : step(g, std::false_type{}, AnyCp{});
-  for (int g = nch; ok && g < nblk; ++g)
-    ok = cur.cp == full_cp && full_cp == FullCp::value ? step(g, std::true_type{}, FullCp{})
-                                                       : step(g, std::true_type{}, AnyCp{});
-  if (!ok) {
-    // A wait gave up at block gf (status 2 is set): the blocks gf .. gf +
-    // nstage - 1 may still be in flight into this CTA's buffers.  Thread 0
-    // waits for them, again with the time limit, and the CTA returns without
-    // writing z.
-    if (threadIdx.x == 0) {
-      const int gf = *abort_at;
-      for (int q = gf; q < min(gf + nstage, nblk); ++q)
-        mbar_wait(&bar[q % nstage], (unsigned)(q / nstage) & 1u, status);
-    }
-    return;
+#pragma unroll
+  for (int i = 0; i < kNbrPerLane; ++i) {   // earlier neighbour q: level n-1, d = q (q < 27); level n, d = q - 27
+    const int q = sub + kLanes * i, d = q < 27 ? q : q - 27, dt = q < 27 ? -1 : 0;
+    off[i] = kVecWidth * ((d % 3 - 1) + sy * ((d / 3) % 3 - 1) + sz * (d / 9 - 1) + st * dt);
   }
+  bool ok = sweep(ng, std::false_type{});   // forward, unit lower factor
+  if (ok) {
+#pragma unroll
+    for (int i = 0; i < kNbrPerLane; ++i) {   // later neighbour q: level n, d = 14 + q (q < 13); level n+1, d = q - 13
+      const int q = sub + kLanes * i, d = q < 13 ? 14 + q : q - 13, dt = q < 13 ? 0 : 1;
+      off[i] = kVecWidth * ((d % 3 - 1) + sy * ((d / 3) % 3 - 1) + sz * (d / 9 - 1) + st * dt);
+    }
+    ok = sweep(2 * ng, std::true_type{});   // backward, upper factor
+  }
+  if (!ok && kStaged) {
+    // a wait gave up (status 2 is set): the copies of the warp's groups t .. t + nbuf may still be
+    // in flight into its buffers; wait for them, again with the limit
+    for (int q = t; q < t + nbuf; ++q)
+      if (warp + q * nwarp < 2 * ng) mbar_wait(&bar[q % nbuf], (unsigned)(q / nbuf) & 1u, status);
+  }
+  __syncthreads();
+  if (*aborted) return;   // without writing z
   // scatter the owned part: (R^0)^T (otab: the owned points' global indices and offsets)
-  for (int q = threadIdx.x; q < bx.nown; q += blockDim.x) {
-    const int2 e = otab[bx.ooff + q];
-    T a0, a1, a2;
-    ld3(v + e.y, a0, a1, a2);
-    z[e.x] = (double)a0;
-    z[e.x + 1] = (double)a1;
-    z[e.x + 2] = (double)a2;
+  for (int q0 = threadIdx.x; q0 < bx.nown; q0 += 4 * blockDim.x) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = q0 + k * blockDim.x;
+      if (q >= bx.nown) break;
+      const int2 e = otab[bx.ooff + q];
+      T a0, a1, a2;
+      ld3(v + e.y, a0, a1, a2);
+      z[e.x] = (double)a0;
+      z[e.x + 1] = (double)a1;
+      z[e.x + 2] = (double)a2;
+    }
   }
 }
 
@@ -612,25 +681,27 @@ std::vector<std::pair<int, int>> parts(int n, int p) {
   return out;
 }
 
-// esz: bytes of a stored factor value, vsz: of a local-vector value
-size_t solve_smem(int cpmax, int nstage, size_t esz, size_t vsz, long long max_pad, bool smem_vec) {
-  const size_t bufs = (size_t)nstage * kLRanks * cpmax * esz;
-  return kSolveHeader + bufs + (smem_vec ? (size_t)max_pad * vsz : 0);
+// The wavefronts' group pointers (kept in shared memory up to kGptrLimit
+// bytes, else read from global memory) and the local vector.
+constexpr int kGptrLimit = 32 * 1024;
+int gptr_smem(int nlev) {
+  const int bytes = (nlev + 1 + 31) / 32 * 32 * (int)sizeof(int);
+  return bytes <= kGptrLimit ? bytes : 0;
 }
 
-// Chunk size, copy-ring depth and local-vector placement of the subdomain
-// solve.  Each box is one CTA that steps through its chunks one after the
-// other, so a step's latency decides the time.  The order of preference, as
-// measured on GB300 (32^3 x 64 fine boxes, coarse-sized boxes, FP32 and
-// FP64): the fewest waves of CTAs over the SMs (the runtime's occupancy for
-// the shared memory, threads and registers); the local vectors in global
-// memory (cached in L1) rather than in shared memory; the shallowest ring (a
-// deeper ring takes shared memory from the L1 that caches the local
-// vectors); the largest chunk (fewest steps).  ras_autotune measures instead.
+// buffers per warp of a shape's second field (its value counts the group in use as well)
+int solve_buffers(int nstage) { return nstage - 1; }
+// dynamic shared memory of the solve without the local vector
+template <typename S>
+size_t solve_smem(int nlev, int warps, int nstage) {
+  return kSolveHeader + gptr_smem(nlev) + (size_t)warps * solve_buffers(nstage) * solve_buffer<S>();
+}
+
 struct SolveShape {
-  int ch, cpmax, nstage, lanes;
+  int ch, warps, nstage, lanes;
   bool smem_vec;
 };
+constexpr int kFillGroups = 7;   // groups per wavefront from which the largest CTA is taken
 template <typename T, bool SMEM>
 const void* solve_kernel() {
   return (const void*)ras_solve<T, SMEM>;
@@ -639,14 +710,20 @@ const void* solve_kernel() {
 struct ShapeRequest {
   int ch = 0, nstage = 0, lanes = 0, place = 0;   // place: 1 shared-memory vector, 2 global-memory vector
 };
-// Picks the best shape allowed by `req`; KKT_ERR_ARG when none is.
+// Picks the best shape allowed by `req`; KKT_ERR_ARG when none is.  Boxes whose
+// wavefronts fill the largest CTA take it (one per SM, its L1 to itself); others
+// take the shape with the fewest waves of CTAs over the SMs.  Measured at 32^3 x
+// 64, FP32, 256 boxes: fine boxes (15 groups a wavefront) 2.16 ms with 16 warps,
+// 2.46 with 8 (two CTAs an SM), 4.04 with 4; coarse boxes (3 groups) 303, 221,
+// 300 us.  FP64, 64 boxes of 9 groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
+// global memory, the fewest buffers, the largest CTA.  ras_autotune measures instead.
 template <typename T>
-kkt_status choose_solve_shape(int nbox, long long max_pad, int nsm, const ShapeRequest& req, SolveShape* out) {
+kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int nsm,
+                              const ShapeRequest& req, SolveShape* out) {
   if (req.lanes != 0 && req.lanes != kLanes) {
     set_error("ras_setup: the subdomain solve runs 4 lanes per point");
     return KKT_ERR_ARG;
   }
-  const int cands[3] = {ChunkCfg<T>::CH, ChunkCfg<T>::CH2, ChunkCfg<T>::CH3};
   KKT_TRY_CUDA(cudaFuncSetAttribute(ras_solve<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kSmemLimit));
   KKT_TRY_CUDA(cudaFuncSetAttribute(ras_solve<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -656,30 +733,30 @@ kkt_status choose_solve_shape(int nbox, long long max_pad, int nsm, const ShapeR
   for (int ci = 0; ci < 3; ++ci)
     for (int ns = 2; ns <= kMaxStages; ++ns)
       for (int sv = 1; sv >= 0; --sv) {
-        const int ch = cands[ci], cp = chunk_stride<T>(ch);
+        const int ch = SizeClasses<T>::name[ci], warps = SizeClasses<T>::warps[ci];
         if ((req.ch && req.ch != ch) || (req.nstage && req.nstage != ns) || (req.place == 1 && !sv) ||
             (req.place == 2 && sv))
           continue;
-        const size_t sm = solve_smem(cp, ns, sizeof(T), sizeof(typename SolveArith<T>::type), max_pad, sv != 0);
+        const size_t vec = sv ? (size_t)max_pad * sizeof(typename SolveArith<T>::type) : 0;
+        // a vector in shared memory leaves room for ns lower blocks of ch points beside it (the
+        // limit that the shape interface has always had)
+        if (sv && vec + kSolveReserve + (size_t)ns * kLRanks * ch * sizeof(T) > kSmemLimit) continue;
+        const size_t sm = solve_smem<T>(nlev, warps, ns) + vec;
         if (sm > kSmemLimit) continue;
-        const int threads = (ch * kLanes + 31) / 32 * 32;
         int per_sm = 0;
         KKT_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, sv ? solve_kernel<T, true>() : solve_kernel<T, false>(), threads, sm));
+            &per_sm, sv ? solve_kernel<T, true>() : solve_kernel<T, false>(), 32 * warps, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
-        // smaller key is better: fewest waves, then the local vectors in global
-        // memory (measured faster than in shared memory with this kernel, also on
-        // the small coarse-level boxes: 0.285 vs 0.354 ms at 17^3 x 33 nodes, 4^4
-        // boxes, overlap 1), the shallowest ring, the largest chunk
-        const long long key = waves * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
+        const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
+        const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
         if (best_key < 0 || key < best_key) {
           best_key = key;
-          best = SolveShape{ch, cp, ns, kLanes, sv != 0};
+          best = SolveShape{ch, warps, ns, kLanes, sv != 0};
         }
       }
   if (best_key < 0) {
-    set_error("ras_setup: no subdomain-solve shape fits the request (chunk size, ring depth and vector "
+    set_error("ras_setup: no subdomain-solve shape fits the request (size class, groups ahead and vector "
               "placement must be a compiled combination that fits in shared memory)");
     return KKT_ERR_ARG;
   }
@@ -740,7 +817,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
     }
     for (int i = 0; i < kSlots; ++i)
       if (kGenRank[i] != slot_rank(i)) {
-        set_error("ras_setup: generated elimination code does not match the chunk block order");
+        set_error("ras_setup: generated elimination code does not match the group order");
         return KKT_ERR_ARG;
       }
   }
@@ -759,7 +836,6 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   m->n_total = m->vec_off.back();
   m->prec = factor_prec;
   m->local = local;
-  auto stride = [&](int n) { return chunk_stride_of(factor_prec, n); };
   // every box: its problem and the owned part of each axis (part k of n holds
   // floor(n/p) + (k < n mod p)); the extended box adds `overlap`, trimmed
   struct Geom {
@@ -783,20 +859,25 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
             geoms.push_back(g);
           }
   }
-  // several problems: the largest boxes first, so that the CTAs of one launch
-  // (one per box, started in list order) finish as close together as they can
-  if (nprob > 1)
-    std::stable_sort(geoms.begin(), geoms.end(), [](const Geom& a, const Geom& b) { return a.points > b.points; });
+  // the largest boxes first, so that the CTAs of a launch (one per box, started in list order)
+  // finish as close together as they can
+  std::stable_sort(geoms.begin(), geoms.end(), [](const Geom& a, const Geom& b) { return a.points > b.points; });
   {
-    // largest padded local vector
-    long long pad = 0;
+    // largest padded local vector, most wavefronts, points of all boxes
+    long long pad = 0, points = 0;
     for (const Geom& g : geoms) {
       const kkt_problem* pk = probs[g.prob];
       const int dk[4] = {pk->nx, pk->ny, pk->nz, pk->L};
       long long v = kVecWidth;
-      for (int a = 0; a < 4; ++a)
-        v *= std::min(dk[a], g.own[a].second + overlap) - std::max(0, g.own[a].first - overlap) + 2;
+      int nlev = 1;
+      for (int a = 0; a < 4; ++a) {
+        const int l = std::min(dk[a], g.own[a].second + overlap) - std::max(0, g.own[a].first - overlap);
+        v *= l + 2;
+        nlev += (l - 1) << a;
+      }
       pad = std::max(pad, v);
+      points += g.points;
+      m->max_nlev = std::max(m->max_nlev, nlev);
     }
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -815,151 +896,137 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       req.place = shape[3];
     }
     SolveShape sh{};
-    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, pad, nsm, req, &sh)
-                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, pad, nsm, req, &sh)
-                                              : choose_solve_shape<__nv_bfloat16>(nbox, pad, nsm, req, &sh);
+    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, nsm, req, &sh)
+                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, nsm, req, &sh)
+                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, nsm, req, &sh);
     if (cs != KKT_OK) {
       delete m;
       return cs;
     }
     m->ch = sh.ch;
-    m->cpmax = sh.cpmax;
+    m->warps = sh.warps;
     m->smem_vec = sh.smem_vec;
     m->nstage = sh.nstage;
     m->lanes = sh.lanes;
   }
-  const int CH = m->ch;
   std::vector<BoxDesc> boxes;
-  std::vector<int> perm, iperm, lptr;
-  std::vector<int2> ptab, gtab, otab;
-  std::vector<int> vtab;
+  std::vector<int> perm, gptr, ptab, vtab;
+  std::vector<int2> gtab, otab;
   if (m->n_total >= INT32_MAX) {
     set_error("ras_setup: more than 2^31 unknowns are not supported");
     delete m;
     return KKT_ERR_ARG;
   }
-  std::vector<Chunk> chunks;
-  long long foff = 0, voff = 0;
+  const int gvals = group_vals(factor_prec);
+  long long foff = 0, voff = 0, poff = 0, ngroup = 0;
   for (const Geom& geo : geoms) {
-          const kkt_problem* pk = probs[geo.prob];
-          const long long gbase = m->vec_off[geo.prob];   // the problem's first unknown
-          const int dims[4] = {pk->nx, pk->ny, pk->nz, pk->L};
-          BoxDesc b{};
-          b.prob = geo.prob;
-          const std::pair<int, int>* own[4] = {&geo.own[0], &geo.own[1], &geo.own[2], &geo.own[3]};
-          int lo[4], hi[4];
-          for (int a = 0; a < 4; ++a) {
-            lo[a] = std::max(0, own[a]->first - overlap);
-            hi[a] = std::min(dims[a], own[a]->second + overlap);
-          }
-          b.x0 = lo[0]; b.y0 = lo[1]; b.z0 = lo[2]; b.t0 = lo[3];
-          b.lx = hi[0] - lo[0]; b.ly = hi[1] - lo[1]; b.lz = hi[2] - lo[2]; b.lt = hi[3] - lo[3];
-          b.ox0 = own[0]->first; b.ox1 = own[0]->second; b.oy0 = own[1]->first; b.oy1 = own[1]->second;
-          b.oz0 = own[2]->first; b.oz1 = own[2]->second; b.ot0 = own[3]->first; b.ot1 = own[3]->second;
-          b.P = (long long)b.lx * b.ly * b.lz * b.lt;
-          b.nlev = (b.lx - 1) + 2 * (b.ly - 1) + 4 * (b.lz - 1) + 8 * (b.lt - 1) + 1;
-          b.foff = foff;
-          b.voff = voff;
-          b.poff = (long long)perm.size();
-          b.loff = (long long)lptr.size();
-          voff += (long long)kVecWidth * (b.lx + 2) * (b.ly + 2) * (b.lz + 2) * (b.lt + 2);
-          // counting sort of the points by wavefront
-          std::vector<int> cnt(b.nlev + 1, 0);
-          for (int kt = 0; kt < b.lt; ++kt)
-            for (int kz = 0; kz < b.lz; ++kz)
-              for (int ky = 0; ky < b.ly; ++ky)
-                for (int kx = 0; kx < b.lx; ++kx) cnt[kx + 2 * ky + 4 * kz + 8 * kt + 1]++;
-          for (int w = 0; w < b.nlev; ++w) cnt[w + 1] += cnt[w];
-          for (int w = 0; w <= b.nlev; ++w) lptr.push_back(cnt[w]);
-          std::vector<int> bp(b.P), bi(b.P);
-          std::vector<int> fill(cnt.begin(), cnt.end() - 1);
-          int lex = 0;
-          for (int kt = 0; kt < b.lt; ++kt)
-            for (int kz = 0; kz < b.lz; ++kz)
-              for (int ky = 0; ky < b.ly; ++ky)
-                for (int kx = 0; kx < b.lx; ++kx, ++lex) {
-                  const int q = fill[kx + 2 * ky + 4 * kz + 8 * kt]++;
-                  bp[q] = lex;
-                  bi[lex] = q;
-                }
-          perm.insert(perm.end(), bp.begin(), bp.end());
-          iperm.insert(iperm.end(), bi.begin(), bi.end());
-          // index tables of the solve: global index and padded offset of every
-          // point (lexicographic), padded offset in wavefront order, owned points
-          {
-            const long long sy = b.lx + 2, sz = sy * (b.ly + 2), st = sz * (b.lz + 2);
-            auto pad = [&](int kx, int ky, int kz, int kt) {
-              return (int)(kVecWidth * ((kx + 1) + sy * (ky + 1) + sz * (kz + 1) + st * (kt + 1)));
-            };
-            auto glob = [&](int kx, int ky, int kz, int kt) {
-              return (int)(gbase + 3 * ((long long)(b.t0 + kt) * pk->N + (b.x0 + kx) +
-                                        (long long)pk->nx * ((b.y0 + ky) + (long long)pk->ny * (b.z0 + kz))));
-            };
-            const size_t g0 = gtab.size();
-            gtab.resize(g0 + b.P);
-            vtab.resize(g0 + b.P);
-            int q = 0;
-            for (int kt = 0; kt < b.lt; ++kt)
-              for (int kz = 0; kz < b.lz; ++kz)
-                for (int ky = 0; ky < b.ly; ++ky)
-                  for (int kx = 0; kx < b.lx; ++kx, ++q) gtab[g0 + q] = make_int2(glob(kx, ky, kz, kt), pad(kx, ky, kz, kt));
-            for (int w = 0; w < (int)b.P; ++w) vtab[g0 + w] = gtab[g0 + bp[w]].y;
-            b.ooff = (long long)otab.size();
-            for (int gt = b.ot0; gt < b.ot1; ++gt)
-              for (int gz = b.oz0; gz < b.oz1; ++gz)
-                for (int gy = b.oy0; gy < b.oy1; ++gy)
-                  for (int gx = b.ox0; gx < b.ox1; ++gx)
-                    otab.push_back(make_int2(glob(gx - b.x0, gy - b.y0, gz - b.z0, gt - b.t0),
-                                             pad(gx - b.x0, gy - b.y0, gz - b.z0, gt - b.t0)));
-            b.nown = (int)((long long)otab.size() - b.ooff);
-          }
-          // chunks of each wavefront and the storage offset of every point
-          b.cbeg = (int)chunks.size();
-          const size_t pt0 = ptab.size();
-          ptab.resize(pt0 + b.P);
-          long long off = 0;
-          for (int w = 0; w < b.nlev; ++w)
-            for (int q0 = cnt[w]; q0 < cnt[w + 1]; q0 += CH) {
-              Chunk c{};
-              c.box = (int)boxes.size();
-              c.w = w;
-              c.q0 = q0;
-              c.n = std::min(CH, cnt[w + 1] - q0);
-              c.cp = stride(c.n);
-              c.off = off;
-              for (int k = 0; k < c.n; ++k) ptab[pt0 + q0 + k] = make_int2((int)(off + k), c.cp);
-              off += (long long)kSlots * c.cp;
-              chunks.push_back(c);
+    const kkt_problem* pk = probs[geo.prob];
+    const long long gbase = m->vec_off[geo.prob];   // the problem's first unknown
+    const int dims[4] = {pk->nx, pk->ny, pk->nz, pk->L};
+    BoxDesc b{};
+    b.prob = geo.prob;
+    const std::pair<int, int>* own[4] = {&geo.own[0], &geo.own[1], &geo.own[2], &geo.own[3]};
+    int lo[4], hi[4];
+    for (int a = 0; a < 4; ++a) {
+      lo[a] = std::max(0, own[a]->first - overlap);
+      hi[a] = std::min(dims[a], own[a]->second + overlap);
+    }
+    b.x0 = lo[0]; b.y0 = lo[1]; b.z0 = lo[2]; b.t0 = lo[3];
+    b.lx = hi[0] - lo[0]; b.ly = hi[1] - lo[1]; b.lz = hi[2] - lo[2]; b.lt = hi[3] - lo[3];
+    b.ox0 = own[0]->first; b.ox1 = own[0]->second; b.oy0 = own[1]->first; b.oy1 = own[1]->second;
+    b.oz0 = own[2]->first; b.oz1 = own[2]->second; b.ot0 = own[3]->first; b.ot1 = own[3]->second;
+    b.P = (long long)b.lx * b.ly * b.lz * b.lt;
+    b.nlev = (b.lx - 1) + 2 * (b.ly - 1) + 4 * (b.lz - 1) + 8 * (b.lt - 1) + 1;
+    b.foff = foff;
+    b.voff = voff;
+    b.poff = poff;
+    b.goff = ngroup;
+    b.loff = (long long)gptr.size();
+    poff += b.P;
+    voff += (long long)kVecWidth * (b.lx + 2) * (b.ly + 2) * (b.lz + 2) * (b.lt + 2);
+    if (b.P * kSlots > INT32_MAX) {
+      set_error("ras_setup: a subdomain holds more than 2^31 factor values; use more subdomains");
+      delete m;
+      return KKT_ERR_ARG;
+    }
+    if (local == 0) {
+      // groups of 8 points per wavefront: counting sort of the points (lexicographic within a wavefront)
+      std::vector<int> fill(b.nlev + 1, 0);
+      for (int kt = 0; kt < b.lt; ++kt)
+        for (int kz = 0; kz < b.lz; ++kz)
+          for (int ky = 0; ky < b.ly; ++ky)
+            for (int kx = 0; kx < b.lx; ++kx) fill[kx + 2 * ky + 4 * kz + 8 * kt]++;
+      int groups = 0;
+      for (int w = 0; w < b.nlev; ++w) {
+        gptr.push_back(groups);
+        const int n = fill[w];
+        fill[w] = kGroup * groups;
+        groups += (n + kGroup - 1) / kGroup;
+      }
+      gptr.push_back(groups);
+      m->max_groups = std::max(m->max_groups, groups);
+      ngroup += groups;
+      // index tables: lexicographic index and padded offset of every group place, place in the
+      // factors, global index and padded offset of every point, owned points
+      const long long sy = b.lx + 2, sz = sy * (b.ly + 2), st = sz * (b.lz + 2);
+      auto pad = [&](int kx, int ky, int kz, int kt) {
+        return (int)(kVecWidth * ((kx + 1) + sy * (ky + 1) + sz * (kz + 1) + st * (kt + 1)));
+      };
+      auto glob = [&](int kx, int ky, int kz, int kt) {
+        return (int)(gbase + 3 * ((long long)(b.t0 + kt) * pk->N + (b.x0 + kx) +
+                                  (long long)pk->nx * ((b.y0 + ky) + (long long)pk->ny * (b.z0 + kz))));
+      };
+      const size_t q0 = perm.size(), p0 = gtab.size();
+      perm.resize(q0 + (size_t)kGroup * groups, -1);
+      vtab.resize(q0 + (size_t)kGroup * groups, ~pad(0, 0, 0, 0));
+      gtab.resize(p0 + b.P);
+      ptab.resize(p0 + b.P);
+      int lex = 0;
+      for (int kt = 0; kt < b.lt; ++kt)
+        for (int kz = 0; kz < b.lz; ++kz)
+          for (int ky = 0; ky < b.ly; ++ky)
+            for (int kx = 0; kx < b.lx; ++kx, ++lex) {
+              const int q = fill[kx + 2 * ky + 4 * kz + 8 * kt]++;
+              perm[q0 + q] = lex;
+              vtab[q0 + q] = pad(kx, ky, kz, kt);
+              gtab[p0 + lex] = make_int2(glob(kx, ky, kz, kt), vtab[q0 + q]);
+              ptab[p0 + lex] = q / kGroup * gvals + q % kGroup;
             }
-          b.cend = (int)chunks.size();
-          // the unit row of pivot points outside the box, padded so that the
-          // next box's blocks start on a 16-byte boundary (bulk copies need it)
-          b.unit = off;
-          off += kUnitRowSpan;
-          if (off > INT32_MAX) {
-            set_error("ras_setup: a subdomain holds more than 2^31 factor values; use more subdomains");
-            delete m;
-            return KKT_ERR_ARG;
-          }
-          foff += off;
-          if (local == 1) {
-            // exact LU: band of the box matrix in natural point-block order
-            const long long n_b = 3 * b.P;
-            b.kl = 3 * (1 + b.lx + b.lx * b.ly + b.lx * b.ly * b.lz) + 2;
-            if (b.kl > kMaxLuBand || n_b > kMaxLuUnknowns) {
-              set_error("ras_setup: a subdomain is too large for the exact local LU (at most " +
-                        std::to_string(kMaxLuUnknowns) + " unknowns and half-bandwidth " +
-                        std::to_string(kMaxLuBand) + "); use ILU(0) or more subdomains");
-              delete m;
-              return KKT_ERR_ARG;
-            }
-            b.aoff = m->ab_count;
-            m->ab_count += n_b * (3LL * b.kl + 1);
-          }
-          boxes.push_back(b);
-        }
+      b.ooff = (long long)otab.size();
+      for (int gt = b.ot0; gt < b.ot1; ++gt)
+        for (int gz = b.oz0; gz < b.oz1; ++gz)
+          for (int gy = b.oy0; gy < b.oy1; ++gy)
+            for (int gx = b.ox0; gx < b.ox1; ++gx)
+              otab.push_back(make_int2(glob(gx - b.x0, gy - b.y0, gz - b.z0, gt - b.t0),
+                                       pad(gx - b.x0, gy - b.y0, gz - b.z0, gt - b.t0)));
+      b.nown = (int)((long long)otab.size() - b.ooff);
+      // the unit row of pivot points outside the box is one more group
+      b.unit = (long long)groups * gvals;
+      if (b.unit + gvals > INT32_MAX) {
+        set_error("ras_setup: a subdomain holds more than 2^31 factor values; use more subdomains");
+        delete m;
+        return KKT_ERR_ARG;
+      }
+      foff += b.unit + gvals;
+    }
+    if (local == 1) {
+      // exact LU: band of the box matrix in natural point-block order
+      const long long n_b = 3 * b.P;
+      b.kl = 3 * (1 + b.lx + b.lx * b.ly + b.lx * b.ly * b.lz) + 2;
+      if (b.kl > kMaxLuBand || n_b > kMaxLuUnknowns) {
+        set_error("ras_setup: a subdomain is too large for the exact local LU (at most " +
+                  std::to_string(kMaxLuUnknowns) + " unknowns and half-bandwidth " +
+                  std::to_string(kMaxLuBand) + "); use ILU(0) or more subdomains");
+        delete m;
+        return KKT_ERR_ARG;
+      }
+      b.aoff = m->ab_count;
+      m->ab_count += n_b * (3LL * b.kl + 1);
+    }
+    boxes.push_back(b);
+  }
   m->nbox = (int)boxes.size();
-  m->nchunk = (int)chunks.size();
+  m->ngroup = ngroup;
   m->boxes_h = boxes;
   m->fcount = foff;
   m->vcount = voff;
@@ -969,35 +1036,24 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   // bytes of a stored factor value and of a local-vector value
   const size_t esz = factor_prec == 64 ? sizeof(double) : (factor_prec == 32 ? sizeof(float) : 2);
   const size_t vsz = factor_prec == 64 ? sizeof(double) : sizeof(float);
-  // every bulk copy of the solve must start on a 16-byte boundary and move a
-  // multiple of 16 bytes: check each chunk's L and U blocks before any launch
-  for (const Chunk& c : chunks) {
-    const long long base = (boxes[c.box].foff + c.off) * (long long)esz;
-    const long long lbytes = (long long)kLRanks * c.cp * (long long)esz;
-    const long long ubytes = (long long)kURanks * c.cp * (long long)esz;
-    if (base % 16 || lbytes % 16 || ubytes % 16) {
-      set_error("ras_setup: internal error: a factor block is not 16-byte aligned");
-      delete m;
-      return KKT_ERR_ARG;
-    }
-  }
+  // every lane vector must start on a 16-byte boundary (group and box offsets are whole groups)
+  static_assert(kGroupVals32 * 2 % 16 == 0 && kLaneL * 32 * 2 % 16 == 0, "16-byte lane vectors");
   auto fail = [&](kkt_status st, const char* what) {
     cudaGetLastError();
     set_error(std::string("ras_setup: ") + what);
     ras_destroy(m);
     return st;
   };
+  auto bytes = [](size_t n, size_t size) { return std::max<size_t>(1, n) * size; };
   if (cudaMalloc(&m->boxes, boxes.size() * sizeof(BoxDesc)) != cudaSuccess ||
-      cudaMalloc(&m->perm, perm.size() * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&m->iperm, iperm.size() * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&m->lptr, lptr.size() * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&m->ptab, ptab.size() * sizeof(int2)) != cudaSuccess ||
-      cudaMalloc(&m->gtab, gtab.size() * sizeof(int2)) != cudaSuccess ||
-      cudaMalloc(&m->otab, std::max<size_t>(1, otab.size()) * sizeof(int2)) != cudaSuccess ||
-      cudaMalloc(&m->vtab, vtab.size() * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&m->chunks, chunks.size() * sizeof(Chunk)) != cudaSuccess ||
-      cudaMalloc(&m->F, (local >= 2 ? 16 : foff) * esz) != cudaSuccess ||
-      cudaMalloc(&m->V, (local >= 2 ? 16 : voff) * vsz) != cudaSuccess ||
+      cudaMalloc(&m->perm, bytes(perm.size(), sizeof(int))) != cudaSuccess ||
+      cudaMalloc(&m->gptr, bytes(gptr.size(), sizeof(int))) != cudaSuccess ||
+      cudaMalloc(&m->ptab, bytes(ptab.size(), sizeof(int))) != cudaSuccess ||
+      cudaMalloc(&m->gtab, bytes(gtab.size(), sizeof(int2))) != cudaSuccess ||
+      cudaMalloc(&m->otab, bytes(otab.size(), sizeof(int2))) != cudaSuccess ||
+      cudaMalloc(&m->vtab, bytes(vtab.size(), sizeof(int))) != cudaSuccess ||
+      cudaMalloc(&m->F, (local != 0 ? 16 : foff) * esz) != cudaSuccess ||
+      cudaMalloc(&m->V, (local != 0 ? 16 : voff) * vsz) != cudaSuccess ||
       (factor_prec == 16 && cudaMalloc(&m->Ffac, foff * sizeof(float)) != cudaSuccess) ||
       cudaMalloc(&m->status, sizeof(int)) != cudaSuccess ||
       cudaMalloc(&m->dprobs, m->probs.size() * sizeof(DevProblem)) != cudaSuccess)
@@ -1011,7 +1067,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       return fail(KKT_ERR_NOMEM, ("the exact local LU needs " + std::to_string((long long)(need / 1e6)) +
                                   " MB of band storage; use ILU(0) or more subdomains").c_str());
     if (cudaMalloc(&m->AB, m->ab_count * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&m->ipiv, 3 * perm.size() * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&m->ipiv, 3 * (size_t)poff * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&m->lu_ju, 2 * boxes.size() * sizeof(int)) != cudaSuccess)
       return fail(KKT_ERR_NOMEM, "device allocation failed (exact LU)");
     int dev = 0, nsm = 1;
@@ -1021,17 +1077,17 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   }
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = cudaMemcpy(m->boxes, boxes.data(), boxes.size() * sizeof(BoxDesc), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->perm, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->iperm, iperm.data(), iperm.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->lptr, lptr.data(), lptr.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->ptab, ptab.data(), ptab.size() * sizeof(int2), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->gtab, gtab.data(), gtab.size() * sizeof(int2), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && !otab.empty())
-    e = cudaMemcpy(m->otab, otab.data(), otab.size() * sizeof(int2), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->vtab, vtab.data(), vtab.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->chunks, chunks.data(), chunks.size() * sizeof(Chunk), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(m->F, 0, (local >= 2 ? 16 : foff) * esz);
-  if (e == cudaSuccess) e = cudaMemset(m->V, 0, (local >= 2 ? 16 : voff) * vsz);
+  auto copy = [&](void* dst, const void* src, size_t n) {
+    if (e == cudaSuccess && n) e = cudaMemcpy(dst, src, n, cudaMemcpyHostToDevice);
+  };
+  copy(m->perm, perm.data(), perm.size() * sizeof(int));
+  copy(m->gptr, gptr.data(), gptr.size() * sizeof(int));
+  copy(m->ptab, ptab.data(), ptab.size() * sizeof(int));
+  copy(m->gtab, gtab.data(), gtab.size() * sizeof(int2));
+  copy(m->otab, otab.data(), otab.size() * sizeof(int2));
+  copy(m->vtab, vtab.data(), vtab.size() * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(m->F, 0, (local != 0 ? 16 : foff) * esz);
+  if (e == cudaSuccess) e = cudaMemset(m->V, 0, (local != 0 ? 16 : voff) * vsz);
   if (e == cudaSuccess && m->Ffac) e = cudaMemset(m->Ffac, 0, foff * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(m->status, 0, sizeof(int));
   if (e != cudaSuccess) return fail(KKT_ERR_CUDA, cudaGetErrorString(e));
@@ -1051,18 +1107,12 @@ template <typename S>
 kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename SolveArith<S>::type* V,
                         cudaStream_t s, const int* gate = nullptr, int gate_stride = 0) {
   using T = typename SolveArith<S>::type;
-  const int threads = (m->ch * kLanes + 31) / 32 * 32;
-  const int bstride = kLRanks * m->cpmax;
+  const int gbytes = gptr_smem(m->max_nlev);
   // (the dynamic shared-memory limit of both instances is raised at set-up, in choose_solve_shape)
-  const size_t smem = solve_smem(m->cpmax, m->nstage, sizeof(S), sizeof(T), m->max_pad, m->smem_vec);
-  if (m->smem_vec)
-    ras_solve<S, true><<<m->nbox, threads, smem, s>>>(m->boxes, m->chunks, (const S*)m->F, V, r, z, m->gtab,
-                                                      m->otab, m->vtab, bstride, m->nstage, m->status, gate,
-                                                      gate_stride);
-  else
-    ras_solve<S, false><<<m->nbox, threads, smem, s>>>(m->boxes, m->chunks, (const S*)m->F, V, r, z, m->gtab,
-                                                       m->otab, m->vtab, bstride, m->nstage, m->status, gate,
-                                                       gate_stride);
+  const size_t smem = solve_smem<S>(m->max_nlev, m->warps, m->nstage) + (m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
+  auto* kernel = m->smem_vec ? ras_solve<S, true> : ras_solve<S, false>;
+  kernel<<<m->nbox, 32 * m->warps, smem, s>>>(m->boxes, m->gptr, (const S*)m->F, V, r, z, m->gtab, m->otab, m->vtab,
+                                              gbytes, solve_buffers(m->nstage), m->status, gate, gate_stride);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
@@ -1259,8 +1309,7 @@ extern "C" void ras_destroy(ras_precond* m) {
   if (!m) return;
   cudaFree(m->boxes);
   cudaFree(m->perm);
-  cudaFree(m->iperm);
-  cudaFree(m->lptr);
+  cudaFree(m->gptr);
   cudaFree(m->ptab);
   cudaFree(m->gtab);
   cudaFree(m->otab);
@@ -1269,7 +1318,6 @@ extern "C" void ras_destroy(ras_precond* m) {
   cudaFree(m->AB);
   cudaFree(m->ipiv);
   cudaFree(m->lu_ju);
-  cudaFree(m->chunks);
   cudaFree(m->F);
   cudaFree(m->V);
   cudaFree(m->status);
@@ -1352,8 +1400,8 @@ extern "C" kkt_status ras_apply_static(ras_precond* m, const double* r, double* 
 }
 
 // ---------------------------------------------------------------------------
-// Autotuner of the subdomain solve's shape: every compiled chunk size with
-// 2 and 3 copy buffers (local vectors placed as the chooser places them) is
+// Autotuner of the subdomain solve's shape: every compiled size class with
+// 2 and 3 in the buffer field (local vectors placed as the chooser places them) is
 // set up on the given problems and timed over `reps` applies with CUDA
 // events; the fastest is returned and, with a cache file, remembered there
 // under a key of the problems' sizes, the split, the precision and the
@@ -1414,16 +1462,9 @@ extern "C" kkt_status ras_autotune(kkt_problem* const* probs, int nprob, const i
       std::fclose(f);
     }
   }
-  int cands[3] = {ChunkCfg<float>::CH, ChunkCfg<float>::CH2, ChunkCfg<float>::CH3};
-  if (factor_prec == 64) {
-    cands[0] = ChunkCfg<double>::CH;
-    cands[1] = ChunkCfg<double>::CH2;
-    cands[2] = ChunkCfg<double>::CH3;
-  } else if (factor_prec == 16) {
-    cands[0] = ChunkCfg<__nv_bfloat16>::CH;
-    cands[1] = ChunkCfg<__nv_bfloat16>::CH2;
-    cands[2] = ChunkCfg<__nv_bfloat16>::CH3;
-  }
+  const int* cands = factor_prec == 64   ? SizeClasses<double>::name
+                     : factor_prec == 16 ? SizeClasses<__nv_bfloat16>::name
+                                         : SizeClasses<float>::name;
   long long n = 0;
   for (int i = 0; i < nprob; ++i) n += probs[i]->n;
   double *r = nullptr, *z = nullptr;

@@ -6,17 +6,27 @@
 // slots per point: C row 2*27*2 = 108, G row 2*(27+1) = 56, f row 3*27*2 = 162
 constexpr int kSlots = 326;
 
-// A run of at most CH points of one wavefront whose factor values form one
-// contiguous block [slot rank][cp] (cp >= n, chosen per precision).
-struct Chunk {
-  int q0;                      // first point (wavefront order, box-local)
-  int n;                       // points
-  int cp;                      // row stride of the block
-  int box;                     // owning box
-  int w;                       // wavefront of the chunk
-  int pad_;
-  long long off;               // element offset of the block within the box
-};
+// The points of a wavefront are stored in groups of 8 (the last one of a
+// wavefront may be ragged): one warp of the subdomain solve takes one group.
+// Values per group: FP64 [slot rank][8] blocks; FP32 and BF16 44 lower and 38
+// upper values for each of the 32 lanes (ras.cu), 326 slots x 8 points plus 16
+// unused places.
+constexpr int kGroup = 8;
+constexpr int kGroupVals64 = kSlots * kGroup;
+constexpr int kLaneL = 44, kLaneU = 38;                        // values per lane of a group
+constexpr int kGroupVals32 = 32 * (kLaneL + kLaneU);
+__host__ __device__ constexpr int group_vals(int prec) { return prec == 64 ? kGroupVals64 : kGroupVals32; }
+
+// Where the solve's lanes keep their values (FP32 and BF16): place of value v
+// of a lane within its group.  A lane's values form 16-byte vectors, vector k
+// of the 32 lanes side by side, so a warp reads 512 contiguous bytes at a
+// time; the last vector is shorter where the count is no multiple.
+template <typename S>
+__host__ __device__ __forceinline__ int lane_place(bool upper, int v, int lane) {
+  constexpr int W = 16 / (int)sizeof(S);
+  const int n = upper ? kLaneU : kLaneL, full = n / W * W, base = upper ? 32 * kLaneL : 0;
+  return base + (v < full ? (v / W * 32 + lane) * W + v % W : full * 32 + lane * (n - full) + (v - full));
+}
 
 struct GpFactor;   // ILU(1) / point-block ILU(0) factors (iluk.cu)
 
@@ -27,12 +37,12 @@ struct BoxDesc {
   int ox0, ox1, oy0, oy1, oz0, oz1, ot0, ot1;   // owned ranges (global, half open)
   int nlev;                    // wavefronts x + 2y + 4z + 8t
   long long P;                 // points of the extended box
-  long long foff;              // offset of the box's chunk blocks (elements)
+  long long foff;              // offset of the box's factor groups (elements)
   long long unit;              // offset of the box's unit row within its factor values (elements)
   long long voff;              // offset of the box's padded local vector (elements)
-  long long poff;              // offset into perm / iperm
+  long long poff;              // offset into the per-point tables (lexicographic)
+  long long goff;              // first group of the box
   long long loff;              // offset into the wavefront pointers
-  int cbeg, cend;              // chunk range
   int nown;                    // owned points
   long long ooff;              // offset into the owned-point table
   int kl;                      // exact LU: half-bandwidth of the box matrix
@@ -57,28 +67,28 @@ struct ras_precond {
   std::vector<DevProblem> dprobs_h;
   int prec = 64;               // factor storage: 64, 32, or 16 (BF16; factorisation and solve in FP32)
   int nbox = 0;
-  int ch = 0;                  // points per chunk of the subdomain solve (chosen per preconditioner)
-  int cpmax = 0;               // largest chunk row stride
+  int ch = 0;                  // size class of the solve's CTA (ras_setup_shape)
+  int warps = 0;               // warps of that CTA
   bool smem_vec = false;       // solve keeps the local vectors in shared memory
-  int nstage = 2;              // buffers of the solve's copy ring
+  int nstage = 2;              // factor groups a warp asks for ahead, itself included (ras_setup_shape)
   int lanes = 4;               // lanes per point in the solve
+  int max_nlev = 0;            // most wavefronts of a box
+  long long ngroup = 0;        // groups of all boxes
+  int max_groups = 0;          // most groups of a box
   long long fcount = 0;        // factor values
   long long max_pad = 0;       // largest padded local vector (elements)
   long long vcount = 0;        // elements of all padded local vectors (the solve's scratch)
   std::vector<BoxDesc> boxes_h;
   BoxDesc* boxes = nullptr;
-  int* perm = nullptr;         // wavefront order -> lexicographic local index
-  int* iperm = nullptr;        // lexicographic -> wavefront order
-  int* lptr = nullptr;         // wavefront pointers per box (nlev + 1 each)
-  Chunk* chunks = nullptr;
-  int nchunk = 0;
+  int* perm = nullptr;         // per group place: lexicographic local index, -1 in a ragged group's empty places
+  int* gptr = nullptr;         // first group of each wavefront per box (nlev + 1 each)
   int2* gtab = nullptr;        // per point (lexicographic): {3 x global point index, padded offset}
   int2* otab = nullptr;        // per owned point: {3 x global point index, padded offset}
-  int* vtab = nullptr;         // per point (wavefront order): padded offset in the box's local vector
-  int2* ptab = nullptr;        // per point (wavefront order): {offset of its column in the box's
-                               // chunk blocks, row stride of its block}
+  int* vtab = nullptr;         // per group place: padded offset in the box's local vector; empty places hold
+                               // the complement of an offset that can be read
+  int* ptab = nullptr;         // per point (lexicographic): offset of its column in the box's factor values
   void* F = nullptr;           // factor values (FP64, FP32 or BF16, as the solve reads them)
-  void* Ffac = nullptr;        // BF16 storage: the FP32 values the factorisation works on
+  void* Ffac = nullptr;        // BF16 storage: the FP32 values the factorisation works on, [slot rank][8] groups
   void* V = nullptr;           // padded local vectors
   int* status = nullptr;
   int local = 0;               // 0: ILU(0) local solves, 1: exact banded LU (FP64)
