@@ -1,22 +1,21 @@
-// ILU(0) factorisation of all subdomain matrices (Sec. 3.2), in place on the
-// chunk layout that the subdomain solve streams.  Included by factor32.cu and
-// factor64.cu, one translation unit per precision (the generated elimination
-// code is large, and the two compile in parallel).
+// FP64 ILU(0) factorisation of all subdomain matrices (Sec. 3.2), in place on
+// the [slot rank][8 points] groups that the subdomain solve reads.  (FP32:
+// factor32.cu.)
 //
-// Values.  gather_chunks forms every slot value of every box point from the
+// Values.  gather_groups forms every slot value of every box point from the
 // stencil coefficients (the principal submatrix of F_h on the extended box,
 // Eq. 10-12; a slot whose column leaves the box holds 0) and writes it to the
-// point's column of its chunk block, row c_gen_rank[slot] (c_gen_rank_of by
-// the slot's offsets).
+// point's column of its group, row c_gen_rank[slot] (c_gen_rank_of by the
+// slot's offsets).
 //
 // Elimination.  One CTA per box steps through the wavefronts
 // w = x + 2y + 4z + 8t with a barrier between them; one thread takes one point
 // of the wavefront and eliminates its C, G and f rows in turn with the
 // straight-line code of ilu_rows.inc.  The thread first lists where the
-// columns of its 41 possible pivot points are (offset and row stride of their
-// chunk blocks); a pivot point outside the box is sent to the box's unit row
-// (stride 1, 1 at the three diagonal ranks, 0 elsewhere).  The diagonal slot
-// of a finished row holds 1/u_kk.
+// columns of its 41 possible pivot points are; a pivot point outside the box
+// is sent to the box's unit row (1 at the three diagonal ranks, 0 elsewhere).
+// The diagonal slot of a finished row holds 1/u_kk.  (One warp per point, as in
+// FP32, would issue 2.5 times the FP64 instructions; the pipe has 2 lanes.)
 #pragma once
 
 #include "slotval.cuh"
@@ -27,10 +26,9 @@ namespace {
 
 constexpr int kGatherThreads = 256;
 // Threads per factor CTA, two CTAs per SM (all 256 boxes of the 4x4x4x4
-// partition resident at once).  FP32 rows fit 192 threads without large
-// spills; FP64 rows need the registers of 128.
+// partition resident at once); the rows need the registers of 128 threads.
 template <typename T>
-constexpr int factor_threads = sizeof(T) == 4 ? 192 : 128;
+constexpr int factor_threads = 128;
 
 // offset of the column of group place q in the box's factor values
 template <typename T>
@@ -38,7 +36,7 @@ __device__ __forceinline__ int group_column(int q) {
   return q / kGroup * group_vals(8 * sizeof(T)) + q % kGroup;
 }
 
-// One thread per point (wavefront order, so the threads of a chunk write
+// One thread per point (wavefront order, so the threads of a group write
 // consecutive addresses); all threads of a warp on the same slot.  Entries are
 // formed in the factor precision, with the arithmetic of slot_value, but one
 // spatial offset at a time: the point's B, S, S^T and K coefficients of that
@@ -47,7 +45,7 @@ __device__ __forceinline__ int group_column(int q) {
 // at n-1, n, n+1), plus the G row's two sensor slots at the centre.  Also
 // writes each box's unit row.
 template <typename T>
-__global__ void __launch_bounds__(kGatherThreads) gather_chunks(const DevProblem* __restrict__ probs,
+__global__ void __launch_bounds__(kGatherThreads) gather_groups(const DevProblem* __restrict__ probs,
                                                                 const BoxDesc* __restrict__ boxes,
                                                                 const int* __restrict__ gptr,
                                                                 const int* __restrict__ perm, T* __restrict__ F) {
@@ -146,19 +144,11 @@ __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDes
       }
       T* own = Fb + group_column<T>(q);
       // the G and f rows read the U parts of this point's C and G rows
-      if constexpr (sizeof(T) == 4) {
-        check_pivot((double)ilu_row0_32<T, NS>(own, Fb, nb), status);
-        asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row1_32<T, NS>(own, Fb, nb), status);
-        asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row2_32<T, NS>(own, Fb, nb), status);
-      } else {
-        check_pivot((double)ilu_row0_64<T, NS>(own, Fb, nb), status);
-        asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row1_64<T, NS>(own, Fb, nb), status);
-        asm volatile("" ::: "memory");
-        check_pivot((double)ilu_row2_64<T, NS>(own, Fb, nb), status);
-      }
+      check_pivot((double)ilu_row0_64<T, NS>(own, Fb, nb), status);
+      asm volatile("" ::: "memory");
+      check_pivot((double)ilu_row1_64<T, NS>(own, Fb, nb), status);
+      asm volatile("" ::: "memory");
+      check_pivot((double)ilu_row2_64<T, NS>(own, Fb, nb), status);
     }
     __syncthreads();
   }
@@ -168,7 +158,7 @@ __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDes
 template <typename T>
 kkt_status factor_launch(ras_precond* m, T* F, cudaStream_t s) {
   const dim3 g((unsigned)((kGroup * (long long)m->max_groups + kGatherThreads - 1) / kGatherThreads), m->nbox);
-  gather_chunks<T><<<g, kGatherThreads, 0, s>>>(m->dprobs, m->boxes, m->gptr, m->perm, F);
+  gather_groups<T><<<g, kGatherThreads, 0, s>>>(m->dprobs, m->boxes, m->gptr, m->perm, F);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   {

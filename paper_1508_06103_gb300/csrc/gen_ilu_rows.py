@@ -1,4 +1,4 @@
-"""Generate ilu_rows.inc: straight-line ILU(0) elimination of one KKT row per thread.
+"""Generate ilu_rows.inc: straight-line FP64 ILU(0) elimination of one KKT row per thread.
 
 (and ilu_slots.inc: the slot list's checksum and each slot's row in a group,
 also indexed by the slot's offsets for the value gather)
@@ -86,8 +86,7 @@ def checksum(slots):
     return h
 
 
-GROUP32 = 8    # entries finished between two rounds of stores, FP32
-GROUP64 = 4    # the same in FP64 (twice the registers per value)
+GROUP64 = 4    # entries finished between two rounds of stores
 
 
 def row_function(c, prec, group, nl, cnt, base, slots, diag, rank, nbrs, contrib):
@@ -224,7 +223,7 @@ def generate() -> str:
         nupd = sum(len(v) for v in contrib.values())
         out.append(f"// row type {'CGf'[c]}: {count[c]} slots, {nl} L-slots, {nupd} updates")
         out.append(f"constexpr int kGenRowUpdates{c} = {nupd};")
-        for prec, gmax in (("32", GROUP32), ("64", GROUP64)):
+        for prec, gmax in (("64", GROUP64),):
             out.extend(row_function(c, prec, gmax, nl, count[c], base[c], slots, diag, rank, nbrs, contrib))
     return "\n".join(hdr) + "\n", "\n".join(out) + "\n"
 

@@ -119,6 +119,7 @@ struct DevProblem {
   double hx, hy, hz;                        // mesh widths (Q1: B and K are tensor products of 1D factors)
   const double *S, *ST, *B, *K;             // [27][N] row coefficients (FP64)
   const float *S32, *ST32, *B32, *K32;      // FP32 copies
+  const float4* pack32;                     // [N][27] FP32 {B, S, ST, K}, node by node (the FP32 factorisation)
   const unsigned char* dir;                 // [N] 1 on Dirichlet nodes
   const double* sens;                       // [N] sensor counts, 0 on Dirichlet nodes
   const int* gate;                          // device flag: the kernels return at once when it reads 0
@@ -202,6 +203,7 @@ struct kkt_problem {
   // device memory
   double* coef64 = nullptr;                 // S, ST, B, K   (4 * 27 * N)
   float* coef32 = nullptr;                  // FP32 copies
+  float4* pack32 = nullptr;                 // FP32 {B, S, ST, K} per node and offset
   unsigned char* dir = nullptr;
   double* sens = nullptr;
   int* sens_ptr = nullptr;                  // CSR: sensors of each node (N+1)

@@ -117,6 +117,7 @@ DevProblem kkt_problem::dev() const {
   d.hx = hx; d.hy = hy; d.hz = hz;
   const size_t c = (size_t)kStencil * N;
   d.S = coef64; d.ST = coef64 + c; d.B = coef64 + 2 * c; d.K = coef64 + 3 * c;
+  d.pack32 = pack32;
   d.S32 = coef32; d.ST32 = coef32 + c; d.B32 = coef32 + 2 * c; d.K32 = coef32 + 3 * c;
   d.dir = dir;
   d.sens = sens;
@@ -268,6 +269,14 @@ __global__ void to_float(const double* __restrict__ x, float* __restrict__ y, si
     y[i] = (float)x[i];
 }
 
+__global__ void pack_float4(const float* __restrict__ c, float4* __restrict__ out, int N) {
+  const size_t n = (size_t)kStencil * N;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t o = i % kStencil * N + i / kStencil;   // S, ST, B, K blocks of [27][N]
+    out[i] = make_float4(c[2 * n + o], c[o], c[n + o], c[3 * n + o]);
+  }
+}
+
 __global__ void rhs_kernel(DevProblem p, const double* __restrict__ c_obs, int nsens, const double* __restrict__ c0,
                            const int* __restrict__ sptr, const int* __restrict__ sidx, double* __restrict__ b) {
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -325,7 +334,8 @@ kkt_status assemble_coefficients(kkt_problem* p, const char* who) {
       assemble_stencils<<<blocks, 128>>>(geo, d_a, d_v, p->coef64, p->coef64 + c, p->coef64 + 2 * c,
                                          p->coef64 + 3 * c);
     to_float<<<1024, 256>>>(p->coef64, p->coef32, ncoef);
-    KKT_COUNT(2);
+    pack_float4<<<1024, 256>>>(p->coef32, p->pack32, (int)N);
+    KKT_COUNT(3);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -411,6 +421,7 @@ kkt_status create_problem(const kkt_grid* g, int nt, double dt, const double* a_
   const size_t ncoef = 4 * (size_t)kStencil * N;
   if (cudaMalloc(&p->coef64, ncoef * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&p->coef32, ncoef * sizeof(float)) != cudaSuccess ||
+      cudaMalloc(&p->pack32, ncoef * sizeof(float)) != cudaSuccess ||
       cudaMalloc(&p->dir, N) != cudaSuccess || cudaMalloc(&p->sens, N * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&p->sens_ptr, (N + 1) * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&p->sens_idx, std::max(nsens, 1) * sizeof(int)) != cudaSuccess) {
@@ -509,6 +520,7 @@ extern "C" void kkt_destroy(kkt_problem* p) {
   if (!p) return;
   cudaFree(p->coef64);
   cudaFree(p->coef32);
+  cudaFree(p->pack32);
   cudaFree(p->dir);
   cudaFree(p->sens);
   cudaFree(p->sens_ptr);

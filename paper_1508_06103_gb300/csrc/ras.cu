@@ -701,7 +701,8 @@ struct SolveShape {
   int ch, warps, nstage, lanes;
   bool smem_vec;
 };
-constexpr int kFillGroups = 7;   // groups per wavefront from which the largest CTA is taken
+// groups per wavefront from which the largest CTA is taken: boxes one per SM, more boxes than SMs
+constexpr int kFillGroups = 7, kFillGroups2 = 12;
 template <typename T, bool SMEM>
 const void* solve_kernel() {
   return (const void*)ras_solve<T, SMEM>;
@@ -748,7 +749,7 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
             &per_sm, sv ? solve_kernel<T, true>() : solve_kernel<T, false>(), 32 * warps, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
-        const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
+        const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * (nbox > nsm ? kFillGroups2 : kFillGroups);
         const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
         if (best_key < 0 || key < best_key) {
           best_key = key;
@@ -980,7 +981,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       perm.resize(q0 + (size_t)kGroup * groups, -1);
       vtab.resize(q0 + (size_t)kGroup * groups, ~pad(0, 0, 0, 0));
       gtab.resize(p0 + b.P);
-      ptab.resize(p0 + b.P);
+      if (factor_prec == 64) ptab.resize(p0 + b.P);
       int lex = 0;
       for (int kt = 0; kt < b.lt; ++kt)
         for (int kz = 0; kz < b.lz; ++kz)
@@ -990,7 +991,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
               perm[q0 + q] = lex;
               vtab[q0 + q] = pad(kx, ky, kz, kt);
               gtab[p0 + lex] = make_int2(glob(kx, ky, kz, kt), vtab[q0 + q]);
-              ptab[p0 + lex] = q / kGroup * gvals + q % kGroup;
+              if (factor_prec == 64) ptab[p0 + lex] = q / kGroup * gvals + q % kGroup;
             }
       b.ooff = (long long)otab.size();
       for (int gt = b.ot0; gt < b.ot1; ++gt)
@@ -1000,14 +1001,14 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
               otab.push_back(make_int2(glob(gx - b.x0, gy - b.y0, gz - b.z0, gt - b.t0),
                                        pad(gx - b.x0, gy - b.y0, gz - b.z0, gt - b.t0)));
       b.nown = (int)((long long)otab.size() - b.ooff);
-      // the unit row of pivot points outside the box is one more group
+      // FP64: the unit row of pivot points outside the box is one more group
       b.unit = (long long)groups * gvals;
-      if (b.unit + gvals > INT32_MAX) {
+      if (factor_prec == 64 && b.unit + gvals > INT32_MAX) {
         set_error("ras_setup: a subdomain holds more than 2^31 factor values; use more subdomains");
         delete m;
         return KKT_ERR_ARG;
       }
-      foff += b.unit + gvals;
+      foff += b.unit + (factor_prec == 64 ? gvals : 0);
     }
     if (local == 1) {
       // exact LU: band of the box matrix in natural point-block order
@@ -1054,7 +1055,6 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       cudaMalloc(&m->vtab, bytes(vtab.size(), sizeof(int))) != cudaSuccess ||
       cudaMalloc(&m->F, (local != 0 ? 16 : foff) * esz) != cudaSuccess ||
       cudaMalloc(&m->V, (local != 0 ? 16 : voff) * vsz) != cudaSuccess ||
-      (factor_prec == 16 && cudaMalloc(&m->Ffac, foff * sizeof(float)) != cudaSuccess) ||
       cudaMalloc(&m->status, sizeof(int)) != cudaSuccess ||
       cudaMalloc(&m->dprobs, m->probs.size() * sizeof(DevProblem)) != cudaSuccess)
     return fail(KKT_ERR_NOMEM, "device allocation failed");
@@ -1088,10 +1088,10 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   copy(m->vtab, vtab.data(), vtab.size() * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(m->F, 0, (local != 0 ? 16 : foff) * esz);
   if (e == cudaSuccess) e = cudaMemset(m->V, 0, (local != 0 ? 16 : voff) * vsz);
-  if (e == cudaSuccess && m->Ffac) e = cudaMemset(m->Ffac, 0, foff * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(m->status, 0, sizeof(int));
   if (e != cudaSuccess) return fail(KKT_ERR_CUDA, cudaGetErrorString(e));
   kkt_status st = local >= 2 ? gp_create(m, local, factor_prec) : KKT_OK;
+  if (st == KKT_OK && local == 0 && factor_prec != 64) st = ras_factor_prepare32(m);
   if (st == KKT_OK) st = ras_factor(m, nullptr);
   if (st != KKT_OK) {
     ras_destroy(m);
@@ -1314,7 +1314,7 @@ extern "C" void ras_destroy(ras_precond* m) {
   cudaFree(m->gtab);
   cudaFree(m->otab);
   cudaFree(m->vtab);
-  cudaFree(m->Ffac);
+  cudaFree(m->rec);
   cudaFree(m->AB);
   cudaFree(m->ipiv);
   cudaFree(m->lu_ju);

@@ -88,9 +88,12 @@ struct ras_precond {
                                // the complement of an offset that can be read
   int* ptab = nullptr;         // per point (lexicographic): offset of its column in the box's factor values
   void* F = nullptr;           // factor values (FP64, FP32 or BF16, as the solve reads them)
-  void* Ffac = nullptr;        // BF16 storage: the FP32 values the factorisation works on, [slot rank][8] groups
   void* V = nullptr;           // padded local vectors
   int* status = nullptr;
+  float* rec = nullptr;        // FP32 factorisation: pivot records of the boxes in work
+  long long rec_floats = 0;    // per cluster
+  int fac_cluster = 1;         // FP32 factorisation: CTAs per box, clusters of the launch
+  int fac_nclusters = 0;
   int local = 0;               // 0: ILU(0) local solves, 1: exact banded LU (FP64)
   double* AB = nullptr;        // exact LU: band factors of all boxes
   long long ab_count = 0;
@@ -122,6 +125,7 @@ kkt_status ras_factor_status(ras_precond* m);                   // after the str
 kkt_status ras_factor_launch32(ras_precond* m, cudaStream_t s);
 kkt_status ras_factor_launch64(ras_precond* m, cudaStream_t s);
 kkt_status ras_factor_launch16(ras_precond* m, cudaStream_t s);   // FP32 factorisation, BF16 store
+kkt_status ras_factor_prepare32(ras_precond* m);                  // launch shape and records of the two above
 // exact banded LU (lu.cu)
 kkt_status ras_lu_factor(ras_precond* m, cudaStream_t s);
 kkt_status ras_lu_solve(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate);
