@@ -11,9 +11,11 @@
 // Mt, Lt are the 1D linear-element time mass and stiffness (tau/6 [1 4 1],
 // [-1 2 -1]/tau, halved diagonals at the end levels).
 //
-// matvec_tiled below computes all three output slots of a space-time point
-// in one pass: four spatial operators applied to six time combinations, B and
-// K by sum factorisation, S and S^T as 27-point stencils.  Under P1 elements
+// matvec_tiled below (FP32, and FP64 under P1 elements) computes all three output
+// slots of a space-time point in one pass: four spatial operators applied to six
+// time combinations, B and K by sum factorisation, S and S^T as 27-point
+// stencils; matvec64_levels (FP64, trilinear elements) applies the operators to
+// the levels and combines them in time at the output nodes.  Under P1 elements
 // on the Kuhn split (kkt_set_element) B and K are no tensor products: all four
 // operators are applied as stencils over the 15 offsets the split couples.
 
@@ -65,9 +67,8 @@ __device__ __forceinline__ Coefs<float> coefs<float>(const DevProblem& p) {
 // nodes: 40 x 40 x 36 / 33^3 = 1.6x the nodes with 8 x 8 x 4 tiles); the host
 // picks the shape with the least estimated work (launch_tiled).
 // Levels per CTA: shorter runs give more CTAs for the same work (two halo
-// levels more per run).  Measured at 32^3 x 64 with the inputs out of L2
-// (runs of 16 / 8 / 4 levels): FP64 1.127 / 1.047 / 1.018 ms, FP32 0.158 /
-// 0.153 / 0.159 ms.
+// levels more per run).  Measured at 32^3 x 64, FP32, with the inputs out of L2
+// (runs of 16 / 8 / 4 levels): 0.158 / 0.153 / 0.159 ms.
 template <typename T>
 __host__ __device__ constexpr int levels_per_cta() {
   return sizeof(T) == 8 ? 4 : 8;
@@ -82,6 +83,7 @@ struct Tile {
 };
 using TileA = Tile<8, 8, 4>;
 using TileB = Tile<11, 11, 2>;
+using TileC = Tile<11, 11, 3>;   // FP64 levels kernel
 
 template <typename T, typename Tl, bool kP1 = false>
 constexpr size_t mv_smem() {
@@ -424,6 +426,298 @@ void launch_tiled(const DevProblem& p, const T* x, T* y, const double* b, cudaSt
   else launch_shape<T, TileA>(p, x, y, b, s);
 }
 
+// ---------------------------------------------------------------------------
+// FP64, trilinear elements.  The FP64 pipe (2 lanes per SM and clock) is the limit,
+// so this kernel spends as few FP64 instructions per point as it can, about 130
+// against 200 in matvec_tiled:
+// - The spatial operators go to the levels themselves, once each, and the time
+//   weights are applied at the output nodes, carried from level to level in
+//   registers; matvec_tiled forms six weighted combinations on every halo node.
+//   With level m in hand the CTA finishes the C row of level m and the G and f rows of
+//   level m - 1.  The mass matrix of the C and G rows is applied to the differences
+//   C^m - C^{m-1}, G^{m-1} - G^m (formed on the halo), as in matvec_tiled: the
+//   difference of two products would lose digits where the solution varies slowly.
+// - The 1D factors of B and K are written [1 c 1] and [1 -c 1] (c = 4, 2 inside, 2, 1 at a
+//   domain face; neighbours outside the domain are zero), two instructions instead of
+//   three, and the products of the widths go into the time weights.
+// A CTA takes a tile of nodes and a run of levels; a run costs about 1.3 levels more
+// (one before and one after, in part), so the host picks long runs that still
+// fill the SMs.
+// Measured against matvec_tiled: 32^3 x 64 1016 -> 650 us (11 x 11 x 3 tiles, runs of 22),
+// 5 x 4 x 3 x 6 56 -> 22.5 us (runs of one level); the error against extended precision is
+// slightly smaller, on random and on smooth fields.
+// ---------------------------------------------------------------------------
+template <typename Tl>
+constexpr size_t mv64_smem() {
+  // C, G: levels m-1, m, m+1; f: m, m+1; the x-pass results; the y-pass results over the differences
+  return sizeof(double) * (8 * Tl::NH + 5 * Tl::NXP + (5 * Tl::NYP > 2 * Tl::NH ? 5 * Tl::NYP : 2 * Tl::NH));
+}
+
+struct Weights64 {
+  double sB;                  // product of the mass factors: B = sB [1 c 1] (x) [1 c 1] (x) [1 c 1]
+  double ry, rz;              // weights of the y and z stiffness against the x stiffness
+  double wt0, wt1;            // tau theta, tau (1 - theta)
+  double eG, eF, eK;          // neighbouring level in the f row: G, f by B; f by K
+  double dG, dF, dK;          // the level itself with one time element beside it
+  double dG2, dF2, dK2;       // with two
+  double th, th1, tau;
+  void init(const DevProblem& p) {
+    const double mo = p.hx / 6.0 * (p.hy / 6.0) * (p.hz / 6.0);
+    const double ax = -6.0 / (p.hx * p.hx), ay = -6.0 / (p.hy * p.hy), az = -6.0 / (p.hz * p.hz);
+    sB = mo;
+    ry = ay / ax;
+    rz = az / ax;
+    tau = p.tau;
+    th = p.theta;
+    th1 = 1.0 - p.theta;
+    wt0 = tau * th;
+    wt1 = tau * th1;
+    const double m6 = tau / 6.0, m3 = tau / 3.0, l1 = 1.0 / tau;
+    eG = -m6 * sB;
+    dG = -m3 * sB;
+    eF = -p.beta1 * l1 * sB;
+    dF = p.beta1 * l1 * sB;
+    eK = p.beta2 * m6 * sB;
+    dK = p.beta2 * m3 * sB;
+    if (p.reg != 0) {   // H1-L2: the beta2 term goes through B
+      eF += eK;
+      dF += dK;
+    } else {
+      eK *= ax;
+      dK *= ax;
+    }
+    dG2 = 2.0 * dG;
+    dF2 = 2.0 * dF;
+    dK2 = 2.0 * dK;
+  }
+};
+
+template <bool kL2, typename Tl>
+__global__ void __launch_bounds__(Tl::kThreads, Tl::kThreads > 256 ? 2 : 3) matvec64_levels(DevProblem p, const double* __restrict__ x,
+                                                                double* __restrict__ y, const double* __restrict__ b,
+                                                                int tiles_x, int tiles_y, int run, Weights64 W) {
+  constexpr int TX = Tl::TX, TY = Tl::TY, TZ = Tl::TZ;
+  constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH, NXP = Tl::NXP, NYP = Tl::NYP, NT = Tl::kThreads;
+  if (gated_off(p.gate)) return;
+  extern __shared__ __align__(16) unsigned char mv_sm[];
+  double* Cs = reinterpret_cast<double*>(mv_sm);   // [3 slots][NH]: level mod 3
+  double* Gs = Cs + 3 * NH;                        // [3 slots][NH]
+  double* Fs = Gs + 3 * NH;                        // [2 slots][NH]: level mod 2
+  double* PX = Fs + 2 * NH;                        // [5][NXP]
+  double* PY = PX + 5 * NXP;                       // [5][NYP]
+  double* U = PY;                                  // [2][NH]: the differences, read before PY is written
+  const int N = p.N, M = p.M;
+  const int tile = blockIdx.x;
+  const int bx0 = (tile % tiles_x) * TX, by0 = ((tile / tiles_x) % tiles_y) * TY, bz0 = (tile / (tiles_x * tiles_y)) * TZ;
+  const int n0 = blockIdx.y * run, n1 = min(n0 + run, M + 1);   // levels of the run
+  const int t = threadIdx.x;
+  const int tx = t % TX, ty = (t / TX) % TY, tz = t / (TX * TY);
+  const int ix = bx0 + tx, iy = by0 + ty, iz = bz0 + tz;
+  const bool own = ix < p.nx && iy < p.ny && iz < p.nz;
+  const int j = own ? ix + p.nx * (iy + p.ny * iz) : 0;
+  const int hc = (tx + 1) + HX * ((ty + 1) + HY * (tz + 1));
+
+  auto prefetch = [&](int m) {   // level m of x on the halo
+    double *dc = Cs + m % 3 * NH, *dg = Gs + m % 3 * NH, *df = Fs + m % 2 * NH;
+    for (int h = t; h < NH; h += NT) {
+      const int hx_ = h % HX, hy_ = (h / HX) % HY, hz_ = h / (HX * HY);
+      const int gx = bx0 - 1 + hx_, gy = by0 - 1 + hy_, gz = bz0 - 1 + hz_;
+      const bool valid = m <= M && gx >= 0 && gx < p.nx && gy >= 0 && gy < p.ny && gz >= 0 && gz < p.nz;
+      const double* src = valid ? x + 3 * ((long long)m * N + gx + (long long)p.nx * (gy + (long long)p.ny * gz)) : x;
+      cp_async_value(dc + h, src, valid);
+      cp_async_value(dg + h, src + (valid ? 1 : 0), valid);
+      cp_async_value(df + h, src + (valid ? 2 : 0), valid);
+    }
+  };
+  // 1D rows: c of the mass [1 c 1] and -c of the stiffness [1 -c 1] at node i of n (selected, not
+  // computed: a conversion is an FP64 instruction)
+  auto inner = [](int i, int n) { return i > 0 && i < n - 1; };
+  const int m0 = max(n0 - 1, 0), m1 = min(n1, M);   // levels read
+  prefetch(m0);
+  cp_async_commit();
+  const bool dirj = own && p.dir[j] != 0;
+  const double sj = own ? p.sens[j] : 0.0;
+  const bool sensor = sj != 0.0;
+  const double zm = inner(iz, p.nz) ? 4.0 : 2.0, zk = inner(iz, p.nz) ? -2.0 : -1.0;
+  double carryC = 0.0, accG = 0.0, accF = 0.0, Eprev = 0.0, yC = 0.0;   // yC: the C row of level m - 1
+  auto put = [&](int n, double c, double g, double f) {
+    const long long o = 3 * ((long long)n * N + j);
+    if (b != nullptr) {
+      y[o] = b[o] - c;
+      y[o + 1] = b[o + 1] - g;
+      y[o + 2] = b[o + 2] - f;
+    } else {
+      y[o] = c;
+      y[o + 1] = g;
+      y[o + 2] = f;
+    }
+  };
+  for (int m = m0; m <= m1; ++m) {
+    cp_async_wait<0>();
+    __syncthreads();   // level m has landed; the last step's reads are done
+    if (m < m1) prefetch(m + 1);
+    cp_async_commit();
+    const double *C0 = Cs + m % 3 * NH, *Cm = Cs + (m + 2) % 3 * NH;
+    const double *G0 = Gs + m % 3 * NH, *Gm = Gs + (m + 2) % 3 * NH;
+    const double* F0 = Fs + m % 2 * NH;
+    // what this level is needed for (a run's first and last level: in part)
+    const bool doC = m >= n0 && m < n1 && m > 0;     // C row of level m
+    const bool doS = m < n1;                         // S C^m: C rows of levels m, m + 1
+    const bool doG = m > n0;                         // G row of level m - 1
+    const bool doT = m >= n0;                        // S^T G^m: G rows of levels m, m - 1
+    if (doC || doG)
+      for (int h = t; h < NH; h += NT) {
+        if (doC) U[h] = C0[h] - Cm[h];
+        if (doG) U[NH + h] = Gm[h] - G0[h];
+      }
+    __syncthreads();
+    for (int e = t; e < NXP; e += NT) {
+      const int ex = e % TX, ey = (e / TX) % HY, ez = e / (TX * HY);
+      const int h = (ex + 1) + HX * (ey + HY * ez);
+      const bool in_ = inner(bx0 + ex, p.nx);
+      const double c = in_ ? 4.0 : 2.0;
+      if (doC) PX[e] = fma(c, U[h], U[h - 1]) + U[h + 1];
+      if (doG) PX[NXP + e] = fma(c, U[NH + h], U[NH + h - 1]) + U[NH + h + 1];
+      PX[2 * NXP + e] = fma(c, G0[h], G0[h - 1]) + G0[h + 1];
+      const double f_ = F0[h], fl = F0[h - 1], fr = F0[h + 1];
+      PX[3 * NXP + e] = fma(c, f_, fl) + fr;
+      if (!kL2) PX[4 * NXP + e] = fma(in_ ? -2.0 : -1.0, f_, fl) + fr;
+    }
+    __syncthreads();
+    for (int e = t; e < NYP; e += NT) {
+      const int ex = e % TX, ey = (e / TX) % TY, ez = e / (TX * TY);
+      const int q = ex + TX * ((ey + 1) + HY * ez);
+      const bool in_ = inner(by0 + ey, p.ny);
+      const double c = in_ ? 4.0 : 2.0;
+      if (doC) PY[e] = fma(c, PX[q], PX[q - TX]) + PX[q + TX];
+      if (doG) PY[NYP + e] = fma(c, PX[NXP + q], PX[NXP + q - TX]) + PX[NXP + q + TX];
+      PY[2 * NYP + e] = fma(c, PX[2 * NXP + q], PX[2 * NXP + q - TX]) + PX[2 * NXP + q + TX];
+      const double f_ = PX[3 * NXP + q], fl = PX[3 * NXP + q - TX], fr = PX[3 * NXP + q + TX];
+      PY[3 * NYP + e] = fma(c, f_, fl) + fr;
+      if (!kL2) {
+        const double k = fma(in_ ? -2.0 : -1.0, f_, fl) + fr;
+        PY[4 * NYP + e] = fma(W.ry, k, fma(c, PX[4 * NXP + q], PX[4 * NXP + q - TX]) + PX[4 * NXP + q + TX]);
+      }
+    }
+    __syncthreads();
+    if (own) {
+      const int q = tx + TX * (ty + TY * (tz + 1));
+      constexpr int zs = TX * TY;
+      // S C^m and S^T G^m, two chains each
+      double S0 = 0.0, S1 = 0.0, T0 = 0.0, T1 = 0.0;
+      if (doS && doT) {
+#pragma unroll
+        for (int d = 0; d < kStencil; ++d) {
+          const int h = hc + d % 3 - 1 + HX * ((d / 3) % 3 - 1 + HY * (d / 9 - 1));
+          const double s_ = p.S[(size_t)d * N + j], st_ = p.ST[(size_t)d * N + j];
+          if (d % 2) {
+            S1 = fma(s_, C0[h], S1);
+            T1 = fma(st_, G0[h], T1);
+          } else {
+            S0 = fma(s_, C0[h], S0);
+            T0 = fma(st_, G0[h], T0);
+          }
+        }
+      } else {
+        const double* A = doS ? p.S : p.ST;
+        const double* v = doS ? C0 : G0;
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int d = 0; d < kStencil; ++d) {
+          const int h = hc + d % 3 - 1 + HX * ((d / 3) % 3 - 1 + HY * (d / 9 - 1));
+          const double s_ = A[(size_t)d * N + j];
+          if (d % 2) s1 = fma(s_, v[h], s1);
+          else s0 = fma(s_, v[h], s0);
+        }
+        if (doS) {
+          S0 = s0;
+          S1 = s1;
+        } else {
+          T0 = s0;
+          T1 = s1;
+        }
+      }
+      const double BG = fma(zm, PY[2 * NYP + q], PY[2 * NYP + q - zs]) + PY[2 * NYP + q + zs];
+      const double f_ = PY[3 * NYP + q], fl = PY[3 * NYP + q - zs], fr = PY[3 * NYP + q + zs];
+      const double Bf = fma(zm, f_, fl) + fr;
+      double E = fma(W.eF, Bf, W.eG * BG);
+      const bool mid = m > 0 && m < M;   // two time elements
+      double Fd = fma(mid ? W.dF2 : W.dF, Bf, fma(mid ? W.dG2 : W.dG, BG, Eprev));
+      if (!kL2) {
+        const double Kf = fma(W.rz, fma(zk, f_, fl) + fr,
+                              fma(zm, PY[4 * NYP + q], PY[4 * NYP + q - zs]) + PY[4 * NYP + q + zs]);
+        E = fma(W.eK, Kf, E);
+        Fd = fma(mid ? W.dK2 : W.dK, Kf, Fd);
+      }
+      if (doG) {   // level m - 1 is complete
+        double g = fma(W.wt1, T0 + T1, accG);
+        g = fma(W.sB, fma(zm, PY[NYP + q], PY[NYP + q - zs]) + PY[NYP + q + zs], g);
+        if (sensor) g += W.tau * sj * (W.th * C0[hc] + W.th1 * Cm[hc]);
+        if (dirj) g = Gm[hc];
+        put(m - 1, yC, g, accF + E);
+      }
+      accF = Fd;
+      Eprev = E;
+      if (doT) accG = W.wt0 * (T0 + T1);
+      if (doS) {
+        const double D = fma(-W.sB, Bf, S0 + S1);
+        if (doC) yC = fma(W.sB, fma(zm, PY[q], PY[q - zs]) + PY[q + zs], fma(W.wt0, D, carryC));
+        if (m == 0 || dirj) yC = C0[hc];
+        carryC = W.wt1 * D;
+      }
+      if (m == M && n1 == M + 1) put(M, yC, G0[hc], accF);   // the last level: G^M is an identity row
+    }
+  }
+  cp_async_wait<0>();
+}
+
+template <bool kL2, typename Tl>
+void launch64_tile(const DevProblem& p, const double* x, double* y, const double* b, int run, cudaStream_t s) {
+  const int tx = (p.nx + Tl::TX - 1) / Tl::TX, ty = (p.ny + Tl::TY - 1) / Tl::TY, tz = (p.nz + Tl::TZ - 1) / Tl::TZ;
+  Weights64 w;
+  w.init(p);
+  matvec64_levels<kL2, Tl><<<dim3(tx * ty * tz, (p.M + run) / run), Tl::kThreads, mv64_smem<Tl>(), s>>>(
+      p, x, y, b, tx, ty, run, w);
+}
+
+// FP64 instructions of the busiest SM with tile shape Tl, and the run length that gives the
+// least: CTAs of an SM share its pipe; one alone leaves it idle at the barriers (measured
+// 0.7 of the rate of two or more).
+template <typename Tl>
+double work64(const DevProblem& p, int* run) {
+  const long long tiles = (long long)((p.nx + Tl::TX - 1) / Tl::TX) * ((p.ny + Tl::TY - 1) / Tl::TY) *
+                          ((p.nz + Tl::TZ - 1) / Tl::TZ);
+  const double level = 2.0 * Tl::NH + 10.0 * Tl::NXP + 13.0 * Tl::NYP + 81.0 * ((Tl::kThreads + 31) / 32 * 32);
+  double best = -1.0;
+  for (int r = 1; r <= p.M + 1; ++r) {
+    const int n = (p.M + r) / r;   // levels per run with r runs
+    const long long per_sm = (tiles * ((p.M + n) / n) + p.nsm - 1) / p.nsm;
+    const double w = per_sm * (n + 1.3) * level * (per_sm == 1 ? 1.0 / 0.7 : 1.0);
+    if (best < 0.0 || w < best) {
+      best = w;
+      *run = n;
+    }
+    if (per_sm > 64) break;   // shorter runs only add levels
+  }
+  return best;
+}
+
+void launch_fp64(const DevProblem& p, const double* x, double* y, const double* b, cudaStream_t s) {
+  if (p.elem == KKT_ELEM_P1) {
+    launch_shape<double, TileA, true>(p, x, y, b, s);
+    return;
+  }
+  int run_a = 1, run_c = 1;
+  const double a = work64<TileA>(p, &run_a), c = work64<TileC>(p, &run_c);
+  if (p.reg != 0) {
+    if (c < a) launch64_tile<true, TileC>(p, x, y, b, run_c, s);
+    else launch64_tile<true, TileA>(p, x, y, b, run_a, s);
+  } else {
+    if (c < a) launch64_tile<false, TileC>(p, x, y, b, run_c, s);
+    else launch64_tile<false, TileA>(p, x, y, b, run_a, s);
+  }
+}
+
 __global__ void d2f(const double* __restrict__ x, float* __restrict__ y, long long n, const int* gate) {
   if (gated_off(gate)) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -454,6 +748,15 @@ kkt_status prepare_shape() {
   return KKT_OK;
 }
 
+template <typename Tl>
+kkt_status prepare64() {
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec64_levels<false, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)mv64_smem<Tl>()));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec64_levels<true, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)mv64_smem<Tl>()));
+  return KKT_OK;
+}
+
 template <typename T>
 kkt_status prepare_p1() {
   KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<T, false, TileA, true>,
@@ -464,8 +767,8 @@ kkt_status prepare_p1() {
 }
 
 kkt_status matvec_prepare() {
-  KKT_TRY((prepare_shape<double, TileA>()));
-  KKT_TRY((prepare_shape<double, TileB>()));
+  KKT_TRY(prepare64<TileA>());
+  KKT_TRY(prepare64<TileC>());
   KKT_TRY((prepare_shape<float, TileA>()));
   KKT_TRY((prepare_shape<float, TileB>()));
   KKT_TRY((prepare_p1<double>()));
@@ -474,7 +777,7 @@ kkt_status matvec_prepare() {
 }
 
 kkt_status launch_matvec64(const DevProblem& p, const double* x, double* y, cudaStream_t s) {
-  launch_tiled<double>(p, x, y, nullptr, s);
+  launch_fp64(p, x, y, nullptr, s);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
@@ -488,7 +791,7 @@ kkt_status launch_matvec32(const DevProblem& p, const float* x, float* y, cudaSt
 }
 
 kkt_status launch_residual(const DevProblem& p, const double* b, const double* x, double* r, cudaStream_t s) {
-  launch_tiled<double>(p, x, r, b, s);
+  launch_fp64(p, x, r, b, s);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
