@@ -701,8 +701,8 @@ struct SolveShape {
   int ch, warps, nstage, lanes;
   bool smem_vec;
 };
-// groups per wavefront from which the largest CTA is taken: boxes one per SM, more boxes than SMs
-constexpr int kFillGroups = 7, kFillGroups2 = 12;
+// groups per wavefront from which the largest CTA is taken
+constexpr int kFillGroups = 4;
 template <typename T, bool SMEM>
 const void* solve_kernel() {
   return (const void*)ras_solve<T, SMEM>;
@@ -715,8 +715,9 @@ struct ShapeRequest {
 // wavefronts fill the largest CTA take it (one per SM, its L1 to itself); others
 // take the shape with the fewest waves of CTAs over the SMs.  Measured at 32^3 x
 // 64, FP32, 256 boxes: fine boxes (15 groups a wavefront) 2.16 ms with 16 warps,
-// 2.46 with 8 (two CTAs an SM), 4.04 with 4; coarse boxes (3 groups) 303, 221,
-// 300 us.  FP64, 64 boxes of 9 groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
+// 2.46 with 8 (two CTAs an SM), 4.04 with 4; coarse boxes (2.5 groups) 303, 221,
+// 300 us; 192 uneven boxes (5.6 groups) 695, 1039, 1633 us.  FP64, 64 boxes of 9
+// groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
 // global memory, the fewest buffers, the largest CTA.  ras_autotune measures instead.
 template <typename T>
 kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int nsm,
@@ -749,7 +750,7 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
             &per_sm, sv ? solve_kernel<T, true>() : solve_kernel<T, false>(), 32 * warps, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
-        const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * (nbox > nsm ? kFillGroups2 : kFillGroups);
+        const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
         const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
         if (best_key < 0 || key < best_key) {
           best_key = key;
