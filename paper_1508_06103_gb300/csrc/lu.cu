@@ -151,17 +151,38 @@ __global__ void __launch_bounds__(kLuThreads) lu_step(const BoxDesc* __restrict_
   }
 }
 
-// z = sum over boxes (R^0)^T M_ij^{-1} R^delta r with the band LU factors
+// z = sum over boxes (R^0)^T M_ij^{-1} R^delta r with the band LU factors.
+//
+// One CTA per box, one column a step, one barrier a step.  Row i belongs to
+// thread i mod 1024: only it writes bvec[i].  What a step needs of other threads' rows
+// -- the pivot row's value and, under an interchange, the value of row j -- their owners
+// publish at the end of the step before, in slots that alternate.  A thread's
+// entries of the next columns are loaded kLuAhead columns ahead into registers and
+// the diagonals' reciprocals formed ahead, so a step's chain is two
+// shared-memory reads, a few FMAs and the barrier.  (With the loads at their use and two
+// barriers a column took 2.3 us.)  What is left is the FP64 pipe: 3 kl FMAs per
+// column and box at 2 a clock.
+constexpr int kLuAhead = 4;
+constexpr int kLuFwd = (kMaxLuBand + kLuThreads - 1) / kLuThreads;       // rows per thread and column, L
+constexpr int kLuBwd = (2 * kMaxLuBand + kLuThreads - 1) / kLuThreads;   // and U
+static_assert((kLuThreads & (kLuThreads - 1)) == 0, "row owners by mask");
+
+// WIDE: a half-bandwidth above kLuThreads (more rows per thread)
+template <bool WIDE>
 __global__ void __launch_bounds__(kLuThreads) lu_solve(const BoxDesc* __restrict__ boxes,
                                                        const double* __restrict__ AB, const int* __restrict__ ipiv,
                                                        const double* __restrict__ r, double* __restrict__ z, int nx,
                                                        int ny, int N, const int* gate) {
   if (gated_off(gate)) return;
-  extern __shared__ __align__(16) double bvec[];
+  constexpr int RF = WIDE ? kLuFwd : 1, RB = WIDE ? kLuBwd : 2;
+  extern __shared__ __align__(16) double lu_sm[];
+  double* pub = lu_sm;        // two alternating slots of {pivot row's value, row j's value} / {x_j}
+  double* bvec = lu_sm + 4;
   const BoxDesc bx = boxes[blockIdx.x];
-  const int n = 3 * (int)bx.P, kl = bx.kl;
+  const int n = 3 * (int)bx.P, kl = bx.kl, ld = 3 * kl + 1, t = threadIdx.x;
   const int* ip = ipiv + 3 * bx.poff;
-  for (int u = threadIdx.x; u < n; u += blockDim.x) {
+  const double* A = AB + bx.aoff + 2 * kl;   // A(i, k) = A[(ld - 1) k + i]
+  for (int u = t; u < n; u += kLuThreads) {
     const int lex = u / 3, c = u - 3 * lex;
     const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
     const int kt = lex / (bx.lx * bx.ly * bx.lz);
@@ -170,31 +191,115 @@ __global__ void __launch_bounds__(kLuThreads) lu_solve(const BoxDesc* __restrict
     bvec[u] = r[g + c];
   }
   __syncthreads();
+  const int mask = kLuThreads - 1;
+
   // forward: interchanges and the unit lower factor
-  for (int j = 0; j < n - 1; ++j) {
-    const int p = ip[j];
-    const double bj = bvec[p];
-    __syncthreads();
-    if (threadIdx.x == 0 && p != j) {
-      bvec[p] = bvec[j];
-      bvec[j] = bj;
+  {
+    double a[kLuAhead][RF];
+    int piv[kLuAhead];
+    auto load = [&](int j, double (&v)[RF], int& pj) {
+      const double* Aj = A + (long long)(ld - 1) * j;
+      const int i = j + 1 + ((t - j - 1) & mask), last = min(j + kl, n - 1);
+#pragma unroll
+      for (int q = 0; q < RF; ++q) v[q] = j < n - 1 && i + q * kLuThreads <= last ? Aj[i + q * kLuThreads] : 0.0;
+      pj = j < n - 1 ? ip[j] : j;
+    };
+#pragma unroll
+    for (int c = 0; c < kLuAhead; ++c) load(c, a[c], piv[c]);
+    if (t == 0) {
+      pub[0] = bvec[piv[0]];
+      pub[1] = bvec[0];
     }
-    const double* Aj = band_col(const_cast<double*>(AB), bx, j);
-    const int km = min(kl, n - 1 - j);
-    for (int t = 1 + threadIdx.x; t <= km; t += blockDim.x)
-      if (j + t != p) bvec[j + t] -= Aj[j + t] * bj;
-    if (threadIdx.x == 0 && p != j) bvec[p] -= Aj[p] * bj;
     __syncthreads();
+    for (int j0 = 0; j0 < n - 1; j0 += kLuAhead) {
+#pragma unroll
+      for (int c = 0; c < kLuAhead; ++c) {
+        const int j = j0 + c;
+        if (j >= n - 1) break;
+        const int p = piv[c];
+        const double bj = pub[2 * (j & 1)], old = pub[2 * (j & 1) + 1];
+        const int i = j + 1 + ((t - j - 1) & mask), last = min(j + kl, n - 1);
+#pragma unroll
+        for (int q = 0; q < RF; ++q) {
+          const int ii = i + q * kLuThreads;
+          if (ii <= last) bvec[ii] = fma(-a[c][q], bj, ii == p ? old : bvec[ii]);
+        }
+        if (t == (j & mask)) bvec[j] = bj;
+        // the next column's pivot row and row, by their owners
+        const int pn = piv[(c + 1) % kLuAhead];   // (loaded: kLuAhead > 1)
+        if (j + 1 < n - 1) {
+          if (t == (pn & mask)) pub[2 * ((j + 1) & 1)] = bvec[pn];
+          if (t == ((j + 1) & mask)) pub[2 * ((j + 1) & 1) + 1] = bvec[j + 1];
+        }
+        load(j + kLuAhead, a[c], piv[c]);
+        __syncthreads();
+      }
+    }
   }
   // backward: U has 2 kl superdiagonals
-  for (int j = n - 1; j >= 0; --j) {
-    const double* Aj = band_col(const_cast<double*>(AB), bx, j);
-    const double xj = bvec[j] / Aj[j];
+  {
+    double a[kLuAhead][RB];
+    auto load = [&](int j, double (&v)[RB]) {
+      const double* Aj = A + (long long)(ld - 1) * j;
+      const int i = j - 1 - ((j - 1 - t) & mask), first = max(0, j - 2 * kl);
+#pragma unroll
+      for (int q = 0; q < RB; ++q) v[q] = j > 0 && i - q * kLuThreads >= first ? Aj[i - q * kLuThreads] : 0.0;
+    };
+    // Diagonals and their reciprocals, a warp's 32 rows at a time: loaded two blocks of 32
+    // columns before they are needed, divided one block before.
+    const int warp = t / 32, warps = kLuThreads / 32;
+    double ahead = 1.0, dg = 1.0, rd = 1.0;
+    auto diag_load = [&](int blk) {
+      if (blk >= 0 && blk % warps == warp) {
+        const int row = 32 * blk + t % 32;
+        ahead = row < n ? A[(long long)(ld - 1) * row + row] : 1.0;
+      }
+    };
+    auto diag_divide = [&](int blk) {
+      if (blk >= 0 && blk % warps == warp) {
+        dg = ahead;
+        rd = 1.0 / dg;
+      }
+    };
+    const int top = (n - 1) / 32;
+    diag_load(top);
+    diag_divide(top);
+    diag_load(top - 1);
+    // x = b / a from the reciprocal, corrected once (as accurate as the division)
+    auto quotient = [&](double v) {
+      const double q = v * rd, e = fma(-dg, q, v);
+      return isfinite(e) ? fma(e, rd, q) : v / dg;
+    };
+#pragma unroll
+    for (int c = 0; c < kLuAhead; ++c)
+      if (n - 1 - c >= 0) load(n - 1 - c, a[c]);
+    if (t == ((n - 1) & mask)) pub[2 * ((n - 1) & 1)] = quotient(bvec[n - 1]);
     __syncthreads();
-    if (threadIdx.x == 0) bvec[j] = xj;
-    const int lo = max(0, j - 2 * kl);
-    for (int i = lo + threadIdx.x; i < j; i += blockDim.x) bvec[i] -= Aj[i] * xj;
-    __syncthreads();
+    for (int j0 = n - 1; j0 >= 0; j0 -= kLuAhead) {
+#pragma unroll
+      for (int c = 0; c < kLuAhead; ++c) {
+        const int j = j0 - c;
+        if (j < 0) break;
+        if (j % 32 == 31 || j == n - 1) {   // a new block of columns: j / 32
+          diag_divide(j / 32 - 1);
+          diag_load(j / 32 - 2);
+        }
+        const double xj = pub[2 * (j & 1)];
+        const int i = j - 1 - ((j - 1 - t) & mask), first = max(0, j - 2 * kl);
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          const int ii = i - q * kLuThreads;
+          if (ii >= first) {
+            const double v = fma(-a[c][q], xj, bvec[ii]);
+            bvec[ii] = v;
+            if (q == 0 && ii == j - 1) pub[2 * ((j - 1) & 1)] = quotient(v);
+          }
+        }
+        if (t == (j & mask)) bvec[j] = xj;
+        if (j - kLuAhead >= 0) load(j - kLuAhead, a[c]);
+        __syncthreads();
+      }
+    }
   }
   // scatter the owned part
   const int ox = bx.ox1 - bx.ox0, oy = bx.oy1 - bx.oy0, oz = bx.oz1 - bx.oz0, ot = bx.ot1 - bx.ot0;
@@ -222,8 +327,10 @@ kkt_status ras_lu_factor(ras_precond* m, cudaStream_t s) {
   }
   // the solve keeps a box's vector in shared memory (at most kMaxLuUnknowns values); the
   // limit is raised here, at set-up, so the solve's launch needs no attribute call
-  KKT_TRY_CUDA(cudaFuncSetAttribute(lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(kMaxLuUnknowns * sizeof(double))));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(lu_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)((kMaxLuUnknowns + 4) * sizeof(double))));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(lu_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)((kMaxLuUnknowns + 4) * sizeof(double))));
   KKT_TRY_CUDA(cudaMemsetAsync(m->AB, 0, m->ab_count * sizeof(double), s));
   KKT_TRY_CUDA(cudaMemsetAsync(m->lu_ju, 0, 2 * m->nbox * sizeof(int), s));
   const dim3 g((unsigned)((pmax + kLuGather - 1) / kLuGather), m->nbox);
@@ -241,10 +348,14 @@ kkt_status ras_lu_factor(ras_precond* m, cudaStream_t s) {
 
 kkt_status ras_lu_solve(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate) {
   const kkt_problem* p = m->prob;
-  int nmax = 0;
-  for (const BoxDesc& b : m->boxes_h) nmax = std::max(nmax, 3 * (int)b.P);
-  const size_t smem = (size_t)nmax * sizeof(double);
-  lu_solve<<<m->nbox, kLuThreads, smem, s>>>(m->boxes, m->AB, m->ipiv, r, z, p->nx, p->ny, p->N, gate);
+  int nmax = 0, klmax = 0;
+  for (const BoxDesc& b : m->boxes_h) {
+    nmax = std::max(nmax, 3 * (int)b.P);
+    klmax = std::max(klmax, b.kl);
+  }
+  const size_t smem = ((size_t)nmax + 4) * sizeof(double);
+  auto* kernel = klmax > kLuThreads ? lu_solve<true> : lu_solve<false>;   // L and U rows per thread: 2 and 4, or 1 and 2
+  kernel<<<m->nbox, kLuThreads, smem, s>>>(m->boxes, m->AB, m->ipiv, r, z, p->nx, p->ny, p->N, gate);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;

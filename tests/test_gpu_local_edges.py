@@ -77,3 +77,30 @@ def test_ras_apply_on_edge_shapes_matches_oracle(api, oracle, name, prec):
         else:
             assert np.linalg.norm(z - zr) <= (1e-3 if prec == 32 else 8 * 2.0**-8) * np.linalg.norm(zr)
         ras.refactor()
+
+
+# exact local LU: bands within one CTA's threads and beyond, fewer unknowns than threads
+LU_CASES = {
+    "few-unknowns": ((1, 1, 1), 3, (1, 1, 1, 1), 0),
+    "band-in-one-pass": ((5, 5, 6), 3, (1, 1, 1, 1), 0),
+    "band-over-one-pass": ((6, 6, 7), 3, (1, 1, 1, 1), 0),
+}
+
+
+@pytest.mark.parametrize("name", LU_CASES)
+def test_exact_lu_on_edge_shapes_matches_oracle(api, name):
+    # bar: 100 cond_1 u max|z|, as in test_gpu_solve.py (both sides backward stable)
+    cells, M, nsub, ov = LU_CASES[name]
+    w = W.random_small(43, cells=cells, M=M, nsens=4, reg="h1l2")
+    beta = max(w.h) ** 2
+    w = dataclasses.replace(w, T=M / 16.0, beta1=beta / 100, beta2=beta)
+    p = okkt.Problem.from_workload(w)
+    F = okkt.assemble(p)
+    ref = osch.RAS(p, F, nsub, ov, "lu")
+    kappa = max(np.linalg.cond(F[idx][:, idx].toarray(), 1) for idx in ref.idx)
+    prob = api.Problem.from_workload(w)
+    ras = api.RAS(prob, nsub, ov, 64, local="lu")
+    for seed in (1, 2):
+        r = W.random_vector(prob.n, seed)
+        z, zr = ras.apply(torch.from_numpy(r).cuda()).cpu().numpy(), ref.apply(r)
+        assert np.abs(z - zr).max() <= 100 * kappa * 2.0**-53 * np.abs(zr).max()
