@@ -31,13 +31,17 @@
 //
 // Solve.  One CTA per box: gather R^delta r, forward and backward sweeps by
 // wavefront over the same slot lists (a warp per point), scatter the owned
-// points.
+// points.  A slot's column comes from a table in shared memory (its offset in the
+// box and the range of positions that have it), the box's vector sits there too
+// where it fits; the point-block rows' values are loaded a point ahead and the
+// three rows' columns together.
 
 #include <algorithm>
 #include <array>
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "ras.cuh"
@@ -231,8 +235,8 @@ struct GpFactor {
 
 namespace {
 
+constexpr int kGpSmemLimit = 112 * 1024;   // two CTAs of the solve per SM
 constexpr int kGpThreads = 192;        // factor CTA (row buffers: 6 warps x 800 slots fit 48 KB in FP64)
-constexpr int kGpSolveThreads = 256;
 
 __device__ __forceinline__ int gp_row_of(const GpTables& tb, int s) {
   return s < tb.base[1] ? 0 : (s < tb.base[2] ? 1 : 2);
@@ -375,64 +379,168 @@ __global__ void __launch_bounds__(kGpThreads) gp_factor(const BoxDesc* __restric
 // wavefront, one warp per point and row, its lanes summing over the slots
 // (slots whose column leaves the box are skipped; dropped entries hold 0),
 // and writes its owned points.
-template <typename T>
-__global__ void __launch_bounds__(kGpSolveThreads) gp_solve(const DevProblem* __restrict__ probs,
-                                                       const BoxDesc* __restrict__ boxes, const GpBox* __restrict__ gb,
-                                                       const int* __restrict__ perm,
-                                                       const int* __restrict__ lptr, GpTables tb,
-                                                       const T* __restrict__ F, T* __restrict__ V,
-                                                       const double* __restrict__ r, double* __restrict__ z,
-                                                       const int* gate) {
+//
+// NIT: 32-slot steps of the longest row half.  BLOCK (the point-block pattern, 4
+// steps): all three rows' values and columns are in registers at once, the values
+// loaded a point ahead; a column of the point itself takes the value just solved.
+// What bounds it is latency: a wavefront of 18 points (16^3 x 32, 4^4 boxes) is a
+// round or two of the CTA's 12 warps.  Measured there, FP32: 5.47 -> 1.12 ms, FP64 7.09 -> 2.84, against
+// index arithmetic per slot, rows one after the other, 8 warps; ILU(1) at 9^3 x 12, 3^4 boxes: 3.71 -> 1.10.
+constexpr int kGpOwn = 1 << 22, kGpComp = 20;   // slot table: the point's own column, component (2 bits)
+template <int NIT>
+constexpr int gp_solve_threads() {
+  return NIT <= 4 ? 384 : 256;
+}
+
+template <typename T, int NIT, bool SMEM>
+__global__ void __launch_bounds__(gp_solve_threads<NIT>(), 2) gp_solve(
+    const DevProblem* __restrict__ probs, const BoxDesc* __restrict__ boxes, const GpBox* __restrict__ gb,
+    const int* __restrict__ perm, const int* __restrict__ lptr, GpTables tb, const T* __restrict__ F,
+    T* __restrict__ V, const double* __restrict__ r, double* __restrict__ z, const int* gate) {
   if (gated_off(gate)) return;
+  constexpr bool BLOCK = NIT <= 4;
+  constexpr int nwarp = gp_solve_threads<NIT>() / 32;
+  extern __shared__ __align__(16) unsigned char gp_sm[];
+  int2* info = reinterpret_cast<int2*>(gp_sm);   // [S]: offset in the box's vector, positions that have the slot
   const BoxDesc bx = boxes[blockIdx.x];
   const GpBox g = gb[blockIdx.x];
-  const DevProblem p = probs[bx.prob];
-  T* Vb = V + g.voff;
+  const int nx = probs[bx.prob].nx, ny = probs[bx.prob].ny, N = probs[bx.prob].N;
+  T* Vb = SMEM ? reinterpret_cast<T*>(info + tb.S) : V + g.voff;
+  const T* Fb = F + g.foff;
+  const int* pm = perm + g.poff;
+  const int* lp = lptr + g.loff;
   const int lane = threadIdx.x & 31, wp = threadIdx.x / 32;
+  for (int s = threadIdx.x; s < tb.S; s += blockDim.x) {
+    const signed char* sl = tb.slot + 5 * s;
+    const int dt = sl[0], dz = sl[1], dy = sl[2], dx = sl[3], cc = sl[4];
+    const bool own = dt == 0 && dz == 0 && dy == 0 && dx == 0;
+    info[s] = make_int2(3 * (dx + bx.lx * (dy + bx.ly * (dz + bx.lz * dt))) + cc,
+                        1 << (dx + 2) | 1 << (dy + 7) | 1 << (dz + 12) | 1 << (dt + 17) | cc << kGpComp | (own ? kGpOwn : 0));
+  }
   auto global_point = [&](int lex) {
     const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
     const int kt = lex / (bx.lx * bx.ly * bx.lz);
-    return (long long)(bx.t0 + kt) * p.N + (bx.x0 + kx) + (long long)p.nx * ((bx.y0 + ky) + (long long)p.ny * (bx.z0 + kz));
+    return (long long)(bx.t0 + kt) * N + (bx.x0 + kx) + (long long)nx * ((bx.y0 + ky) + (long long)ny * (bx.z0 + kz));
   };
   for (int lex = threadIdx.x; lex < g.P; lex += blockDim.x) {   // R^delta r
     const long long gi = 3 * global_point(lex);
     for (int c = 0; c < 3; ++c) Vb[3 * lex + c] = (T)r[gi + c];
   }
   __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
+  // offsets -2..2 that stay inside an axis of n at position k
+  auto inside = [](int k, int n) {
+    int m = 0;
+#pragma unroll
+    for (int d = -2; d <= 2; ++d) m |= (k + d >= 0 && k + d < n ? 1 : 0) << (d + 2);
+    return m;
+  };
+  auto sweep = [&](auto pass_tag) {
+    constexpr int pass = decltype(pass_tag)::value;   // 0 forward, 1 backward
+    auto first = [&](int c) { return pass == 0 ? 0 : tb.diag[c] + 1; };
+    auto count = [&](int c) { return pass == 0 ? tb.diag[c] : tb.cnt[c] - tb.diag[c] - 1; };
+    T v[BLOCK ? 3 : 1][NIT];
+    auto values = [&](int lex, int c, T (&o)[NIT]) {
+      const T* Fp = Fb + (long long)lex * tb.S + tb.base[c] + first(c);
+      const int n = count(c);
+#pragma unroll
+      for (int k = 0; k < NIT; ++k) o[k] = 32 * k + lane < n ? Fp[32 * k + lane] : (T)0;
+    };
+    // the warp's first point of a wavefront, its values loaded before the wavefront before ends
+    auto wave = [&](int wi) { return pass == 0 ? wi : g.nlev - 1 - wi; };
+    int q = lp[wave(0)] + wp, q1 = lp[wave(0) + 1], lex = q < q1 ? pm[q] : -1;
+    if (BLOCK && lex >= 0)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) values(lex, c, v[BLOCK ? c : 0]);
     for (int wi = 0; wi < g.nlev; ++wi) {
-      const int w = pass == 0 ? wi : g.nlev - 1 - wi;
-      const int l0 = lptr[g.loff + w], l1 = lptr[g.loff + w + 1];
-      for (int q = l0 + wp; q < l1; q += kGpSolveThreads / 32) {
-        const int lex = perm[g.poff + q];
+      const int wn = wave(min(wi + 1, g.nlev - 1)), qn = lp[wn] + wp, qn1 = wi + 1 < g.nlev ? lp[wn + 1] : 0;
+      while (q < q1) {
         const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
         const int kt = lex / (bx.lx * bx.ly * bx.lz);
-        const T* Fp = F + g.foff + (long long)lex * tb.S;
-        for (int ci = 0; ci < 3; ++ci) {
-          const int c = pass == 0 ? ci : 2 - ci;
-          const int b = tb.base[c], dg = tb.diag[c];
-          const int s0 = pass == 0 ? 0 : dg + 1, s1 = pass == 0 ? dg : tb.cnt[c];
+        const int here = inside(kx, bx.lx) | inside(ky, bx.ly) << 5 | inside(kz, bx.lz) << 10 | inside(kt, bx.lt) << 15;
+        const T* Vp = Vb + 3 * lex;
+        T x[BLOCK ? 3 : 1][NIT], sol[3] = {0, 0, 0}, old[3], inv[3];
+        int own_k[3], own_c[3];   // the lane's slot of the point itself in row c: step (or -1) and component
+        auto columns = [&](int c, T (&o)[NIT]) {
+          const int n = count(c), b = tb.base[c] + first(c);
+          own_k[c] = -1;
+          own_c[c] = 0;
+#pragma unroll
+          for (int k = 0; k < NIT; ++k) {
+            o[k] = (T)0;
+            if (32 * k + lane < n) {
+              const int2 e = info[b + 32 * k + lane];
+              if (e.y & kGpOwn) {
+                own_k[c] = k;
+                own_c[c] = e.y >> kGpComp & 3;
+              } else if ((e.y & here) == (e.y & 0xfffff)) {
+                o[k] = Vp[e.x];
+              }
+            }
+          }
+        };
+        const T* Fp = Fb + (long long)lex * tb.S;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          old[c] = Vp[c];
+          inv[c] = pass == 1 ? Fp[tb.base[c] + tb.diag[c]] : (T)1;
+        }
+        if (BLOCK)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) columns(c, x[BLOCK ? c : 0]);
+        // the next point's index (and, point-block, its values, once this point's are used)
+        int qx = q + nwarp, lexn = -1;
+        if (qx < q1) lexn = pm[qx];
+        else if (qn < qn1) lexn = pm[qn];
+        auto row = [&](int c) {
+          if (!BLOCK) {
+            values(lex, c, v[0]);
+            columns(c, x[0]);
+          }
           T part = (T)0;
-#pragma unroll 4
-          for (int s = s0 + lane; s < s1; s += 32) {
-            // the column from the slot table alone, so the value and vector loads are independent
-            const signed char* sl = tb.slot + 5 * (b + s);
-            const int cl = gp_col_lex(bx, sl, kx, ky, kz, kt);
-            const T v = Fp[b + s];
-            if (cl >= 0) part += v * Vb[3 * cl + sl[4]];
+#pragma unroll
+          for (int k = 0; k < NIT; ++k) {
+            T xk = x[BLOCK ? c : 0][k];
+            if (k == own_k[c]) xk = own_c[c] == 0 ? sol[0] : own_c[c] == 1 ? sol[1] : sol[2];
+            part += v[BLOCK ? c : 0][k] * xk;
           }
           for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-          if (lane == 0) {
-            T acc = Vb[3 * lex + c] - part;
-            if (pass == 1) acc *= Fp[b + dg];   // the stored 1 / u_ii
-            Vb[3 * lex + c] = acc;
-          }
-          __syncwarp();
+          T acc = old[c] - part;
+          if (pass == 1) acc *= inv[c];   // the stored 1 / u_ii
+          sol[c] = acc;
+        };
+        if (pass == 0) {
+          row(0);
+          row(1);
+          row(2);
+        } else {
+          row(2);
+          row(1);
+          row(0);
         }
+        if (lane < 3) Vb[3 * lex + lane] = lane == 0 ? sol[0] : lane == 1 ? sol[1] : sol[2];
+        if (BLOCK && lexn >= 0)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) values(lexn, c, v[BLOCK ? c : 0]);
+        q = qx;
+        if (q < q1) lex = lexn;
       }
       __syncthreads();
+      // (a warp without a point in this wavefront has not looked at the next one yet)
+      if (wi + 1 < g.nlev) {
+        const bool had = lp[wave(wi)] + wp < q1;
+        q = qn;
+        q1 = qn1;
+        if (q < q1) {
+          lex = pm[q];
+          if (BLOCK && !had)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) values(lex, c, v[BLOCK ? c : 0]);
+        }
+      }
     }
-  }
+  };
+  sweep(std::integral_constant<int, 0>{});
+  sweep(std::integral_constant<int, 1>{});
   for (int lex = threadIdx.x; lex < g.P; lex += blockDim.x) {   // (R^0)^T: owned points only
     const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
     const int kt = lex / (bx.lx * bx.ly * bx.lz);
@@ -470,17 +578,45 @@ kkt_status gp_factor(ras_precond* m, cudaStream_t s) {
   return m->gp->prec == 64 ? gp_factor_t<double>(m, s) : gp_factor_t<float>(m, s);
 }
 
-kkt_status gp_solve(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate) {
+namespace {
+
+// shared memory of the solve: the slot table, and the largest box vector where two CTAs fit an SM with it
+size_t gp_solve_smem(const GpFactor* f, bool* vec) {
+  int pmax = 0;
+  for (const GpBox& b : f->boxes_h) pmax = std::max(pmax, b.P);
+  const size_t table = (size_t)f->tab.S * sizeof(int2);
+  const size_t v = 3 * (size_t)pmax * (f->prec == 64 ? sizeof(double) : sizeof(float));
+  *vec = table + v <= kGpSmemLimit;
+  return table + (*vec ? v : 0);
+}
+
+template <typename T, int NIT>
+kkt_status gp_solve_launch(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate) {
   GpFactor* f = m->gp;
-  if (f->prec == 64)
-    gp_solve<double><<<m->nbox, kGpSolveThreads, 0, s>>>(m->dprobs, m->boxes, f->boxes, f->perm, f->lptr, f->tab,
-                                                    (const double*)f->F, (double*)f->V, r, z, gate);
-  else
-    gp_solve<float><<<m->nbox, kGpSolveThreads, 0, s>>>(m->dprobs, m->boxes, f->boxes, f->perm, f->lptr, f->tab,
-                                                   (const float*)f->F, (float*)f->V, r, z, gate);
+  bool vec = false;
+  const size_t smem = gp_solve_smem(f, &vec);
+  auto* kernel = vec ? gp_solve<T, NIT, true> : gp_solve<T, NIT, false>;
+  kernel<<<m->nbox, gp_solve_threads<NIT>(), smem, s>>>(m->dprobs, m->boxes, f->boxes, f->perm, f->lptr, f->tab,
+                                                        (const T*)f->F, (T*)f->V, r, z, gate);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
+}
+
+template <typename T, int NIT>
+kkt_status gp_solve_prepare() {   // raises the shared-memory limit, at set-up
+  KKT_TRY_CUDA(cudaFuncSetAttribute(gp_solve<T, NIT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGpSmemLimit));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(gp_solve<T, NIT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGpSmemLimit));
+  return KKT_OK;
+}
+
+}  // namespace
+
+kkt_status gp_solve(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate) {
+  const bool block = m->gp->local == 3;
+  if (m->gp->prec == 64)
+    return block ? gp_solve_launch<double, 4>(m, r, z, s, gate) : gp_solve_launch<double, 14>(m, r, z, s, gate);
+  return block ? gp_solve_launch<float, 4>(m, r, z, s, gate) : gp_solve_launch<float, 14>(m, r, z, s, gate);
 }
 
 void gp_destroy(ras_precond* m) {
@@ -645,6 +781,13 @@ kkt_status gp_create(ras_precond* m, int local, int prec) {
     set_error("ras_setup: device allocation failed (" + std::to_string(f->fcount) + " factor values)");
     return KKT_ERR_NOMEM;
   }
+  for (int c = 0; c < 3; ++c)
+    if (std::max(tb.diag[c], tb.cnt[c] - tb.diag[c] - 1) > 32 * (local == 3 ? 4 : 14)) {
+      set_error("ras_setup: internal error: a pattern row exceeds the solve's steps");
+      return KKT_ERR_ARG;
+    }
+  KKT_TRY((prec == 64 ? (local == 3 ? gp_solve_prepare<double, 4>() : gp_solve_prepare<double, 14>())
+                      : (local == 3 ? gp_solve_prepare<float, 4>() : gp_solve_prepare<float, 14>())));
   tb.slot = f->slot;
   tb.smap = f->smap;
   tb.tptr = f->tptr;
