@@ -246,7 +246,7 @@ __global__ void wait_selftest(int* status, unsigned long long limit_ns) {
 // warp's own buffers in shared memory, asked for while the warp still works on
 // the groups before.  (Loads through L1 into registers ahead of their use were
 // measured slower, 2.30 against 2.16 ms at 32^3 x 64: the neighbours' loads wait
-// behind them in L1's queue.)  The warps of a box do not meet at
+// behind them in L1's queue.  Chunks of 52 points with a CTA barrier each: 2.81.)  The warps of a box do not meet at
 // wavefronts: a counter of finished groups in shared memory tells a warp when
 // the wavefronts before its group's are done.  What does not depend on the
 // last of them -- all neighbours but those one wavefront away -- is loaded and
@@ -386,19 +386,34 @@ __host__ __device__ constexpr int dep_lanes(bool upper, int i) {
   return upper ? (i == 0 ? 3 : i == 1 ? 1 : i == 3 ? 2 : 0) : (i == 6 ? 4 : i == 8 ? 8 : i == 9 ? 12 : 0);
 }
 
+// The ring of wavefronts (FP32, BF16 where it fits): the solved values of the last 16
+// wavefronts, 4 values a point, wavefront w in slot w mod 16 at the places of its
+// groups, and one point of zeros for columns outside the box.  No neighbour lies
+// more than 15 wavefronts away.  A table holds the ring place of every neighbour (10
+// of 16 bits a lane, sweep and group, 12 % more bytes than the FP32 values) and comes with
+// the factor values.  Through L1 a group's 10 neighbour loads touch 16 to 24 lines
+// each.  Measured, one apply: 32^3 x 64 FP32 2150 -> 2047 us, BF16 2038 -> 1857; coarse 16^3 x
+// 32 FP32 211 -> 191; 40^3 x 39 BF16 1433 -> 1345; 192 uneven boxes 695 -> 597; 16 boxes 638 ->
+// 650 (not used there).  What is left is the latency of a group's 600 instructions.
+constexpr int kNbrBytes = 32 * kNbrPerLane * 2;
+constexpr int kRingWaves = 16;
+constexpr int kMaxRingPlaces = 65535 / kRingWaves - 1;   // places a wavefront, in 16 bits
+
 // Bytes of a warp's factor buffer (the lower half of a group is the larger one).
 template <typename S>
-constexpr int solve_buffer() {
-  return LaneFactors<S>::kStaged ? 32 * kLaneL * (int)sizeof(S) : 0;
+constexpr int solve_buffer(bool ring) {
+  return LaneFactors<S>::kStaged ? 32 * kLaneL * (int)sizeof(S) + (ring ? kNbrBytes : 0) : 0;
 }
+constexpr unsigned kPollNs = 20;
 constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter of finished groups, abort word
 
-template <typename S, bool SMEM>
+template <typename S, bool SMEM, bool RING>
 __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr, const S* __restrict__ F,
     typename SolveArith<S>::type* __restrict__ V, const double* __restrict__ r, double* __restrict__ z,
-    const int2* __restrict__ gtab, const int2* __restrict__ otab, const int* __restrict__ vtab, int gptr_bytes,
-    int nbuf, int* __restrict__ status, const int* gate, int gate_stride) {
+    const int2* __restrict__ gtab, const int2* __restrict__ otab, const int* __restrict__ vtab,
+    const unsigned short* __restrict__ ntab, int wcap, int gptr_bytes, int nbuf, int* __restrict__ status,
+    const int* gate, int gate_stride) {
   using T = typename SolveArith<S>::type;
   constexpr bool kStaged = LaneFactors<S>::kStaged;
   // the box's problem gate (one problem: gate_stride 0, every box reads gate[0])
@@ -417,8 +432,10 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   const int sub = lane & (kLanes - 1);
   // shared memory: header, group pointers, the warps' factor buffers, the local vector
   unsigned char* bufs = smem + kSolveHeader + gptr_bytes;
-  T* v = SMEM ? reinterpret_cast<T*>(bufs + (size_t)nwarp * nbuf * solve_buffer<S>()) : V + bx.voff;
-  S* mine = reinterpret_cast<S*>(bufs + (size_t)warp * nbuf * solve_buffer<S>());
+  unsigned char* rest = bufs + (size_t)nwarp * nbuf * solve_buffer<S>(RING);   // the ring or the local vector
+  T* v = SMEM ? reinterpret_cast<T*>(rest) : V + bx.voff;
+  T* ring = reinterpret_cast<T*>(rest);   // RING: [16][wcap] points and the zeros
+  unsigned char* mine = bufs + (size_t)warp * nbuf * solve_buffer<S>(RING);
   unsigned long long* bar = bars + warp * (kMaxStages - 1);
   const int* gp = gptr + bx.loff;   // first group of every wavefront
   if (gptr_bytes) {
@@ -431,6 +448,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     mbar_fence_init();
   }
   if (threadIdx.x == 0) *finished = *aborted = 0;
+  if (RING && threadIdx.x < kVecWidth) ring[kVecWidth * kRingWaves * wcap + threadIdx.x] = (T)0;
   if (SMEM)
     for (int i = threadIdx.x; i < kVecWidth * st * (bx.lt + 2); i += blockDim.x) v[i] = (T)0;
   __syncthreads();
@@ -445,16 +463,20 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     if (kStaged && k < 2 * ng && lane == 0) {
       const bool up = k >= ng;
       const unsigned bytes = 32 * (up ? kLaneU : kLaneL) * (unsigned)sizeof(S);
+      unsigned char* to = mine + (t % nbuf) * solve_buffer<S>(RING);
       fence_proxy_async();
-      mbar_expect_tx(&bar[t % nbuf], bytes);
-      bulk_g2s(mine + (t % nbuf) * (solve_buffer<S>() / (int)sizeof(S)),
-               Fb + (long long)group(k) * kGroupVals32 + (up ? 32 * kLaneL : 0), bytes, &bar[t % nbuf]);
+      mbar_expect_tx(&bar[t % nbuf], bytes + (RING ? kNbrBytes : 0));
+      bulk_g2s(to, Fb + (long long)group(k) * kGroupVals32 + (up ? 32 * kLaneL : 0), bytes, &bar[t % nbuf]);
+      if (RING)
+        bulk_g2s(to + 32 * kLaneL * sizeof(S), ntab + (2 * (bx.goff + group(k)) + (up ? 1 : 0)) * (kNbrBytes / 2),
+                 kNbrBytes, &bar[t % nbuf]);
     }
   };
   for (int t = 0; t < nbuf; ++t) issue(warp + t * nwarp, t);
-  // the point of the group after the next one is loaded a group ahead: the neighbours' addresses
-  // come from it
-  int vq = warp < 2 * ng ? vt[kGroup * group(warp) + lane / kLanes] : 0;
+  // the points of the warp's next two groups: the neighbours' and the own point's addresses
+  // come from them
+  auto point = [&](int k) { return k < 2 * ng ? vt[kGroup * group(k) + lane / kLanes] : 0; };
+  int vq = point(warp), vq2 = point(warp + nwarp);
   // R^delta r into the padded local vector (gtab: per box point, its global unknown index and
   // its padded offset); four points at a time, so that their loads overlap
   for (int q0 = threadIdx.x; q0 < P; q0 += 4 * blockDim.x) {
@@ -479,6 +501,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   auto wait_done = [&](int n) -> bool {
     unsigned long long t0 = 0;
     for (unsigned it = 0; ld_acquire_cta(finished) < n; ++it) {
+      __nanosleep(kPollNs);   // a warp that polls without a pause takes issue slots from those at work
       if ((it & 255u) == 255u) {
         const unsigned long long now = global_ns();
         if (t0 == 0) t0 = now;
@@ -495,6 +518,8 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   int off[kNbrPerLane];   // offsets of the lane's neighbours in the padded local vector
   int s = 0, t = 0;       // step of the warp's group, number of its groups so far
   int k = warp;
+  T v0 = 0, v1 = 0, v2 = 0, a0 = 0, a1 = 0, a2 = 0;   // the own point's values, of this group and the next
+  bool ahead = false;                                 // the next one's are loaded
   // one sweep: the warp's groups k < kend
   auto sweep = [&](int kend, auto upper_tag) -> bool {
     constexpr bool kUpper = decltype(upper_tag)::value;
@@ -502,13 +527,20 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       while (k >= before(s + 1)) ++s;
       const bool act = vq >= 0;
       T* vp = v + (act ? vq : ~vq);
-      if (k + nwarp < 2 * ng) vq = vt[kGroup * group(k + nwarp) + lane / kLanes];
+      vq = vq2;
+      vq2 = point(k + 2 * nwarp);
+      unsigned places[kNbrPerLane / 2];   // RING: the neighbours' places, two a word
       if (kStaged) {
         if (!mbar_wait(&bar[t % nbuf], (unsigned)(t / nbuf) & 1u, status)) {
           atomicExch(aborted, 1);
           return false;
         }
-        fac.load(mine + (t % nbuf) * (solve_buffer<S>() / (int)sizeof(S)), kUpper, lane);
+        const unsigned char* from = mine + (t % nbuf) * solve_buffer<S>(RING);
+        fac.load(reinterpret_cast<const S*>(from), kUpper, lane);
+        if constexpr (RING)
+#pragma unroll
+          for (int i = 0; i < kNbrPerLane / 2; ++i)
+            places[i] = reinterpret_cast<const unsigned*>(from + 32 * kLaneL * sizeof(S))[kNbrPerLane / 2 * lane + i];
         __syncwarp();
         issue(k + nbuf * nwarp, t + nbuf);
       } else {
@@ -517,19 +549,34 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       // neighbours two and more wavefronts away (at the first backward step the own point is one
       // of the last wavefront's)
       if (!wait_done(s == nlev ? ng : before(max(s - 1, 0)))) return false;
-      T v0, v1, v2;
-      ld3(vp, v0, v1, v2);
+      if (RING && ahead) {
+        v0 = a0;
+        v1 = a1;
+        v2 = a2;
+      } else {
+        ld3(vp, v0, v1, v2);
+      }
+      if constexpr (RING) {   // the next own point's (in the backward sweep all forward values are there by now)
+        ahead = k + nwarp < kend;
+        if (ahead) ld3(v + (vq >= 0 ? vq : ~vq), a0, a1, a2);
+      }
       T nc[kNbrPerLane], nG[kNbrPerLane], nf[kNbrPerLane];   // the neighbours' unknowns
+      auto neighbour = [&](int i) {
+        if constexpr (RING)
+          ld3(ring + kVecWidth * (i % 2 ? places[i / 2] >> 16 : places[i / 2] & 0xffffu), nc[i], nG[i], nf[i]);
+        else
+          ld3(vp + off[i], nc[i], nG[i], nf[i]);
+      };
 #pragma unroll
       for (int i = 0; i < kNbrPerLane; ++i)
-        if (!(dep_lanes(kUpper, i) >> sub & 1)) ld3(vp + off[i], nc[i], nG[i], nf[i]);
+        if (!(dep_lanes(kUpper, i) >> sub & 1)) neighbour(i);
       T sc = 0, sg = 0, sf = 0;
       T rc = 0, rg = 0, rf = 0, cf = 0, own_c = 0, own_g = 0;
       if constexpr (sizeof(T) == 8) {
         if (!wait_done(before(s))) return false;
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i)
-          if (dep_lanes(kUpper, i) >> sub & 1) ld3(vp + off[i], nc[i], nG[i], nf[i]);
+          if (dep_lanes(kUpper, i) >> sub & 1) neighbour(i);
         // one FMA per product into two chains per sum (the FP64 pipe is the limit)
         T sc1 = 0, sf1 = 0;
 #pragma unroll
@@ -591,7 +638,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
         if (!wait_done(before(s))) return false;
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i)
-          if (dep_lanes(kUpper, i) >> sub & 1) ld3(vp + off[i], nc[i], nG[i], nf[i]);
+          if (dep_lanes(kUpper, i) >> sub & 1) neighbour(i);
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i)
           if (dep_lanes(kUpper, i) >> sub & 1) products(i);
@@ -611,6 +658,10 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       sc = lane_sum(sc);
       sg = lane_sum(sg);
       sf = lane_sum(sf);
+      auto place = [&]() {   // of the point in the ring
+        const int w = s < nlev ? s : 2 * nlev - 1 - s;
+        return kVecWidth * (w % kRingWaves * wcap + kGroup * (group(k) - gp[w]) + lane / kLanes);
+      };
       if (act && sub == 0) {
         if constexpr (!kUpper) {
           // own-point terms in C, G, f order: the G row's own-C and the f row's own-G slot
@@ -618,12 +669,14 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
           const T yg = v1 - sg - own_c * yc;
           const T yf = v2 - sf - own_g * yg;
           st3(vp, yc, yg, yf);
+          if (RING) st3(ring + place(), yc, yg, yf);
         } else {
           // the C row's own-point f column is applied after the f row is solved
           const T zf = (v2 - sf) * rf;
           const T zg = (v1 - sg) * rg;
           const T zc = (v0 - sc - cf * zf) * rc;
           st3(vp, zc, zg, zf);
+          if (RING) st3(ring + place(), zc, zg, zf);
         }
       }
       __syncwarp();
@@ -637,6 +690,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     off[i] = kVecWidth * ((d % 3 - 1) + sy * ((d / 3) % 3 - 1) + sz * (d / 9 - 1) + st * dt);
   }
   bool ok = sweep(ng, std::false_type{});   // forward, unit lower factor
+  ahead = false;
   if (ok) {
 #pragma unroll
     for (int i = 0; i < kNbrPerLane; ++i) {   // later neighbour q: level n, d = 14 + q (q < 13); level n+1, d = q - 13
@@ -669,6 +723,56 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   }
 }
 
+// Ring places of every neighbour of every group place (see kNbrBytes): one thread per lane and
+// group.  inv: group place of every box point.
+__global__ void place_points(const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr,
+                             const int* __restrict__ perm, int* __restrict__ inv) {
+  const BoxDesc bx = boxes[blockIdx.y];
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= kGroup * gptr[bx.loff + bx.nlev]) return;
+  const int lex = perm[kGroup * bx.goff + q];
+  if (lex >= 0) inv[bx.poff + lex] = q;
+}
+__global__ void neighbour_places(const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr,
+                                 const int* __restrict__ perm, const int* __restrict__ inv, int wcap,
+                                 unsigned short* __restrict__ out) {
+  const BoxDesc bx = boxes[blockIdx.y];
+  const int* gp = gptr + bx.loff;
+  const int g = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32, sub = lane % kLanes;
+  if (g >= gp[bx.nlev]) return;
+  const int lex = perm[kGroup * (bx.goff + g) + lane / kLanes];
+  const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
+  const int kt = lex / (bx.lx * bx.ly * bx.lz);
+  for (int up = 0; up < 2; ++up)
+    for (int i = 0; i < kNbrPerLane; ++i) {
+      const int q = sub + kLanes * i;
+      const int d = up ? (q < 13 ? 14 + q : q - 13) : (q < 27 ? q : q - 27), dt = up ? (q < 13 ? 0 : 1) : (q < 27 ? -1 : 0);
+      const int x = kx + d % 3 - 1, y = ky + d / 3 % 3 - 1, z = kz + d / 9 - 1, t = kt + dt;
+      int place = kRingWaves * wcap;
+      if (lex >= 0 && x >= 0 && x < bx.lx && y >= 0 && y < bx.ly && z >= 0 && z < bx.lz && t >= 0 && t < bx.lt) {
+        const int w = x + 2 * y + 4 * z + 8 * t;
+        place = w % kRingWaves * wcap + inv[bx.poff + x + bx.lx * (y + bx.ly * (z + bx.lz * t))] - kGroup * gp[w];
+      }
+      out[((2 * (bx.goff + g) + up) * 32 + lane) * kNbrPerLane + i] = (unsigned short)place;
+    }
+}
+
+// places of the largest wavefront of a box (whole groups)
+int widest_wavefront(const int l[4]) {
+  std::vector<int> h(1, 1);
+  for (int a = 0; a < 4; ++a) {
+    const int step = 1 << a;
+    std::vector<int> n(h.size() + (size_t)step * (l[a] - 1), 0);
+    for (size_t i = 0; i < n.size(); ++i) {   // n[i] = sum over k < l[a] of h[i - step k]
+      n[i] = (i >= (size_t)step ? n[i - step] : 0) + (i < h.size() ? h[i] : 0);
+      const size_t out = (size_t)step * l[a];
+      if (i >= out && i - out < h.size()) n[i] -= h[i - out];
+    }
+    h.swap(n);
+  }
+  return (*std::max_element(h.begin(), h.end()) + kGroup - 1) / kGroup * kGroup;
+}
+
 std::vector<std::pair<int, int>> parts(int n, int p) {
   std::vector<std::pair<int, int>> out;
   const int base = n / p, extra = n % p;
@@ -693,19 +797,22 @@ int gptr_smem(int nlev) {
 int solve_buffers(int nstage) { return nstage - 1; }
 // dynamic shared memory of the solve without the local vector
 template <typename S>
-size_t solve_smem(int nlev, int warps, int nstage) {
-  return kSolveHeader + gptr_smem(nlev) + (size_t)warps * solve_buffers(nstage) * solve_buffer<S>();
+size_t solve_smem(int nlev, int warps, int nstage, bool ring) {
+  return kSolveHeader + gptr_smem(nlev) + (size_t)warps * solve_buffers(nstage) * solve_buffer<S>(ring);
 }
+size_t ring_smem(int wcap) { return ((size_t)kRingWaves * wcap + 1) * kVecWidth * sizeof(float); }
 
 struct SolveShape {
   int ch, warps, nstage, lanes;
-  bool smem_vec;
+  bool smem_vec, ring;
 };
 // groups per wavefront from which the largest CTA is taken
 constexpr int kFillGroups = 4;
-template <typename T, bool SMEM>
-const void* solve_kernel() {
-  return (const void*)ras_solve<T, SMEM>;
+template <typename T>
+const void* solve_kernel(bool smem_vec, bool ring) {
+  if constexpr (LaneFactors<T>::kStaged)
+    if (ring) return (const void*)ras_solve<T, false, true>;
+  return smem_vec ? (const void*)ras_solve<T, true, false> : (const void*)ras_solve<T, false, false>;
 }
 // A requested shape (ras_setup_shape): 0 in a field leaves it to the chooser.
 struct ShapeRequest {
@@ -713,23 +820,22 @@ struct ShapeRequest {
 };
 // Picks the best shape allowed by `req`; KKT_ERR_ARG when none is.  Boxes whose
 // wavefronts fill the largest CTA take it (one per SM, its L1 to itself); others
-// take the shape with the fewest waves of CTAs over the SMs.  Measured at 32^3 x
-// 64, FP32, 256 boxes: fine boxes (15 groups a wavefront) 2.16 ms with 16 warps,
+// take the shape with the fewest waves of CTAs over the SMs.  Measured (before
+// the ring below) at 32^3 x 64, FP32, 256 boxes: fine boxes (15 groups a wavefront) 2.16 ms with 16 warps,
 // 2.46 with 8 (two CTAs an SM), 4.04 with 4; coarse boxes (2.5 groups) 303, 221,
 // 300 us; 192 uneven boxes (5.6 groups) 695, 1039, 1633 us.  FP64, 64 boxes of 9
 // groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
 // global memory, the fewest buffers, the largest CTA.  ras_autotune measures instead.
 template <typename T>
-kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int nsm,
+kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int wcap, int nsm,
                               const ShapeRequest& req, SolveShape* out) {
   if (req.lanes != 0 && req.lanes != kLanes) {
     set_error("ras_setup: the subdomain solve runs 4 lanes per point");
     return KKT_ERR_ARG;
   }
-  KKT_TRY_CUDA(cudaFuncSetAttribute(ras_solve<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSmemLimit));
-  KKT_TRY_CUDA(cudaFuncSetAttribute(ras_solve<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSmemLimit));
+  for (int form = 0; form < 3; ++form)
+    KKT_TRY_CUDA(cudaFuncSetAttribute(solve_kernel<T>(form == 1, form == 2),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
   SolveShape best{};
   long long best_key = -1;
   for (int ci = 0; ci < 3; ++ci)
@@ -743,18 +849,25 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
         // a vector in shared memory leaves room for ns lower blocks of ch points beside it (the
         // limit that the shape interface has always had)
         if (sv && vec + kSolveReserve + (size_t)ns * kLRanks * ch * sizeof(T) > kSmemLimit) continue;
-        const size_t sm = solve_smem<T>(nlev, warps, ns) + vec;
+        size_t sm = solve_smem<T>(nlev, warps, ns, false) + vec;
+        bool ring = false;
+        // (fewer boxes than a quarter of the SMs: their vectors stay in L1, measured 2 to 3 % faster)
+        if (LaneFactors<T>::kStaged && !sv && wcap <= kMaxRingPlaces && 4 * nbox >= nsm) {
+          const size_t with = solve_smem<T>(nlev, warps, ns, true) + ring_smem(wcap);
+          ring = with <= kSmemLimit;
+          if (ring) sm = with;
+        }
         if (sm > kSmemLimit) continue;
         int per_sm = 0;
         KKT_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, sv ? solve_kernel<T, true>() : solve_kernel<T, false>(), 32 * warps, sm));
+            &per_sm, solve_kernel<T>(sv != 0, ring), 32 * warps, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
         const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
         const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
         if (best_key < 0 || key < best_key) {
           best_key = key;
-          best = SolveShape{ch, warps, ns, kLanes, sv != 0};
+          best = SolveShape{ch, warps, ns, kLanes, sv != 0, ring};
         }
       }
   if (best_key < 0) {
@@ -871,12 +984,13 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       const kkt_problem* pk = probs[g.prob];
       const int dk[4] = {pk->nx, pk->ny, pk->nz, pk->L};
       long long v = kVecWidth;
-      int nlev = 1;
+      int nlev = 1, len[4];
       for (int a = 0; a < 4; ++a) {
-        const int l = std::min(dk[a], g.own[a].second + overlap) - std::max(0, g.own[a].first - overlap);
+        const int l = len[a] = std::min(dk[a], g.own[a].second + overlap) - std::max(0, g.own[a].first - overlap);
         v *= l + 2;
         nlev += (l - 1) << a;
       }
+      if (local == 0) m->wcap = std::max(m->wcap, widest_wavefront(len));
       pad = std::max(pad, v);
       points += g.points;
       m->max_nlev = std::max(m->max_nlev, nlev);
@@ -898,9 +1012,9 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       req.place = shape[3];
     }
     SolveShape sh{};
-    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, nsm, req, &sh)
-                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, nsm, req, &sh)
-                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, nsm, req, &sh);
+    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, m->wcap, nsm, req, &sh)
+                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, m->wcap, nsm, req, &sh)
+                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, m->wcap, nsm, req, &sh);
     if (cs != KKT_OK) {
       delete m;
       return cs;
@@ -908,6 +1022,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
     m->ch = sh.ch;
     m->warps = sh.warps;
     m->smem_vec = sh.smem_vec;
+    m->ring = sh.ring;
     m->nstage = sh.nstage;
     m->lanes = sh.lanes;
   }
@@ -1091,6 +1206,20 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   if (e == cudaSuccess) e = cudaMemset(m->V, 0, (local != 0 ? 16 : voff) * vsz);
   if (e == cudaSuccess) e = cudaMemset(m->status, 0, sizeof(int));
   if (e != cudaSuccess) return fail(KKT_ERR_CUDA, cudaGetErrorString(e));
+  if (local == 0 && m->ring) {
+    int* inv = nullptr;
+    if (cudaMalloc(&m->ntab, (size_t)ngroup * 2 * kNbrBytes) != cudaSuccess ||
+        cudaMalloc(&inv, (size_t)poff * sizeof(int)) != cudaSuccess)
+      return fail(KKT_ERR_NOMEM, "device allocation failed (neighbour places)");
+    place_points<<<dim3((kGroup * m->max_groups + 255) / 256, m->nbox), 256>>>(m->boxes, m->gptr, m->perm, inv);
+    neighbour_places<<<dim3((m->max_groups + 7) / 8, m->nbox), 256>>>(m->boxes, m->gptr, m->perm, inv, m->wcap,
+                                                                      m->ntab);
+    KKT_COUNT(2);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    cudaFree(inv);
+    if (e != cudaSuccess) return fail(KKT_ERR_CUDA, cudaGetErrorString(e));
+  }
   kkt_status st = local >= 2 ? gp_create(m, local, factor_prec) : KKT_OK;
   if (st == KKT_OK && local == 0 && factor_prec != 64) st = ras_factor_prepare32(m);
   if (st == KKT_OK) st = ras_factor(m, nullptr);
@@ -1110,10 +1239,14 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
   using T = typename SolveArith<S>::type;
   const int gbytes = gptr_smem(m->max_nlev);
   // (the dynamic shared-memory limit of both instances is raised at set-up, in choose_solve_shape)
-  const size_t smem = solve_smem<S>(m->max_nlev, m->warps, m->nstage) + (m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
-  auto* kernel = m->smem_vec ? ras_solve<S, true> : ras_solve<S, false>;
+  const size_t smem = solve_smem<S>(m->max_nlev, m->warps, m->nstage, m->ring) +
+                      (m->ring ? ring_smem(m->wcap) : m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
+  auto* kernel = m->smem_vec ? ras_solve<S, true, false> : ras_solve<S, false, false>;
+  if constexpr (LaneFactors<S>::kStaged)
+    if (m->ring) kernel = ras_solve<S, false, true>;
   kernel<<<m->nbox, 32 * m->warps, smem, s>>>(m->boxes, m->gptr, (const S*)m->F, V, r, z, m->gtab, m->otab, m->vtab,
-                                              gbytes, solve_buffers(m->nstage), m->status, gate, gate_stride);
+                                              m->ntab, m->wcap, gbytes, solve_buffers(m->nstage), m->status, gate,
+                                              gate_stride);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
@@ -1315,6 +1448,7 @@ extern "C" void ras_destroy(ras_precond* m) {
   cudaFree(m->gtab);
   cudaFree(m->otab);
   cudaFree(m->vtab);
+  cudaFree(m->ntab);
   cudaFree(m->rec);
   cudaFree(m->AB);
   cudaFree(m->ipiv);

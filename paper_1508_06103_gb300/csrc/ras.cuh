@@ -72,6 +72,8 @@ struct ras_precond {
   bool smem_vec = false;       // solve keeps the local vectors in shared memory
   int nstage = 2;              // factor groups a warp asks for ahead, itself included (ras_setup_shape)
   int lanes = 4;               // lanes per point in the solve
+  bool ring = false;           // solve keeps the last wavefronts in shared memory
+  int wcap = 0;                // group places of the widest wavefront
   int max_nlev = 0;            // most wavefronts of a box
   long long ngroup = 0;        // groups of all boxes
   int max_groups = 0;          // most groups of a box
@@ -86,6 +88,7 @@ struct ras_precond {
   int2* otab = nullptr;        // per owned point: {3 x global point index, padded offset}
   int* vtab = nullptr;         // per group place: padded offset in the box's local vector; empty places hold
                                // the complement of an offset that can be read
+  unsigned short* ntab = nullptr;   // ring: place of every neighbour per group, sweep and lane
   int* ptab = nullptr;         // per point (lexicographic): offset of its column in the box's factor values
   void* F = nullptr;           // factor values (FP64, FP32 or BF16, as the solve reads them)
   void* V = nullptr;           // padded local vectors
