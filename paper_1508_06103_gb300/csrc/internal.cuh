@@ -221,10 +221,9 @@ kkt_status matvec_prepare();   // raises the kernels' shared-memory limit on the
 kkt_status launch_matvec64(const DevProblem& p, const double* x, double* y, cudaStream_t s);
 kkt_status launch_matvec32(const DevProblem& p, const float* x, float* y, cudaStream_t s);
 kkt_status launch_residual(const DevProblem& p, const double* b, const double* x, double* r, cudaStream_t s);
-kkt_status launch_residual32(const DevProblem& p, const double* b, const double* x, double* r,
-                             float* x32, float* y32, cudaStream_t s);
-kkt_status launch_matvec32_d(const DevProblem& p, const double* x, double* y, float* x32, float* y32,
-                             cudaStream_t s);
+kkt_status launch_residual32(const DevProblem& p, const double* b, const float* x, double* r, cudaStream_t s);
+kkt_status launch_matvec32_d(const DevProblem& p, const float* x, double* y, cudaStream_t s);
+kkt_status launch_narrow(const double* x, float* y, long long n, cudaStream_t s, const int* gate);
 
 // problem.cu
 kkt_status create_problem(const kkt_grid* g, int nt, double dt, const double* a_cell, const double* v_cell,

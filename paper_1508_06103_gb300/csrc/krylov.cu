@@ -122,9 +122,10 @@ __global__ void copy_kernel(double* __restrict__ y, const double* __restrict__ x
 // ---------------------------------------------------------------------------
 
 // First call of a solve: ||b|| from its squared norm; the iteration budget.
-__global__ void gm_init(GmresState* st, double rtol, int maxit, const int* parent) {
+__global__ void gm_init(GmresState* st, double rtol, int maxit, const int* parent, bool zero_guess) {
   if (threadIdx.x != 0) return;
   st->bnorm = sqrt(st->b2);
+  if (zero_guess) st->r2 = st->b2;   // r = b
   st->rtol = rtol;
   st->maxit = maxit;
   st->iters = 0;
@@ -254,14 +255,14 @@ kkt_status launched(int n = 1) {
 // r = b - A x and its squared norm.  Every launch is stream-ordered on s and
 // nothing reads the device state on the host, so the cycle can be captured.
 kkt_status enqueue_cycle(Operator& A, Operator* M, const double* b, double* x, GmresWork& ws, int m,
-                         bool check_true, const int* parent, cudaStream_t s) {
+                         bool check_true, const int* parent, cudaStream_t s, const double* r0 = nullptr) {
   const long long n = ws.n;
   GmresState* st = ws.st;
   const int* active = &st->active;
   const int* ran = &st->ran;
   gm_begin<<<1, 32, 0, s>>>(st, ws.g(), m, parent);
   KKT_TRY(launched());
-  scale_dev<<<kVecBlocks, 256, 0, s>>>(ws.V, ws.r, &st->inv, n, active);
+  scale_dev<<<kVecBlocks, 256, 0, s>>>(ws.V, r0 ? r0 : ws.r, &st->inv, n, active);
   KKT_TRY(launched());
   // the outer cycle tags its captured timing pairs with the step (the inner coarse cycle
   // runs inside an outer step and leaves the tag alone)
@@ -484,17 +485,15 @@ kkt_status gmres_run(Operator& A, Operator* M, const double* b, double* x, Gmres
   if (!check_true) {
     // inner solve (the coarse level): one cycle from a zero guess, enqueued only
     KKT_TRY(vec_zero(x, n, s));
-    KKT_TRY(vec_copy(ws.r, b, n, s, parent));
     KKT_TRY(multidot(b, 0, 1, b, n, ws.part, &st->b2, s, parent));
-    KKT_TRY(multidot(b, 0, 1, b, n, ws.part, &st->r2, s, parent));
-    gm_init<<<1, 32, 0, s>>>(st, rtol, maxit, parent);
+    gm_init<<<1, 32, 0, s>>>(st, rtol, maxit, parent, true);
     KKT_TRY(launched());
-    return enqueue_cycle(A, M, b, x, ws, m, false, parent, s);
+    return enqueue_cycle(A, M, b, x, ws, m, false, parent, s, b);
   }
 
   // outer solve: ||b|| and the initial residual, then one host round trip per cycle
   KKT_TRY(multidot(b, 0, 1, b, n, ws.part, &st->b2, s, nullptr));
-  gm_init<<<1, 32, 0, s>>>(st, rtol, maxit, nullptr);
+  gm_init<<<1, 32, 0, s>>>(st, rtol, maxit, nullptr, false);
   KKT_TRY(launched());
   KKT_TRY(read_state(ws, s));
   const double bnorm = ws.st_host->bnorm;
@@ -705,8 +704,7 @@ kkt_status gmres_run_batch(std::vector<Operator*>& A, Operator& M, const double*
   for (int k = 0; k < np; ++k) {
     const long long o = bw.off[k], nk = bw.off[k + 1] - o;
     KKT_TRY(multidot(b + o, 0, 1, b + o, nk, ws.part, &bw.st[k].b2, s, nullptr));
-    KKT_TRY(multidot(b + o, 0, 1, b + o, nk, ws.part, &bw.st[k].r2, s, nullptr));
-    gm_init<<<1, 32, 0, s>>>(bw.st + k, rtol, maxit, nullptr);
+    gm_init<<<1, 32, 0, s>>>(bw.st + k, rtol, maxit, nullptr, true);
     KKT_TRY(launched());
   }
   KKT_TRY_CUDA(cudaMemcpyAsync(bw.st_host, bw.st, np * sizeof(GmresState), cudaMemcpyDeviceToHost, s));

@@ -183,10 +183,11 @@ __device__ __forceinline__ void cp_async_wait() {
 // kL2: the H1-L2 regularisation (its beta2 term goes through B), a template
 // argument so the H1-H1 kernel carries no test for it.  kP1: P1 elements, B and
 // K as stored 15-point stencils (no x and y passes, two barriers per level).
-template <typename T, bool kL2, typename Tl, bool kP1 = false>
+// kWide (FP32): the product, or b minus it, written as FP64 values to yd.
+template <typename T, bool kL2, typename Tl, bool kP1 = false, bool kWide = false>
 __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const T* __restrict__ x,
                                                              T* __restrict__ y, const double* __restrict__ b,
-                                                             int tiles_x, int tiles_y, Axis1D<T> ax, Axis1D<T> ay,
+                                                             double* __restrict__ yd, int tiles_x, int tiles_y, Axis1D<T> ax, Axis1D<T> ay,
                                                              Axis1D<T> az, LevelW<T> W) {
   constexpr int TX = Tl::TX, TY = Tl::TY, TZ = Tl::TZ;
   constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH, NXP = Tl::NXP, NYP = Tl::NYP;
@@ -220,6 +221,23 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
       cp_async_value(dst + h, src, valid);
       cp_async_value(dst + NH + h, src + (valid ? 1 : 0), valid);
       cp_async_value(dst + 2 * NH + h, src + (valid ? 2 : 0), valid);
+    }
+  };
+  // F x, b - F x, or (FP32) either of them as FP64 values
+  auto put = [&](int n, T c_, T g_, T f_) {
+    const long long o = 3 * ((long long)n * N + j);
+    if constexpr (kWide) {
+      yd[o] = b != nullptr ? b[o] - (double)c_ : (double)c_;
+      yd[o + 1] = b != nullptr ? b[o + 1] - (double)g_ : (double)g_;
+      yd[o + 2] = b != nullptr ? b[o + 2] - (double)f_ : (double)f_;
+    } else if (b != nullptr) {
+      y[o] = (T)(b[o] - (double)c_);
+      y[o + 1] = (T)(b[o + 1] - (double)g_);
+      y[o + 2] = (T)(b[o + 2] - (double)f_);
+    } else {
+      y[o] = c_;
+      y[o + 1] = g_;
+      y[o + 2] = f_;
     }
   };
   // S and S^T (and under P1, B and K) of the thread's node: registers in
@@ -305,16 +323,7 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
         if (n == 0 || dirj) yc = C0;
         if (n == M || dirj) yg = G0;
         else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
-        const long long o = 3 * ((long long)n * N + j);
-        if (b != nullptr) {
-          y[o] = (T)(b[o] - (double)yc);
-          y[o + 1] = (T)(b[o + 1] - (double)yg);
-          y[o + 2] = (T)(b[o + 2] - (double)yf);
-        } else {
-          y[o] = yc;
-          y[o + 1] = yg;
-          y[o + 2] = yf;
-        }
+        put(n, yc, yg, yf);
       }
       continue;
     }
@@ -375,16 +384,7 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
       if (n == 0 || dirj) yc = C0;
       if (n == M || dirj) yg = G0;
       else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
-      const long long o = 3 * ((long long)n * N + j);
-      if (b != nullptr) {
-        y[o] = (T)(b[o] - (double)yc);
-        y[o + 1] = (T)(b[o + 1] - (double)yg);
-        y[o + 2] = (T)(b[o + 2] - (double)yf);
-      } else {
-        y[o] = yc;
-        y[o + 1] = yg;
-        y[o + 2] = yf;
-      }
+      put(n, yc, yg, yf);
     }
   }
   cp_async_wait<0>();
@@ -401,7 +401,7 @@ double tile_work(const DevProblem& p) {
 }
 
 template <typename T, typename Tl, bool kP1 = false>
-void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaStream_t s) {
+void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaStream_t s, double* yd = nullptr) {
   const int tx = (p.nx + Tl::TX - 1) / Tl::TX, ty = (p.ny + Tl::TY - 1) / Tl::TY, tz = (p.nz + Tl::TZ - 1) / Tl::TZ;
   constexpr int NT = levels_per_cta<T>();
   dim3 grid(tx * ty * tz, (p.M + 1 + NT - 1) / NT);
@@ -413,17 +413,17 @@ void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaSt
   w.init(p.tau, p.theta, p.beta1, p.beta2);
   // (the dynamic shared-memory limits are raised once, in matvec_prepare)
   constexpr size_t smem = mv_smem<T, Tl, kP1>();
-  if (p.reg != 0)
-    matvec_tiled<T, true, Tl, kP1><<<grid, Tl::kThreads, smem, s>>>(p, x, y, b, tx, ty, ax, ay, az, w);
-  else
-    matvec_tiled<T, false, Tl, kP1><<<grid, Tl::kThreads, smem, s>>>(p, x, y, b, tx, ty, ax, ay, az, w);
+  auto* kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1> : matvec_tiled<T, false, Tl, kP1>;
+  if constexpr (sizeof(T) == 4)
+    if (yd) kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1, true> : matvec_tiled<T, false, Tl, kP1, true>;
+  kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, y, b, yd, tx, ty, ax, ay, az, w);
 }
 
 template <typename T>
-void launch_tiled(const DevProblem& p, const T* x, T* y, const double* b, cudaStream_t s) {
-  if (p.elem == KKT_ELEM_P1) launch_shape<T, TileA, true>(p, x, y, b, s);
-  else if (tile_work<TileB>(p) < tile_work<TileA>(p)) launch_shape<T, TileB>(p, x, y, b, s);
-  else launch_shape<T, TileA>(p, x, y, b, s);
+void launch_tiled(const DevProblem& p, const T* x, T* y, const double* b, cudaStream_t s, double* yd = nullptr) {
+  if (p.elem == KKT_ELEM_P1) launch_shape<T, TileA, true>(p, x, y, b, s, yd);
+  else if (tile_work<TileB>(p) < tile_work<TileA>(p)) launch_shape<T, TileB>(p, x, y, b, s, yd);
+  else launch_shape<T, TileA>(p, x, y, b, s, yd);
 }
 
 // ---------------------------------------------------------------------------
@@ -724,27 +724,14 @@ __global__ void d2f(const double* __restrict__ x, float* __restrict__ y, long lo
     y[i] = (float)x[i];
 }
 
-__global__ void f2d(const float* __restrict__ x, double* __restrict__ y, long long n, const int* gate) {
-  if (gated_off(gate)) return;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = (double)x[i];
-}
-
-__global__ void sub_f2d(const double* __restrict__ b, const float* __restrict__ y, double* __restrict__ r, long long n,
-                        const int* gate) {
-  if (gated_off(gate)) return;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    r[i] = b[i] - (double)y[i];
-}
-
 }  // namespace
 
-template <typename T, typename Tl>
-kkt_status prepare_shape() {
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<T, false, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)mv_smem<T, Tl>()));
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<T, true, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)mv_smem<T, Tl>()));
+template <typename Tl, bool kP1, bool kWide>
+kkt_status prepare32() {
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<float, false, Tl, kP1, kWide>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<float, Tl, kP1>()));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<float, true, Tl, kP1, kWide>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<float, Tl, kP1>()));
   return KKT_OK;
 }
 
@@ -757,22 +744,24 @@ kkt_status prepare64() {
   return KKT_OK;
 }
 
-template <typename T>
-kkt_status prepare_p1() {
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<T, false, TileA, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<T, TileA, true>()));
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<T, true, TileA, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<T, TileA, true>()));
+kkt_status prepare64_p1() {
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<double, false, TileA, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<double, TileA, true>()));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<double, true, TileA, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<double, TileA, true>()));
   return KKT_OK;
 }
 
 kkt_status matvec_prepare() {
   KKT_TRY(prepare64<TileA>());
   KKT_TRY(prepare64<TileC>());
-  KKT_TRY((prepare_shape<float, TileA>()));
-  KKT_TRY((prepare_shape<float, TileB>()));
-  KKT_TRY((prepare_p1<double>()));
-  KKT_TRY((prepare_p1<float>()));
+  KKT_TRY(prepare64_p1());
+  KKT_TRY((prepare32<TileA, false, false>()));
+  KKT_TRY((prepare32<TileA, false, true>()));
+  KKT_TRY((prepare32<TileB, false, false>()));
+  KKT_TRY((prepare32<TileB, false, true>()));
+  KKT_TRY((prepare32<TileA, true, false>()));
+  KKT_TRY((prepare32<TileA, true, true>()));
   return KKT_OK;
 }
 
@@ -797,26 +786,26 @@ kkt_status launch_residual(const DevProblem& p, const double* b, const double* x
   return KKT_OK;
 }
 
-// r = b - F x with the product in FP32 (x32, y32: scratch of 3P floats).
-kkt_status launch_residual32(const DevProblem& p, const double* b, const double* x, double* r, float* x32,
-                             float* y32, cudaStream_t s) {
-  const long long n = 3 * p.P;
-  d2f<<<1216, 256, 0, s>>>(x, x32, n, p.gate);
-  launch_tiled<float>(p, x32, y32, nullptr, s);
-  sub_f2d<<<1216, 256, 0, s>>>(b, y32, r, n, p.gate);
-  KKT_COUNT(3);
+// r = b - F x (FP64) with the product in FP32 of x in FP32.
+kkt_status launch_residual32(const DevProblem& p, const double* b, const float* x, double* r, cudaStream_t s) {
+  launch_tiled<float>(p, x, nullptr, b, s, r);
+  KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
 }
 
-// y = F x for FP64 vectors with the product in FP32 (x32, y32: scratch of 3P floats).
-kkt_status launch_matvec32_d(const DevProblem& p, const double* x, double* y, float* x32, float* y32,
-                             cudaStream_t s) {
-  const long long n = 3 * p.P;
-  d2f<<<1216, 256, 0, s>>>(x, x32, n, p.gate);
-  launch_tiled<float>(p, x32, y32, nullptr, s);
-  f2d<<<1216, 256, 0, s>>>(y32, y, n, p.gate);
-  KKT_COUNT(3);
+// y = F x (FP64) with the product in FP32 of x in FP32.
+kkt_status launch_matvec32_d(const DevProblem& p, const float* x, double* y, cudaStream_t s) {
+  launch_tiled<float>(p, x, nullptr, nullptr, s, y);
+  KKT_COUNT(1);
+  KKT_TRY_CUDA(cudaGetLastError());
+  return KKT_OK;
+}
+
+// y = (float)x
+kkt_status launch_narrow(const double* x, float* y, long long n, cudaStream_t s, const int* gate) {
+  d2f<<<1216, 256, 0, s>>>(x, y, n, gate);
+  KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
 }

@@ -110,10 +110,7 @@ const SlotTables& tables() {
 constexpr int kCBase = 0, kCDiag = 80, kCEnd = 108;
 constexpr int kGBase = 108, kGDiag = 122, kGEnd = 164;
 constexpr int kFBase = 164, kFDiag = 245, kFEnd = 326;
-// span of a box's unit row: kSlots rounded up to whole 16-byte units in FP32 and FP64
-constexpr int kUnitRowSpan = (kSlots + 3) / 4 * 4;
 constexpr int kLRanks = 175;        // L-slots of the three rows
-constexpr int kURanks = 151;        // diagonals and U-slots of the three rows
 
 // rank of slot s in a group: L-slots of C, G, f, then diag+U of C, G, f
 int slot_rank(int s) {
@@ -413,7 +410,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     typename SolveArith<S>::type* __restrict__ V, const double* __restrict__ r, double* __restrict__ z,
     const int2* __restrict__ gtab, const int2* __restrict__ otab, const int* __restrict__ vtab,
     const unsigned short* __restrict__ ntab, int wcap, int gptr_bytes, int nbuf, int* __restrict__ status,
-    const int* gate, int gate_stride) {
+    const int* gate, int gate_stride, RasExtra extra) {
   using T = typename SolveArith<S>::type;
   constexpr bool kStaged = LaneFactors<S>::kStaged;
   // the box's problem gate (one problem: gate_stride 0, every box reads gate[0])
@@ -529,7 +526,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       T* vp = v + (act ? vq : ~vq);
       vq = vq2;
       vq2 = point(k + 2 * nwarp);
-      unsigned places[kNbrPerLane / 2];   // RING: the neighbours' places, two a word
+      [[maybe_unused]] unsigned places[kNbrPerLane / 2];   // RING: the neighbours' places, two a word
       if (kStaged) {
         if (!mbar_wait(&bar[t % nbuf], (unsigned)(t / nbuf) & 1u, status)) {
           atomicExch(aborted, 1);
@@ -716,9 +713,20 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       const int2 e = otab[bx.ooff + q];
       T a0, a1, a2;
       ld3(v + e.y, a0, a1, a2);
-      z[e.x] = (double)a0;
-      z[e.x + 1] = (double)a1;
-      z[e.x + 2] = (double)a2;
+      double d0 = (double)a0, d1 = (double)a1, d2 = (double)a2;
+      if (extra.add != nullptr) {
+        d0 += extra.add[e.x];
+        d1 += extra.add[e.x + 1];
+        d2 += extra.add[e.x + 2];
+      }
+      z[e.x] = d0;
+      z[e.x + 1] = d1;
+      z[e.x + 2] = d2;
+      if (extra.z32 != nullptr) {
+        extra.z32[e.x] = (float)d0;
+        extra.z32[e.x + 1] = (float)d1;
+        extra.z32[e.x + 2] = (float)d2;
+      }
     }
   }
 }
@@ -1235,7 +1243,8 @@ namespace {
 
 template <typename S>
 kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename SolveArith<S>::type* V,
-                        cudaStream_t s, const int* gate = nullptr, int gate_stride = 0) {
+                        cudaStream_t s, const int* gate = nullptr, int gate_stride = 0,
+                        const RasExtra& extra = RasExtra()) {
   using T = typename SolveArith<S>::type;
   const int gbytes = gptr_smem(m->max_nlev);
   // (the dynamic shared-memory limit of both instances is raised at set-up, in choose_solve_shape)
@@ -1246,7 +1255,7 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
     if (m->ring) kernel = ras_solve<S, false, true>;
   kernel<<<m->nbox, 32 * m->warps, smem, s>>>(m->boxes, m->gptr, (const S*)m->F, V, r, z, m->gtab, m->otab, m->vtab,
                                               m->ntab, m->wcap, gbytes, solve_buffers(m->nstage), m->status, gate,
-                                              gate_stride);
+                                              gate_stride, extra);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
@@ -1285,13 +1294,20 @@ kkt_status ras_factor(ras_precond* m, cudaStream_t s) {
 }
 
 kkt_status ras_launch(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate,
-                      int gate_stride) {
-  TimedScope timed(&m->timing, s);
-  if (m->gp) return gp_solve(m, r, z, s, gate);
-  if (m->local == 1) return ras_lu_solve(m, r, z, s, gate);
-  if (m->prec == 64) return launch_solve<double>(m, r, z, (double*)m->V, s, gate, gate_stride);
-  if (m->prec == 32) return launch_solve<float>(m, r, z, (float*)m->V, s, gate, gate_stride);
-  return launch_solve<__nv_bfloat16>(m, r, z, (float*)m->V, s, gate, gate_stride);
+                      int gate_stride, const RasExtra& extra) {
+  if (m->local == 0) {
+    TimedScope timed(&m->timing, s);
+    if (m->prec == 64) return launch_solve<double>(m, r, z, (double*)m->V, s, gate, gate_stride, extra);
+    if (m->prec == 32) return launch_solve<float>(m, r, z, (float*)m->V, s, gate, gate_stride, extra);
+    return launch_solve<__nv_bfloat16>(m, r, z, (float*)m->V, s, gate, gate_stride, extra);
+  }
+  {
+    TimedScope timed(&m->timing, s);
+    KKT_TRY(m->gp ? gp_solve(m, r, z, s, gate) : ras_lu_solve(m, r, z, s, gate));
+  }
+  if (extra.add) KKT_TRY(vec_axpby(z, 1.0, extra.add, 1.0, m->n_total, s, gate));
+  if (extra.z32) KKT_TRY(launch_narrow(z, extra.z32, m->n_total, s, gate));
+  return KKT_OK;
 }
 
 kkt_status ras_check(ras_precond* m) {

@@ -135,6 +135,12 @@ kkt_status ras_lu_solve(ras_precond* m, const double* r, double* z, cudaStream_t
 // the subdomain solve z = M^{-1} r on s; its kernel returns at once while *gate reads 0
 // gate_stride: distance (ints) between the gates of consecutive problems; box b
 // reads gate[prob(b) * gate_stride]
+// z = M^{-1} r + add (where given); z32 (where given) also gets z rounded to FP32 (exact without add
+// where the solve runs in FP32)
+struct RasExtra {
+  const double* add = nullptr;
+  float* z32 = nullptr;
+};
 kkt_status ras_launch(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate = nullptr,
-                      int gate_stride = 0);
+                      int gate_stride = 0, const RasExtra& extra = RasExtra());
 kkt_status ras_check(ras_precond* m);

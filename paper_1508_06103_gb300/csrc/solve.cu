@@ -30,8 +30,9 @@ struct coarse_level {
   int c_maxit = 4;
   double *rc = nullptr, *yc = nullptr, *y = nullptr, *t = nullptr;
   int prec = 64;                     // precision of everything inside the preconditioner
-  float *cx32 = nullptr, *cy32 = nullptr;   // coarse FP32 scratch
-  float *fx32 = nullptr, *fy32 = nullptr;   // fine FP32 scratch
+  float* cx32 = nullptr;             // FP32 copy of the coarse matvec's argument
+  float4* yc4 = nullptr;             // y_c in FP32, 4 values a point
+  float* fx32 = nullptr;             // FP32 copy of y
   GmresWork ws;
   cudaStream_t aux = nullptr;        // two_level_refactor: stream of the coarse factorisation
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -126,6 +127,50 @@ __global__ void restrict_kernel(Grid4 f, Grid4 c, int rx, int ry, int rz, int rt
   rc[3 * idx + 2] = a2;
 }
 
+// y_c in FP32, 4 values a point, for interp32
+__global__ void pack_coarse(const double* __restrict__ yc, float4* __restrict__ out, long long P, const int* gate) {
+  if (gated_off(gate)) return;
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i < P) out[i] = make_float4((float)yc[3 * i], (float)yc[3 * i + 1], (float)yc[3 * i + 2], 0.f);
+}
+
+// interp_kernel<float> from the packed coarse values, writing y and its FP32 copy (the argument of the
+// residual's FP32 product).  Corners of weight 0 are left out; the sums' order is interp_kernel's.
+// interp_kernel<float> spent 156 us at 32^3 x 64 on 48 eight-byte loads and conversions a point.
+__global__ void interp32(Grid4 f, Grid4 c, int rx, int ry, int rz, int rt, const float4* __restrict__ yc,
+                         double* __restrict__ y, float* __restrict__ y32, const int* gate) {
+  if (gated_off(gate)) return;
+  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (idx >= (long long)f.N * f.L) return;
+  const int n = (int)(idx / f.N);
+  const int j = (int)(idx - (long long)n * f.N);
+  const int ix = j % f.nx, iy = (j / f.nx) % f.ny, iz = j / (f.nx * f.ny);
+  const int X0 = ix / rx, Y0 = iy / ry, Z0 = iz / rz, T0 = n / rt;
+  const float wx = (float)(ix - X0 * rx) / (float)rx, wy = (float)(iy - Y0 * ry) / (float)ry;
+  const float wz = (float)(iz - Z0 * rz) / (float)rz, wt = (float)(n - T0 * rt) / (float)rt;
+  const int ex = wx > 0.f ? 2 : 1, ey = wy > 0.f ? 2 : 1, ez = wz > 0.f ? 2 : 1, et = wt > 0.f ? 2 : 1;
+  float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+  for (int at = 0; at < et; ++at)
+    for (int az = 0; az < ez; ++az)
+      for (int ay = 0; ay < ey; ++ay) {
+        const float w3 = (at ? wt : 1.f - wt) * (az ? wz : 1.f - wz) * (ay ? wy : 1.f - wy);
+        const float4* src = yc + (long long)(T0 + at) * c.N + X0 + c.nx * (Y0 + ay + c.ny * (Z0 + az));
+        for (int ax = 0; ax < ex; ++ax) {
+          const float w = w3 * (ax ? wx : 1.f - wx);
+          const float4 q = __ldg(src + ax);
+          a0 += w * q.x;
+          a1 += w * q.y;
+          a2 += w * q.z;
+        }
+      }
+  y[3 * idx] = a0;
+  y[3 * idx + 1] = a1;
+  y[3 * idx + 2] = a2;
+  y32[3 * idx] = a0;
+  y32[3 * idx + 1] = a1;
+  y32[3 * idx + 2] = a2;
+}
+
 Grid4 grid_of(const kkt_problem* p) { return Grid4{p->nx, p->ny, p->nz, p->L, p->N}; }
 
 // The outer operator: FP64 KKT matvec (timed for the roofline report).
@@ -146,22 +191,31 @@ struct KktOp : Operator {
 struct CoarseOp : Operator {
   kkt_problem* p;
   int prec;
-  float *x32, *y32;
-  CoarseOp(kkt_problem* p_, int prec_, float* a, float* b) : p(p_), prec(prec_), x32(a), y32(b) {}
+  float* x32;                        // FP32 copy of the argument
+  const double* copied = nullptr;    // the vector whose copy x32 holds already (the RAS before wrote it)
+  CoarseOp(kkt_problem* p_, int prec_, float* a) : p(p_), prec(prec_), x32(a) {}
   kkt_status apply(const double* x, double* y, cudaStream_t s, const int* gate) override {
     DevProblem d = p->dev();
     d.gate = gate;
     if (prec == 64) return launch_matvec64(d, x, y, s);
-    return launch_matvec32_d(d, x, y, x32, y32, s);
+    if (x != copied) KKT_TRY(launch_narrow(x, x32, p->n, s, gate));
+    copied = nullptr;
+    return launch_matvec32_d(d, x32, y, s);
   }
   unsigned long long uid() const override { return p->uid * 4 + (unsigned long long)(p->reg + 2 * p->elem); }
 };
 
 struct RasOp : Operator {
   ras_precond* m;
-  explicit RasOp(ras_precond* m_) : m(m_) {}
+  CoarseOp* next;   // the coarse operator applied to the result next, or nullptr
+  explicit RasOp(ras_precond* m_, CoarseOp* next_ = nullptr) : m(m_), next(next_) {}
   kkt_status apply(const double* x, double* y, cudaStream_t s, const int* gate) override {
-    return ras_launch(m, x, y, s, gate);
+    RasExtra extra;
+    if (next && next->prec != 64) {
+      extra.z32 = next->x32;
+      next->copied = y;
+    }
+    return ras_launch(m, x, y, s, gate, 0, extra);
   }
   unsigned long long uid() const override { return m->uid; }
 };
@@ -181,23 +235,26 @@ kkt_status two_level(coarse_level* c, ras_precond* fine, const double* x, double
     restrict_kernel<float><<<rblocks, 256, 0, s>>>(gf, gc, c->rx, c->ry, c->rz, c->rt, x, c->rc, gate);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
-  CoarseOp Ac(pc, c->prec, c->cx32, c->cy32);
-  RasOp Mc(c->cras);
+  CoarseOp Ac(pc, c->prec, c->cx32);
+  RasOp Mc(c->cras, &Ac);
   GmresResult r;
   KKT_TRY(gmres_run(Ac, &Mc, c->rc, c->yc, c->ws, c->c_maxit, c->c_rtol, c->c_maxit, false, true, &r, s, gate));
-  if (c->prec == 64)
+  if (c->prec == 64) {
     interp_kernel<double><<<iblocks, 256, 0, s>>>(gf, gc, c->rx, c->ry, c->rz, c->rt, c->yc, c->y, gate);
-  else
-    interp_kernel<float><<<iblocks, 256, 0, s>>>(gf, gc, c->rx, c->ry, c->rz, c->rt, c->yc, c->y, gate);
+  } else {
+    pack_coarse<<<rblocks, 256, 0, s>>>(c->yc, c->yc4, pc->P, gate);
+    KKT_COUNT(1);
+    interp32<<<iblocks, 256, 0, s>>>(gf, gc, c->rx, c->ry, c->rz, c->rt, c->yc4, c->y, c->fx32, gate);
+  }
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   DevProblem df = pf->dev();
   df.gate = gate;
   if (c->prec == 64) KKT_TRY(launch_residual(df, x, c->y, c->t, s));   // t = x - F_h y
-  else KKT_TRY(launch_residual32(df, x, c->y, c->t, c->fx32, c->fy32, s));
-  KKT_TRY(ras_launch(fine, c->t, z, s, gate));
-  KKT_TRY(vec_axpby(z, 1.0, c->y, 1.0, pf->n, s, gate));   // z = M^{-1} t + y
-  return KKT_OK;
+  else KKT_TRY(launch_residual32(df, x, c->fx32, c->t, s));
+  RasExtra extra;
+  extra.add = c->y;   // z = M^{-1} t + y
+  return ras_launch(fine, c->t, z, s, gate, 0, extra);
 }
 
 // The one-level RAS of several problems: one subdomain solve over all their
@@ -286,9 +343,8 @@ extern "C" kkt_status coarse_setup(kkt_problem* fine, int ccx, int ccy, int ccz,
        cudaMalloc(&c->y, fine->n * sizeof(double)) != cudaSuccess ||
        cudaMalloc(&c->t, fine->n * sizeof(double)) != cudaSuccess ||
        (c->prec == 32 && (cudaMalloc(&c->cx32, c->cp->n * sizeof(float)) != cudaSuccess ||
-                          cudaMalloc(&c->cy32, c->cp->n * sizeof(float)) != cudaSuccess ||
-                          cudaMalloc(&c->fx32, fine->n * sizeof(float)) != cudaSuccess ||
-                          cudaMalloc(&c->fy32, fine->n * sizeof(float)) != cudaSuccess)))) {
+                          cudaMalloc(&c->yc4, c->cp->P * sizeof(float4)) != cudaSuccess ||
+                          cudaMalloc(&c->fx32, fine->n * sizeof(float)) != cudaSuccess)))) {
     cudaGetLastError();
     set_error("coarse_setup: device allocation failed");
     st = KKT_ERR_NOMEM;
@@ -358,9 +414,8 @@ extern "C" void coarse_destroy(coarse_level* c) {
   cudaFree(c->y);
   cudaFree(c->t);
   cudaFree(c->cx32);
-  cudaFree(c->cy32);
+  cudaFree(c->yc4);
   cudaFree(c->fx32);
-  cudaFree(c->fy32);
   c->ws.release();
   delete c;
 }
