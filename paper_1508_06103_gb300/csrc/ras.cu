@@ -39,7 +39,7 @@
 // slot of a factored row stores 1/u_kk, so both the factorisation and the
 // backward sweep multiply instead of divide.
 //
-// Solve.  One CTA per box; a warp takes a group of 8 points of the wavefront.
+// Solve.  One CTA per box, or a cluster of 2 to 8 where few boxes leave SMs idle; a warp takes a group of 8 points of the wavefront.
 // The local vector of each box has a ghost layer of zeros one point wide in
 // every direction, so the triangular sweeps need no bounds tests: a slot whose
 // column leaves the box reads 0 and has factor value 0.
@@ -177,6 +177,22 @@ __device__ __forceinline__ int ld_acquire_cta(const int* p) {
 }
 __device__ __forceinline__ void add_release_cta(int* p, int v) {
   asm volatile("red.release.cta.shared::cta.add.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+// the same across a cluster: a counter of CTA `rank`, given by its place in this CTA
+__device__ __forceinline__ int ld_acquire_cluster(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cluster.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void add_release_cluster(int* p, int v, int rank) {
+  asm volatile(
+      "{\n .reg .b32 a;\n mapa.shared::cluster.u32 a, %0, %2;\n red.release.cluster.shared::cluster.add.s32 [a], %1;\n}\n" ::"r"(
+          smem_u32(p)),
+      "r"(v), "r"(rank)
+      : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
   unsigned done;
@@ -404,7 +420,10 @@ constexpr int solve_buffer(bool ring) {
 constexpr unsigned kPollNs = 20;
 constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter of finished groups, abort word
 
-template <typename S, bool SMEM, bool RING>
+// CS: CTAs of a cluster that share a box: the groups go round the warps of all of them, the
+// local vector stays in global memory (the L2 holds it), and each CTA has its own counter of
+// the box's finished groups, to which every group adds.  The bits are those of one CTA.
+template <typename S, bool SMEM, bool RING, int CS>
 __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr, const S* __restrict__ F,
     typename SolveArith<S>::type* __restrict__ V, const double* __restrict__ r, double* __restrict__ z,
@@ -414,26 +433,31 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   using T = typename SolveArith<S>::type;
   constexpr bool kStaged = LaneFactors<S>::kStaged;
   // the box's problem gate (one problem: gate_stride 0, every box reads gate[0])
-  if (gate != nullptr && gate[boxes[blockIdx.x].prob * gate_stride] == 0) return;
+  if (gate != nullptr && gate[boxes[blockIdx.x / CS].prob * gate_stride] == 0) return;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned long long* bars = reinterpret_cast<unsigned long long*>(smem);
   int* finished = reinterpret_cast<int*>(smem + 8 * kSolveWarpsMax * (kMaxStages - 1));   // groups done
   int* aborted = finished + 1;
-  const BoxDesc bx = boxes[blockIdx.x];
+  const BoxDesc bx = boxes[blockIdx.x / CS];
   const int P = (int)bx.P, nlev = bx.nlev;
   const S* Fb = F + bx.foff;
   const int* vt = vtab + kGroup * bx.goff;
   const int px = bx.lx + 2, py = bx.ly + 2, pz = bx.lz + 2;
   const int sy = px, sz = px * py, st = px * py * pz;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x / 32, nwarp = blockDim.x / 32;
-  const int sub = lane & (kLanes - 1);
+  const int lane = threadIdx.x & 31, sub = lane & (kLanes - 1);
+  const int rank = CS == 1 ? 0 : blockIdx.x % CS, local_warp = threadIdx.x / 32;
+  const int warp = local_warp * CS + rank, nwarp = blockDim.x / 32 * CS;   // of all CTAs of the box
+  auto box_sync = [&]() {
+    if constexpr (CS == 1) __syncthreads();
+    else cluster_sync();
+  };
   // shared memory: header, group pointers, the warps' factor buffers, the local vector
   unsigned char* bufs = smem + kSolveHeader + gptr_bytes;
-  unsigned char* rest = bufs + (size_t)nwarp * nbuf * solve_buffer<S>(RING);   // the ring or the local vector
+  unsigned char* rest = bufs + (size_t)(blockDim.x / 32) * nbuf * solve_buffer<S>(RING);   // the ring or the local vector
   T* v = SMEM ? reinterpret_cast<T*>(rest) : V + bx.voff;
   T* ring = reinterpret_cast<T*>(rest);   // RING: [16][wcap] points and the zeros
-  unsigned char* mine = bufs + (size_t)warp * nbuf * solve_buffer<S>(RING);
-  unsigned long long* bar = bars + warp * (kMaxStages - 1);
+  unsigned char* mine = bufs + (size_t)local_warp * nbuf * solve_buffer<S>(RING);
+  unsigned long long* bar = bars + local_warp * (kMaxStages - 1);
   const int* gp = gptr + bx.loff;   // first group of every wavefront
   if (gptr_bytes) {
     int* copy = reinterpret_cast<int*>(smem + kSolveHeader);
@@ -476,12 +500,13 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   int vq = point(warp), vq2 = point(warp + nwarp);
   // R^delta r into the padded local vector (gtab: per box point, its global unknown index and
   // its padded offset); four points at a time, so that their loads overlap
-  for (int q0 = threadIdx.x; q0 < P; q0 += 4 * blockDim.x) {
+  const int member = rank * blockDim.x + threadIdx.x, members = CS * blockDim.x;   // threads of the box
+  for (int q0 = member; q0 < P; q0 += 4 * members) {
     int2 e[4];
     T a[4][3];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int q = q0 + k * blockDim.x;
+      const int q = q0 + k * members;
       e[k] = q < P ? gtab[bx.poff + q] : make_int2(-1, 0);
     }
 #pragma unroll
@@ -492,19 +517,21 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     for (int k = 0; k < 4; ++k)
       if (e[k].x >= 0) st3(v + e[k].y, a[k][0], a[k][1], a[k][2]);
   }
-  __syncthreads();
+  box_sync();
 
   // waits until n groups are done; false when the limit ran out here or in another warp
   auto wait_done = [&](int n) -> bool {
     unsigned long long t0 = 0;
-    for (unsigned it = 0; ld_acquire_cta(finished) < n; ++it) {
+    for (unsigned it = 0; (CS == 1 ? ld_acquire_cta(finished) : ld_acquire_cluster(finished)) < n; ++it) {
       __nanosleep(kPollNs);   // a warp that polls without a pause takes issue slots from those at work
       if ((it & 255u) == 255u) {
         const unsigned long long now = global_ns();
         if (t0 == 0) t0 = now;
         else if (now - t0 > kWaitLimitNs) {
           atomicExch(status, 2);
-          atomicExch(aborted, 1);
+          if constexpr (CS == 1) atomicExch(aborted, 1);
+          else
+            for (int c = 0; c < CS; ++c) add_release_cluster(aborted, 1, c);
         }
         if (*(volatile int*)aborted) return false;
       }
@@ -677,7 +704,11 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
         }
       }
       __syncwarp();
-      if (lane == 0) add_release_cta(finished, 1);
+      if constexpr (CS == 1) {
+        if (lane == 0) add_release_cta(finished, 1);
+      } else {
+        if (lane < CS) add_release_cluster(finished, 1, lane);
+      }
     }
     return true;
   };
@@ -702,13 +733,13 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     for (int q = t; q < t + nbuf; ++q)
       if (warp + q * nwarp < 2 * ng) mbar_wait(&bar[q % nbuf], (unsigned)(q / nbuf) & 1u, status);
   }
-  __syncthreads();
+  box_sync();             // (no CTA of the box ends while another may still count in its counter)
   if (*aborted) return;   // without writing z
   // scatter the owned part: (R^0)^T (otab: the owned points' global indices and offsets)
-  for (int q0 = threadIdx.x; q0 < bx.nown; q0 += 4 * blockDim.x) {
+  for (int q0 = member; q0 < bx.nown; q0 += 4 * members) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int q = q0 + k * blockDim.x;
+      const int q = q0 + k * members;
       if (q >= bx.nown) break;
       const int2 e = otab[bx.ooff + q];
       T a0, a1, a2;
@@ -735,8 +766,8 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
 // group.  inv: group place of every box point.
 __global__ void place_points(const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr,
                              const int* __restrict__ perm, int* __restrict__ inv) {
-  const BoxDesc bx = boxes[blockIdx.y];
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  const BoxDesc bx = boxes[blockIdx.x];
+  const int q = blockIdx.y * blockDim.x + threadIdx.x;
   if (q >= kGroup * gptr[bx.loff + bx.nlev]) return;
   const int lex = perm[kGroup * bx.goff + q];
   if (lex >= 0) inv[bx.poff + lex] = q;
@@ -744,9 +775,9 @@ __global__ void place_points(const BoxDesc* __restrict__ boxes, const int* __res
 __global__ void neighbour_places(const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr,
                                  const int* __restrict__ perm, const int* __restrict__ inv, int wcap,
                                  unsigned short* __restrict__ out) {
-  const BoxDesc bx = boxes[blockIdx.y];
+  const BoxDesc bx = boxes[blockIdx.x];
   const int* gp = gptr + bx.loff;
-  const int g = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32, sub = lane % kLanes;
+  const int g = blockIdx.y * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32, sub = lane % kLanes;
   if (g >= gp[bx.nlev]) return;
   const int lex = perm[kGroup * (bx.goff + g) + lane / kLanes];
   const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
@@ -813,14 +844,53 @@ size_t ring_smem(int wcap) { return ((size_t)kRingWaves * wcap + 1) * kVecWidth 
 struct SolveShape {
   int ch, warps, nstage, lanes;
   bool smem_vec, ring;
+  int cluster;
 };
 // groups per wavefront from which the largest CTA is taken
 constexpr int kFillGroups = 4;
 template <typename T>
-const void* solve_kernel(bool smem_vec, bool ring) {
+const void* solve_kernel(bool smem_vec, bool ring, int cluster) {
   if constexpr (LaneFactors<T>::kStaged)
-    if (ring) return (const void*)ras_solve<T, false, true>;
-  return smem_vec ? (const void*)ras_solve<T, true, false> : (const void*)ras_solve<T, false, false>;
+    if (ring) return (const void*)ras_solve<T, false, true, 1>;
+  if (smem_vec) return (const void*)ras_solve<T, true, false, 1>;
+  return cluster == 8   ? (const void*)ras_solve<T, false, false, 8>
+         : cluster == 4 ? (const void*)ras_solve<T, false, false, 4>
+         : cluster == 2 ? (const void*)ras_solve<T, false, false, 2>
+                        : (const void*)ras_solve<T, false, false, 1>;
+}
+// CTAs (a cluster) per box where the boxes alone leave SMs idle: the most whose clusters all
+// run at once and that have 2.5 groups of a wavefront each; FP32 and BF16, less bound by
+// arithmetic, 4 or 8 only.  Counting in every CTA's counter and waiting for the
+// other SMs costs more than fewer groups give.  Measured, FP64 (FP32) us a solve with 1, 2, 4, 8 CTAs a box:
+//   16 boxes, 2.1 groups a wavefront:   553   715   711  1167   ( 105  217  201  350)
+//   64 boxes, 6.8:                     1471  1419  2604         (the wait for a second wave)
+//   16 boxes, 9.2:                     1962  1655  1493  2637   ( 425  513  456  809)
+//   64 boxes, 9.0:                     3048  2626  4691
+//   16 boxes, 15.6:                    3878  2470  1974  3374   ( 827  849  635 1027)
+//   1 box, 21.9:                       5653  3708  2376  1932   (1154 1138  761  638)
+//   8 boxes, 82:                      28476 16691  9412  5708   (7447 6086 3368 2029)
+template <typename T>
+kkt_status choose_cluster(int nbox, double groups, int warps, size_t smem, int* out) {
+  *out = 1;
+  for (int cs = 8; cs >= (sizeof(T) == 8 ? 2 : 4); cs /= 2) {
+    if (groups < 2.5 * cs) continue;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(nbox * cs);
+    cfg.blockDim = dim3(32 * warps);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim = {(unsigned)cs, 1, 1};
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    KKT_TRY_CUDA(cudaOccupancyMaxActiveClusters(&fit, solve_kernel<T>(false, false, cs), &cfg));
+    if (nbox <= fit) {
+      *out = cs;
+      return KKT_OK;
+    }
+  }
+  return KKT_OK;
 }
 // A requested shape (ras_setup_shape): 0 in a field leaves it to the chooser.
 struct ShapeRequest {
@@ -841,8 +911,8 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
     set_error("ras_setup: the subdomain solve runs 4 lanes per point");
     return KKT_ERR_ARG;
   }
-  for (int form = 0; form < 3; ++form)
-    KKT_TRY_CUDA(cudaFuncSetAttribute(solve_kernel<T>(form == 1, form == 2),
+  for (int form = 0; form < 6; ++form)
+    KKT_TRY_CUDA(cudaFuncSetAttribute(solve_kernel<T>(form == 1, form == 2, form > 2 ? 1 << (form - 2) : 1),
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
   SolveShape best{};
   long long best_key = -1;
@@ -868,14 +938,14 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
         if (sm > kSmemLimit) continue;
         int per_sm = 0;
         KKT_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, solve_kernel<T>(sv != 0, ring), 32 * warps, sm));
+            &per_sm, solve_kernel<T>(sv != 0, ring, 1), 32 * warps, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
         const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
         const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
         if (best_key < 0 || key < best_key) {
           best_key = key;
-          best = SolveShape{ch, warps, ns, kLanes, sv != 0, ring};
+          best = SolveShape{ch, warps, ns, kLanes, sv != 0, ring, 1};
         }
       }
   if (best_key < 0) {
@@ -883,6 +953,9 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
               "placement must be a compiled combination that fits in shared memory)");
     return KKT_ERR_ARG;
   }
+  if (best.ch == SizeClasses<T>::name[0] && !best.smem_vec && !best.ring)
+    KKT_TRY(choose_cluster<T>(nbox, (double)points / ((double)nbox * nlev * kGroup), best.warps,
+                              solve_smem<T>(nlev, best.warps, best.nstage, false), &best.cluster));
   *out = best;
   return KKT_OK;
 }
@@ -1031,6 +1104,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
     m->warps = sh.warps;
     m->smem_vec = sh.smem_vec;
     m->ring = sh.ring;
+    m->cluster = sh.cluster;
     m->nstage = sh.nstage;
     m->lanes = sh.lanes;
   }
@@ -1215,16 +1289,23 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   if (e == cudaSuccess) e = cudaMemset(m->status, 0, sizeof(int));
   if (e != cudaSuccess) return fail(KKT_ERR_CUDA, cudaGetErrorString(e));
   if (local == 0 && m->ring) {
+    // without room for the table (a quarter of what is free at most, so that a problem sized to the
+    // memory still finds its Krylov vectors) the solve reads its neighbours from global memory
     int* inv = nullptr;
-    if (cudaMalloc(&m->ntab, (size_t)ngroup * 2 * kNbrBytes) != cudaSuccess ||
-        cudaMalloc(&inv, (size_t)poff * sizeof(int)) != cudaSuccess)
-      return fail(KKT_ERR_NOMEM, "device allocation failed (neighbour places)");
-    place_points<<<dim3((kGroup * m->max_groups + 255) / 256, m->nbox), 256>>>(m->boxes, m->gptr, m->perm, inv);
-    neighbour_places<<<dim3((m->max_groups + 7) / 8, m->nbox), 256>>>(m->boxes, m->gptr, m->perm, inv, m->wcap,
-                                                                      m->ntab);
-    KKT_COUNT(2);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    const size_t tab = (size_t)ngroup * 2 * kNbrBytes, invb = (size_t)poff * sizeof(int);
+    size_t free_b = 0, total_b = 0;
+    m->ring = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && tab + invb <= free_b / 4 &&
+              cudaMalloc(&inv, invb) == cudaSuccess && cudaMalloc(&m->ntab, tab) == cudaSuccess;
+    if (m->ring) {
+      place_points<<<dim3(m->nbox, (kGroup * m->max_groups + 255) / 256), 256>>>(m->boxes, m->gptr, m->perm, inv);
+      neighbour_places<<<dim3(m->nbox, (m->max_groups + 7) / 8), 256>>>(m->boxes, m->gptr, m->perm, inv, m->wcap,
+                                                                        m->ntab);
+      KKT_COUNT(2);
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    } else {
+      cudaGetLastError();
+    }
     cudaFree(inv);
     if (e != cudaSuccess) return fail(KKT_ERR_CUDA, cudaGetErrorString(e));
   }
@@ -1250,12 +1331,28 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
   // (the dynamic shared-memory limit of both instances is raised at set-up, in choose_solve_shape)
   const size_t smem = solve_smem<S>(m->max_nlev, m->warps, m->nstage, m->ring) +
                       (m->ring ? ring_smem(m->wcap) : m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
-  auto* kernel = m->smem_vec ? ras_solve<S, true, false> : ras_solve<S, false, false>;
-  if constexpr (LaneFactors<S>::kStaged)
-    if (m->ring) kernel = ras_solve<S, false, true>;
-  kernel<<<m->nbox, 32 * m->warps, smem, s>>>(m->boxes, m->gptr, (const S*)m->F, V, r, z, m->gtab, m->otab, m->vtab,
-                                              m->ntab, m->wcap, gbytes, solve_buffers(m->nstage), m->status, gate,
-                                              gate_stride, extra);
+  const void* kernel = solve_kernel<S>(m->smem_vec, m->ring, m->cluster);
+  const BoxDesc* boxes = m->boxes;
+  const S* F = (const S*)m->F;
+  const int *gptr = m->gptr, *vtab = m->vtab;
+  const int2 *gtab = m->gtab, *otab = m->otab;
+  const unsigned short* ntab = m->ntab;
+  int wcap = m->wcap, nbuf = solve_buffers(m->nstage);
+  int* status = m->status;
+  RasExtra ex = extra;
+  void* args[] = {&boxes, &gptr, &F,    &V,      &r,    &z,      &gtab, &otab,        &vtab,
+                  &ntab,  &wcap, (void*)&gbytes, &nbuf, &status, &gate, &gate_stride, &ex};
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(m->nbox * m->cluster);
+  cfg.blockDim = dim3(32 * m->warps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim = {(unsigned)m->cluster, 1, 1};
+  cfg.attrs = &attr;
+  cfg.numAttrs = m->cluster > 1 ? 1 : 0;
+  KKT_TRY_CUDA(cudaLaunchKernelExC(&cfg, kernel, args));
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;

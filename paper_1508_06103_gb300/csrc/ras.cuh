@@ -72,6 +72,7 @@ struct ras_precond {
   bool smem_vec = false;       // solve keeps the local vectors in shared memory
   int nstage = 2;              // factor groups a warp asks for ahead, itself included (ras_setup_shape)
   int lanes = 4;               // lanes per point in the solve
+  int cluster = 1;             // CTAs per box of the solve
   bool ring = false;           // solve keeps the last wavefronts in shared memory
   int wcap = 0;                // group places of the widest wavefront
   int max_nlev = 0;            // most wavefronts of a box

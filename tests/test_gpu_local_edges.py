@@ -104,3 +104,26 @@ def test_exact_lu_on_edge_shapes_matches_oracle(api, name):
         r = W.random_vector(prob.n, seed)
         z, zr = ras.apply(torch.from_numpy(r).cuda()).cpu().numpy(), ref.apply(r)
         assert np.abs(z - zr).max() <= 100 * kappa * 2.0**-53 * np.abs(zr).max()
+
+
+# boxes solved by one CTA, by a cluster of 2, 4 and 8 CTAs (FP64; FP32 and BF16: 1, 1, 4, 8)
+CLUSTER_CELLS = {"2": (10, 9, 9, 8), "4": (20, 11, 8, 6), "8": (27, 15, 9, 6)}
+
+
+@pytest.mark.parametrize("prec", [64, 32, 16])
+@pytest.mark.parametrize("name", CLUSTER_CELLS)
+def test_box_shared_by_ctas_has_the_bits_of_one_cta(api, name, prec):
+    # the same groups with the same operations in the same order: no tolerance.  Enough copies of
+    # the problem in one batch leave every box to a CTA of its own.
+    *cells, M = CLUSTER_CELLS[name]
+    w = W.random_small(44, cells=tuple(cells), M=M, nsens=4, reg="h1l2")
+    beta = max(w.h) ** 2
+    w = dataclasses.replace(w, T=M / 16.0, beta1=beta / 100, beta2=beta)
+    probs = [api.Problem.from_workload(w) for _ in range(80)]
+    many = api.BatchRAS(probs, (1, 1, 1, 1), 0, prec)
+    one = api.RAS(probs[0], (1, 1, 1, 1), 0, prec)
+    r = torch.from_numpy(W.random_vector(probs[0].n, 6)).cuda()
+    z = one.apply(r)
+    assert torch.isfinite(z).all() and z.abs().max() > 0
+    assert torch.equal(many.apply(r.repeat(80))[-probs[0].n:], z)
+    assert one.status() == 0
