@@ -11,12 +11,13 @@
 // Mt, Lt are the 1D linear-element time mass and stiffness (tau/6 [1 4 1],
 // [-1 2 -1]/tau, halved diagonals at the end levels).
 //
-// matvec_levels (trilinear elements) applies the four spatial operators to the
-// levels and combines them in time at the output nodes: B and K by sum
-// factorisation, S and S^T as 27-point stencils.  Under P1 elements on the Kuhn
-// split (kkt_set_element) B and K are no tensor products: matvec_p1 applies all
-// four operators as stencils over the 15 offsets the split couples, to six time
-// combinations.
+// matvec_tiled below (FP32, and FP64 under P1 elements) computes all three output
+// slots of a space-time point in one pass: four spatial operators applied to six
+// time combinations, B and K by sum factorisation, S and S^T as 27-point
+// stencils; matvec64_levels (FP64, trilinear elements) applies the operators to
+// the levels and combines them in time at the output nodes.  Under P1 elements
+// on the Kuhn split (kkt_set_element) B and K are no tensor products: all four
+// operators are applied as stencils over the 15 offsets the split couples.
 
 #include "internal.cuh"
 
@@ -38,10 +39,40 @@ __device__ __forceinline__ Coefs<float> coefs<float>(const DevProblem& p) {
   return {p.S32, p.ST32, p.B32, p.K32};
 }
 
-// Tile shapes (nodes per CTA along x, y, z): 8 x 8 x 4, or 11 x 11 x 2 and 11 x 11 x 3, which
-// cover grids of 11 k nodes per axis without ragged tiles (33^3 and 65^3 nodes: 40 x 40 x 36 /
-// 33^3 = 1.6x the nodes with 8 x 8 x 4 tiles); the host picks the shape with the least
-// estimated work (work_levels).
+// ---------------------------------------------------------------------------
+// Tiled matvec: one CTA owns a TX x TY x TZ tile of nodes and a run of NT time
+// levels (NT = levels_per_cta<T>(): 4 in FP64, 8 in FP32); one thread per
+// output node.  Per level the six time combinations
+//   u1 = (C^n - C^{n-1}) - tau (theta f^n + (1-theta) f^{n-1})   (C row, via B)
+//   u2 = tau (theta C^n + (1-theta) C^{n-1})                        (C row, via S)
+//   u3 = G^n - G^{n+1}                                              (G row, via B)
+//   u4 = tau (theta G^n + (1-theta) G^{n+1})                        (G row, via S^T)
+//   u5 = -(Mt G)_n + beta1 (Lt f)_n                                 (f row, via B)
+//   u6 = beta2 (Mt f)_n                                             (f row, via K;
+//        via B, added to u5, under the H1-L2 regularisation)
+// are formed once per halo node.  B = Mx (x) My (x) Mz and K = Kx My Mz +
+// Mx Ky Mz + Mx My Kz are tensor products of the 1D linear-element mass and
+// stiffness matrices on the uniform grid, so B u1, B u3, B u5 and K u6 are
+// applied by sum factorisation: a pass along x over the tile and its y, z
+// halo, one along y, one along z, with 1D factors computed from the mesh
+// widths (no coefficient loads).  S and S^T, whose coefficients vary from
+// node to node, are applied as 27-point stencils; in FP32 each thread keeps
+// its node's 54 coefficients in registers for all NT levels.  Levels of x
+// stream into a ring of four shared-memory slots with cp.async two levels
+// ahead of their use; halo nodes outside the domain are zero-filled, so the
+// passes need no bounds tests.
+// ---------------------------------------------------------------------------
+// Tile shapes (nodes per CTA along x, y, z): 8 x 8 x 4, or 11 x 11 x 2, which
+// covers grids of 11 k nodes per axis without ragged tiles (33^3 and 65^3
+// nodes: 40 x 40 x 36 / 33^3 = 1.6x the nodes with 8 x 8 x 4 tiles); the host
+// picks the shape with the least estimated work (launch_tiled).
+// Levels per CTA: shorter runs give more CTAs for the same work (two halo
+// levels more per run).  Measured at 32^3 x 64, FP32, with the inputs out of L2
+// (runs of 16 / 8 / 4 levels): 0.158 / 0.153 / 0.159 ms.
+template <typename T>
+__host__ __device__ constexpr int levels_per_cta() {
+  return sizeof(T) == 8 ? 4 : 8;
+}
 template <int TX_, int TY_, int TZ_>
 struct Tile {
   static constexpr int TX = TX_, TY = TY_, TZ = TZ_;
@@ -52,11 +83,12 @@ struct Tile {
 };
 using TileA = Tile<8, 8, 4>;
 using TileB = Tile<11, 11, 2>;
-using TileC = Tile<11, 11, 3>;
+using TileC = Tile<11, 11, 3>;   // FP64 levels kernel
 
-template <typename T, typename Tl>
-constexpr size_t p1_smem() {
-  return sizeof(T) * (4 * 3 * Tl::NH + 6 * Tl::NH);
+template <typename T, typename Tl, bool kP1 = false>
+constexpr size_t mv_smem() {
+  return kP1 ? sizeof(T) * (4 * 3 * Tl::NH + 6 * Tl::NH)
+             : sizeof(T) * (4 * 3 * Tl::NH + 6 * Tl::NH + 5 * Tl::NXP + 5 * Tl::NYP);
 }
 
 // Stencil offset d = (dx+1) + 3 (dy+1) + 9 (dz+1) is an edge of the Kuhn split
@@ -65,6 +97,45 @@ __host__ __device__ constexpr bool kuhn_offset(int d) {
   const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
   return !((dx > 0 || dy > 0 || dz > 0) && (dx < 0 || dy < 0 || dz < 0));
 }
+
+// 1D linear-element mass and stiffness rows on one axis of n nodes with
+// width h: row i has (i > 0) + (i < n - 1) elements; the entries are chosen
+// from values formed once on the host (no arithmetic per node).
+template <typename T>
+struct Axis1D {
+  int n;
+  T m1, m2, mo, k1, k2, ko;   // mass diagonal (one / two elements), off-diagonal; the same for stiffness
+  T hh;                       // the width
+  __host__ __device__ void init(int n_, double h) {
+    n = n_;
+    m1 = (T)(h / 3.0);
+    m2 = (T)(2.0 * h / 3.0);
+    mo = (T)(h / 6.0);
+    k1 = (T)(1.0 / h);
+    k2 = (T)(2.0 / h);
+    ko = (T)(-1.0 / h);
+    hh = (T)h;
+  }
+  // entries (i, i-1), (i, i), (i, i+1) of the mass (m) and stiffness (k) rows
+  __device__ __forceinline__ void row(int i, T& m_, T& m0, T& mp, T& k_, T& k0, T& kp) const {
+    const bool lo = i > 0, hi = i < n - 1;
+    if constexpr (sizeof(T) == 8) {   // FP64: select only (the FP64 pipe is the limit)
+      m_ = lo ? mo : (T)0;
+      mp = hi ? mo : (T)0;
+      m0 = lo && hi ? m2 : (lo || hi ? m1 : (T)0);
+      k_ = lo ? ko : (T)0;
+      kp = hi ? ko : (T)0;
+      k0 = lo && hi ? k2 : (lo || hi ? k1 : (T)0);
+    } else {                          // FP32: from the width per node (measured 4 % faster)
+      m0 = (T)((i > 0) + (i < n - 1)) * hh / (T)3;
+      m_ = lo ? hh / (T)6 : (T)0;
+      mp = hi ? hh / (T)6 : (T)0;
+      k0 = (T)((i > 0) + (i < n - 1)) / hh;
+      k_ = lo ? -(T)1 / hh : (T)0;
+      kp = hi ? -(T)1 / hh : (T)0;
+    }
+  }
+};
 
 // Weights of the six time combinations: the theta weights and the rows of
 // the 1D linear-element time mass Mt (tau/6 [1 4 1]) and stiffness Lt
@@ -109,37 +180,23 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// ---------------------------------------------------------------------------
-// P1 elements.  One CTA owns a tile of nodes and a run of levels_per_cta<T>() time levels, one
-// thread per output node.  Per level the six time combinations
-//   u1 = (C^n - C^{n-1}) - tau (theta f^n + (1-theta) f^{n-1})   (C row, via B)
-//   u2 = tau (theta C^n + (1-theta) C^{n-1})                        (C row, via S)
-//   u3 = G^n - G^{n+1}                                              (G row, via B)
-//   u4 = tau (theta G^n + (1-theta) G^{n+1})                        (G row, via S^T)
-//   u5 = -(Mt G)_n + beta1 (Lt f)_n                                 (f row, via B)
-//   u6 = beta2 (Mt f)_n                                             (f row, via K;
-//        via B, added to u5, under the H1-L2 regularisation)
-// are formed once per halo node and the 15-point stencils applied to them.  Levels of x
-// stream into a ring of four shared-memory slots with cp.async two levels ahead of their use;
-// halo nodes outside the domain are zero-filled.
-// ---------------------------------------------------------------------------
-template <typename T>
-__host__ __device__ constexpr int levels_per_cta() {
-  return sizeof(T) == 8 ? 4 : 8;
-}
 // kL2: the H1-L2 regularisation (its beta2 term goes through B), a template
-// argument so the H1-H1 kernel carries no test for it.
+// argument so the H1-H1 kernel carries no test for it.  kP1: P1 elements, B and
+// K as stored 15-point stencils (no x and y passes, two barriers per level).
 // kWide (FP32): the product, or b minus it, written as FP64 values to yd.
-template <typename T, bool kL2, typename Tl, bool kWide = false>
-__global__ void __launch_bounds__(Tl::kThreads) matvec_p1(DevProblem p, const T* __restrict__ x, T* __restrict__ y,
-                                                          const double* __restrict__ b, double* __restrict__ yd,
-                                                          int tiles_x, int tiles_y, LevelW<T> W) {
+template <typename T, bool kL2, typename Tl, bool kP1 = false, bool kWide = false>
+__global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const T* __restrict__ x,
+                                                             T* __restrict__ y, const double* __restrict__ b,
+                                                             double* __restrict__ yd, int tiles_x, int tiles_y, Axis1D<T> ax, Axis1D<T> ay,
+                                                             Axis1D<T> az, LevelW<T> W) {
   constexpr int TX = Tl::TX, TY = Tl::TY, TZ = Tl::TZ;
-  constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH;
+  constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH, NXP = Tl::NXP, NYP = Tl::NYP;
   if (gated_off(p.gate)) return;
   extern __shared__ __align__(16) unsigned char mv_sm[];
   T* Xs = reinterpret_cast<T*>(mv_sm);   // [4 slots][3 components][NH]
   T* U = Xs + 4 * 3 * NH;                // [6][NH]
+  T* PX = U + 6 * NH;                    // [5][NXP]
+  T* PY = PX + 5 * NXP;                  // [5][NYP]
   const int N = p.N, M = p.M;
   const int tile = blockIdx.x;
   const int bx0 = (tile % tiles_x) * TX, by0 = ((tile / tiles_x) % tiles_y) * TY, bz0 = (tile / (tiles_x * tiles_y)) * TZ;
@@ -183,16 +240,19 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_p1(DevProblem p, const T*
       y[o + 2] = f_;
     }
   };
-  // S, S^T, B and K of the thread's node: registers in FP32, reloaded per level in FP64
+  // S and S^T (and under P1, B and K) of the thread's node: registers in
+  // FP32, reloaded per level in FP64
   T cS[kStencil], cST[kStencil], cB[kStencil], cK[kStencil];
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int d = 0; d < kStencil; ++d) {
-      if (!kuhn_offset(d)) continue;
+      if (kP1 && !kuhn_offset(d)) continue;
       cS[d] = own ? c.S[(size_t)d * N + j] : (T)0;
       cST[d] = own ? c.ST[(size_t)d * N + j] : (T)0;
-      cB[d] = own ? c.B[(size_t)d * N + j] : (T)0;
-      cK[d] = own ? c.K[(size_t)d * N + j] : (T)0;
+      if constexpr (kP1) {
+        cB[d] = own ? c.B[(size_t)d * N + j] : (T)0;
+        cK[d] = own ? c.K[(size_t)d * N + j] : (T)0;
+      }
     }
   }
   prefetch(n0 - 1);
@@ -233,29 +293,91 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_p1(DevProblem p, const T*
     __syncthreads();
     if (n + 3 <= n1) prefetch(n + 3);    // into the slot of level n - 1, no longer read
     cp_async_commit();
+    if constexpr (kP1) {
+      if (own) {
+        T yc = (T)0, yg = (T)0, yf = (T)0;
+#pragma unroll
+        for (int d = 0; d < kStencil; ++d) {
+          if (!kuhn_offset(d)) continue;
+          const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
+          const int h = hc + dx + HX * (dy + HY * dz);
+          T s_, st_, b_, k_;
+          if constexpr (sizeof(T) == 4) {
+            s_ = cS[d];
+            st_ = cST[d];
+            b_ = cB[d];
+            k_ = cK[d];
+          } else {
+            s_ = c.S[(size_t)d * N + j];
+            st_ = c.ST[(size_t)d * N + j];
+            b_ = c.B[(size_t)d * N + j];
+            k_ = kL2 ? (T)0 : c.K[(size_t)d * N + j];
+          }
+          yc += b_ * U[h] + s_ * U[NH + h];
+          yg += b_ * U[2 * NH + h] + st_ * U[3 * NH + h];
+          yf += b_ * U[4 * NH + h];
+          if constexpr (!kL2) yf += k_ * U[5 * NH + h];
+        }
+        const bool dirj = p.dir[j] != 0;
+        const T C0 = X0[hc], G0 = X0[NH + hc], Cp = Xp[hc];
+        if (n == 0 || dirj) yc = C0;
+        if (n == M || dirj) yg = G0;
+        else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
+        put(n, yc, yg, yf);
+      }
+      continue;
+    }
+    // x pass: Mx on u1, u3, u5, u6 and Kx on u6
+    for (int e = t; e < NXP; e += blockDim.x) {
+      const int ex = e % TX, ey = (e / TX) % HY, ez = e / (TX * HY);
+      const int h = (ex + 1) + HX * (ey + HY * ez);
+      T m_, m0, mp, k_, k0, kp;
+      ax.row(bx0 + ex, m_, m0, mp, k_, k0, kp);
+      PX[e] = m_ * U[h - 1] + m0 * U[h] + mp * U[h + 1];
+      PX[NXP + e] = m_ * U[2 * NH + h - 1] + m0 * U[2 * NH + h] + mp * U[2 * NH + h + 1];
+      PX[2 * NXP + e] = m_ * U[4 * NH + h - 1] + m0 * U[4 * NH + h] + mp * U[4 * NH + h + 1];
+      PX[3 * NXP + e] = m_ * U[5 * NH + h - 1] + m0 * U[5 * NH + h] + mp * U[5 * NH + h + 1];
+      PX[4 * NXP + e] = k_ * U[5 * NH + h - 1] + k0 * U[5 * NH + h] + kp * U[5 * NH + h + 1];
+    }
+    __syncthreads();
+    // y pass: My on the four Mx results; My (Kx u6) + Ky (Mx u6)
+    for (int e = t; e < NYP; e += blockDim.x) {
+      const int ex = e % TX, ey = (e / TX) % TY, ez = e / (TX * TY);
+      const int q = ex + TX * ((ey + 1) + HY * ez);
+      T m_, m0, mp, k_, k0, kp;
+      ay.row(by0 + ey, m_, m0, mp, k_, k0, kp);
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        PY[f * NYP + e] = m_ * PX[f * NXP + q - TX] + m0 * PX[f * NXP + q] + mp * PX[f * NXP + q + TX];
+      PY[4 * NYP + e] = m_ * PX[4 * NXP + q - TX] + m0 * PX[4 * NXP + q] + mp * PX[4 * NXP + q + TX] +
+                        k_ * PX[3 * NXP + q - TX] + k0 * PX[3 * NXP + q] + kp * PX[3 * NXP + q + TX];
+    }
+    __syncthreads();
     if (own) {
-      T yc = (T)0, yg = (T)0, yf = (T)0;
+      // z pass and the S, S^T stencils
+      const int qz = tx + TX * (ty + TY * (tz + 1));
+      T m_, m0, mp, k_, k0, kp;
+      az.row(iz, m_, m0, mp, k_, k0, kp);
+      constexpr int zs = TX * TY;
+      T yc = m_ * PY[qz - zs] + m0 * PY[qz] + mp * PY[qz + zs];
+      T yg = m_ * PY[NYP + qz - zs] + m0 * PY[NYP + qz] + mp * PY[NYP + qz + zs];
+      T yf = m_ * PY[2 * NYP + qz - zs] + m0 * PY[2 * NYP + qz] + mp * PY[2 * NYP + qz + zs];
+      yf += m_ * PY[4 * NYP + qz - zs] + m0 * PY[4 * NYP + qz] + mp * PY[4 * NYP + qz + zs];
+      yf += k_ * PY[3 * NYP + qz - zs] + k0 * PY[3 * NYP + qz] + kp * PY[3 * NYP + qz + zs];
 #pragma unroll
       for (int d = 0; d < kStencil; ++d) {
-        if (!kuhn_offset(d)) continue;
         const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
         const int h = hc + dx + HX * (dy + HY * dz);
-        T s_, st_, b_, k_;
+        T s_, st_;
         if constexpr (sizeof(T) == 4) {
           s_ = cS[d];
           st_ = cST[d];
-          b_ = cB[d];
-          k_ = cK[d];
         } else {
           s_ = c.S[(size_t)d * N + j];
           st_ = c.ST[(size_t)d * N + j];
-          b_ = c.B[(size_t)d * N + j];
-          k_ = kL2 ? (T)0 : c.K[(size_t)d * N + j];
         }
-        yc += b_ * U[h] + s_ * U[NH + h];
-        yg += b_ * U[2 * NH + h] + st_ * U[3 * NH + h];
-        yf += b_ * U[4 * NH + h];
-        if constexpr (!kL2) yf += k_ * U[5 * NH + h];
+        yc += s_ * U[NH + h];
+        yg += st_ * U[3 * NH + h];
       }
       const bool dirj = p.dir[j] != 0;
       const T C0 = X0[hc], G0 = X0[NH + hc], Cp = Xp[hc];
@@ -268,110 +390,122 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_p1(DevProblem p, const T*
   cp_async_wait<0>();
 }
 
-template <typename T, typename TO>
-void launch_p1(const DevProblem& p, const T* x, TO* y, const double* b, cudaStream_t s) {
-  using Tl = TileA;
+// Estimated multiply-adds of one level over the grid with tile shape Tl: the
+// six time combinations on every halo node, the x and y passes, and the z pass
+// with the two 27-point stencils per tile node (ragged tiles count in full).
+template <typename Tl>
+double tile_work(const DevProblem& p) {
+  const double tiles = (double)((p.nx + Tl::TX - 1) / Tl::TX) * ((p.ny + Tl::TY - 1) / Tl::TY) *
+                       ((p.nz + Tl::TZ - 1) / Tl::TZ);
+  return tiles * (25.0 * Tl::NH + 30.0 * Tl::NXP + 36.0 * Tl::NYP + 138.0 * Tl::kThreads);
+}
+
+template <typename T, typename Tl, bool kP1 = false>
+void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaStream_t s, double* yd = nullptr) {
   const int tx = (p.nx + Tl::TX - 1) / Tl::TX, ty = (p.ny + Tl::TY - 1) / Tl::TY, tz = (p.nz + Tl::TZ - 1) / Tl::TZ;
   constexpr int NT = levels_per_cta<T>();
   dim3 grid(tx * ty * tz, (p.M + 1 + NT - 1) / NT);
+  Axis1D<T> ax, ay, az;
+  ax.init(p.nx, p.hx);
+  ay.init(p.ny, p.hy);
+  az.init(p.nz, p.hz);
   LevelW<T> w;
   w.init(p.tau, p.theta, p.beta1, p.beta2);
   // (the dynamic shared-memory limits are raised once, in matvec_prepare)
-  constexpr size_t smem = p1_smem<T, Tl>();
-  if constexpr (sizeof(T) == sizeof(TO)) {
-    auto* kernel = p.reg != 0 ? matvec_p1<T, true, Tl> : matvec_p1<T, false, Tl>;
-    kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, y, b, nullptr, tx, ty, w);
-  } else {
-    auto* kernel = p.reg != 0 ? matvec_p1<T, true, Tl, true> : matvec_p1<T, false, Tl, true>;
-    kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, nullptr, b, y, tx, ty, w);
-  }
+  constexpr size_t smem = mv_smem<T, Tl, kP1>();
+  auto* kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1> : matvec_tiled<T, false, Tl, kP1>;
+  if constexpr (sizeof(T) == 4)
+    if (yd) kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1, true> : matvec_tiled<T, false, Tl, kP1, true>;
+  kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, y, b, yd, tx, ty, ax, ay, az, w);
+}
+
+template <typename T>
+void launch_tiled(const DevProblem& p, const T* x, T* y, const double* b, cudaStream_t s, double* yd = nullptr) {
+  if (p.elem == KKT_ELEM_P1) launch_shape<T, TileA, true>(p, x, y, b, s, yd);
+  else if (tile_work<TileB>(p) < tile_work<TileA>(p)) launch_shape<T, TileB>(p, x, y, b, s, yd);
+  else launch_shape<T, TileA>(p, x, y, b, s, yd);
 }
 
 // ---------------------------------------------------------------------------
-// Trilinear elements.  In FP64 the FP64 pipe (2 lanes per SM and clock) is the limit,
-// so this kernel spends few instructions per point, in FP64 about 130 against 200 with
-// the operators applied to six time combinations formed on every halo node:
+// FP64, trilinear elements.  The FP64 pipe (2 lanes per SM and clock) is the limit,
+// so this kernel spends as few FP64 instructions per point as it can, about 130
+// against 200 in matvec_tiled:
 // - The spatial operators go to the levels themselves, once each, and the time
 //   weights are applied at the output nodes, carried from level to level in
-//   registers.  With level m in hand the CTA finishes the C row of level m and the
-//   G and f rows of level m - 1.  The mass matrix of the C and G rows is applied to the
-//   differences C^m - C^{m-1}, G^{m-1} - G^m (formed on the halo): the
+//   registers; matvec_tiled forms six weighted combinations on every halo node.
+//   With level m in hand the CTA finishes the C row of level m and the G and f rows of
+//   level m - 1.  The mass matrix of the C and G rows is applied to the differences
+//   C^m - C^{m-1}, G^{m-1} - G^m (formed on the halo), as in matvec_tiled: the
 //   difference of two products would lose digits where the solution varies slowly.
 // - The 1D factors of B and K are written [1 c 1] and [1 -c 1] (c = 4, 2 inside, 2, 1 at a
 //   domain face; neighbours outside the domain are zero), two instructions instead of
 //   three, and the products of the widths go into the time weights.
 // A CTA takes a tile of nodes and a run of levels; a run costs about 1.3 levels more
 // (one before and one after, in part), so the host picks long runs that still
-// fill the SMs.  FP32 keeps a node's 54 coefficients of S and S^T in registers and takes
-// 8 x 8 x 4 or 11 x 11 x 2 tiles (two CTAs of 128 registers a thread on an SM); shared-memory
-// reads (about 150 a point) and the four barriers a level bound it.
-// Measured against the six combinations, FP64: 32^3 x 64 1016 -> 650 us (11 x 11 x 3 tiles,
-// runs of 22), 5 x 4 x 3 x 6 56 -> 22.5 us (runs of one level).  FP32: 64^3 x 64 1064 -> 828 us,
-// 40^3 x 39 190 -> 166, 32^3 x 64 148 -> 132, 16^3 x 32 28.9 -> 25.0, 8^3 x 16 25.9 -> 10.3.  The
-// error against extended precision is smaller in both, on random and on smooth fields
-// (FP32, of the f rows: 1.2e-7 -> 0.9e-7, 1.2e-7 -> 0.7e-7 in the relative 2-norm).
+// fill the SMs.
+// Measured against matvec_tiled: 32^3 x 64 1016 -> 650 us (11 x 11 x 3 tiles, runs of 22),
+// 5 x 4 x 3 x 6 56 -> 22.5 us (runs of one level); the error against extended precision is
+// slightly smaller, on random and on smooth fields.
 // ---------------------------------------------------------------------------
-template <typename T, typename Tl>
-constexpr size_t levels_smem() {
+template <typename Tl>
+constexpr size_t mv64_smem() {
   // C, G: levels m-1, m, m+1; f: m, m+1; the x-pass results; the y-pass results over the differences
-  return sizeof(T) * (8 * Tl::NH + 5 * Tl::NXP + (5 * Tl::NYP > 2 * Tl::NH ? 5 * Tl::NYP : 2 * Tl::NH));
+  return sizeof(double) * (8 * Tl::NH + 5 * Tl::NXP + (5 * Tl::NYP > 2 * Tl::NH ? 5 * Tl::NYP : 2 * Tl::NH));
 }
 
-template <typename T>
-struct LevelWeights {
-  T sB;                  // product of the mass factors: B = sB [1 c 1] (x) [1 c 1] (x) [1 c 1]
-  T ry, rz;              // weights of the y and z stiffness against the x stiffness
-  T wt0, wt1;            // tau theta, tau (1 - theta)
-  T eG, eF, eK;          // neighbouring level in the f row: G, f by B; f by K
-  T dG, dF, dK;          // the level itself with one time element beside it
-  T dG2, dF2, dK2;       // with two
-  T th, th1, tau;
-  void init(const DevProblem& p) {   // formed in FP64
+struct Weights64 {
+  double sB;                  // product of the mass factors: B = sB [1 c 1] (x) [1 c 1] (x) [1 c 1]
+  double ry, rz;              // weights of the y and z stiffness against the x stiffness
+  double wt0, wt1;            // tau theta, tau (1 - theta)
+  double eG, eF, eK;          // neighbouring level in the f row: G, f by B; f by K
+  double dG, dF, dK;          // the level itself with one time element beside it
+  double dG2, dF2, dK2;       // with two
+  double th, th1, tau;
+  void init(const DevProblem& p) {
     const double mo = p.hx / 6.0 * (p.hy / 6.0) * (p.hz / 6.0);
     const double ax = -6.0 / (p.hx * p.hx), ay = -6.0 / (p.hy * p.hy), az = -6.0 / (p.hz * p.hz);
-    sB = (T)mo;
-    ry = (T)(ay / ax);
-    rz = (T)(az / ax);
-    tau = (T)p.tau;
-    th = (T)p.theta;
-    th1 = (T)(1.0 - p.theta);
-    wt0 = (T)(p.tau * p.theta);
-    wt1 = (T)(p.tau * (1.0 - p.theta));
-    const double m6 = p.tau / 6.0, m3 = p.tau / 3.0, l1 = 1.0 / p.tau;
-    double f6 = -p.beta1 * l1 * mo, f3 = p.beta1 * l1 * mo, k6 = p.beta2 * m6 * mo, k3 = p.beta2 * m3 * mo;
+    sB = mo;
+    ry = ay / ax;
+    rz = az / ax;
+    tau = p.tau;
+    th = p.theta;
+    th1 = 1.0 - p.theta;
+    wt0 = tau * th;
+    wt1 = tau * th1;
+    const double m6 = tau / 6.0, m3 = tau / 3.0, l1 = 1.0 / tau;
+    eG = -m6 * sB;
+    dG = -m3 * sB;
+    eF = -p.beta1 * l1 * sB;
+    dF = p.beta1 * l1 * sB;
+    eK = p.beta2 * m6 * sB;
+    dK = p.beta2 * m3 * sB;
     if (p.reg != 0) {   // H1-L2: the beta2 term goes through B
-      f6 += k6;
-      f3 += k3;
+      eF += eK;
+      dF += dK;
     } else {
-      k6 *= ax;
-      k3 *= ax;
+      eK *= ax;
+      dK *= ax;
     }
-    eG = (T)(-m6 * mo);
-    dG = (T)(-m3 * mo);
-    eF = (T)f6;
-    dF = (T)f3;
-    eK = (T)k6;
-    dK = (T)k3;
-    dG2 = 2 * dG;
-    dF2 = 2 * dF;
-    dK2 = 2 * dK;
+    dG2 = 2.0 * dG;
+    dF2 = 2.0 * dF;
+    dK2 = 2.0 * dK;
   }
 };
 
-template <typename T, typename TO, bool kL2, typename Tl>
-__global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads > 256 ? 2 : 3)
-    matvec_levels(DevProblem p, const T* __restrict__ x, TO* __restrict__ y, const double* __restrict__ b, int tiles_x,
-                  int tiles_y, int run, LevelWeights<T> W) {
+template <bool kL2, typename Tl>
+__global__ void __launch_bounds__(Tl::kThreads, Tl::kThreads > 256 ? 2 : 3) matvec64_levels(DevProblem p, const double* __restrict__ x,
+                                                                double* __restrict__ y, const double* __restrict__ b,
+                                                                int tiles_x, int tiles_y, int run, Weights64 W) {
   constexpr int TX = Tl::TX, TY = Tl::TY, TZ = Tl::TZ;
   constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH, NXP = Tl::NXP, NYP = Tl::NYP, NT = Tl::kThreads;
   if (gated_off(p.gate)) return;
   extern __shared__ __align__(16) unsigned char mv_sm[];
-  T* Cs = reinterpret_cast<T*>(mv_sm);   // [3 slots][NH]: level mod 3
-  T* Gs = Cs + 3 * NH;                        // [3 slots][NH]
-  T* Fs = Gs + 3 * NH;                        // [2 slots][NH]: level mod 2
-  T* PX = Fs + 2 * NH;                        // [5][NXP]
-  T* PY = PX + 5 * NXP;                       // [5][NYP]
-  T* U = PY;                                  // [2][NH]: the differences, read before PY is written
+  double* Cs = reinterpret_cast<double*>(mv_sm);   // [3 slots][NH]: level mod 3
+  double* Gs = Cs + 3 * NH;                        // [3 slots][NH]
+  double* Fs = Gs + 3 * NH;                        // [2 slots][NH]: level mod 2
+  double* PX = Fs + 2 * NH;                        // [5][NXP]
+  double* PY = PX + 5 * NXP;                       // [5][NYP]
+  double* U = PY;                                  // [2][NH]: the differences, read before PY is written
   const int N = p.N, M = p.M;
   const int tile = blockIdx.x;
   const int bx0 = (tile % tiles_x) * TX, by0 = ((tile / tiles_x) % tiles_y) * TY, bz0 = (tile / (tiles_x * tiles_y)) * TZ;
@@ -384,12 +518,12 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
   const int hc = (tx + 1) + HX * ((ty + 1) + HY * (tz + 1));
 
   auto prefetch = [&](int m) {   // level m of x on the halo
-    T *dc = Cs + m % 3 * NH, *dg = Gs + m % 3 * NH, *df = Fs + m % 2 * NH;
+    double *dc = Cs + m % 3 * NH, *dg = Gs + m % 3 * NH, *df = Fs + m % 2 * NH;
     for (int h = t; h < NH; h += NT) {
       const int hx_ = h % HX, hy_ = (h / HX) % HY, hz_ = h / (HX * HY);
       const int gx = bx0 - 1 + hx_, gy = by0 - 1 + hy_, gz = bz0 - 1 + hz_;
       const bool valid = m <= M && gx >= 0 && gx < p.nx && gy >= 0 && gy < p.ny && gz >= 0 && gz < p.nz;
-      const T* src = valid ? x + 3 * ((long long)m * N + gx + (long long)p.nx * (gy + (long long)p.ny * gz)) : x;
+      const double* src = valid ? x + 3 * ((long long)m * N + gx + (long long)p.nx * (gy + (long long)p.ny * gz)) : x;
       cp_async_value(dc + h, src, valid);
       cp_async_value(dg + h, src + (valid ? 1 : 0), valid);
       cp_async_value(df + h, src + (valid ? 2 : 0), valid);
@@ -402,31 +536,20 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
   prefetch(m0);
   cp_async_commit();
   const bool dirj = own && p.dir[j] != 0;
-  const T sj = own ? (T)p.sens[j] : (T)0;
-  const bool sensor = sj != (T)0;
-  const T zm = inner(iz, p.nz) ? (T)4 : (T)2, zk = inner(iz, p.nz) ? (T)-2 : (T)-1;
-  T carryC = (T)0, accG = (T)0, accF = (T)0, Eprev = (T)0, yC = (T)0;   // yC: the C row of level m - 1
-  // FP32 keeps its coefficients in registers (converted once); FP64 reads them at every level
-  float cS[sizeof(T) == 4 ? kStencil : 1], cST[sizeof(T) == 4 ? kStencil : 1];
-  if constexpr (sizeof(T) == 4) {
-#pragma unroll
-    for (int d = 0; d < kStencil; ++d) {
-      cS[d] = p.S32[(size_t)d * N + j];
-      cST[d] = p.ST32[(size_t)d * N + j];
-    }
-  }
-  auto coef = [&](int d) -> T { if constexpr (sizeof(T) == 4) return cS[d]; else return p.S[(size_t)d * N + j]; };
-  auto coefT = [&](int d) -> T { if constexpr (sizeof(T) == 4) return cST[d]; else return p.ST[(size_t)d * N + j]; };
-  auto put = [&](int n, T c_, T g_, T f_) {
+  const double sj = own ? p.sens[j] : 0.0;
+  const bool sensor = sj != 0.0;
+  const double zm = inner(iz, p.nz) ? 4.0 : 2.0, zk = inner(iz, p.nz) ? -2.0 : -1.0;
+  double carryC = 0.0, accG = 0.0, accF = 0.0, Eprev = 0.0, yC = 0.0;   // yC: the C row of level m - 1
+  auto put = [&](int n, double c, double g, double f) {
     const long long o = 3 * ((long long)n * N + j);
     if (b != nullptr) {
-      y[o] = (TO)(b[o] - (double)c_);
-      y[o + 1] = (TO)(b[o + 1] - (double)g_);
-      y[o + 2] = (TO)(b[o + 2] - (double)f_);
+      y[o] = b[o] - c;
+      y[o + 1] = b[o + 1] - g;
+      y[o + 2] = b[o + 2] - f;
     } else {
-      y[o] = c_;
-      y[o + 1] = g_;
-      y[o + 2] = f_;
+      y[o] = c;
+      y[o + 1] = g;
+      y[o + 2] = f;
     }
   };
   for (int m = m0; m <= m1; ++m) {
@@ -434,9 +557,9 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
     __syncthreads();   // level m has landed; the last step's reads are done
     if (m < m1) prefetch(m + 1);
     cp_async_commit();
-    const T *C0 = Cs + m % 3 * NH, *Cm = Cs + (m + 2) % 3 * NH;
-    const T *G0 = Gs + m % 3 * NH, *Gm = Gs + (m + 2) % 3 * NH;
-    const T* F0 = Fs + m % 2 * NH;
+    const double *C0 = Cs + m % 3 * NH, *Cm = Cs + (m + 2) % 3 * NH;
+    const double *G0 = Gs + m % 3 * NH, *Gm = Gs + (m + 2) % 3 * NH;
+    const double* F0 = Fs + m % 2 * NH;
     // what this level is needed for (a run's first and last level: in part)
     const bool doC = m >= n0 && m < n1 && m > 0;     // C row of level m
     const bool doS = m < n1;                         // S C^m: C rows of levels m, m + 1
@@ -452,27 +575,27 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
       const int ex = e % TX, ey = (e / TX) % HY, ez = e / (TX * HY);
       const int h = (ex + 1) + HX * (ey + HY * ez);
       const bool in_ = inner(bx0 + ex, p.nx);
-      const T c = in_ ? (T)4 : (T)2;
+      const double c = in_ ? 4.0 : 2.0;
       if (doC) PX[e] = fma(c, U[h], U[h - 1]) + U[h + 1];
       if (doG) PX[NXP + e] = fma(c, U[NH + h], U[NH + h - 1]) + U[NH + h + 1];
       PX[2 * NXP + e] = fma(c, G0[h], G0[h - 1]) + G0[h + 1];
-      const T f_ = F0[h], fl = F0[h - 1], fr = F0[h + 1];
+      const double f_ = F0[h], fl = F0[h - 1], fr = F0[h + 1];
       PX[3 * NXP + e] = fma(c, f_, fl) + fr;
-      if (!kL2) PX[4 * NXP + e] = fma(in_ ? (T)-2 : (T)-1, f_, fl) + fr;
+      if (!kL2) PX[4 * NXP + e] = fma(in_ ? -2.0 : -1.0, f_, fl) + fr;
     }
     __syncthreads();
     for (int e = t; e < NYP; e += NT) {
       const int ex = e % TX, ey = (e / TX) % TY, ez = e / (TX * TY);
       const int q = ex + TX * ((ey + 1) + HY * ez);
       const bool in_ = inner(by0 + ey, p.ny);
-      const T c = in_ ? (T)4 : (T)2;
+      const double c = in_ ? 4.0 : 2.0;
       if (doC) PY[e] = fma(c, PX[q], PX[q - TX]) + PX[q + TX];
       if (doG) PY[NYP + e] = fma(c, PX[NXP + q], PX[NXP + q - TX]) + PX[NXP + q + TX];
       PY[2 * NYP + e] = fma(c, PX[2 * NXP + q], PX[2 * NXP + q - TX]) + PX[2 * NXP + q + TX];
-      const T f_ = PX[3 * NXP + q], fl = PX[3 * NXP + q - TX], fr = PX[3 * NXP + q + TX];
+      const double f_ = PX[3 * NXP + q], fl = PX[3 * NXP + q - TX], fr = PX[3 * NXP + q + TX];
       PY[3 * NYP + e] = fma(c, f_, fl) + fr;
       if (!kL2) {
-        const T k = fma(in_ ? (T)-2 : (T)-1, f_, fl) + fr;
+        const double k = fma(in_ ? -2.0 : -1.0, f_, fl) + fr;
         PY[4 * NYP + e] = fma(W.ry, k, fma(c, PX[4 * NXP + q], PX[4 * NXP + q - TX]) + PX[4 * NXP + q + TX]);
       }
     }
@@ -481,12 +604,12 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
       const int q = tx + TX * (ty + TY * (tz + 1));
       constexpr int zs = TX * TY;
       // S C^m and S^T G^m, two chains each
-      T S0 = (T)0, S1 = (T)0, T0 = (T)0, T1 = (T)0;
+      double S0 = 0.0, S1 = 0.0, T0 = 0.0, T1 = 0.0;
       if (doS && doT) {
 #pragma unroll
         for (int d = 0; d < kStencil; ++d) {
           const int h = hc + d % 3 - 1 + HX * ((d / 3) % 3 - 1 + HY * (d / 9 - 1));
-          const T s_ = coef(d), st_ = coefT(d);
+          const double s_ = p.S[(size_t)d * N + j], st_ = p.ST[(size_t)d * N + j];
           if (d % 2) {
             S1 = fma(s_, C0[h], S1);
             T1 = fma(st_, G0[h], T1);
@@ -496,16 +619,13 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
           }
         }
       } else {
-        const T* A = nullptr;
-        if constexpr (sizeof(T) == 8) A = doS ? p.S : p.ST;
-        const T* v = doS ? C0 : G0;
-        T s0 = (T)0, s1 = (T)0;
+        const double* A = doS ? p.S : p.ST;
+        const double* v = doS ? C0 : G0;
+        double s0 = 0.0, s1 = 0.0;
 #pragma unroll
         for (int d = 0; d < kStencil; ++d) {
           const int h = hc + d % 3 - 1 + HX * ((d / 3) % 3 - 1 + HY * (d / 9 - 1));
-          T s_;
-          if constexpr (sizeof(T) == 4) s_ = doS ? cS[d] : cST[d];
-          else s_ = A[(size_t)d * N + j];
+          const double s_ = A[(size_t)d * N + j];
           if (d % 2) s1 = fma(s_, v[h], s1);
           else s0 = fma(s_, v[h], s0);
         }
@@ -517,20 +637,20 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
           T1 = s1;
         }
       }
-      const T BG = fma(zm, PY[2 * NYP + q], PY[2 * NYP + q - zs]) + PY[2 * NYP + q + zs];
-      const T f_ = PY[3 * NYP + q], fl = PY[3 * NYP + q - zs], fr = PY[3 * NYP + q + zs];
-      const T Bf = fma(zm, f_, fl) + fr;
-      T E = fma(W.eF, Bf, W.eG * BG);
+      const double BG = fma(zm, PY[2 * NYP + q], PY[2 * NYP + q - zs]) + PY[2 * NYP + q + zs];
+      const double f_ = PY[3 * NYP + q], fl = PY[3 * NYP + q - zs], fr = PY[3 * NYP + q + zs];
+      const double Bf = fma(zm, f_, fl) + fr;
+      double E = fma(W.eF, Bf, W.eG * BG);
       const bool mid = m > 0 && m < M;   // two time elements
-      T Fd = fma(mid ? W.dF2 : W.dF, Bf, fma(mid ? W.dG2 : W.dG, BG, Eprev));
+      double Fd = fma(mid ? W.dF2 : W.dF, Bf, fma(mid ? W.dG2 : W.dG, BG, Eprev));
       if (!kL2) {
-        const T Kf = fma(W.rz, fma(zk, f_, fl) + fr,
+        const double Kf = fma(W.rz, fma(zk, f_, fl) + fr,
                               fma(zm, PY[4 * NYP + q], PY[4 * NYP + q - zs]) + PY[4 * NYP + q + zs]);
         E = fma(W.eK, Kf, E);
         Fd = fma(mid ? W.dK2 : W.dK, Kf, Fd);
       }
       if (doG) {   // level m - 1 is complete
-        T g = fma(W.wt1, T0 + T1, accG);
+        double g = fma(W.wt1, T0 + T1, accG);
         g = fma(W.sB, fma(zm, PY[NYP + q], PY[NYP + q - zs]) + PY[NYP + q + zs], g);
         if (sensor) g += W.tau * sj * (W.th * C0[hc] + W.th1 * Cm[hc]);
         if (dirj) g = Gm[hc];
@@ -540,7 +660,7 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
       Eprev = E;
       if (doT) accG = W.wt0 * (T0 + T1);
       if (doS) {
-        const T D = fma(-W.sB, Bf, S0 + S1);
+        const double D = fma(-W.sB, Bf, S0 + S1);
         if (doC) yC = fma(W.sB, fma(zm, PY[q], PY[q - zs]) + PY[q + zs], fma(W.wt0, D, carryC));
         if (m == 0 || dirj) yC = C0[hc];
         carryC = W.wt1 * D;
@@ -551,20 +671,20 @@ __global__ void __launch_bounds__(Tl::kThreads, sizeof(T) == 4 || Tl::kThreads >
   cp_async_wait<0>();
 }
 
-template <typename T, typename TO, bool kL2, typename Tl>
-void launch_levels_tile(const DevProblem& p, const T* x, TO* y, const double* b, int run, cudaStream_t s) {
+template <bool kL2, typename Tl>
+void launch64_tile(const DevProblem& p, const double* x, double* y, const double* b, int run, cudaStream_t s) {
   const int tx = (p.nx + Tl::TX - 1) / Tl::TX, ty = (p.ny + Tl::TY - 1) / Tl::TY, tz = (p.nz + Tl::TZ - 1) / Tl::TZ;
-  LevelWeights<T> w;
+  Weights64 w;
   w.init(p);
-  matvec_levels<T, TO, kL2, Tl><<<dim3(tx * ty * tz, (p.M + run) / run), Tl::kThreads, levels_smem<T, Tl>(), s>>>(
+  matvec64_levels<kL2, Tl><<<dim3(tx * ty * tz, (p.M + run) / run), Tl::kThreads, mv64_smem<Tl>(), s>>>(
       p, x, y, b, tx, ty, run, w);
 }
 
-// Instructions of the busiest SM with tile shape Tl, and the run length that gives the
+// FP64 instructions of the busiest SM with tile shape Tl, and the run length that gives the
 // least: CTAs of an SM share its pipe; one alone leaves it idle at the barriers (measured
 // 0.7 of the rate of two or more).
 template <typename Tl>
-double work_levels(const DevProblem& p, int* run) {
+double work64(const DevProblem& p, int* run) {
   const long long tiles = (long long)((p.nx + Tl::TX - 1) / Tl::TX) * ((p.ny + Tl::TY - 1) / Tl::TY) *
                           ((p.nz + Tl::TZ - 1) / Tl::TZ);
   const double level = 2.0 * Tl::NH + 10.0 * Tl::NXP + 13.0 * Tl::NYP + 81.0 * ((Tl::kThreads + 31) / 32 * 32);
@@ -582,28 +702,20 @@ double work_levels(const DevProblem& p, int* run) {
   return best;
 }
 
-template <typename T, typename TO, typename T1, typename T2>
-void launch_levels(const DevProblem& p, const T* x, TO* y, const double* b, cudaStream_t s) {
-  int run1 = 1, run2 = 1;
-  const bool second = work_levels<T2>(p, &run2) < work_levels<T1>(p, &run1);
-  if (p.reg != 0) {
-    if (second) launch_levels_tile<T, TO, true, T2>(p, x, y, b, run2, s);
-    else launch_levels_tile<T, TO, true, T1>(p, x, y, b, run1, s);
-  } else {
-    if (second) launch_levels_tile<T, TO, false, T2>(p, x, y, b, run2, s);
-    else launch_levels_tile<T, TO, false, T1>(p, x, y, b, run1, s);
-  }
-}
-
 void launch_fp64(const DevProblem& p, const double* x, double* y, const double* b, cudaStream_t s) {
-  if (p.elem == KKT_ELEM_P1) launch_p1<double, double>(p, x, y, b, s);
-  else launch_levels<double, double, TileA, TileC>(p, x, y, b, s);
-}
-
-template <typename TO>
-void launch_fp32(const DevProblem& p, const float* x, TO* y, const double* b, cudaStream_t s) {
-  if (p.elem == KKT_ELEM_P1) launch_p1<float, TO>(p, x, y, b, s);
-  else launch_levels<float, TO, TileA, TileB>(p, x, y, b, s);
+  if (p.elem == KKT_ELEM_P1) {
+    launch_shape<double, TileA, true>(p, x, y, b, s);
+    return;
+  }
+  int run_a = 1, run_c = 1;
+  const double a = work64<TileA>(p, &run_a), c = work64<TileC>(p, &run_c);
+  if (p.reg != 0) {
+    if (c < a) launch64_tile<true, TileC>(p, x, y, b, run_c, s);
+    else launch64_tile<true, TileA>(p, x, y, b, run_a, s);
+  } else {
+    if (c < a) launch64_tile<false, TileC>(p, x, y, b, run_c, s);
+    else launch64_tile<false, TileA>(p, x, y, b, run_a, s);
+  }
 }
 
 __global__ void d2f(const double* __restrict__ x, float* __restrict__ y, long long n, const int* gate) {
@@ -614,34 +726,42 @@ __global__ void d2f(const double* __restrict__ x, float* __restrict__ y, long lo
 
 }  // namespace
 
-template <typename T, typename TO, typename Tl>
-kkt_status prepare_levels() {
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_levels<T, TO, false, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)levels_smem<T, Tl>()));
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_levels<T, TO, true, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)levels_smem<T, Tl>()));
+template <typename Tl, bool kP1, bool kWide>
+kkt_status prepare32() {
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<float, false, Tl, kP1, kWide>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<float, Tl, kP1>()));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<float, true, Tl, kP1, kWide>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<float, Tl, kP1>()));
   return KKT_OK;
 }
 
-template <typename T, bool kWide>
-kkt_status prepare_p1() {
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_p1<T, false, TileA, kWide>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p1_smem<T, TileA>()));
-  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_p1<T, true, TileA, kWide>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p1_smem<T, TileA>()));
+template <typename Tl>
+kkt_status prepare64() {
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec64_levels<false, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)mv64_smem<Tl>()));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec64_levels<true, Tl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)mv64_smem<Tl>()));
+  return KKT_OK;
+}
+
+kkt_status prepare64_p1() {
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<double, false, TileA, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<double, TileA, true>()));
+  KKT_TRY_CUDA(cudaFuncSetAttribute(matvec_tiled<double, true, TileA, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mv_smem<double, TileA, true>()));
   return KKT_OK;
 }
 
 kkt_status matvec_prepare() {
-  KKT_TRY((prepare_levels<double, double, TileA>()));
-  KKT_TRY((prepare_levels<double, double, TileC>()));
-  KKT_TRY((prepare_levels<float, float, TileA>()));
-  KKT_TRY((prepare_levels<float, float, TileB>()));
-  KKT_TRY((prepare_levels<float, double, TileA>()));
-  KKT_TRY((prepare_levels<float, double, TileB>()));
-  KKT_TRY((prepare_p1<double, false>()));
-  KKT_TRY((prepare_p1<float, false>()));
-  KKT_TRY((prepare_p1<float, true>()));
+  KKT_TRY(prepare64<TileA>());
+  KKT_TRY(prepare64<TileC>());
+  KKT_TRY(prepare64_p1());
+  KKT_TRY((prepare32<TileA, false, false>()));
+  KKT_TRY((prepare32<TileA, false, true>()));
+  KKT_TRY((prepare32<TileB, false, false>()));
+  KKT_TRY((prepare32<TileB, false, true>()));
+  KKT_TRY((prepare32<TileA, true, false>()));
+  KKT_TRY((prepare32<TileA, true, true>()));
   return KKT_OK;
 }
 
@@ -653,7 +773,7 @@ kkt_status launch_matvec64(const DevProblem& p, const double* x, double* y, cuda
 }
 
 kkt_status launch_matvec32(const DevProblem& p, const float* x, float* y, cudaStream_t s) {
-  launch_fp32(p, x, y, nullptr, s);
+  launch_tiled<float>(p, x, y, nullptr, s);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
@@ -668,7 +788,7 @@ kkt_status launch_residual(const DevProblem& p, const double* b, const double* x
 
 // r = b - F x (FP64) with the product in FP32 of x in FP32.
 kkt_status launch_residual32(const DevProblem& p, const double* b, const float* x, double* r, cudaStream_t s) {
-  launch_fp32(p, x, r, b, s);
+  launch_tiled<float>(p, x, nullptr, b, s, r);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
@@ -676,7 +796,7 @@ kkt_status launch_residual32(const DevProblem& p, const double* b, const float* 
 
 // y = F x (FP64) with the product in FP32 of x in FP32.
 kkt_status launch_matvec32_d(const DevProblem& p, const float* x, double* y, cudaStream_t s) {
-  launch_fp32(p, x, y, nullptr, s);
+  launch_tiled<float>(p, x, nullptr, nullptr, s, y);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;

@@ -1,8 +1,8 @@
-"""KKT matvec (FP64, FP32) and residual where tiles and level runs end, against the oracle's assembled F_h.
+"""FP64 KKT matvec and residual where tiles and level runs end, against the oracle's assembled F_h.
 
 Grids of one cell, of exactly one tile and of one node more, ragged tiles, one step, runs of one
 level (few tiles) and of several with a ragged last one (many tiles), both regularisers, both time
-schemes.  Bar in FP64: |y - y_ref| <= 1e-12 (|F||x|)_i per output, as in test_gpu_kkt.py (each side's
+schemes.  Bar: |y - y_ref| <= 1e-12 (|F||x|)_i per output, as in test_gpu_kkt.py (each side's
 rounding is below 330 u (|F||x|)_i).
 """
 
@@ -45,16 +45,3 @@ def test_fp64_matvec_and_residual_match_oracle(api, cells, M, reg, theta):
     assert np.all(np.abs(y - F @ x) <= bound)
     r = prob.residual(bd, xd).cpu().numpy()
     assert np.all(np.abs(r - (b - F @ x)) <= bound + 1e-15 * np.abs(b))
-
-
-@pytest.mark.parametrize("reg,theta", [("h1h1", 0.5), ("h1l2", 1.0)])
-@pytest.mark.parametrize("cells,M", CASES, ids=[f"{'x'.join(map(str, c))}x{m}" for c, m in CASES])
-def test_fp32_matvec_matches_oracle(api, cells, M, reg, theta):
-    # bar: 331 u (|F||x|)_i < 3e-5 (|F||x|)_i with u = 2^-24, the rounding of x included
-    w = W.random_small(51, cells=cells, M=M, theta=theta, reg=reg, nsens=5,
-                       dirichlet_faces=W.FACE_X0 if max(cells) > 1 else W.FACE_Z1)
-    F = okkt.assemble(okkt.Problem.from_workload(w))
-    prob = api.Problem.from_workload(w)
-    x = W.random_vector(prob.n, 3)
-    y = prob.apply(torch.from_numpy(x).float().cuda()).double().cpu().numpy()
-    assert np.all(np.abs(y - F @ x) <= 3e-5 * (abs(F) @ np.abs(x)) + 1e-300)
