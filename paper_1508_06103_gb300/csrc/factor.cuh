@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDes
   }
 }
 
-// gather, then factor, in place on F (chunk layout); both on stream s
+// gather, then factor, in place on F (groups of 8 points); both on stream s
 template <typename T>
 kkt_status factor_launch(ras_precond* m, T* F, cudaStream_t s) {
   const dim3 g((unsigned)((kGroup * (long long)m->max_groups + kGatherThreads - 1) / kGatherThreads), m->nbox);

@@ -183,11 +183,11 @@ __device__ __forceinline__ void cp_async_wait() {
 // kL2: the H1-L2 regularisation (its beta2 term goes through B), a template
 // argument so the H1-H1 kernel carries no test for it.  kP1: P1 elements, B and
 // K as stored 15-point stencils (no x and y passes, two barriers per level).
-// kWide (FP32): the product, or b minus it, written as FP64 values to yd.
+// kWide (FP32): the product, or b minus it, written as FP64 values (y points to doubles).
 template <typename T, bool kL2, typename Tl, bool kP1 = false, bool kWide = false>
 __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const T* __restrict__ x,
                                                              T* __restrict__ y, const double* __restrict__ b,
-                                                             double* __restrict__ yd, int tiles_x, int tiles_y, Axis1D<T> ax, Axis1D<T> ay,
+                                                             int tiles_x, int tiles_y, Axis1D<T> ax, Axis1D<T> ay,
                                                              Axis1D<T> az, LevelW<T> W) {
   constexpr int TX = Tl::TX, TY = Tl::TY, TZ = Tl::TZ;
   constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH, NXP = Tl::NXP, NYP = Tl::NYP;
@@ -221,23 +221,6 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
       cp_async_value(dst + h, src, valid);
       cp_async_value(dst + NH + h, src + (valid ? 1 : 0), valid);
       cp_async_value(dst + 2 * NH + h, src + (valid ? 2 : 0), valid);
-    }
-  };
-  // F x, b - F x, or (FP32) either of them as FP64 values
-  auto put = [&](int n, T c_, T g_, T f_) {
-    const long long o = 3 * ((long long)n * N + j);
-    if constexpr (kWide) {
-      yd[o] = b != nullptr ? b[o] - (double)c_ : (double)c_;
-      yd[o + 1] = b != nullptr ? b[o + 1] - (double)g_ : (double)g_;
-      yd[o + 2] = b != nullptr ? b[o + 2] - (double)f_ : (double)f_;
-    } else if (b != nullptr) {
-      y[o] = (T)(b[o] - (double)c_);
-      y[o + 1] = (T)(b[o + 1] - (double)g_);
-      y[o + 2] = (T)(b[o + 2] - (double)f_);
-    } else {
-      y[o] = c_;
-      y[o + 1] = g_;
-      y[o + 2] = f_;
     }
   };
   // S and S^T (and under P1, B and K) of the thread's node: registers in
@@ -323,7 +306,21 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
         if (n == 0 || dirj) yc = C0;
         if (n == M || dirj) yg = G0;
         else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
-        put(n, yc, yg, yf);
+        const long long o = 3 * ((long long)n * N + j);
+        if constexpr (kWide) {
+          double* yd = reinterpret_cast<double*>(y);
+          yd[o] = b != nullptr ? b[o] - (double)yc : (double)yc;
+          yd[o + 1] = b != nullptr ? b[o + 1] - (double)yg : (double)yg;
+          yd[o + 2] = b != nullptr ? b[o + 2] - (double)yf : (double)yf;
+        } else if (b != nullptr) {
+          y[o] = (T)(b[o] - (double)yc);
+          y[o + 1] = (T)(b[o + 1] - (double)yg);
+          y[o + 2] = (T)(b[o + 2] - (double)yf);
+        } else {
+          y[o] = yc;
+          y[o + 1] = yg;
+          y[o + 2] = yf;
+        }
       }
       continue;
     }
@@ -384,7 +381,21 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
       if (n == 0 || dirj) yc = C0;
       if (n == M || dirj) yg = G0;
       else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
-      put(n, yc, yg, yf);
+      const long long o = 3 * ((long long)n * N + j);
+      if constexpr (kWide) {
+        double* yd = reinterpret_cast<double*>(y);
+        yd[o] = b != nullptr ? b[o] - (double)yc : (double)yc;
+        yd[o + 1] = b != nullptr ? b[o + 1] - (double)yg : (double)yg;
+        yd[o + 2] = b != nullptr ? b[o + 2] - (double)yf : (double)yf;
+      } else if (b != nullptr) {
+        y[o] = (T)(b[o] - (double)yc);
+        y[o + 1] = (T)(b[o + 1] - (double)yg);
+        y[o + 2] = (T)(b[o + 2] - (double)yf);
+      } else {
+        y[o] = yc;
+        y[o + 1] = yg;
+        y[o + 2] = yf;
+      }
     }
   }
   cp_async_wait<0>();
@@ -416,7 +427,7 @@ void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaSt
   auto* kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1> : matvec_tiled<T, false, Tl, kP1>;
   if constexpr (sizeof(T) == 4)
     if (yd) kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1, true> : matvec_tiled<T, false, Tl, kP1, true>;
-  kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, y, b, yd, tx, ty, ax, ay, az, w);
+  kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, yd ? reinterpret_cast<T*>(yd) : y, b, tx, ty, ax, ay, az, w);
 }
 
 template <typename T>
