@@ -115,16 +115,16 @@ struct DevProblem {
   long long P;                              // points N * (M+1)
   double tau, theta, beta1, beta2;
   int reg;                                  // beta2 term: 0 stiffness K (H1-H1), 1 mass B (H1-L2)
-  int nsm;                                  // SMs of the device
   int elem;                                 // KKT_ELEM_Q1 or KKT_ELEM_P1 (kkt_set_element)
   double hx, hy, hz;                        // mesh widths (Q1: B and K are tensor products of 1D factors)
   const double *S, *ST, *B, *K;             // [27][N] row coefficients (FP64)
   const float *S32, *ST32, *B32, *K32;      // FP32 copies
-  const float4* pack32;                     // [N][27] FP32 {B, S, ST, K}, node by node (the FP32 factorisation)
   const unsigned char* dir;                 // [N] 1 on Dirichlet nodes
   const double* sens;                       // [N] sensor counts, 0 on Dirichlet nodes
   const int* gate;                          // device flag: the kernels return at once when it reads 0
                                             // (an Arnoldi step after convergence); nullptr = always run
+  const float4* pack32;                     // [N][27] FP32 {B, S, ST, K}, node by node (the FP32 factorisation)
+  int nsm;                                  // SMs of the device
 };
 
 // True when a gated kernel should return without work.
