@@ -281,13 +281,24 @@ kkt_status ras_status(ras_precond* m, int* code, void* stream);
 
 /*
  * ras_selftest_wait -- test hook for the bounded waits (no counterpart in the
- *   paper): launches one thread that waits, for limit_ms milliseconds
+ *   paper): launches one warp that waits, for limit_ms milliseconds
  *   (0 < limit_ms <= 1000), on an mbarrier that nothing completes, with the
  *   same bounded wait the subdomain solve uses; the wait gives up, sets the
  *   status word of m to 2 and the kernel returns.  Nothing is copied; the
  *   device and the handle stay usable (ras_refactor clears the word).
  */
 kkt_status ras_selftest_wait(ras_precond* m, double limit_ms, void* stream);
+
+/*
+ * ras_selftest_lanes -- test hook for the verdict of those waits (no
+ *   counterpart in the paper): a warp whose lanes are given different limits
+ *   waits on an mbarrier (kind 0) or on a counter of finished groups (kind 1)
+ *   that is completed after the shorter limit and before the longer one;
+ *   verdict[i] gets what lane i was told (1 = arrived, 0 = gave up).  All lanes
+ *   must be told the same.  Sets the status word of m to 2 when the warp gave
+ *   up (ras_refactor clears it).  Synchronous.
+ */
+kkt_status ras_selftest_lanes(ras_precond* m, int kind, int verdict[32], void* stream);
 
 /*
  * ras_apply -- z = sum_ij (R^0_ij)^T M_ij^{-1} R^delta_ij r (restricted prolongation,

@@ -177,6 +177,12 @@ class RAS:
         """Run the bounded-wait self-test kernel (ras_selftest_wait)."""
         check(self._lib.ras_selftest_wait(self.h, float(limit_ms), _stream(stream)), "ras_selftest_wait")
 
+    def selftest_lanes(self, kind: int, stream=None):
+        """Verdict of each lane of a warp whose lanes' wait limits differ (ras_selftest_lanes)."""
+        v = (C.c_int * 32)()
+        check(self._lib.ras_selftest_lanes(self.h, int(kind), v, _stream(stream)), "ras_selftest_lanes")
+        return list(v)
+
     def timing(self, kernel: int = 0):
         """(total ms, launches) since the last reset: kernel 0 subdomain solve, 1 factorisation."""
         ms, n = C.c_double(), C.c_longlong()

@@ -208,38 +208,95 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded wait on phase `parity` of an mbarrier: gives up after limit_ns
-// nanoseconds of polling, records status 2 in *failed and returns false.
+// Bounded waits of a warp.  All 32 lanes call them and all get the same verdict, by a vote: lanes
+// that went different ways would leave the others at the next full-warp shuffle for good.  The
+// timer is read only every so many polls, so what arrives within the first polls is seen without
+// its latency.
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s: copies and wavefronts take microseconds
+constexpr unsigned kAllLanes = 0xffffffffu;
+// Phase `parity` of an mbarrier; gives up after limit_ns nanoseconds of polling, records status 2 in
+// *failed and returns false.
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, int* failed,
                                           unsigned long long limit_ns = kWaitLimitNs) {
-  // the timer is read only every 64 polls, so a copy that lands within the
-  // first polls is seen without the timer's latency
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (__all_sync(kAllLanes, mbar_try_wait(bar, parity))) return true;
     if ((it & 63u) == 63u) {
       const unsigned long long t = global_ns();
       if (t0 == 0) {
         t0 = t;
-      } else if (t - t0 > limit_ns) {
+      } else if (__any_sync(kAllLanes, t - t0 > limit_ns)) {
         atomicExch(failed, 2);
         return false;
       }
     }
   }
 }
+// At least n groups in the counter `finished`; false, with status 2 in *failed and give_up() called,
+// when the limit ran out here, and false when *aborted says that it ran out in another warp.
+// CLUSTER: the counter is written by other CTAs of the cluster too.
+constexpr unsigned kPollNs = 20;   // a warp that polls without a pause takes issue slots from those at work
+template <bool CLUSTER, typename GiveUp>
+__device__ __forceinline__ bool count_wait(const int* finished, int n, const int* aborted, int* failed,
+                                           unsigned long long limit_ns, GiveUp&& give_up) {
+  unsigned long long t0 = 0;
+  for (unsigned it = 0; !__all_sync(kAllLanes, (CLUSTER ? ld_acquire_cluster(finished) : ld_acquire_cta(finished)) >= n);
+       ++it) {
+    __nanosleep(kPollNs);
+    if ((it & 255u) == 255u) {
+      const unsigned long long now = global_ns();
+      if (t0 == 0) {
+        t0 = now;
+      } else if (__any_sync(kAllLanes, now - t0 > limit_ns)) {
+        atomicExch(failed, 2);
+        give_up();
+        return false;
+      }
+      if (__any_sync(kAllLanes, *(const volatile int*)aborted != 0)) return false;
+    }
+  }
+  return true;
+}
 
-// Self-test of the bounded wait (ras_selftest_wait): one thread initialises an
-// mbarrier that expects one arrival, which nothing makes, and waits on it for
-// limit_ns; the wait gives up, sets *status = 2 and the kernel returns.  No
-// copy is issued, so nothing is in flight when the CTA exits.
+// Self-test of the bounded wait (ras_selftest_wait): one warp waits for
+// limit_ns on an mbarrier that expects one arrival, which nothing makes; the
+// wait gives up, sets *status = 2 and the kernel returns.  No copy is issued,
+// so nothing is in flight when the CTA exits.
 __global__ void wait_selftest(int* status, unsigned long long limit_ns) {
   __shared__ __align__(8) unsigned long long bar;
-  if (threadIdx.x != 0) return;
-  mbar_init(&bar, 1);
-  mbar_fence_init();
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    mbar_fence_init();
+  }
+  __syncwarp();
   mbar_wait(&bar, 0u, status, limit_ns);
+}
+
+// Self-test of the verdict (ras_selftest_lanes): the first warp waits, on an mbarrier (KIND 0) or a
+// counter (1), half of its lanes for `limit_ns` and half for 100 times that; the second warp
+// completes what it waits for after 3 limit_ns.  verdict: what each lane got.
+template <int KIND>
+__global__ void lane_selftest(int* status, unsigned long long limit_ns, int* verdict) {
+  __shared__ __align__(8) unsigned long long bar;
+  __shared__ int finished, aborted;
+  const int lane = threadIdx.x % 32;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    mbar_fence_init();
+    finished = aborted = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const unsigned long long limit = lane < 16 ? limit_ns : 100 * limit_ns;
+    const bool ok = KIND == 0 ? mbar_wait(&bar, 0u, status, limit)
+                              : count_wait<false>(&finished, 1, &aborted, status, limit, [] {});
+    verdict[lane] = ok;
+  } else if (lane == 0) {
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < 3 * limit_ns) __nanosleep(1000);
+    if (KIND == 0) mbar_expect_tx(&bar, 0);
+    else add_release_cta(&finished, 1);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -417,7 +474,6 @@ template <typename S>
 constexpr int solve_buffer(bool ring) {
   return LaneFactors<S>::kStaged ? 32 * kLaneL * (int)sizeof(S) + (ring ? kNbrBytes : 0) : 0;
 }
-constexpr unsigned kPollNs = 20;
 constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter of finished groups, abort word
 
 // CS: CTAs of a cluster that share a box: the groups go round the warps of all of them, the
@@ -521,22 +577,11 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
 
   // waits until n groups are done; false when the limit ran out here or in another warp
   auto wait_done = [&](int n) -> bool {
-    unsigned long long t0 = 0;
-    for (unsigned it = 0; (CS == 1 ? ld_acquire_cta(finished) : ld_acquire_cluster(finished)) < n; ++it) {
-      __nanosleep(kPollNs);   // a warp that polls without a pause takes issue slots from those at work
-      if ((it & 255u) == 255u) {
-        const unsigned long long now = global_ns();
-        if (t0 == 0) t0 = now;
-        else if (now - t0 > kWaitLimitNs) {
-          atomicExch(status, 2);
-          if constexpr (CS == 1) atomicExch(aborted, 1);
-          else
-            for (int c = 0; c < CS; ++c) add_release_cluster(aborted, 1, c);
-        }
-        if (*(volatile int*)aborted) return false;
-      }
-    }
-    return true;
+    return count_wait<(CS > 1)>(finished, n, aborted, status, kWaitLimitNs, [&]() {
+      if constexpr (CS == 1) atomicExch(aborted, 1);
+      else
+        for (int c = 0; c < CS; ++c) add_release_cluster(aborted, 1, c);
+    });
   };
   LaneFactors<S> fac;
   int off[kNbrPerLane];   // offsets of the lane's neighbours in the padded local vector
@@ -1504,6 +1549,26 @@ extern "C" kkt_status ras_selftest_wait(ras_precond* m, double limit_ms, void* s
   wait_selftest<<<1, 32, 0, (cudaStream_t)stream>>>(m->status, (unsigned long long)(limit_ms * 1e6));
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
+  return KKT_OK;
+}
+
+extern "C" kkt_status ras_selftest_lanes(ras_precond* m, int kind, int verdict[32], void* stream) {
+  if (!m || !verdict || kind < 0 || kind > 1) {
+    set_error("ras_selftest_lanes: null argument or kind not 0 (mbarrier) / 1 (counter)");
+    return KKT_ERR_ARG;
+  }
+  const cudaStream_t s = (cudaStream_t)stream;
+  constexpr unsigned long long limit_ns = 5000000ull;
+  int* d = nullptr;
+  KKT_TRY_CUDA(cudaMalloc(&d, 32 * sizeof(int)));
+  if (kind == 0) lane_selftest<0><<<1, 64, 0, s>>>(m->status, limit_ns, d);
+  else lane_selftest<1><<<1, 64, 0, s>>>(m->status, limit_ns, d);
+  KKT_COUNT(1);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(verdict, d, 32 * sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFree(d);
+  KKT_TRY_CUDA(e);
   return KKT_OK;
 }
 
