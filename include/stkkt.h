@@ -269,6 +269,15 @@ kkt_status ras_info(const ras_precond* m, int* nbox, long long* points, long lon
 kkt_status ras_solve_shape(const ras_precond* m, int* chunk_points, int* stages, int* lanes, int* smem_vectors);
 
 /*
+ * ras_solve_form -- which of its forms the ILU(0) subdomain solve takes: warps
+ *   of a box's CTA, buffers of factor values a warp has in shared memory (0 in
+ *   FP64, which reads them from global memory), CTAs (a cluster) that share a
+ *   box, and 1 if the last wavefronts are kept in shared memory.  Any output
+ *   may be NULL.  Reporting only; the paper has no counterpart.
+ */
+kkt_status ras_solve_form(const ras_precond* m, int* warps, int* buffers, int* cluster, int* ring);
+
+/*
  * ras_status -- the preconditioner's device status word, read on `stream`
  *   (synchronises that stream): 0 = fine; 1 = the last factorisation met a
  *   zero or non-finite pivot (returns ZERO_PIVOT); 2 = a subdomain solve gave

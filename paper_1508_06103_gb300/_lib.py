@@ -56,6 +56,7 @@ SIGNATURES = {
                                   C.POINTER(C.c_void_p)]),
     "ras_solve_shape": (C.c_int, [C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int),
                                   C.POINTER(C.c_int)]),
+    "ras_solve_form": (C.c_int, [C.c_void_p] + [C.POINTER(C.c_int)] * 4),
     "ras_status": (C.c_int, [C.c_void_p, C.POINTER(C.c_int), C.c_void_p]),
     "ras_setup_batch": (C.c_int, [C.POINTER(C.c_void_p), C.c_int, C.POINTER(C.c_int), C.c_int, C.c_int,
                                   C.POINTER(C.c_int), C.POINTER(C.c_void_p)]),

@@ -167,6 +167,12 @@ class RAS:
               "ras_solve_shape")
         return dict(chunk_points=ch.value, stages=ns.value, lanes=ln.value, smem_vectors=bool(sv.value))
 
+    def solve_form(self):
+        """dict(warps, buffers, cluster, ring) of the ILU(0) subdomain solve (ras_solve_form)."""
+        v = [C.c_int() for _ in range(4)]
+        check(self._lib.ras_solve_form(self.h, *(C.byref(x) for x in v)), "ras_solve_form")
+        return dict(warps=v[0].value, buffers=v[1].value, cluster=v[2].value, ring=bool(v[3].value))
+
     def status(self, stream=None) -> int:
         """The device status word (ras_status); raises KktError for 1 (zero pivot) and 2 (copy wait gave up)."""
         code = C.c_int()

@@ -1520,6 +1520,18 @@ extern "C" kkt_status ras_solve_shape(const ras_precond* m, int* chunk_points, i
   return KKT_OK;
 }
 
+extern "C" kkt_status ras_solve_form(const ras_precond* m, int* warps, int* buffers, int* cluster, int* ring) {
+  if (!m) {
+    set_error("ras_solve_form: null argument");
+    return KKT_ERR_ARG;
+  }
+  if (warps) *warps = m->warps;
+  if (buffers) *buffers = m->local == 0 && m->prec != 64 ? solve_buffers(m->nstage) : 0;
+  if (cluster) *cluster = m->cluster;
+  if (ring) *ring = m->local == 0 && m->ring ? 1 : 0;
+  return KKT_OK;
+}
+
 extern "C" kkt_status ras_status(ras_precond* m, int* code, void* stream) {
   if (!m || !code) {
     set_error("ras_status: null argument");

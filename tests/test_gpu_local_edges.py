@@ -127,3 +127,38 @@ def test_box_shared_by_ctas_has_the_bits_of_one_cta(api, name, prec):
     assert torch.isfinite(z).all() and z.abs().max() > 0
     assert torch.equal(many.apply(r.repeat(80))[-probs[0].n:], z)
     assert one.status() == 0
+
+
+# the forms the chooser takes: clusters for the few boxes above, one CTA a box for many of them
+@pytest.mark.parametrize("prec", [64, 32, 16])
+@pytest.mark.parametrize("name", CLUSTER_CELLS)
+def test_few_boxes_take_a_cluster_and_many_do_not(api, name, prec):
+    *cells, M = CLUSTER_CELLS[name]
+    w = W.random_small(44, cells=tuple(cells), M=M, nsens=4, reg="h1l2")
+    beta = max(w.h) ** 2
+    w = dataclasses.replace(w, T=M / 16.0, beta1=beta / 100, beta2=beta)
+    probs = [api.Problem.from_workload(w) for _ in range(80)]
+    form = api.RAS(probs[0], (1, 1, 1, 1), 0, prec).solve_form()
+    assert form["cluster"] == (1 if prec != 64 and name == "2" else int(name)) and not form["ring"]
+    form = api.BatchRAS(probs, (1, 1, 1, 1), 0, prec).solve_form()
+    # the ring of "8" (508 points in a wavefront) beside 16 FP32 buffers would take 233,104 of 232,448 bytes
+    assert form["cluster"] == 1 and form["ring"] == (prec == 16 or (prec == 32 and name != "8"))
+
+
+# the ring of wavefronts in shared memory is taken from a quarter as many boxes as SMs: enough
+# copies of the problem in one batch
+@pytest.mark.parametrize("prec", [32, 16])
+@pytest.mark.parametrize("name", CASES)
+def test_ring_of_wavefronts_on_edge_shapes_matches_oracle(api, oracle, name, prec):
+    _, _, nsub, ov = CASES[name]
+    w, r, zr = oracle(name)
+    copies = -(-40 // int(np.prod(nsub)))
+    probs = [api.Problem.from_workload(w) for _ in range(copies)]
+    ras = api.BatchRAS(probs, nsub, ov, prec)
+    form = ras.solve_form()
+    assert form["ring"] and form["cluster"] == 1 and form["buffers"] >= 1
+    z = ras.apply(torch.from_numpy(r).cuda().repeat(copies)).view(copies, -1)
+    assert torch.equal(z, z[:1].expand_as(z))
+    z0 = z[0].cpu().numpy()
+    assert np.linalg.norm(z0 - zr) <= (1e-3 if prec == 32 else 8 * 2.0**-8) * np.linalg.norm(zr)
+    assert ras.status() == 0
