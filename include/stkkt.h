@@ -310,6 +310,21 @@ kkt_status ras_selftest_wait(ras_precond* m, double limit_ms, void* stream);
 kkt_status ras_selftest_lanes(ras_precond* m, int kind, int verdict[32], void* stream);
 
 /*
+ * ras_selftest_solve -- test hook for the solve's way out when a wait runs out
+ *   (no counterpart in the paper): ras_apply (ILU(0), FP32 factors) with the waits of
+ *   one CTA of every box's cluster (cta; 0 where a box has one) held up.
+ *   hold 1: its counter of finished groups stays one short.  Those waits give
+ *   up after limit_ms milliseconds (0 < limit_ms <= 1000), the kernel returns,
+ *   the status word is 2 and z is left unwritten.  *drained (may be NULL) gets
+ *   the sum, over the copies of factor values in flight then, of the 1-based
+ *   numbers (in the order of the sweeps) of the groups they belong to, as the
+ *   warps waited for them before they left.  Synchronous; ras_refactor clears
+ *   the word.
+ */
+kkt_status ras_selftest_solve(ras_precond* m, const double* r, double* z, double limit_ms, int hold, int cta,
+                              int* drained, void* stream);
+
+/*
  * ras_apply -- z = sum_ij (R^0_ij)^T M_ij^{-1} R^delta_ij r (restricted prolongation,
  *   Cai-Sarkis form cited in Sec. 3.2); all boxes in one launch.  r, z FP64,
  *   3*N*(M+1) values each; the two spans must not overlap (ERR_ARG).  Does not

@@ -66,6 +66,8 @@ SIGNATURES = {
                                     C.c_double, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_double),
                                     C.POINTER(C.c_int), C.c_void_p]),
     "ras_selftest_wait": (C.c_int, [C.c_void_p, C.c_double, C.c_void_p]),
+    "ras_selftest_solve": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_double, C.c_int, C.c_int,
+                                     C.POINTER(C.c_int), C.c_void_p]),
     "ras_selftest_lanes": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int), C.c_void_p]),
     "coarse_refactor": (C.c_int, [C.c_void_p, C.c_void_p]),
     "two_level_refactor": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p]),

@@ -183,6 +183,14 @@ class RAS:
         """Run the bounded-wait self-test kernel (ras_selftest_wait)."""
         check(self._lib.ras_selftest_wait(self.h, float(limit_ms), _stream(stream)), "ras_selftest_wait")
 
+    def selftest_solve(self, r: torch.Tensor, z: torch.Tensor, limit_ms: float, hold: int = 1, cta: int = 0,
+                       stream=None) -> int:
+        """An apply whose waits run out (ras_selftest_solve); returns what its warps waited for on leaving."""
+        d = C.c_int()
+        check(self._lib.ras_selftest_solve(self.h, _ptr(r), _ptr(z), float(limit_ms), int(hold), int(cta), C.byref(d),
+                                           _stream(stream)), "ras_selftest_solve")
+        return d.value
+
     def selftest_lanes(self, kind: int, stream=None):
         """Verdict of each lane of a warp whose lanes' wait limits differ (ras_selftest_lanes)."""
         v = (C.c_int * 32)()

@@ -212,12 +212,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // that went different ways would leave the others at the next full-warp shuffle for good.  The
 // timer is read only every so many polls, so what arrives within the first polls is seen without
 // its latency.
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s: copies and wavefronts take microseconds
 constexpr unsigned kAllLanes = 0xffffffffu;
-// Phase `parity` of an mbarrier; gives up after limit_ns nanoseconds of polling, records status 2 in
-// *failed and returns false.
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, int* failed,
-                                          unsigned long long limit_ns = kWaitLimitNs) {
+// Phase `parity` of an mbarrier; gives up after limit_ns() nanoseconds of polling, records status 2
+// in *failed and returns false.
+template <typename Limit>
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, int* failed, Limit&& limit_ns) {
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
     if (__all_sync(kAllLanes, mbar_try_wait(bar, parity))) return true;
@@ -225,7 +224,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
       const unsigned long long t = global_ns();
       if (t0 == 0) {
         t0 = t;
-      } else if (__any_sync(kAllLanes, t - t0 > limit_ns)) {
+      } else if (__any_sync(kAllLanes, t - t0 > limit_ns())) {
         atomicExch(failed, 2);
         return false;
       }
@@ -236,9 +235,9 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 // when the limit ran out here, and false when *aborted says that it ran out in another warp.
 // CLUSTER: the counter is written by other CTAs of the cluster too.
 constexpr unsigned kPollNs = 20;   // a warp that polls without a pause takes issue slots from those at work
-template <bool CLUSTER, typename GiveUp>
+template <bool CLUSTER, typename Limit, typename GiveUp>
 __device__ __forceinline__ bool count_wait(const int* finished, int n, const int* aborted, int* failed,
-                                           unsigned long long limit_ns, GiveUp&& give_up) {
+                                           Limit&& limit_ns, GiveUp&& give_up) {
   unsigned long long t0 = 0;
   for (unsigned it = 0; !__all_sync(kAllLanes, (CLUSTER ? ld_acquire_cluster(finished) : ld_acquire_cta(finished)) >= n);
        ++it) {
@@ -247,7 +246,7 @@ __device__ __forceinline__ bool count_wait(const int* finished, int n, const int
       const unsigned long long now = global_ns();
       if (t0 == 0) {
         t0 = now;
-      } else if (__any_sync(kAllLanes, now - t0 > limit_ns)) {
+      } else if (__any_sync(kAllLanes, now - t0 > limit_ns())) {
         atomicExch(failed, 2);
         give_up();
         return false;
@@ -269,7 +268,7 @@ __global__ void wait_selftest(int* status, unsigned long long limit_ns) {
     mbar_fence_init();
   }
   __syncwarp();
-  mbar_wait(&bar, 0u, status, limit_ns);
+  mbar_wait(&bar, 0u, status, [=] { return limit_ns; });
 }
 
 // Self-test of the verdict (ras_selftest_lanes): the first warp waits, on an mbarrier (KIND 0) or a
@@ -287,7 +286,7 @@ __global__ void lane_selftest(int* status, unsigned long long limit_ns, int* ver
   }
   __syncthreads();
   if (threadIdx.x < 32) {
-    const unsigned long long limit = lane < 16 ? limit_ns : 100 * limit_ns;
+    auto limit = [=] { return lane < 16 ? limit_ns : 100 * limit_ns; };
     const bool ok = KIND == 0 ? mbar_wait(&bar, 0u, status, limit)
                               : count_wait<false>(&finished, 1, &aborted, status, limit, [] {});
     verdict[lane] = ok;
@@ -479,7 +478,9 @@ constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter
 // CS: CTAs of a cluster that share a box: the groups go round the warps of all of them, the
 // local vector stays in global memory (the L2 holds it), and each CTA has its own counter of
 // the box's finished groups, to which every group adds.  The bits are those of one CTA.
-template <typename S, bool SMEM, bool RING, int CS>
+// HOLD: the self-test's instance, in which waits of one CTA of a box run out (RasExtra).  (The limit and
+// the hold as run-time arguments of the others cost 1 % through the registers they were given.)
+template <typename S, bool SMEM, bool RING, int CS, bool HOLD = false>
 __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr, const S* __restrict__ F,
     typename SolveArith<S>::type* __restrict__ V, const double* __restrict__ r, double* __restrict__ z,
@@ -524,7 +525,10 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     mbar_init(&bar[lane], 1);
     mbar_fence_init();
   }
-  if (threadIdx.x == 0) *finished = *aborted = 0;
+  if (threadIdx.x == 0) {
+    *finished = HOLD && extra.hold == kHoldCounter && rank == extra.hold_cta ? -1 : 0;   // -1: one group short for good
+    *aborted = 0;
+  }
   if (RING && threadIdx.x < kVecWidth) ring[kVecWidth * kRingWaves * wcap + threadIdx.x] = (T)0;
   if (SMEM)
     for (int i = threadIdx.x; i < kVecWidth * st * (bx.lt + 2); i += blockDim.x) v[i] = (T)0;
@@ -576,8 +580,9 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   box_sync();
 
   // waits until n groups are done; false when the limit ran out here or in another warp
+  auto limit = [&]() { return HOLD && rank == extra.hold_cta ? extra.limit_ns : kWaitLimitNs; };
   auto wait_done = [&](int n) -> bool {
-    return count_wait<(CS > 1)>(finished, n, aborted, status, kWaitLimitNs, [&]() {
+    return count_wait<(CS > 1)>(finished, n, aborted, status, limit, [&]() {
       if constexpr (CS == 1) atomicExch(aborted, 1);
       else
         for (int c = 0; c < CS; ++c) add_release_cluster(aborted, 1, c);
@@ -590,7 +595,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   T v0 = 0, v1 = 0, v2 = 0, a0 = 0, a1 = 0, a2 = 0;   // the own point's values, of this group and the next
   bool ahead = false;                                 // the next one's are loaded
   // one sweep: the warp's groups k < kend
-  auto sweep = [&](int kend, auto upper_tag) -> bool {
+  auto sweep = [&](int kend, auto upper_tag) -> int {
     constexpr bool kUpper = decltype(upper_tag)::value;
     for (; k < kend; k += nwarp, ++t) {
       while (k >= before(s + 1)) ++s;
@@ -600,9 +605,9 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       vq2 = point(k + 2 * nwarp);
       [[maybe_unused]] unsigned places[kNbrPerLane / 2];   // RING: the neighbours' places, two a word
       if (kStaged) {
-        if (!mbar_wait(&bar[t % nbuf], (unsigned)(t / nbuf) & 1u, status)) {
+        if (!mbar_wait(&bar[t % nbuf], (unsigned)(t / nbuf) & 1u, status, limit)) {
           atomicExch(aborted, 1);
-          return false;
+          return 1;
         }
         const unsigned char* from = mine + (t % nbuf) * solve_buffer<S>(RING);
         fac.load(reinterpret_cast<const S*>(from), kUpper, lane);
@@ -617,7 +622,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       }
       // neighbours two and more wavefronts away (at the first backward step the own point is one
       // of the last wavefront's)
-      if (!wait_done(s == nlev ? ng : before(max(s - 1, 0)))) return false;
+      if (!wait_done(s == nlev ? ng : before(max(s - 1, 0)))) return 2;
       if (RING && ahead) {
         v0 = a0;
         v1 = a1;
@@ -642,7 +647,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       T sc = 0, sg = 0, sf = 0;
       T rc = 0, rg = 0, rf = 0, cf = 0, own_c = 0, own_g = 0;
       if constexpr (sizeof(T) == 8) {
-        if (!wait_done(before(s))) return false;
+        if (!wait_done(before(s))) return 2;
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i)
           if (dep_lanes(kUpper, i) >> sub & 1) neighbour(i);
@@ -704,7 +709,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
           rc = __shfl_down_sync(0xffffffffu, fac.at(36), 3);
           cf = __shfl_down_sync(0xffffffffu, fac.at(37), 3);
         }
-        if (!wait_done(before(s))) return false;
+        if (!wait_done(before(s))) return 2;
 #pragma unroll
         for (int i = 0; i < kNbrPerLane; ++i)
           if (dep_lanes(kUpper, i) >> sub & 1) neighbour(i);
@@ -755,28 +760,31 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
         if (lane < CS) add_release_cluster(finished, 1, lane);
       }
     }
-    return true;
+    return 0;
   };
 #pragma unroll
   for (int i = 0; i < kNbrPerLane; ++i) {   // earlier neighbour q: level n-1, d = q (q < 27); level n, d = q - 27
     const int q = sub + kLanes * i, d = q < 27 ? q : q - 27, dt = q < 27 ? -1 : 0;
     off[i] = kVecWidth * ((d % 3 - 1) + sy * ((d / 3) % 3 - 1) + sz * (d / 9 - 1) + st * dt);
   }
-  bool ok = sweep(ng, std::false_type{});   // forward, unit lower factor
+  int gave_up = sweep(ng, std::false_type{});   // forward, unit lower factor
   ahead = false;
-  if (ok) {
+  if (!gave_up) {
 #pragma unroll
     for (int i = 0; i < kNbrPerLane; ++i) {   // later neighbour q: level n, d = 14 + q (q < 13); level n+1, d = q - 13
       const int q = sub + kLanes * i, d = q < 13 ? 14 + q : q - 13, dt = q < 13 ? 0 : 1;
       off[i] = kVecWidth * ((d % 3 - 1) + sy * ((d / 3) % 3 - 1) + sz * (d / 9 - 1) + st * dt);
     }
-    ok = sweep(2 * ng, std::true_type{});   // backward, upper factor
+    gave_up = sweep(2 * ng, std::true_type{});   // backward, upper factor
   }
-  if (!ok && kStaged) {
-    // a wait gave up (status 2 is set): the copies of the warp's groups t .. t + nbuf may still be
-    // in flight into its buffers; wait for them, again with the limit
-    for (int q = t; q < t + nbuf; ++q)
-      if (warp + q * nwarp < 2 * ng) mbar_wait(&bar[q % nbuf], (unsigned)(q / nbuf) & 1u, status);
+  if (kStaged && gave_up) {
+    const int first = t + gave_up - 1;
+    // a wait gave up (status 2 is set): nbuf copies may still be in flight into the warp's buffers;
+    // wait for them, again with the limit
+    for (int q = first; q < first + nbuf; ++q)
+      if (warp + q * nwarp < 2 * ng && mbar_wait(&bar[q % nbuf], (unsigned)(q / nbuf) & 1u, status, limit) &&
+          HOLD && lane == 0)
+        atomicAdd(extra.drained, warp + q * nwarp + 1);
   }
   box_sync();             // (no CTA of the box ends while another may still count in its counter)
   if (*aborted) return;   // without writing z
@@ -893,15 +901,15 @@ struct SolveShape {
 };
 // groups per wavefront from which the largest CTA is taken
 constexpr int kFillGroups = 4;
-template <typename T>
+template <typename T, bool HOLD = false>
 const void* solve_kernel(bool smem_vec, bool ring, int cluster) {
   if constexpr (LaneFactors<T>::kStaged)
-    if (ring) return (const void*)ras_solve<T, false, true, 1>;
-  if (smem_vec) return (const void*)ras_solve<T, true, false, 1>;
-  return cluster == 8   ? (const void*)ras_solve<T, false, false, 8>
-         : cluster == 4 ? (const void*)ras_solve<T, false, false, 4>
-         : cluster == 2 ? (const void*)ras_solve<T, false, false, 2>
-                        : (const void*)ras_solve<T, false, false, 1>;
+    if (ring) return (const void*)ras_solve<T, false, true, 1, HOLD>;
+  if (smem_vec) return (const void*)ras_solve<T, true, false, 1, HOLD>;
+  return cluster == 8   ? (const void*)ras_solve<T, false, false, 8, HOLD>
+         : cluster == 4 ? (const void*)ras_solve<T, false, false, 4, HOLD>
+         : cluster == 2 ? (const void*)ras_solve<T, false, false, 2, HOLD>
+                        : (const void*)ras_solve<T, false, false, 1, HOLD>;
 }
 // CTAs (a cluster) per box where the boxes alone leave SMs idle: the most whose clusters all
 // run at once and that have 2.5 groups of a wavefront each; FP32 and BF16, less bound by
@@ -1377,6 +1385,8 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
   const size_t smem = solve_smem<S>(m->max_nlev, m->warps, m->nstage, m->ring) +
                       (m->ring ? ring_smem(m->wcap) : m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
   const void* kernel = solve_kernel<S>(m->smem_vec, m->ring, m->cluster);
+  if constexpr (std::is_same_v<S, float>)
+    if (extra.hold != kHoldNone) kernel = solve_kernel<S, true>(m->smem_vec, m->ring, m->cluster);
   const BoxDesc* boxes = m->boxes;
   const S* F = (const S*)m->F;
   const int *gptr = m->gptr, *vtab = m->vtab;
@@ -1562,6 +1572,35 @@ extern "C" kkt_status ras_selftest_wait(ras_precond* m, double limit_ms, void* s
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
+}
+
+extern "C" kkt_status ras_selftest_solve(ras_precond* m, const double* r, double* z, double limit_ms, int hold, int cta,
+                                         int* drained, void* stream) {
+  if (!m || !r || !z || !(limit_ms > 0.0) || limit_ms > 1000.0 || hold != kHoldCounter || cta < 0 ||
+      m->local != 0 || m->prec != 32 || cta >= m->cluster || spans_overlap(r, z, m->n_total)) {
+    set_error("ras_selftest_solve: null argument, limit_ms outside (0, 1000], hold not 1, cta outside the cluster, "
+              "r and z overlap, or not an ILU(0) preconditioner with FP32 factors");
+    return KKT_ERR_ARG;
+  }
+  const cudaStream_t s = (cudaStream_t)stream;
+  int* d = nullptr;
+  KKT_TRY_CUDA(cudaMalloc(&d, sizeof(int)));
+  RasExtra extra;
+  extra.limit_ns = (unsigned long long)(limit_ms * 1e6);
+  extra.hold = hold;
+  extra.hold_cta = cta;
+  extra.drained = d;
+  cudaError_t e = cudaFuncSetAttribute(solve_kernel<float, true>(m->smem_vec, m->ring, m->cluster),
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(int), s);
+  const kkt_status st = e == cudaSuccess ? ras_launch(m, r, z, s, nullptr, 0, extra) : KKT_OK;
+  int sum = 0;
+  if (e == cudaSuccess && st == KKT_OK) e = cudaMemcpyAsync(&sum, d, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && st == KKT_OK) e = cudaStreamSynchronize(s);
+  cudaFree(d);
+  KKT_TRY_CUDA(e);
+  if (drained) *drained = sum;
+  return st;
 }
 
 extern "C" kkt_status ras_selftest_lanes(ras_precond* m, int kind, int verdict[32], void* stream) {

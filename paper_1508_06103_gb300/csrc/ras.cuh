@@ -138,10 +138,16 @@ kkt_status ras_lu_solve(ras_precond* m, const double* r, double* z, cudaStream_t
 // reads gate[prob(b) * gate_stride]
 // z = M^{-1} r + add (where given); z32 (where given) also gets z rounded to FP32 (exact without add
 // where the solve runs in FP32)
+constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s: copies and wavefronts take microseconds
 struct RasExtra {
   const double* add = nullptr;
   float* z32 = nullptr;
+  // ras_selftest_solve: makes waits of one CTA of every box run out (RasHold), after limit_ns there
+  unsigned long long limit_ns = kWaitLimitNs;
+  int hold = 0, hold_cta = 0;
+  int* drained = nullptr;   // sum of the 1-based numbers of the groups whose copies were waited for on leaving
 };
+enum RasHold : int { kHoldNone = 0, kHoldCounter = 1 };
 kkt_status ras_launch(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate = nullptr,
                       int gate_stride = 0, const RasExtra& extra = RasExtra());
 kkt_status ras_check(ras_precond* m);
