@@ -313,7 +313,9 @@ kkt_status ras_selftest_lanes(ras_precond* m, int kind, int verdict[32], void* s
  * ras_selftest_solve -- test hook for the solve's way out when a wait runs out
  *   (no counterpart in the paper): ras_apply (ILU(0), FP32 factors) with the waits of
  *   one CTA of every box's cluster (cta; 0 where a box has one) held up.
- *   hold 1: its counter of finished groups stays one short.  Those waits give
+ *   hold 1: its counter of finished groups stays one short; hold 2: its copies
+ *   of factor values are waited for in vain (they land, but their barriers
+ *   expect one arrival more).  Those waits give
  *   up after limit_ms milliseconds (0 < limit_ms <= 1000), the kernel returns,
  *   the status word is 2 and z is left unwritten.  *drained (may be NULL) gets
  *   the sum, over the copies of factor values in flight then, of the 1-based

@@ -522,7 +522,8 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     gp = copy;
   }
   if (kStaged && lane < nbuf) {
-    mbar_init(&bar[lane], 1);
+    // (2: an arrival that never comes)
+    mbar_init(&bar[lane], HOLD && extra.hold == kHoldCopies && rank == extra.hold_cta ? 2 : 1);
     mbar_fence_init();
   }
   if (threadIdx.x == 0) {
@@ -579,14 +580,15 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   }
   box_sync();
 
+  auto abort_box = [&]() {   // in every CTA of the box: none may write its part of z
+    if constexpr (CS == 1) atomicExch(aborted, 1);
+    else
+      for (int c = 0; c < CS; ++c) add_release_cluster(aborted, 1, c);
+  };
   // waits until n groups are done; false when the limit ran out here or in another warp
   auto limit = [&]() { return HOLD && rank == extra.hold_cta ? extra.limit_ns : kWaitLimitNs; };
   auto wait_done = [&](int n) -> bool {
-    return count_wait<(CS > 1)>(finished, n, aborted, status, limit, [&]() {
-      if constexpr (CS == 1) atomicExch(aborted, 1);
-      else
-        for (int c = 0; c < CS; ++c) add_release_cluster(aborted, 1, c);
-    });
+    return count_wait<(CS > 1)>(finished, n, aborted, status, limit, abort_box);
   };
   LaneFactors<S> fac;
   int off[kNbrPerLane];   // offsets of the lane's neighbours in the padded local vector
@@ -606,7 +608,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       [[maybe_unused]] unsigned places[kNbrPerLane / 2];   // RING: the neighbours' places, two a word
       if (kStaged) {
         if (!mbar_wait(&bar[t % nbuf], (unsigned)(t / nbuf) & 1u, status, limit)) {
-          atomicExch(aborted, 1);
+          abort_box();
           return 1;
         }
         const unsigned char* from = mine + (t % nbuf) * solve_buffer<S>(RING);
@@ -1576,9 +1578,9 @@ extern "C" kkt_status ras_selftest_wait(ras_precond* m, double limit_ms, void* s
 
 extern "C" kkt_status ras_selftest_solve(ras_precond* m, const double* r, double* z, double limit_ms, int hold, int cta,
                                          int* drained, void* stream) {
-  if (!m || !r || !z || !(limit_ms > 0.0) || limit_ms > 1000.0 || hold != kHoldCounter || cta < 0 ||
+  if (!m || !r || !z || !(limit_ms > 0.0) || limit_ms > 1000.0 || hold < kHoldCounter || hold > kHoldCopies || cta < 0 ||
       m->local != 0 || m->prec != 32 || cta >= m->cluster || spans_overlap(r, z, m->n_total)) {
-    set_error("ras_selftest_solve: null argument, limit_ms outside (0, 1000], hold not 1, cta outside the cluster, "
+    set_error("ras_selftest_solve: null argument, limit_ms outside (0, 1000], hold not 1 or 2, cta outside the cluster, "
               "r and z overlap, or not an ILU(0) preconditioner with FP32 factors");
     return KKT_ERR_ARG;
   }

@@ -147,7 +147,7 @@ struct RasExtra {
   int hold = 0, hold_cta = 0;
   int* drained = nullptr;   // sum of the 1-based numbers of the groups whose copies were waited for on leaving
 };
-enum RasHold : int { kHoldNone = 0, kHoldCounter = 1 };
+enum RasHold : int { kHoldNone = 0, kHoldCounter = 1, kHoldCopies = 2 };
 kkt_status ras_launch(ras_precond* m, const double* r, double* z, cudaStream_t s, const int* gate = nullptr,
                       int gate_stride = 0, const RasExtra& extra = RasExtra());
 kkt_status ras_check(ras_precond* m);

@@ -1,9 +1,12 @@
 """The subdomain solve's bounded waits when they run out: one verdict per warp, and every copy into
-shared memory waited for before a CTA leaves.
+shared memory waited for before a CTA leaves, and none of a box's CTAs writes z.
 
 Every wait ends (limits of milliseconds), every kernel returns, and after ras_refactor the handle
 gives the bits it gave before.
 """
+
+import dataclasses
+import time
 
 import numpy as np
 import pytest
@@ -75,6 +78,33 @@ def test_a_solve_that_gives_up_waits_for_its_copies(api, stages, nsub, place):
     for ng in _groups((6, 5, 4, 6), nsub, 1):
         expect += sum(range(form["warps"] + 1, min(2 * ng, (form["buffers"] + 1) * form["warps"]) + 1))
     assert ras.selftest_solve(r, z, 5.0) == expect > 0
+    assert (z == 7.0).all()
+    with pytest.raises(KktError) as e:
+        ras.status()
+    assert e.value.status == -3
+    ras.refactor()
+    assert ras.status() == 0 and torch.equal(ras.apply(r), z0)
+
+
+@pytest.mark.parametrize("cta", [0, 1, 3])
+@pytest.mark.parametrize("hold", [1, 2], ids=["counter", "copies"])
+def test_one_cta_that_gives_up_ends_its_whole_cluster(api, hold, cta):
+    # the other CTAs keep the 2 s limit, so a return within a second means that they were told
+    from paper_1508_06103_gb300._lib import KktError
+
+    w = W.random_small(44, cells=(20, 11, 8), M=6, nsens=4, reg="h1l2")
+    beta = max(w.h) ** 2
+    w = dataclasses.replace(w, T=6 / 16.0, beta1=beta / 100, beta2=beta)
+    prob = api.Problem.from_workload(w)
+    ras = api.RAS(prob, (1, 1, 1, 1), 0, 32)
+    assert ras.solve_form()["cluster"] == 4
+    r = torch.from_numpy(W.random_vector(prob.n, 3)).cuda()
+    z0 = ras.apply(r).clone()
+    z = torch.full_like(r, 7.0)
+    torch.cuda.synchronize()
+    t = time.perf_counter()
+    ras.selftest_solve(r, z, 5.0, hold=hold, cta=cta)
+    assert time.perf_counter() - t < 1.0
     assert (z == 7.0).all()
     with pytest.raises(KktError) as e:
         ras.status()
