@@ -211,10 +211,14 @@ kkt_status ras_setup(kkt_problem* p, const int nsub[4], int overlap, int local, 
  *             points (FP64: 34, 26, 18; FP32: 52, 36, 20; BF16: 72, 40, 8): 16,
  *             8 or 4 warps, each taking 8 points of a wavefront at a time
  *   shape[1]  2..4: groups of 8 points whose factor values a warp holds, the one
- *             in use included (one less are buffers in shared memory; FP64 reads
- *             its factors from global memory and takes the field as given)
+ *             in use included (one less are buffers in shared memory, fewer
+ *             where they do not fit; FP64 reads its factors from global memory
+ *             and takes the field as given)
  *   shape[2]  lanes per point: 4 (the one compiled)
- *   shape[3]  1 = local vectors in shared memory, 2 = in global memory
+ *   shape[3]  1 = local vectors in shared memory, 2 = in global memory.  A
+ *             vector fits with 2048 + 175 shape[0] shape[1] x (bytes of a factor
+ *             value) bytes beside it in 227 KB; the CTA has fewer warps where
+ *             that leaves no room for all
  *   A 0 in a field leaves that choice to the library (as ras_setup does).
  *   Errors: ARG when no compiled shape matches or the chosen one does not fit
  *   the device's shared memory; otherwise those of ras_setup.

@@ -887,17 +887,16 @@ int gptr_smem(int nlev) {
   return bytes <= kGptrLimit ? bytes : 0;
 }
 
-// buffers per warp of a shape's second field (its value counts the group in use as well)
-int solve_buffers(int nstage) { return nstage - 1; }
-// dynamic shared memory of the solve without the local vector
+// dynamic shared memory of the solve without the ring and the local vector
 template <typename S>
-size_t solve_smem(int nlev, int warps, int nstage, bool ring) {
-  return kSolveHeader + gptr_smem(nlev) + (size_t)warps * solve_buffers(nstage) * solve_buffer<S>(ring);
+size_t solve_smem(int gptr_bytes, int warps, int nbuf, bool ring) {
+  return kSolveHeader + gptr_bytes + (size_t)warps * nbuf * solve_buffer<S>(ring);
 }
 size_t ring_smem(int wcap) { return ((size_t)kRingWaves * wcap + 1) * kVecWidth * sizeof(float); }
 
 struct SolveShape {
-  int ch, warps, nstage, lanes;
+  int ch, nstage, lanes;          // as the shape interface names them
+  int warps, nbuf, gptr_bytes;    // as the kernel runs: a warp's buffers, group pointers in shared memory
   bool smem_vec, ring;
   int cluster;
 };
@@ -979,28 +978,41 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
             (req.place == 2 && sv))
           continue;
         const size_t vec = sv ? (size_t)max_pad * sizeof(typename SolveArith<T>::type) : 0;
-        // a vector in shared memory leaves room for ns lower blocks of ch points beside it (the
-        // limit that the shape interface has always had)
+        // the interface's limit: a vector in shared memory leaves room for ns lower blocks of ch points
         if (sv && vec + kSolveReserve + (size_t)ns * kLRanks * ch * sizeof(T) > kSmemLimit) continue;
-        size_t sm = solve_smem<T>(nlev, warps, ns, false) + vec;
+        // The warps' buffers can take more than those blocks (16 warps x 3 x 5632 bytes against
+        // 4 x 36,400).  Where they do not fit, there are fewer of them a warp, then the group
+        // pointers stay in global memory, then there are fewer warps.
+        // (fewer boxes than a quarter of the SMs: their vectors stay in L1 without the ring, measured 2 to 3 % faster)
+        const bool can_ring = LaneFactors<T>::kStaged && !sv && wcap <= kMaxRingPlaces && 4 * nbox >= nsm;
+        int w = warps, nbuf = 0, gbytes = gptr_smem(nlev);
         bool ring = false;
-        // (fewer boxes than a quarter of the SMs: their vectors stay in L1, measured 2 to 3 % faster)
-        if (LaneFactors<T>::kStaged && !sv && wcap <= kMaxRingPlaces && 4 * nbox >= nsm) {
-          const size_t with = solve_smem<T>(nlev, warps, ns, true) + ring_smem(wcap);
-          ring = with <= kSmemLimit;
-          if (ring) sm = with;
+        size_t sm = 0;
+        auto fits = [&]() {
+          for (nbuf = ns - 1; nbuf >= 1; --nbuf)
+            for (int without = can_ring ? 0 : 1; without < 2; ++without) {
+              ring = !without;
+              sm = solve_smem<T>(gbytes, w, nbuf, ring) + (ring ? ring_smem(wcap) : vec);
+              if (sm <= kSmemLimit) return true;
+            }
+          return false;
+        };
+        bool ok = fits();
+        if (!ok) {
+          gbytes = 0;
+          while (!(ok = fits()) && w > 1) --w;
         }
-        if (sm > kSmemLimit) continue;
+        if (!ok) continue;
         int per_sm = 0;
         KKT_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, solve_kernel<T>(sv != 0, ring, 1), 32 * warps, sm));
+            &per_sm, solve_kernel<T>(sv != 0, ring, 1), 32 * w, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
         const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
         const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
         if (best_key < 0 || key < best_key) {
           best_key = key;
-          best = SolveShape{ch, warps, ns, kLanes, sv != 0, ring, 1};
+          best = SolveShape{ch, ns, kLanes, w, nbuf, gbytes, sv != 0, ring, 1};
         }
       }
   if (best_key < 0) {
@@ -1010,7 +1022,7 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
   }
   if (best.ch == SizeClasses<T>::name[0] && !best.smem_vec && !best.ring)
     KKT_TRY(choose_cluster<T>(nbox, (double)points / ((double)nbox * nlev * kGroup), best.warps,
-                              solve_smem<T>(nlev, best.warps, best.nstage, false), &best.cluster));
+                              solve_smem<T>(best.gptr_bytes, best.warps, best.nbuf, false), &best.cluster));
   *out = best;
   return KKT_OK;
 }
@@ -1157,6 +1169,8 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
     }
     m->ch = sh.ch;
     m->warps = sh.warps;
+    m->nbuf = sh.nbuf;
+    m->gptr_bytes = sh.gptr_bytes;
     m->smem_vec = sh.smem_vec;
     m->ring = sh.ring;
     m->cluster = sh.cluster;
@@ -1382,9 +1396,9 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
                         cudaStream_t s, const int* gate = nullptr, int gate_stride = 0,
                         const RasExtra& extra = RasExtra()) {
   using T = typename SolveArith<S>::type;
-  const int gbytes = gptr_smem(m->max_nlev);
+  const int gbytes = m->gptr_bytes;
   // (the dynamic shared-memory limit of both instances is raised at set-up, in choose_solve_shape)
-  const size_t smem = solve_smem<S>(m->max_nlev, m->warps, m->nstage, m->ring) +
+  const size_t smem = solve_smem<S>(gbytes, m->warps, m->nbuf, m->ring) +
                       (m->ring ? ring_smem(m->wcap) : m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
   const void* kernel = solve_kernel<S>(m->smem_vec, m->ring, m->cluster);
   if constexpr (std::is_same_v<S, float>)
@@ -1394,7 +1408,7 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
   const int *gptr = m->gptr, *vtab = m->vtab;
   const int2 *gtab = m->gtab, *otab = m->otab;
   const unsigned short* ntab = m->ntab;
-  int wcap = m->wcap, nbuf = solve_buffers(m->nstage);
+  int wcap = m->wcap, nbuf = m->nbuf;
   int* status = m->status;
   RasExtra ex = extra;
   void* args[] = {&boxes, &gptr, &F,    &V,      &r,    &z,      &gtab, &otab,        &vtab,
@@ -1538,7 +1552,7 @@ extern "C" kkt_status ras_solve_form(const ras_precond* m, int* warps, int* buff
     return KKT_ERR_ARG;
   }
   if (warps) *warps = m->warps;
-  if (buffers) *buffers = m->local == 0 && m->prec != 64 ? solve_buffers(m->nstage) : 0;
+  if (buffers) *buffers = m->local == 0 && m->prec != 64 ? m->nbuf : 0;
   if (cluster) *cluster = m->cluster;
   if (ring) *ring = m->local == 0 && m->ring ? 1 : 0;
   return KKT_OK;

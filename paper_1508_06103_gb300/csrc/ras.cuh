@@ -70,7 +70,9 @@ struct ras_precond {
   int ch = 0;                  // size class of the solve's CTA (ras_setup_shape)
   int warps = 0;               // warps of that CTA
   bool smem_vec = false;       // solve keeps the local vectors in shared memory
-  int nstage = 2;              // factor groups a warp asks for ahead, itself included (ras_setup_shape)
+  int nstage = 2;              // factor groups a warp holds, the one in use included (ras_setup_shape)
+  int nbuf = 1;                // buffers a warp has for them: one less, fewer where they do not fit
+  int gptr_bytes = 0;          // wavefront pointers in the solve's shared memory (0: read from global memory)
   int lanes = 4;               // lanes per point in the solve
   int cluster = 1;             // CTAs per box of the solve
   bool ring = false;           // solve keeps the last wavefronts in shared memory
