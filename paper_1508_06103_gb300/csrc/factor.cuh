@@ -1,5 +1,5 @@
 // FP64 ILU(0) factorisation of all subdomain matrices (Sec. 3.2), in place on
-// the [slot rank][8 points] groups that the subdomain solve reads.  (FP32:
+// the [slot rank][G points] groups that the subdomain solve reads.  (FP32:
 // factor32.cu.)
 //
 // Values.  gather_groups forms every slot value of every box point from the
@@ -31,9 +31,9 @@ template <typename T>
 constexpr int factor_threads = 128;
 
 // offset of the column of group place q in the box's factor values
-template <typename T>
+template <typename T, int G>
 __device__ __forceinline__ int group_column(int q) {
-  return q / kGroup * group_vals(8 * sizeof(T)) + q % kGroup;
+  return q / G * group_vals(8 * sizeof(T), G) + q % G;
 }
 
 // One thread per point (wavefront order, so the threads of a group write
@@ -44,7 +44,7 @@ __device__ __forceinline__ int group_column(int q) {
 // columns at levels n-1, n; G row: G column at n, n+1; f row: G and f columns
 // at n-1, n, n+1), plus the G row's two sensor slots at the centre.  Also
 // writes each box's unit row.
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(kGatherThreads) gather_groups(const DevProblem* __restrict__ probs,
                                                                 const BoxDesc* __restrict__ boxes,
                                                                 const int* __restrict__ gptr,
@@ -54,21 +54,21 @@ __global__ void __launch_bounds__(kGatherThreads) gather_groups(const DevProblem
   T* Fb = F + bx.foff;
   if (blockIdx.x == 0)
     for (int s = threadIdx.x; s < kSlots; s += blockDim.x)
-      Fb[bx.unit + c_gen_rank[s] * kGroup] = (s == kDiagC || s == kDiagG || s == kDiagF) ? (T)1 : (T)0;
+      Fb[bx.unit + c_gen_rank[s] * G] = (s == kDiagC || s == kDiagG || s == kDiagF) ? (T)1 : (T)0;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= kGroup * gptr[bx.loff + bx.nlev]) return;
-  const int lex = perm[kGroup * bx.goff + q];
+  if (q >= G * gptr[bx.loff + bx.nlev]) return;
+  const int lex = perm[G * bx.goff + q];
   if (lex < 0) return;
   const Coefs<T> cf = coefs<T>(p);
   const PointRow<T> pr = point_row<T>(p, bx, lex);
-  T* dst = Fb + group_column<T>(q);
+  T* dst = Fb + group_column<T, G>(q);
   const T tau = (T)p.tau, th = (T)p.theta, th1 = (T)(1.0 - p.theta), b1 = (T)p.beta1, b2 = (T)p.beta2;
   const T mt1 = tau / (T)6, lt1 = -(T)1 / tau;
   const bool idC = pr.n == 0 || pr.dirj, idG = pr.n == p.M || pr.dirj;   // identity rows
   const bool tm = pr.kt > 0, tp = pr.kt + 1 < bx.lt;                      // levels n-1, n+1 in the box
   const T z = (T)0;
   // slot (row type c, level offset dt, spatial offset d, column component cc)
-#define PUT(c, dt, d, cc, v) dst[c_gen_rank_of[c][(dt) + 1][d][cc] * kGroup] = (v)
+#define PUT(c, dt, d, cc, v) dst[c_gen_rank_of[c][(dt) + 1][d][cc] * G] = (v)
 #pragma unroll
   for (int d = 0; d < kStencil; ++d) {
     const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
@@ -110,7 +110,7 @@ __device__ __forceinline__ void check_pivot(double d, int* status) {
   if (!(fabs(d) > 1e-300) || !isfinite(d)) atomicExch(status, 1);
 }
 
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDesc* __restrict__ boxes,
                                                                     const int* __restrict__ gptr,
                                                                     const int* __restrict__ perm,
@@ -122,13 +122,13 @@ __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDes
   const BoxDesc bx = boxes[blockIdx.x];
   T* Fb = F + bx.foff;
   const int* gp = gptr + bx.loff;
-  const int* pm = perm + kGroup * bx.goff;
+  const int* pm = perm + G * bx.goff;
   const int* pb = ptab + bx.poff;
   int* nb = nbs + threadIdx.x;
   const int unit = (int)bx.unit;
   for (int w = 0; w < bx.nlev; ++w) {
-    const int q1 = kGroup * gp[w + 1];
-    for (int q = kGroup * gp[w] + threadIdx.x; q < q1; q += blockDim.x) {
+    const int q1 = G * gp[w + 1];
+    for (int q = G * gp[w] + threadIdx.x; q < q1; q += blockDim.x) {
       const int lex = pm[q];
       if (lex < 0) continue;
       const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
@@ -142,28 +142,28 @@ __global__ void __launch_bounds__(factor_threads<T>, 2) ilu0_factor(const BoxDes
           e = pb[ax + bx.lx * (ay + bx.ly * (az + bx.lz * at))];
         nb[i * NS] = e;
       }
-      T* own = Fb + group_column<T>(q);
+      T* own = Fb + group_column<T, G>(q);
       // the G and f rows read the U parts of this point's C and G rows
-      check_pivot((double)ilu_row0_64<T, NS>(own, Fb, nb), status);
+      check_pivot((double)ilu_row0_64<T, NS, G>(own, Fb, nb), status);
       asm volatile("" ::: "memory");
-      check_pivot((double)ilu_row1_64<T, NS>(own, Fb, nb), status);
+      check_pivot((double)ilu_row1_64<T, NS, G>(own, Fb, nb), status);
       asm volatile("" ::: "memory");
-      check_pivot((double)ilu_row2_64<T, NS>(own, Fb, nb), status);
+      check_pivot((double)ilu_row2_64<T, NS, G>(own, Fb, nb), status);
     }
     __syncthreads();
   }
 }
 
-// gather, then factor, in place on F (groups of 8 points); both on stream s
-template <typename T>
+// gather, then factor, in place on F (groups of G points); both on stream s
+template <typename T, int G>
 kkt_status factor_launch(ras_precond* m, T* F, cudaStream_t s) {
-  const dim3 g((unsigned)((kGroup * (long long)m->max_groups + kGatherThreads - 1) / kGatherThreads), m->nbox);
-  gather_groups<T><<<g, kGatherThreads, 0, s>>>(m->dprobs, m->boxes, m->gptr, m->perm, F);
+  const dim3 g((unsigned)((G * (long long)m->max_groups + kGatherThreads - 1) / kGatherThreads), m->nbox);
+  gather_groups<T, G><<<g, kGatherThreads, 0, s>>>(m->dprobs, m->boxes, m->gptr, m->perm, F);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   {
     TimedScope timed(&m->factor_timing, s);
-    ilu0_factor<T><<<m->nbox, factor_threads<T>, 0, s>>>(m->boxes, m->gptr, m->perm, m->ptab, F,
+    ilu0_factor<T, G><<<m->nbox, factor_threads<T>, 0, s>>>(m->boxes, m->gptr, m->perm, m->ptab, F,
                                                       m->status);
   }
   KKT_COUNT(1);

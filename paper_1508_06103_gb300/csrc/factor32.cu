@@ -170,8 +170,8 @@ struct BoxConst {
   const double* sens;
 };
 
-// S: stored type.  CS: CTAs (a cluster) that share a box.
-template <typename S, int CS>
+// S: stored type.  CS: CTAs (a cluster) that share a box.  G: points per group.
+template <typename S, int CS, int G>
 __global__ void __launch_bounds__(32 * kFacWarps, 1) ilu0_factor32(
     const DevProblem* __restrict__ probs, const BoxDesc* __restrict__ boxes, int nbox, const int* __restrict__ gptr,
     const int* __restrict__ perm, S* __restrict__ F, float* __restrict__ recs, long long rec_floats,
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(32 * kFacWarps, 1) ilu0_factor32(
     }
     const int nlev = bx.nlev;
     const int* gp = gptr + bx.loff;
-    const int* pm = perm + kGroup * bx.goff;
+    const int* pm = perm + G * bx.goff;
     S* Fb = F + bx.foff;
     __syncthreads();
     auto start = [&](int lex) {
@@ -373,48 +373,48 @@ __global__ void __launch_bounds__(32 * kFacWarps, 1) ilu0_factor32(
       // the factors, in the lanes' order (LaneFactors, ras.cu); places formed here, not kept
       int d = lane;
       asm volatile("" : "+r"(d));
-      S* g = Fb + (long long)(idx / kGroup) * kGroupVals32;
-      const int pt = idx % kGroup * 4;
+      S* g = Fb + (long long)(idx / G) * group_vals(32, G);
+      const int pt = idx % G * 4;
       if (lane < 27) {
-        put4(g + lane_place<S>(false, d & ~3, pt + (d & 3)), Cm * imC, cm * imF, Hm * imG, fm * imF);
+        put4(g + lane_place<S, G>(false, d & ~3, pt + (d & 3)), Cm * imC, cm * imF, Hm * imG, fm * imF);
         if (d < 13) {
           const int q = 27 + d;
           const float l = G0 * i0G;
-          put4(g + lane_place<S>(false, q & ~3, pt + (q & 3)), C0 * i0C, c0 * i0F, H0 * i0G, f0 * i0F);
-          put1(g + lane_place<S>(false, 34 + q / 4, pt + (q & 3)), l);
+          put4(g + lane_place<S, G>(false, q & ~3, pt + (q & 3)), C0 * i0C, c0 * i0F, H0 * i0G, f0 * i0F);
+          put1(g + lane_place<S, G>(false, 34 + q / 4, pt + (q & 3)), l);
         } else if (d > 13) {
           const int q = d - 14, l = pt + (q & 3), i = q / 4;
-          put2(g + lane_place<S>(true, 2 * i, l), H0, f0);
-          put1(g + lane_place<S>(true, 20 + i, l), G0);
-          put2(g + lane_place<S>(true, 30 + 2 * i, l), C0, c0);
+          put2(g + lane_place<S, G>(true, 2 * i, l), H0, f0);
+          put1(g + lane_place<S, G>(true, 20 + i, l), G0);
+          put2(g + lane_place<S, G>(true, 30 + 2 * i, l), C0, c0);
         }
         const int q = d + 13, l = pt + (q & 3), i = q / 4;
-        put2(g + lane_place<S>(true, 2 * i, l), Hp, fp);
-        put1(g + lane_place<S>(true, 20 + i, l), Gp);
+        put2(g + lane_place<S, G>(true, 2 * i, l), Hp, fp);
+        put1(g + lane_place<S, G>(true, 20 + i, l), Gp);
       } else if (lane == 27) {
-        put1(g + lane_place<S>(false, 40, pt), lgc);
-        put1(g + lane_place<S>(false, 40, pt + 1), lfg);
+        put1(g + lane_place<S, G>(false, 40, pt), lgc);
+        put1(g + lane_place<S, G>(false, 40, pt + 1), lfg);
       } else if (lane == 28) {
-        put2(g + lane_place<S>(true, 36, pt + 1), iF, iG);
+        put2(g + lane_place<S, G>(true, 36, pt + 1), iF, iG);
       } else if (lane == 29) {
-        put2(g + lane_place<S>(true, 36, pt + 2), gcp, 0.f);
+        put2(g + lane_place<S, G>(true, 36, pt + 2), gcp, 0.f);
       } else if (lane == 30) {
-        put2(g + lane_place<S>(true, 36, pt + 3), iC, ownf);
+        put2(g + lane_place<S, G>(true, 36, pt + 3), iC, ownf);
       }
     };
     // Loaded ahead of their use: the wavefront pointers two wavefronts, the lexicographic index of
     // a place two points (a wavefront's first two from the start of the one before), the
     // coefficients one point.
     auto gp_at = [&](int w) { return gp[min(w, nlev)]; };
-    auto lex_at = [&](int i, int end) { return i < kGroup * end ? pm[i] : -1; };
+    auto lex_at = [&](int i, int end) { return i < G * end ? pm[i] : -1; };
     int g1 = gp[1], g2 = gp_at(2);
-    int idx = kGroup * gp[0] + wid;
+    int idx = G * gp[0] + wid;
     Start next = start(lex_at(idx, g1));
     int lex2 = lex_at(idx + nw, g1);
     for (int w = 0; w < nlev; ++w) {
-      const int g3 = gp_at(w + 3), first = kGroup * g1 + wid;
+      const int g3 = gp_at(w + 3), first = G * g1 + wid;
       const int lex3 = lex_at(first, g2), lex4 = lex_at(first + nw, g2);
-      for (; idx < kGroup * g1; idx += nw) {
+      for (; idx < G * g1; idx += nw) {
         const Start cur = next;
         next = start(lex2);
         lex2 = lex_at(idx + 2 * nw, g1);
@@ -432,11 +432,12 @@ __global__ void __launch_bounds__(32 * kFacWarps, 1) ilu0_factor32(
 }
 
 template <typename S>
-const void* kernel_of(int cs) {
-  return cs == 1   ? (const void*)ilu0_factor32<S, 1>
-         : cs == 2 ? (const void*)ilu0_factor32<S, 2>
-         : cs == 4 ? (const void*)ilu0_factor32<S, 4>
-                   : (const void*)ilu0_factor32<S, 8>;
+const void* kernel_of(int cs, int group) {
+  if (group != kGroup) return (const void*)ilu0_factor32<S, 1, narrow_group(32)>;
+  return cs == 1   ? (const void*)ilu0_factor32<S, 1, kGroup>
+         : cs == 2 ? (const void*)ilu0_factor32<S, 2, kGroup>
+         : cs == 4 ? (const void*)ilu0_factor32<S, 4, kGroup>
+                   : (const void*)ilu0_factor32<S, 8, kGroup>;
 }
 
 cudaLaunchConfig_t config_of(int cs, int ncl, cudaStream_t s, cudaLaunchAttribute* attr) {
@@ -465,7 +466,7 @@ kkt_status factor32_launch(ras_precond* m, S* F, cudaStream_t s) {
   void* args[] = {&probs, &boxes, &nbox, &gptr, &perm, &F, &rec, &rf, &status};
   {
     TimedScope timed(&m->factor_timing, s);
-    KKT_TRY_CUDA(cudaLaunchKernelExC(&cfg, kernel_of<S>(m->fac_cluster), args));
+    KKT_TRY_CUDA(cudaLaunchKernelExC(&cfg, kernel_of<S>(m->fac_cluster, m->group), args));
   }
   KKT_COUNT(1);
   return KKT_OK;
@@ -496,13 +497,13 @@ kkt_status ras_factor_prepare32(ras_precond* m) {
     waves += b.nlev;
   }
   int cs = 1;
-  while (cs < 8 && 2 * cs * 21 * waves <= points) cs *= 2;
+  while (m->group == kGroup && cs < 8 && 2 * cs * 21 * waves <= points) cs *= 2;
   m->fac_cluster = cs;
   cudaLaunchAttribute attr{};
   const cudaLaunchConfig_t cfg = config_of(cs, m->nbox, nullptr, &attr);
   int most = 0;
   KKT_TRY_CUDA(cudaOccupancyMaxActiveClusters(
-      &most, m->prec == 16 ? kernel_of<__nv_bfloat16>(cs) : kernel_of<float>(cs), &cfg));
+      &most, m->prec == 16 ? kernel_of<__nv_bfloat16>(cs, m->group) : kernel_of<float>(cs, m->group), &cfg));
   m->fac_nclusters = std::max(1, std::min(most, m->nbox));
   for (;; m->fac_nclusters /= 2) {   // fewer boxes at a time where memory is short
     if (cudaMalloc(&m->rec, (size_t)m->fac_nclusters * rec * sizeof(float)) == cudaSuccess) return KKT_OK;

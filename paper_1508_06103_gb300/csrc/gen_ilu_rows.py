@@ -101,7 +101,7 @@ def row_function(c, prec, group, nl, cnt, base, slots, diag, rank, nbrs, contrib
     o = [
         "// own: the point's column in its group; F + nb[i * NS]: pivot point i's column (the unit row",
         "// outside the box).  Stores 1/pivot in the diagonal slot and returns the pivot.",
-        "template <typename T, int NS>",
+        "template <typename T, int NS, int G>",
         f"__device__ __forceinline__ T ilu_row{c}_{prec}(T* __restrict__ own, const T* __restrict__ F, "
         "const int* __restrict__ nb) {",
         f"  T l[{nl}], u[{group}], d;",
@@ -109,13 +109,13 @@ def row_function(c, prec, group, nl, cnt, base, slots, diag, rank, nbrs, contrib
 
     def accumulate(x, dst):
         o.append("  {")
-        o.append(f"    T acc = own[{rank[base + x]} * 8];")
+        o.append(f"    T acc = own[{rank[base + x]} * G];")
         for (s, i, t) in contrib[x]:
-            o.append(f"    acc -= l[{s}] * F[nb[{i} * NS] + {rank[t]} * 8];")
+            o.append(f"    acc -= l[{s}] * F[nb[{i} * NS] + {rank[t]} * G];")
         if x < nl:
             dt, dz, dy, dx, ck = slots[base + x]
             i = nbrs.index((dt, dz, dy, dx))
-            o.append(f"    l[{x}] = acc * F[nb[{i} * NS] + {rank[diag[ck]]} * 8];")
+            o.append(f"    l[{x}] = acc * F[nb[{i} * NS] + {rank[diag[ck]]} * G];")
         else:
             o.append(f"    {dst} = acc;")
         o.append("  }")
@@ -131,7 +131,7 @@ def row_function(c, prec, group, nl, cnt, base, slots, diag, rank, nbrs, contrib
             o.append("  u[0] = (T)1 / u[0];")
         for x in range(g0, g1):
             val = f"l[{x}]" if x < nl else f"u[{x - g0}]"
-            o.append(f"  own[{rank[base + x]} * 8] = {val};")
+            o.append(f"  own[{rank[base + x]} * G] = {val};")
     o.append("  return d;")
     o.append("}")
     o.append("")
@@ -198,7 +198,7 @@ def generate() -> str:
     out = [
         "// Generated by gen_ilu_rows.py from the KKT row stencils -- do not edit by hand.",
         "// ILU(0) elimination of one row of each type (C, G, f), one target entry at a time,",
-        "// in place on groups of 8 points (slot s of a point at offset 8 kGenRank[s]).",
+        "// in place on groups of G points (slot s of a point at offset G kGenRank[s]).",
         "#pragma once",
         "",
         f"constexpr int kGenNbrs = {len(nbrs)};",

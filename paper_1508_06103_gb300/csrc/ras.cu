@@ -17,12 +17,12 @@
 // outside the box hold 0, which is the same as leaving them out of the
 // pattern.
 //
-// Layout in HBM.  The points of each wavefront are stored in groups of 8, one
-// after the other; the values of a group form one block, the L-slots first,
+// Layout in HBM.  The points of each wavefront are stored in groups of 8 (fewer
+// in boxes of a few points a wavefront: ras.cuh), one after the other; the values of a group form one block, the L-slots first,
 // then the diagonals and U-slots, so the forward sweep streams the lower
 // halves of the groups in order and the backward sweep the upper halves.  In
 // FP32 and BF16 a half is ordered by the lanes of the solve (lane_place, ras.cuh),
-// in FP64 by slot rank ([rank][8 points]).
+// in FP64 by slot rank ([rank][points of a group]).
 //
 // Ordering and parallelism.  Points are processed in the natural
 // (lexicographic) order of the box; with this stencil every lower-triangular
@@ -363,30 +363,30 @@ __device__ __forceinline__ T lane_sum(T v) {
 // C and f columns (q < 13), and what lanes 1 to 3 hold in place of c(3, .):
 // lane 1 1/u of the f and G rows, lane 2 the G row's C column at level n+1
 // (q = 26), lane 3 1/u of the C row and its own-point f column.
-template <typename S>
+template <typename S, int G>
 struct LaneFactors;
 
-template <>
-struct LaneFactors<float> {
+template <int G>
+struct LaneFactors<float, G> {
   static constexpr bool kStaged = true;   // comes through shared memory
   float v[kLaneL];
-  __device__ __forceinline__ void load(const float* G, bool upper, int lane) {
+  __device__ __forceinline__ void load(const float* F, bool upper, int lane) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const float4 w = *reinterpret_cast<const float4*>(G + 4 * lane + 128 * k);
+      const float4 w = *reinterpret_cast<const float4*>(F + 4 * lane + 16 * G * k);
       v[4 * k] = w.x;
       v[4 * k + 1] = w.y;
       v[4 * k + 2] = w.z;
       v[4 * k + 3] = w.w;
     }
     if (upper) {
-      const float2 w = *reinterpret_cast<const float2*>(G + 32 * 36 + 2 * lane);
+      const float2 w = *reinterpret_cast<const float2*>(F + 4 * G * 36 + 2 * lane);
       v[36] = w.x;
       v[37] = w.y;
     } else {
 #pragma unroll
       for (int k = 9; k < 11; ++k) {
-        const float4 w = *reinterpret_cast<const float4*>(G + 4 * lane + 128 * k);
+        const float4 w = *reinterpret_cast<const float4*>(F + 4 * lane + 16 * G * k);
         v[4 * k] = w.x;
         v[4 * k + 1] = w.y;
         v[4 * k + 2] = w.z;
@@ -397,14 +397,14 @@ struct LaneFactors<float> {
   __device__ __forceinline__ float at(int i) const { return v[i]; }
 };
 
-template <>
-struct LaneFactors<__nv_bfloat16> {
+template <int G>
+struct LaneFactors<__nv_bfloat16, G> {
   static constexpr bool kStaged = true;
   unsigned v[kLaneL / 2];   // pairs: value 2 k in the low half
-  __device__ __forceinline__ void load(const __nv_bfloat16* G, bool upper, int lane) {
+  __device__ __forceinline__ void load(const __nv_bfloat16* F, bool upper, int lane) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const uint4 w = *reinterpret_cast<const uint4*>(G + 8 * lane + 256 * k);
+      const uint4 w = *reinterpret_cast<const uint4*>(F + 8 * lane + 32 * G * k);
       v[4 * k] = w.x;
       v[4 * k + 1] = w.y;
       v[4 * k + 2] = w.z;
@@ -412,14 +412,14 @@ struct LaneFactors<__nv_bfloat16> {
     }
     if (upper) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) v[16 + k] = *reinterpret_cast<const unsigned*>(G + 32 * 32 + 6 * lane + 2 * k);
+      for (int k = 0; k < 3; ++k) v[16 + k] = *reinterpret_cast<const unsigned*>(F + 4 * G * 32 + 6 * lane + 2 * k);
     } else {
-      const uint4 w = *reinterpret_cast<const uint4*>(G + 8 * lane + 1024);
+      const uint4 w = *reinterpret_cast<const uint4*>(F + 8 * lane + 128 * G);
       v[16] = w.x;
       v[17] = w.y;
       v[18] = w.z;
       v[19] = w.w;
-      const uint2 t = *reinterpret_cast<const uint2*>(G + 32 * 40 + 4 * lane);
+      const uint2 t = *reinterpret_cast<const uint2*>(F + 4 * G * 40 + 4 * lane);
       v[20] = t.x;
       v[21] = t.y;
     }
@@ -429,16 +429,16 @@ struct LaneFactors<__nv_bfloat16> {
   }
 };
 
-// FP64: the values stay in global memory ([slot rank][8] groups) until they
+// FP64: the values stay in global memory ([slot rank][G] groups) until they
 // are used; the FP64 pipe is the limit, and other warps hide the loads.
-template <>
-struct LaneFactors<double> {
+template <int G>
+struct LaneFactors<double, G> {
   static constexpr bool kStaged = false;
   const double* p;
-  __device__ __forceinline__ void load(const double* G, bool upper, int lane) {
-    p = G + (upper ? kLRanks * kGroup : 0) + lane / kLanes;
+  __device__ __forceinline__ void load(const double* F, bool upper, int lane) {
+    p = F + (upper ? kLRanks * G : 0) + lane / kLanes;
   }
-  __device__ __forceinline__ double rank(int r) const { return __ldcs(p + r * kGroup); }
+  __device__ __forceinline__ double rank(int r) const { return __ldcs(p + r * G); }
 };
 
 // S: type of the stored factor values; T: arithmetic and local-vector type.
@@ -470,8 +470,8 @@ constexpr int kMaxRingPlaces = 65535 / kRingWaves - 1;   // places a wavefront, 
 
 // Bytes of a warp's factor buffer (the lower half of a group is the larger one).
 template <typename S>
-constexpr int solve_buffer(bool ring) {
-  return LaneFactors<S>::kStaged ? 32 * kLaneL * (int)sizeof(S) + (ring ? kNbrBytes : 0) : 0;
+__host__ __device__ constexpr int solve_buffer(int group, bool ring) {
+  return LaneFactors<S, kGroup>::kStaged ? 4 * group * kLaneL * (int)sizeof(S) + (ring ? kNbrBytes : 0) : 0;
 }
 constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter of finished groups, abort word
 
@@ -480,7 +480,7 @@ constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter
 // the box's finished groups, to which every group adds.  The bits are those of one CTA.
 // HOLD: the self-test's instance, in which waits of one CTA of a box run out (RasExtra).  (The limit and
 // the hold as run-time arguments of the others cost 1 % through the registers they were given.)
-template <typename S, bool SMEM, bool RING, int CS, bool HOLD = false>
+template <typename S, bool SMEM, bool RING, int CS, bool HOLD = false, int G = kGroup>
 __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr, const S* __restrict__ F,
     typename SolveArith<S>::type* __restrict__ V, const double* __restrict__ r, double* __restrict__ z,
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
     const unsigned short* __restrict__ ntab, int wcap, int gptr_bytes, int nbuf, int* __restrict__ status,
     const int* gate, int gate_stride, RasExtra extra) {
   using T = typename SolveArith<S>::type;
-  constexpr bool kStaged = LaneFactors<S>::kStaged;
+  constexpr bool kStaged = LaneFactors<S, G>::kStaged;
   // the box's problem gate (one problem: gate_stride 0, every box reads gate[0])
   if (gate != nullptr && gate[boxes[blockIdx.x / CS].prob * gate_stride] == 0) return;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -498,10 +498,11 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   const BoxDesc bx = boxes[blockIdx.x / CS];
   const int P = (int)bx.P, nlev = bx.nlev;
   const S* Fb = F + bx.foff;
-  const int* vt = vtab + kGroup * bx.goff;
+  const int* vt = vtab + G * bx.goff;
   const int px = bx.lx + 2, py = bx.ly + 2, pz = bx.lz + 2;
   const int sy = px, sz = px * py, st = px * py * pz;
   const int lane = threadIdx.x & 31, sub = lane & (kLanes - 1);
+  const int flane = G == kGroup ? lane : min(lane, kLanes * G - 1);   // whose values the lane reads (idle ones: the last's)
   const int rank = CS == 1 ? 0 : blockIdx.x % CS, local_warp = threadIdx.x / 32;
   const int warp = local_warp * CS + rank, nwarp = blockDim.x / 32 * CS;   // of all CTAs of the box
   auto box_sync = [&]() {
@@ -510,10 +511,10 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   };
   // shared memory: header, group pointers, the warps' factor buffers, the local vector
   unsigned char* bufs = smem + kSolveHeader + gptr_bytes;
-  unsigned char* rest = bufs + (size_t)(blockDim.x / 32) * nbuf * solve_buffer<S>(RING);   // the ring or the local vector
+  unsigned char* rest = bufs + (size_t)(blockDim.x / 32) * nbuf * solve_buffer<S>(G, RING);   // the ring or the local vector
   T* v = SMEM ? reinterpret_cast<T*>(rest) : V + bx.voff;
   T* ring = reinterpret_cast<T*>(rest);   // RING: [16][wcap] points and the zeros
-  unsigned char* mine = bufs + (size_t)local_warp * nbuf * solve_buffer<S>(RING);
+  unsigned char* mine = bufs + (size_t)local_warp * nbuf * solve_buffer<S>(G, RING);
   unsigned long long* bar = bars + local_warp * (kMaxStages - 1);
   const int* gp = gptr + bx.loff;   // first group of every wavefront
   if (gptr_bytes) {
@@ -544,20 +545,24 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   auto issue = [&](int k, int t) {   // copy of group k, the warp's t-th, into its buffer
     if (kStaged && k < 2 * ng && lane == 0) {
       const bool up = k >= ng;
-      const unsigned bytes = 32 * (up ? kLaneU : kLaneL) * (unsigned)sizeof(S);
-      unsigned char* to = mine + (t % nbuf) * solve_buffer<S>(RING);
+      const unsigned bytes = kLanes * G * (up ? kLaneU : kLaneL) * (unsigned)sizeof(S);
+      unsigned char* to = mine + (t % nbuf) * solve_buffer<S>(G, RING);
       fence_proxy_async();
       mbar_expect_tx(&bar[t % nbuf], bytes + (RING ? kNbrBytes : 0));
-      bulk_g2s(to, Fb + (long long)group(k) * kGroupVals32 + (up ? 32 * kLaneL : 0), bytes, &bar[t % nbuf]);
+      bulk_g2s(to, Fb + (long long)group(k) * group_vals(32, G) + (up ? kLanes * G * kLaneL : 0), bytes, &bar[t % nbuf]);
       if (RING)
-        bulk_g2s(to + 32 * kLaneL * sizeof(S), ntab + (2 * (bx.goff + group(k)) + (up ? 1 : 0)) * (kNbrBytes / 2),
+        bulk_g2s(to + kLanes * G * kLaneL * sizeof(S), ntab + (2 * (bx.goff + group(k)) + (up ? 1 : 0)) * (kNbrBytes / 2),
                  kNbrBytes, &bar[t % nbuf]);
     }
   };
   for (int t = 0; t < nbuf; ++t) issue(warp + t * nwarp, t);
   // the points of the warp's next two groups: the neighbours' and the own point's addresses
   // come from them
-  auto point = [&](int k) { return k < 2 * ng ? vt[kGroup * group(k) + lane / kLanes] : 0; };
+  auto point = [&](int k) {
+    int q = k < 2 * ng ? vt[G * group(k) + flane / kLanes] : 0;
+    if (G < kGroup && lane >= kLanes * G && q >= 0) q = ~q;   // an idle lane: as in an empty place
+    return q;
+  };
   int vq = point(warp), vq2 = point(warp + nwarp);
   // R^delta r into the padded local vector (gtab: per box point, its global unknown index and
   // its padded offset); four points at a time, so that their loads overlap
@@ -590,7 +595,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
   auto wait_done = [&](int n) -> bool {
     return count_wait<(CS > 1)>(finished, n, aborted, status, limit, abort_box);
   };
-  LaneFactors<S> fac;
+  LaneFactors<S, G> fac;
   int off[kNbrPerLane];   // offsets of the lane's neighbours in the padded local vector
   int s = 0, t = 0;       // step of the warp's group, number of its groups so far
   int k = warp;
@@ -611,16 +616,16 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
           abort_box();
           return 1;
         }
-        const unsigned char* from = mine + (t % nbuf) * solve_buffer<S>(RING);
-        fac.load(reinterpret_cast<const S*>(from), kUpper, lane);
+        const unsigned char* from = mine + (t % nbuf) * solve_buffer<S>(G, RING);
+        fac.load(reinterpret_cast<const S*>(from), kUpper, flane);
         if constexpr (RING)
 #pragma unroll
           for (int i = 0; i < kNbrPerLane / 2; ++i)
-            places[i] = reinterpret_cast<const unsigned*>(from + 32 * kLaneL * sizeof(S))[kNbrPerLane / 2 * lane + i];
+            places[i] = reinterpret_cast<const unsigned*>(from + kLanes * G * kLaneL * sizeof(S))[kNbrPerLane / 2 * lane + i];
         __syncwarp();
         issue(k + nbuf * nwarp, t + nbuf);
       } else {
-        fac.load(Fb + (long long)group(k) * group_vals(64), kUpper, lane);
+        fac.load(Fb + (long long)group(k) * group_vals(64, G), kUpper, flane);
       }
       // neighbours two and more wavefronts away (at the first backward step the own point is one
       // of the last wavefront's)
@@ -736,7 +741,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
       sf = lane_sum(sf);
       auto place = [&]() {   // of the point in the ring
         const int w = s < nlev ? s : 2 * nlev - 1 - s;
-        return kVecWidth * (w % kRingWaves * wcap + kGroup * (group(k) - gp[w]) + lane / kLanes);
+        return kVecWidth * (w % kRingWaves * wcap + G * (group(k) - gp[w]) + lane / kLanes);
       };
       if (act && sub == 0) {
         if constexpr (!kUpper) {
@@ -820,21 +825,21 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
 // Ring places of every neighbour of every group place (see kNbrBytes): one thread per lane and
 // group.  inv: group place of every box point.
 __global__ void place_points(const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr,
-                             const int* __restrict__ perm, int* __restrict__ inv) {
+                             const int* __restrict__ perm, int G, int* __restrict__ inv) {
   const BoxDesc bx = boxes[blockIdx.x];
   const int q = blockIdx.y * blockDim.x + threadIdx.x;
-  if (q >= kGroup * gptr[bx.loff + bx.nlev]) return;
-  const int lex = perm[kGroup * bx.goff + q];
+  if (q >= G * gptr[bx.loff + bx.nlev]) return;
+  const int lex = perm[G * bx.goff + q];
   if (lex >= 0) inv[bx.poff + lex] = q;
 }
 __global__ void neighbour_places(const BoxDesc* __restrict__ boxes, const int* __restrict__ gptr,
-                                 const int* __restrict__ perm, const int* __restrict__ inv, int wcap,
+                                 const int* __restrict__ perm, const int* __restrict__ inv, int G, int wcap,
                                  unsigned short* __restrict__ out) {
   const BoxDesc bx = boxes[blockIdx.x];
   const int* gp = gptr + bx.loff;
   const int g = blockIdx.y * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32, sub = lane % kLanes;
   if (g >= gp[bx.nlev]) return;
-  const int lex = perm[kGroup * (bx.goff + g) + lane / kLanes];
+  const int lex = lane / kLanes < G ? perm[G * (bx.goff + g) + lane / kLanes] : -1;
   const int kx = lex % bx.lx, ky = (lex / bx.lx) % bx.ly, kz = (lex / (bx.lx * bx.ly)) % bx.lz;
   const int kt = lex / (bx.lx * bx.ly * bx.lz);
   for (int up = 0; up < 2; ++up)
@@ -845,14 +850,14 @@ __global__ void neighbour_places(const BoxDesc* __restrict__ boxes, const int* _
       int place = kRingWaves * wcap;
       if (lex >= 0 && x >= 0 && x < bx.lx && y >= 0 && y < bx.ly && z >= 0 && z < bx.lz && t >= 0 && t < bx.lt) {
         const int w = x + 2 * y + 4 * z + 8 * t;
-        place = w % kRingWaves * wcap + inv[bx.poff + x + bx.lx * (y + bx.ly * (z + bx.lz * t))] - kGroup * gp[w];
+        place = w % kRingWaves * wcap + inv[bx.poff + x + bx.lx * (y + bx.ly * (z + bx.lz * t))] - G * gp[w];
       }
       out[((2 * (bx.goff + g) + up) * 32 + lane) * kNbrPerLane + i] = (unsigned short)place;
     }
 }
 
-// places of the largest wavefront of a box (whole groups)
-int widest_wavefront(const int l[4]) {
+// points of every wavefront of a box
+std::vector<int> wavefronts(const int l[4]) {
   std::vector<int> h(1, 1);
   for (int a = 0; a < 4; ++a) {
     const int step = 1 << a;
@@ -864,7 +869,7 @@ int widest_wavefront(const int l[4]) {
     }
     h.swap(n);
   }
-  return (*std::max_element(h.begin(), h.end()) + kGroup - 1) / kGroup * kGroup;
+  return h;
 }
 
 std::vector<std::pair<int, int>> parts(int n, int p) {
@@ -889,8 +894,8 @@ int gptr_smem(int nlev) {
 
 // dynamic shared memory of the solve without the ring and the local vector
 template <typename S>
-size_t solve_smem(int gptr_bytes, int warps, int nbuf, bool ring) {
-  return kSolveHeader + gptr_bytes + (size_t)warps * nbuf * solve_buffer<S>(ring);
+size_t solve_smem(int gptr_bytes, int warps, int nbuf, int group, bool ring) {
+  return kSolveHeader + gptr_bytes + (size_t)warps * nbuf * solve_buffer<S>(group, ring);
 }
 size_t ring_smem(int wcap) { return ((size_t)kRingWaves * wcap + 1) * kVecWidth * sizeof(float); }
 
@@ -903,8 +908,15 @@ struct SolveShape {
 // groups per wavefront from which the largest CTA is taken
 constexpr int kFillGroups = 4;
 template <typename T, bool HOLD = false>
-const void* solve_kernel(bool smem_vec, bool ring, int cluster) {
-  if constexpr (LaneFactors<T>::kStaged)
+const void* solve_kernel(int group, bool smem_vec, bool ring, int cluster) {
+  constexpr int N = narrow_group(8 * sizeof(T));
+  if (!HOLD && group != kGroup) {   // (boxes of narrow groups have too few of them for a cluster)
+    if constexpr (LaneFactors<T, N>::kStaged)
+      if (ring) return (const void*)ras_solve<T, false, true, 1, false, N>;
+    return smem_vec ? (const void*)ras_solve<T, true, false, 1, false, N>
+                    : (const void*)ras_solve<T, false, false, 1, false, N>;
+  }
+  if constexpr (LaneFactors<T, kGroup>::kStaged)
     if (ring) return (const void*)ras_solve<T, false, true, 1, HOLD>;
   if (smem_vec) return (const void*)ras_solve<T, true, false, 1, HOLD>;
   return cluster == 8   ? (const void*)ras_solve<T, false, false, 8, HOLD>
@@ -938,7 +950,7 @@ kkt_status choose_cluster(int nbox, double groups, int warps, size_t smem, int* 
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int fit = 0;
-    KKT_TRY_CUDA(cudaOccupancyMaxActiveClusters(&fit, solve_kernel<T>(false, false, cs), &cfg));
+    KKT_TRY_CUDA(cudaOccupancyMaxActiveClusters(&fit, solve_kernel<T>(kGroup, false, false, cs), &cfg));
     if (nbox <= fit) {
       *out = cs;
       return KKT_OK;
@@ -959,14 +971,14 @@ struct ShapeRequest {
 // groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
 // global memory, the fewest buffers, the largest CTA.  ras_autotune measures instead.
 template <typename T>
-kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int wcap, int nsm,
+kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int group, int wcap, int nsm,
                               const ShapeRequest& req, SolveShape* out) {
   if (req.lanes != 0 && req.lanes != kLanes) {
     set_error("ras_setup: the subdomain solve runs 4 lanes per point");
     return KKT_ERR_ARG;
   }
   for (int form = 0; form < 6; ++form)
-    KKT_TRY_CUDA(cudaFuncSetAttribute(solve_kernel<T>(form == 1, form == 2, form > 2 ? 1 << (form - 2) : 1),
+    KKT_TRY_CUDA(cudaFuncSetAttribute(solve_kernel<T>(group, form == 1, form == 2, form > 2 ? 1 << (form - 2) : 1),
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
   SolveShape best{};
   long long best_key = -1;
@@ -984,7 +996,7 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
         // 4 x 36,400).  Where they do not fit, there are fewer of them a warp, then the group
         // pointers stay in global memory, then there are fewer warps.
         // (fewer boxes than a quarter of the SMs: their vectors stay in L1 without the ring, measured 2 to 3 % faster)
-        const bool can_ring = LaneFactors<T>::kStaged && !sv && wcap <= kMaxRingPlaces && 4 * nbox >= nsm;
+        const bool can_ring = LaneFactors<T, kGroup>::kStaged && !sv && wcap <= kMaxRingPlaces && 4 * nbox >= nsm;
         int w = warps, nbuf = 0, gbytes = gptr_smem(nlev);
         bool ring = false;
         size_t sm = 0;
@@ -992,7 +1004,7 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
           for (nbuf = ns - 1; nbuf >= 1; --nbuf)
             for (int without = can_ring ? 0 : 1; without < 2; ++without) {
               ring = !without;
-              sm = solve_smem<T>(gbytes, w, nbuf, ring) + (ring ? ring_smem(wcap) : vec);
+              sm = solve_smem<T>(gbytes, w, nbuf, group, ring) + (ring ? ring_smem(wcap) : vec);
               if (sm <= kSmemLimit) return true;
             }
           return false;
@@ -1005,7 +1017,7 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
         if (!ok) continue;
         int per_sm = 0;
         KKT_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, solve_kernel<T>(sv != 0, ring, 1), 32 * w, sm));
+            &per_sm, solve_kernel<T>(group, sv != 0, ring, 1), 32 * w, sm));
         if (per_sm < 1) continue;
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
         const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
@@ -1020,9 +1032,9 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
               "placement must be a compiled combination that fits in shared memory)");
     return KKT_ERR_ARG;
   }
-  if (best.ch == SizeClasses<T>::name[0] && !best.smem_vec && !best.ring)
+  if (group == kGroup && best.ch == SizeClasses<T>::name[0] && !best.smem_vec && !best.ring)
     KKT_TRY(choose_cluster<T>(nbox, (double)points / ((double)nbox * nlev * kGroup), best.warps,
-                              solve_smem<T>(best.gptr_bytes, best.warps, best.nbuf, false), &best.cluster));
+                              solve_smem<T>(best.gptr_bytes, best.warps, best.nbuf, group, false), &best.cluster));
   *out = best;
   return KKT_OK;
 }
@@ -1126,8 +1138,10 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   // finish as close together as they can
   std::stable_sort(geoms.begin(), geoms.end(), [](const Geom& a, const Geom& b) { return a.points > b.points; });
   {
-    // largest padded local vector, most wavefronts, points of all boxes
-    long long pad = 0, points = 0;
+    // largest padded local vector, most wavefronts, points of all boxes, groups of 8 and of the narrow
+    // size, whether a box of groups of 8 has too many values for the FP64 factorisation's offsets
+    long long pad = 0, points = 0, wide = 0;
+    bool too_large = false;
     for (const Geom& g : geoms) {
       const kkt_problem* pk = probs[g.prob];
       const int dk[4] = {pk->nx, pk->ny, pk->nz, pk->L};
@@ -1138,11 +1152,25 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
         v *= l + 2;
         nlev += (l - 1) << a;
       }
-      if (local == 0) m->wcap = std::max(m->wcap, widest_wavefront(len));
+      if (local == 0) {
+        long long groups = 0;
+        for (int n : wavefronts(len)) {
+          groups += (n + kGroup - 1) / kGroup;
+          m->wcap = std::max(m->wcap, (n + kGroup - 1) / kGroup * kGroup);   // places of the widest wavefront
+        }
+        wide += groups;
+        too_large = too_large || (groups + 1) * group_vals(64, kGroup) > INT32_MAX;
+      }
       pad = std::max(pad, v);
       points += g.points;
       m->max_nlev = std::max(m->max_nlev, nlev);
     }
+    // Narrow groups where groups of 8 would be filled by less than a third (FP64) or a half (FP32,
+    // BF16).  Factor values a point, groups of 8 and narrow ones: boxes of one node in two or three
+    // axes, or of two nodes a side, FP64 2608 and 652, FP32 2624 and 1312; 17 x 1 x 1 x 65 nodes FP64
+    // 1249 and 349, FP32 1256 and 628; 3 x 3 x 3 x 3 FP64 998 and 411, FP32 1004 and 567.
+    if (local == 0 && (wide * kGroup > (factor_prec == 64 ? 3 : 2) * points || (factor_prec == 64 && too_large)))
+      m->group = narrow_group(factor_prec);
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) {
@@ -1160,9 +1188,9 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       req.place = shape[3];
     }
     SolveShape sh{};
-    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, m->wcap, nsm, req, &sh)
-                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, m->wcap, nsm, req, &sh)
-                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, m->wcap, nsm, req, &sh);
+    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, m->group, m->wcap, nsm, req, &sh)
+                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, m->group, m->wcap, nsm, req, &sh)
+                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, m->group, m->wcap, nsm, req, &sh);
     if (cs != KKT_OK) {
       delete m;
       return cs;
@@ -1185,7 +1213,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
     delete m;
     return KKT_ERR_ARG;
   }
-  const int gvals = group_vals(factor_prec);
+  const int G = m->group, gvals = group_vals(factor_prec, G);
   long long foff = 0, voff = 0, poff = 0, ngroup = 0;
   for (const Geom& geo : geoms) {
     const kkt_problem* pk = probs[geo.prob];
@@ -1218,7 +1246,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       return KKT_ERR_ARG;
     }
     if (local == 0) {
-      // groups of 8 points per wavefront: counting sort of the points (lexicographic within a wavefront)
+      // groups of G points per wavefront: counting sort of the points (lexicographic within a wavefront)
       std::vector<int> fill(b.nlev + 1, 0);
       for (int kt = 0; kt < b.lt; ++kt)
         for (int kz = 0; kz < b.lz; ++kz)
@@ -1228,8 +1256,8 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       for (int w = 0; w < b.nlev; ++w) {
         gptr.push_back(groups);
         const int n = fill[w];
-        fill[w] = kGroup * groups;
-        groups += (n + kGroup - 1) / kGroup;
+        fill[w] = G * groups;
+        groups += (n + G - 1) / G;
       }
       gptr.push_back(groups);
       m->max_groups = std::max(m->max_groups, groups);
@@ -1245,8 +1273,8 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
                                   (long long)pk->nx * ((b.y0 + ky) + (long long)pk->ny * (b.z0 + kz))));
       };
       const size_t q0 = perm.size(), p0 = gtab.size();
-      perm.resize(q0 + (size_t)kGroup * groups, -1);
-      vtab.resize(q0 + (size_t)kGroup * groups, ~pad(0, 0, 0, 0));
+      perm.resize(q0 + (size_t)G * groups, -1);
+      vtab.resize(q0 + (size_t)G * groups, ~pad(0, 0, 0, 0));
       gtab.resize(p0 + b.P);
       if (factor_prec == 64) ptab.resize(p0 + b.P);
       int lex = 0;
@@ -1258,7 +1286,7 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
               perm[q0 + q] = lex;
               vtab[q0 + q] = pad(kx, ky, kz, kt);
               gtab[p0 + lex] = make_int2(glob(kx, ky, kz, kt), vtab[q0 + q]);
-              if (factor_prec == 64) ptab[p0 + lex] = q / kGroup * gvals + q % kGroup;
+              if (factor_prec == 64) ptab[p0 + lex] = q / G * gvals + q % G;
             }
       b.ooff = (long long)otab.size();
       for (int gt = b.ot0; gt < b.ot1; ++gt)
@@ -1305,7 +1333,8 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   const size_t esz = factor_prec == 64 ? sizeof(double) : (factor_prec == 32 ? sizeof(float) : 2);
   const size_t vsz = factor_prec == 64 ? sizeof(double) : sizeof(float);
   // every lane vector must start on a 16-byte boundary (group and box offsets are whole groups)
-  static_assert(kGroupVals32 * 2 % 16 == 0 && kLaneL * 32 * 2 % 16 == 0, "16-byte lane vectors");
+  static_assert(group_vals(32, kGroup) * 2 % 16 == 0 && group_vals(32, narrow_group(32)) * 2 % 16 == 0 &&
+                kLanes * narrow_group(32) * kLaneL * 2 % 16 == 0, "16-byte lane vectors");
   auto fail = [&](kkt_status st, const char* what) {
     cudaGetLastError();
     set_error(std::string("ras_setup: ") + what);
@@ -1366,9 +1395,10 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
     m->ring = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && tab + invb <= free_b / 4 &&
               cudaMalloc(&inv, invb) == cudaSuccess && cudaMalloc(&m->ntab, tab) == cudaSuccess;
     if (m->ring) {
-      place_points<<<dim3(m->nbox, (kGroup * m->max_groups + 255) / 256), 256>>>(m->boxes, m->gptr, m->perm, inv);
-      neighbour_places<<<dim3(m->nbox, (m->max_groups + 7) / 8), 256>>>(m->boxes, m->gptr, m->perm, inv, m->wcap,
-                                                                        m->ntab);
+      place_points<<<dim3(m->nbox, (m->group * m->max_groups + 255) / 256), 256>>>(m->boxes, m->gptr, m->perm, m->group,
+                                                                                   inv);
+      neighbour_places<<<dim3(m->nbox, (m->max_groups + 7) / 8), 256>>>(m->boxes, m->gptr, m->perm, inv, m->group,
+                                                                        m->wcap, m->ntab);
       KKT_COUNT(2);
       e = cudaGetLastError();
       if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -1398,11 +1428,11 @@ kkt_status launch_solve(ras_precond* m, const double* r, double* z, typename Sol
   using T = typename SolveArith<S>::type;
   const int gbytes = m->gptr_bytes;
   // (the dynamic shared-memory limit of both instances is raised at set-up, in choose_solve_shape)
-  const size_t smem = solve_smem<S>(gbytes, m->warps, m->nbuf, m->ring) +
+  const size_t smem = solve_smem<S>(gbytes, m->warps, m->nbuf, m->group, m->ring) +
                       (m->ring ? ring_smem(m->wcap) : m->smem_vec ? (size_t)m->max_pad * sizeof(T) : 0);
-  const void* kernel = solve_kernel<S>(m->smem_vec, m->ring, m->cluster);
+  const void* kernel = solve_kernel<S>(m->group, m->smem_vec, m->ring, m->cluster);
   if constexpr (std::is_same_v<S, float>)
-    if (extra.hold != kHoldNone) kernel = solve_kernel<S, true>(m->smem_vec, m->ring, m->cluster);
+    if (extra.hold != kHoldNone) kernel = solve_kernel<S, true>(m->group, m->smem_vec, m->ring, m->cluster);
   const BoxDesc* boxes = m->boxes;
   const S* F = (const S*)m->F;
   const int *gptr = m->gptr, *vtab = m->vtab;
@@ -1593,9 +1623,9 @@ extern "C" kkt_status ras_selftest_wait(ras_precond* m, double limit_ms, void* s
 extern "C" kkt_status ras_selftest_solve(ras_precond* m, const double* r, double* z, double limit_ms, int hold, int cta,
                                          int* drained, void* stream) {
   if (!m || !r || !z || !(limit_ms > 0.0) || limit_ms > 1000.0 || hold < kHoldCounter || hold > kHoldCopies || cta < 0 ||
-      m->local != 0 || m->prec != 32 || cta >= m->cluster || spans_overlap(r, z, m->n_total)) {
+      m->local != 0 || m->prec != 32 || m->group != kGroup || cta >= m->cluster || spans_overlap(r, z, m->n_total)) {
     set_error("ras_selftest_solve: null argument, limit_ms outside (0, 1000], hold not 1 or 2, cta outside the cluster, "
-              "r and z overlap, or not an ILU(0) preconditioner with FP32 factors");
+              "r and z overlap, or not an ILU(0) preconditioner with FP32 factors in groups of 8");
     return KKT_ERR_ARG;
   }
   const cudaStream_t s = (cudaStream_t)stream;
@@ -1606,7 +1636,7 @@ extern "C" kkt_status ras_selftest_solve(ras_precond* m, const double* r, double
   extra.hold = hold;
   extra.hold_cta = cta;
   extra.drained = d;
-  cudaError_t e = cudaFuncSetAttribute(solve_kernel<float, true>(m->smem_vec, m->ring, m->cluster),
+  cudaError_t e = cudaFuncSetAttribute(solve_kernel<float, true>(m->group, m->smem_vec, m->ring, m->cluster),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
   if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(int), s);
   const kkt_status st = e == cudaSuccess ? ras_launch(m, r, z, s, nullptr, 0, extra) : KKT_OK;

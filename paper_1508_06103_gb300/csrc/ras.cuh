@@ -6,26 +6,30 @@
 // slots per point: C row 2*27*2 = 108, G row 2*(27+1) = 56, f row 3*27*2 = 162
 constexpr int kSlots = 326;
 
-// The points of a wavefront are stored in groups of 8 (the last one of a
+// The points of a wavefront are stored in groups of G = 8 (the last one of a
 // wavefront may be ragged): one warp of the subdomain solve takes one group.
-// Values per group: FP64 [slot rank][8] blocks; FP32 and BF16 44 lower and 38
-// upper values for each of the 32 lanes (ras.cu), 326 slots x 8 points plus 16
+// Where groups of 8 would be mostly empty (boxes of a few points a wavefront:
+// lines, thin plates, a few nodes a side) G is narrow_group: the same kernels
+// with some lanes idle, for a half or a quarter of the memory.
+// Values per group: FP64 [slot rank][G] blocks; FP32 and BF16 44 lower and 38
+// upper values for each of 4 G lanes (ras.cu), 326 slots x G points plus 2 G
 // unused places.
 constexpr int kGroup = 8;
-constexpr int kGroupVals64 = kSlots * kGroup;
+__host__ __device__ constexpr int narrow_group(int prec) { return prec == 64 ? 2 : 4; }
 constexpr int kLaneL = 44, kLaneU = 38;                        // values per lane of a group
-constexpr int kGroupVals32 = 32 * (kLaneL + kLaneU);
-__host__ __device__ constexpr int group_vals(int prec) { return prec == 64 ? kGroupVals64 : kGroupVals32; }
+__host__ __device__ constexpr int group_vals(int prec, int G) {
+  return prec == 64 ? kSlots * G : 4 * G * (kLaneL + kLaneU);
+}
 
 // Where the solve's lanes keep their values (FP32 and BF16): place of value v
 // of a lane within its group.  A lane's values form 16-byte vectors, vector k
-// of the 32 lanes side by side, so a warp reads 512 contiguous bytes at a
+// of the 4 G lanes side by side, so a warp reads up to 512 contiguous bytes at a
 // time; the last vector is shorter where the count is no multiple.
-template <typename S>
+template <typename S, int G>
 __host__ __device__ __forceinline__ int lane_place(bool upper, int v, int lane) {
-  constexpr int W = 16 / (int)sizeof(S);
-  const int n = upper ? kLaneU : kLaneL, full = n / W * W, base = upper ? 32 * kLaneL : 0;
-  return base + (v < full ? (v / W * 32 + lane) * W + v % W : full * 32 + lane * (n - full) + (v - full));
+  constexpr int W = 16 / (int)sizeof(S), L = 4 * G;
+  const int n = upper ? kLaneU : kLaneL, full = n / W * W, base = upper ? L * kLaneL : 0;
+  return base + (v < full ? (v / W * L + lane) * W + v % W : full * L + lane * (n - full) + (v - full));
 }
 
 struct GpFactor;   // ILU(1) / point-block ILU(0) factors (iluk.cu)
@@ -74,6 +78,7 @@ struct ras_precond {
   int nbuf = 1;                // buffers a warp has for them: one less, fewer where they do not fit
   int gptr_bytes = 0;          // wavefront pointers in the solve's shared memory (0: read from global memory)
   int lanes = 4;               // lanes per point in the solve
+  int group = kGroup;          // points per group
   int cluster = 1;             // CTAs per box of the solve
   bool ring = false;           // solve keeps the last wavefronts in shared memory
   int wcap = 0;                // group places of the widest wavefront
@@ -130,6 +135,7 @@ kkt_status ras_factor_status(ras_precond* m);                   // after the str
 // gather and ILU(0) launches of factor32.cu / factor64.cu
 kkt_status ras_factor_launch32(ras_precond* m, cudaStream_t s);
 kkt_status ras_factor_launch64(ras_precond* m, cudaStream_t s);
+kkt_status ras_factor_launch64_narrow(ras_precond* m, cudaStream_t s);   // groups of narrow_group points
 kkt_status ras_factor_launch16(ras_precond* m, cudaStream_t s);   // FP32 factorisation, BF16 store
 kkt_status ras_factor_prepare32(ras_precond* m);                  // launch shape and records of the two above
 // exact banded LU (lu.cu)

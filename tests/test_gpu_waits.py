@@ -58,15 +58,16 @@ def _groups(dims, nsub, overlap):
                     yield sum(-(-int(c) // 8) for c in np.bincount((x + 2 * y + 4 * z + 8 * t).ravel()))
 
 
-@pytest.mark.parametrize("nsub, place", [((2, 2, 1, 2), 1), ((2, 2, 1, 2), 2), ((3, 2, 2, 4), 2)],
+@pytest.mark.parametrize("dims, nsub, place", [((6, 5, 4, 6), (2, 2, 1, 2), 1), ((6, 5, 4, 6), (2, 2, 1, 2), 2),
+                                               ((12, 10, 8, 16), (3, 2, 2, 4), 2)],
                          ids=["vectors-in-smem", "plain", "ring"])
 @pytest.mark.parametrize("stages", [2, 3, 4])
-def test_a_solve_that_gives_up_waits_for_its_copies(api, stages, nsub, place):
+def test_a_solve_that_gives_up_waits_for_its_copies(api, stages, dims, nsub, place):
     # every warp gives up at its first group: that one's copy has landed, the next `buffers` groups'
     # are in flight
     from paper_1508_06103_gb300._lib import KktError
 
-    w = W.random_small(41, cells=(5, 4, 3), M=5, nsens=4)
+    w = W.random_small(41, cells=tuple(n - 1 for n in dims[:3]), M=dims[3] - 1, nsens=4)
     prob = api.Problem.from_workload(w)
     ras = api.RAS(prob, nsub, 1, 32, shape=(20, stages, 0, place))
     form = ras.solve_form()
@@ -75,7 +76,7 @@ def test_a_solve_that_gives_up_waits_for_its_copies(api, stages, nsub, place):
     z0 = ras.apply(r).clone()
     z = torch.full_like(r, 7.0)
     expect = 0
-    for ng in _groups((6, 5, 4, 6), nsub, 1):
+    for ng in _groups(dims, nsub, 1):
         expect += sum(range(form["warps"] + 1, min(2 * ng, (form["buffers"] + 1) * form["warps"]) + 1))
     assert ras.selftest_solve(r, z, 5.0) == expect > 0
     assert (z == 7.0).all()
