@@ -209,7 +209,8 @@ kkt_status ras_setup(kkt_problem* p, const int nsub[4], int overlap, int local, 
  *   shape applies the same ILU(0) factors.
  *   shape[0]  size class of a box's CTA, by names from when it was a number of
  *             points (FP64: 34, 26, 18; FP32: 52, 36, 20; BF16: 72, 40, 8): 16,
- *             8 or 4 warps, each taking 8 points of a wavefront at a time
+ *             8 or 4 warps, each taking 8 points of a wavefront at a time (fewer
+ *             than 4 where very many boxes have a few points a wavefront)
  *   shape[1]  2..4: groups of 8 points whose factor values a warp holds, the one
  *             in use included (one less are buffers in shared memory, fewer
  *             where they do not fit; FP64 reads its factors from global memory

@@ -971,8 +971,8 @@ struct ShapeRequest {
 // groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
 // global memory, the fewest buffers, the largest CTA.  ras_autotune measures instead.
 template <typename T>
-kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int group, int wcap, int nsm,
-                              const ShapeRequest& req, SolveShape* out) {
+kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int group, double gpw, int wcap,
+                              int nsm, const ShapeRequest& req, SolveShape* out) {
   if (req.lanes != 0 && req.lanes != kLanes) {
     set_error("ras_setup: the subdomain solve runs 4 lanes per point");
     return KKT_ERR_ARG;
@@ -1022,9 +1022,31 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
         const long long waves = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm);
         const bool filled = ci == 0 && points > (long long)nbox * nlev * kGroup * kFillGroups;
         const long long key = (filled ? 0 : waves) * 100000000LL + (sv ? 1000000 : 0) + (ns - 2) * 1000 + (100 - ch);
-        if (best_key < 0 || key < best_key) {
-          best_key = key;
-          best = SolveShape{ch, ns, kLanes, w, nbuf, gbytes, sv != 0, ring, 1};
+        if (best_key >= 0 && key >= best_key) continue;
+        best_key = key;
+        best = SolveShape{ch, ns, kLanes, w, nbuf, gbytes, sv != 0, ring, 1};
+        if (ci < 2 || waves < 2 || (sizeof(T) == 4 && group == kGroup)) continue;
+        // Boxes beyond what the SMs hold at a time, with hardly more than a group a wavefront: fewer warps
+        // each, more boxes at a time.  A wave of CTAs of w warps with g groups a wavefront was measured
+        // to take about 1 + 5 g / w.  us an apply with 1, 2, 3, 4 warps, FP64 (FP32; BF16):
+        //   9537 lines of 17 points:         1013 1153 1663 2034   (221 240 277 306; 214 234 273 307)
+        //   4913 lines of 33 levels:         1228 1365 1771 2222   (364 370 421 461; 341 359 415 455)
+        //   4096 boxes of 2^4 points:         426  520  691  802   (106 112 124 136;  99 108 122 136)
+        //   1296 boxes of 3^4 points:         485  623  561  733   (103 111  87 105; 101 105  83 102)
+        //   4096 boxes of 3 or 4 a side:     1276 1661 2258 2674   (381 369 364 367; 297 291 307 326)
+        //   256 boxes of 3 or 4 a side:       421  366  364  365   (171  93  68  58; 161  87  64  54)
+        // The last are one wave in any case; the last but one are FP32's groups of 8, bound by their bytes.
+        double cost = waves * (1 + 5 * gpw / w);
+        for (int fewer = w - 1; fewer >= 1 && fewer >= gpw; --fewer) {
+          const size_t less = solve_smem<T>(gbytes, fewer, nbuf, group, ring) + (ring ? ring_smem(wcap) : vec);
+          KKT_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+              &per_sm, solve_kernel<T>(group, sv != 0, ring, 1), 32 * fewer, less));
+          if (per_sm < 1) continue;
+          const double c = (nbox + (long long)nsm * per_sm - 1) / ((long long)nsm * per_sm) * (1 + 5 * gpw / fewer);
+          if (c < cost) {
+            cost = c;
+            best.warps = fewer;
+          }
         }
       }
   if (best_key < 0) {
@@ -1139,8 +1161,8 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
   std::stable_sort(geoms.begin(), geoms.end(), [](const Geom& a, const Geom& b) { return a.points > b.points; });
   {
     // largest padded local vector, most wavefronts, points of all boxes, groups of 8 and of the narrow
-    // size, whether a box of groups of 8 has too many values for the FP64 factorisation's offsets
-    long long pad = 0, points = 0, wide = 0;
+    // size, wavefronts with points, whether a box of groups of 8 has too many values for the FP64 factorisation's offsets
+    long long pad = 0, points = 0, wide = 0, narrow = 0, fronts = 0;
     bool too_large = false;
     for (const Geom& g : geoms) {
       const kkt_problem* pk = probs[g.prob];
@@ -1156,6 +1178,8 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
         long long groups = 0;
         for (int n : wavefronts(len)) {
           groups += (n + kGroup - 1) / kGroup;
+          narrow += (n + narrow_group(factor_prec) - 1) / narrow_group(factor_prec);
+          fronts += n > 0;
           m->wcap = std::max(m->wcap, (n + kGroup - 1) / kGroup * kGroup);   // places of the widest wavefront
         }
         wide += groups;
@@ -1165,12 +1189,14 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       points += g.points;
       m->max_nlev = std::max(m->max_nlev, nlev);
     }
-    // Narrow groups where groups of 8 would be filled by less than a third (FP64) or a half (FP32,
-    // BF16).  Factor values a point, groups of 8 and narrow ones: boxes of one node in two or three
-    // axes, or of two nodes a side, FP64 2608 and 652, FP32 2624 and 1312; 17 x 1 x 1 x 65 nodes FP64
-    // 1249 and 349, FP32 1256 and 628; 3 x 3 x 3 x 3 FP64 998 and 411, FP32 1004 and 567.
-    if (local == 0 && (wide * kGroup > (factor_prec == 64 ? 3 : 2) * points || (factor_prec == 64 && too_large)))
+    // Narrow groups where groups of 8 would be filled by less than a third, in FP32 a half (BF16 at a
+    // half: 256 boxes of 3 or 4 nodes a side 43.5 -> 45.5 us an apply).  Factor values a point with groups
+    // of 8 and narrow ones: boxes of one node in two or three axes, or of two nodes a side, FP64 2608 and
+    // 652, FP32 2624 and 1312; 17 x 1 x 1 x 65 nodes FP64 1249 and 349, FP32 1256 and 628; 3 x 3 x 3 x 3
+    // FP64 998 and 411, FP32 1004 and 567.
+    if (local == 0 && (wide * kGroup > (factor_prec == 32 ? 2 : 3) * points || (factor_prec == 64 && too_large)))
       m->group = narrow_group(factor_prec);
+    const double gpw = (double)(m->group == kGroup ? wide : narrow) / std::max(fronts, 1LL);   // groups a wavefront
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) {
@@ -1188,9 +1214,9 @@ kkt_status ras_create(kkt_problem* const* probs, int nprob, const int nsub[4], i
       req.place = shape[3];
     }
     SolveShape sh{};
-    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, m->group, m->wcap, nsm, req, &sh)
-                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, m->group, m->wcap, nsm, req, &sh)
-                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, m->group, m->wcap, nsm, req, &sh);
+    const kkt_status cs = factor_prec == 64   ? choose_solve_shape<double>(nbox, points, pad, m->max_nlev, m->group, gpw, m->wcap, nsm, req, &sh)
+                          : factor_prec == 32 ? choose_solve_shape<float>(nbox, points, pad, m->max_nlev, m->group, gpw, m->wcap, nsm, req, &sh)
+                                              : choose_solve_shape<__nv_bfloat16>(nbox, points, pad, m->max_nlev, m->group, gpw, m->wcap, nsm, req, &sh);
     if (cs != KKT_OK) {
       delete m;
       return cs;

@@ -83,10 +83,10 @@ def test_narrow_boxes_match_oracle(api, name, prec):
 @pytest.mark.parametrize("prec", [64, 32, 16])
 @pytest.mark.parametrize("name", CASES)
 def test_narrow_boxes_take_no_more_than_a_third_beyond_short_rows(api, name, prec):
-    # the yardstick: a wavefront's rows padded to 2 points in FP64 (4 in FP32) when it has no more,
-    # to the next 8 k + 2 (16 k + 4) when it has
+    # the yardstick: a wavefront's rows padded to 2 points in FP64 (4 in FP32, 8 in BF16) when it has no
+    # more, to the next 8 k + 2 (16 k + 4, 32 k + 8) when it has
     dims, nsub, ov = CASES[name]
-    first, step = (2, 8) if prec == 64 else (4, 16)
+    first, step = {64: (2, 8), 32: (4, 16), 16: (8, 32)}[prec]
     places = boxes = 0
     for h in _wavefronts(dims, nsub, ov):
         boxes += 1
@@ -94,3 +94,21 @@ def test_narrow_boxes_take_no_more_than_a_third_beyond_short_rows(api, name, pre
     values = api.RAS(api.Problem.from_workload(_problem(dims)), nsub, ov, prec).info()["factor_values"]
     # 328 values a point in FP32 and BF16 (2 places unused), a unit row a box in FP64
     assert values <= 4 / 3 * places * (326 if prec == 64 else 328) + (boxes * 326 * 2 if prec == 64 else 0)
+
+
+# many boxes of one group a wavefront: CTAs of fewer warps than the smallest size class has
+@pytest.mark.parametrize("prec", [64, 32, 16])
+@pytest.mark.parametrize("dims, nsub", [((17, 17, 17, 9), (1, 17, 17, 9)), ((18, 18, 18, 18), (6, 6, 6, 6))],
+                         ids=["lines", "cubes"])
+def test_many_narrow_boxes_take_fewer_warps(api, dims, nsub, prec):
+    w = _problem(dims)
+    prob = api.Problem.from_workload(w)
+    ras = api.RAS(prob, nsub, 0, prec)
+    assert ras.solve_form()["warps"] in (1, 2, 3)
+    # the same groups in the same order on 16 warps: the same bits (16 warps are held to the oracle elsewhere)
+    few = api.RAS(prob, nsub, 0, prec, shape=({64: 34, 32: 52, 16: 72}[prec], 0, 0, 2))
+    assert few.solve_form()["warps"] == 16
+    r = torch.from_numpy(W.random_vector(prob.n, 5)).cuda()
+    z = ras.apply(r)
+    assert torch.isfinite(z).all() and z.abs().max() > 0 and torch.equal(z, few.apply(r))
+    assert ras.status() == 0
