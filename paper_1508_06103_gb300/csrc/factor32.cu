@@ -505,7 +505,12 @@ kkt_status ras_factor_prepare32(ras_precond* m) {
   KKT_TRY_CUDA(cudaOccupancyMaxActiveClusters(
       &most, m->prec == 16 ? kernel_of<__nv_bfloat16>(cs, m->group) : kernel_of<float>(cs, m->group), &cfg));
   m->fac_nclusters = std::max(1, std::min(most, m->nbox));
-  for (;; m->fac_nclusters /= 2) {   // fewer boxes at a time where memory is short
+  // fewer boxes at a time where their records would take more than a quarter of the free memory, which
+  // a problem sized to the memory needs for its Krylov vectors
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess)
+    while (m->fac_nclusters > 1 && (size_t)m->fac_nclusters * rec * sizeof(float) > free_b / 4) m->fac_nclusters /= 2;
+  for (;; m->fac_nclusters /= 2) {
     if (cudaMalloc(&m->rec, (size_t)m->fac_nclusters * rec * sizeof(float)) == cudaSuccess) return KKT_OK;
     cudaGetLastError();
     m->rec = nullptr;
