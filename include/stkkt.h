@@ -332,6 +332,13 @@ kkt_status ras_selftest_solve(ras_precond* m, const double* r, double* z, double
                               int* drained, void* stream);
 
 /*
+ * lu_selftest_quotient -- test hook (no counterpart in the paper): q[i] =
+ *   v[i] / d[i] for n device values, as the exact local LU's backward sweep
+ *   divides by its diagonals.  Does not synchronise.
+ */
+kkt_status lu_selftest_quotient(const double* v, const double* d, double* q, long long n, void* stream);
+
+/*
  * ras_apply -- z = sum_ij (R^0_ij)^T M_ij^{-1} R^delta_ij r (restricted prolongation,
  *   Cai-Sarkis form cited in Sec. 3.2); all boxes in one launch.  r, z FP64,
  *   3*N*(M+1) values each; the two spans must not overlap (ERR_ARG).  Does not

@@ -66,6 +66,7 @@ SIGNATURES = {
                                     C.c_double, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_double),
                                     C.POINTER(C.c_int), C.c_void_p]),
     "ras_selftest_wait": (C.c_int, [C.c_void_p, C.c_double, C.c_void_p]),
+    "lu_selftest_quotient": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
     "ras_selftest_solve": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_double, C.c_int, C.c_int,
                                      C.POINTER(C.c_int), C.c_void_p]),
     "ras_selftest_lanes": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int), C.c_void_p]),

@@ -167,6 +167,22 @@ constexpr int kLuFwd = (kMaxLuBand + kLuThreads - 1) / kLuThreads;       // rows
 constexpr int kLuBwd = (2 * kMaxLuBand + kLuThreads - 1) / kLuThreads;   // and U
 static_assert((kLuThreads & (kLuThreads - 1)) == 0, "row owners by mask");
 
+// v / d from r = 1 / d (rounded to nearest): the product and one correction by its exact residual,
+// the last step of the division by Newton iteration of P. Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34 (1990).  The bits of the
+// division, or one unit in the last place away where a value is subnormal; infinities, NaN and a
+// reciprocal that overflows take the division itself.
+__device__ __forceinline__ double quotient(double v, double d, double r) {
+  const double q = v * r, e = fma(-d, q, v);
+  return isfinite(e) ? fma(e, r, q) : v / d;
+}
+
+__global__ void quotient_selftest(const double* __restrict__ v, const double* __restrict__ d, double* __restrict__ q,
+                                  long long n) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i < n) q[i] = quotient(v[i], d[i], 1.0 / d[i]);
+}
+
 // WIDE: a half-bandwidth above kLuThreads (more rows per thread)
 template <bool WIDE>
 __global__ void __launch_bounds__(kLuThreads) lu_solve(const BoxDesc* __restrict__ boxes,
@@ -265,15 +281,10 @@ __global__ void __launch_bounds__(kLuThreads) lu_solve(const BoxDesc* __restrict
     diag_load(top);
     diag_divide(top);
     diag_load(top - 1);
-    // x = b / a from the reciprocal, corrected once (as accurate as the division)
-    auto quotient = [&](double v) {
-      const double q = v * rd, e = fma(-dg, q, v);
-      return isfinite(e) ? fma(e, rd, q) : v / dg;
-    };
 #pragma unroll
     for (int c = 0; c < kLuAhead; ++c)
       if (n - 1 - c >= 0) load(n - 1 - c, a[c]);
-    if (t == ((n - 1) & mask)) pub[2 * ((n - 1) & 1)] = quotient(bvec[n - 1]);
+    if (t == ((n - 1) & mask)) pub[2 * ((n - 1) & 1)] = quotient(bvec[n - 1], dg, rd);
     __syncthreads();
     for (int j0 = n - 1; j0 >= 0; j0 -= kLuAhead) {
 #pragma unroll
@@ -292,7 +303,7 @@ __global__ void __launch_bounds__(kLuThreads) lu_solve(const BoxDesc* __restrict
           if (ii >= first) {
             const double v = fma(-a[c][q], xj, bvec[ii]);
             bvec[ii] = v;
-            if (q == 0 && ii == j - 1) pub[2 * ((j - 1) & 1)] = quotient(v);
+            if (q == 0 && ii == j - 1) pub[2 * ((j - 1) & 1)] = quotient(v, dg, rd);
           }
         }
         if (t == (j & mask)) bvec[j] = xj;
@@ -356,6 +367,17 @@ kkt_status ras_lu_solve(ras_precond* m, const double* r, double* z, cudaStream_t
   const size_t smem = ((size_t)nmax + 4) * sizeof(double);
   auto* kernel = klmax > kLuThreads ? lu_solve<true> : lu_solve<false>;   // L and U rows per thread: 2 and 4, or 1 and 2
   kernel<<<m->nbox, kLuThreads, smem, s>>>(m->boxes, m->AB, m->ipiv, r, z, p->nx, p->ny, p->N, gate);
+  KKT_COUNT(1);
+  KKT_TRY_CUDA(cudaGetLastError());
+  return KKT_OK;
+}
+
+extern "C" kkt_status lu_selftest_quotient(const double* v, const double* d, double* q, long long n, void* stream) {
+  if (!v || !d || !q || n < 1 || n > (1LL << 30)) {
+    set_error("lu_selftest_quotient: null argument or n outside [1, 2^30]");
+    return KKT_ERR_ARG;
+  }
+  quotient_selftest<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(v, d, q, n);
   KKT_COUNT(1);
   KKT_TRY_CUDA(cudaGetLastError());
   return KKT_OK;
