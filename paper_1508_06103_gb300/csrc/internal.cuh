@@ -125,6 +125,7 @@ struct DevProblem {
                                             // (an Arnoldi step after convergence); nullptr = always run
   const float4* pack32;                     // [N][27] FP32 {B, S, ST, K}, node by node (the FP32 factorisation)
   int nsm;                                  // SMs of the device
+  int plan64;                               // FP64 matvec: levels of a run, < 0 with the other tile (matvec64_plan)
 };
 
 // True when a gated kernel should return without work.
@@ -199,6 +200,7 @@ struct kkt_problem {
   int reg = 0;                              // kkt_set_regularization
   int elem = 0;                             // kkt_set_element
   int nsm = 1;                              // SMs of the device
+  int plan64 = 1;                           // matvec64_plan of the grid
   // host copies used by the coarse level and by kkt_set_element
   std::vector<double> a_cell, v_cell;
   std::vector<int> sensor_node;
@@ -218,6 +220,7 @@ struct kkt_problem {
 
 // matvec.cu (kernels return at once while *p.gate reads 0)
 kkt_status matvec_prepare();   // raises the kernels' shared-memory limit on the current device
+int matvec64_plan(const DevProblem& p);   // tile and run length of the FP64 matvec on this grid and device
 kkt_status launch_matvec64(const DevProblem& p, const double* x, double* y, cudaStream_t s);
 kkt_status launch_matvec32(const DevProblem& p, const float* x, float* y, cudaStream_t s);
 kkt_status launch_residual(const DevProblem& p, const double* b, const double* x, double* r, cudaStream_t s);

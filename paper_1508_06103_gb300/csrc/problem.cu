@@ -113,7 +113,7 @@ extern "C" const char* kkt_version(void) { return "stkkt 0.1 (sm_103a)"; }
 DevProblem kkt_problem::dev() const {
   DevProblem d;
   d.nx = nx; d.ny = ny; d.nz = nz; d.N = N; d.M = M; d.L = L; d.P = P;
-  d.tau = tau; d.theta = theta; d.beta1 = beta1; d.beta2 = beta2; d.reg = reg; d.elem = elem; d.nsm = nsm;
+  d.tau = tau; d.theta = theta; d.beta1 = beta1; d.beta2 = beta2; d.reg = reg; d.elem = elem; d.nsm = nsm; d.plan64 = plan64;
   d.hx = hx; d.hy = hy; d.hz = hz;
   const size_t c = (size_t)kStencil * N;
   d.S = coef64; d.ST = coef64 + c; d.B = coef64 + 2 * c; d.K = coef64 + 3 * c;
@@ -452,6 +452,7 @@ kkt_status create_problem(const kkt_grid* g, int nt, double dt, const double* a_
       set_error("kkt_create: cannot query the current device");
       return fail(KKT_ERR_CUDA);
     }
+    p->plan64 = matvec64_plan(p->dev());
   }
   *out = p;
   return KKT_OK;
