@@ -170,6 +170,10 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
+// asks for bytes (a multiple of 16, from a 16-byte boundary) in L2; nothing waits for them
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ int ld_acquire_cta(const int* p) {
   int v;
   asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
@@ -430,7 +434,12 @@ struct LaneFactors<__nv_bfloat16, G> {
 };
 
 // FP64: the values stay in global memory ([slot rank][G] groups) until they
-// are used; the FP64 pipe is the limit, and other warps hide the loads.
+// are used; a warp has its next group's brought to L2 while it works on one, by one bulk
+// prefetch.  (Without it every wavefront waited for HBM: boxes of two or three groups a
+// wavefront were slower than with chunks copied to shared memory.  us an apply, with / without /
+// chunks: 64 boxes, 2.9 groups 813 / 970 / 835, 1.5 groups 574 / 707 / 621; 128 boxes, 2.7 groups
+// 787 / 924 / 801; 64 boxes, 8.4 groups 2383 / 2628 / 4866; 32^3 x 64 9242 / 9840 / 12600.  Prefetches
+// of the own group to L1 before the wait, alone or besides: 1 to 4 % slower than this.)
 template <int G>
 struct LaneFactors<double, G> {
   static constexpr bool kStaged = false;
@@ -626,6 +635,11 @@ __global__ void __launch_bounds__(32 * kSolveWarpsMax) ras_solve(
         issue(k + nbuf * nwarp, t + nbuf);
       } else {
         fac.load(Fb + (long long)group(k) * group_vals(64, G), kUpper, flane);
+        if (const int kn = k + nwarp; lane == 0 && kn < 2 * ng) {   // the warp's next group
+          const bool up = kn >= ng;
+          bulk_prefetch_l2(Fb + (long long)group(kn) * group_vals(64, G) + (up ? kLRanks * G : 0),
+                           (up ? kSlots - kLRanks : kLRanks) * G * (unsigned)sizeof(S));
+        }
       }
       // neighbours two and more wavefronts away (at the first backward step the own point is one
       // of the last wavefront's)
