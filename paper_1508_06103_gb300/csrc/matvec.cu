@@ -101,43 +101,19 @@ __host__ __device__ constexpr bool kuhn_offset(int d) {
 }
 
 // 1D linear-element mass and stiffness rows on one axis of n nodes with
-// width h: row i has (i > 0) + (i < n - 1) elements; the entries are chosen
-// from values formed once on the host (no arithmetic per node).
-template <typename T>
-struct Axis1D {
-  int n;
-  T m1, m2, mo, k1, k2, ko;   // mass diagonal (one / two elements), off-diagonal; the same for stiffness
-  T hh;                       // the width
-  __host__ __device__ void init(int n_, double h) {
-    n = n_;
-    m1 = (T)(h / 3.0);
-    m2 = (T)(2.0 * h / 3.0);
-    mo = (T)(h / 6.0);
-    k1 = (T)(1.0 / h);
-    k2 = (T)(2.0 / h);
-    ko = (T)(-1.0 / h);
-    hh = (T)h;
-  }
+// width hh: row i has (i > 0) + (i < n - 1) elements.  Formed per node (against
+// choosing from stored values: measured 4 % faster).
+__device__ __forceinline__ void axis_row(int n, float hh, int i, float& m_, float& m0, float& mp, float& k_, float& k0,
+                                         float& kp) {
   // entries (i, i-1), (i, i), (i, i+1) of the mass (m) and stiffness (k) rows
-  __device__ __forceinline__ void row(int i, T& m_, T& m0, T& mp, T& k_, T& k0, T& kp) const {
-    const bool lo = i > 0, hi = i < n - 1;
-    if constexpr (sizeof(T) == 8) {   // FP64: select only (the FP64 pipe is the limit)
-      m_ = lo ? mo : (T)0;
-      mp = hi ? mo : (T)0;
-      m0 = lo && hi ? m2 : (lo || hi ? m1 : (T)0);
-      k_ = lo ? ko : (T)0;
-      kp = hi ? ko : (T)0;
-      k0 = lo && hi ? k2 : (lo || hi ? k1 : (T)0);
-    } else {                          // FP32: from the width per node (measured 4 % faster)
-      m0 = (T)((i > 0) + (i < n - 1)) * hh / (T)3;
-      m_ = lo ? hh / (T)6 : (T)0;
-      mp = hi ? hh / (T)6 : (T)0;
-      k0 = (T)((i > 0) + (i < n - 1)) / hh;
-      k_ = lo ? -(T)1 / hh : (T)0;
-      kp = hi ? -(T)1 / hh : (T)0;
-    }
-  }
-};
+  const bool lo = i > 0, hi = i < n - 1;
+  m0 = (float)((i > 0) + (i < n - 1)) * hh / 3.f;
+  m_ = lo ? hh / 6.f : 0.f;
+  mp = hi ? hh / 6.f : 0.f;
+  k0 = (float)((i > 0) + (i < n - 1)) / hh;
+  k_ = lo ? -1.f / hh : 0.f;
+  kp = hi ? -1.f / hh : 0.f;
+}
 
 // Weights of the six time combinations: the theta weights and the rows of
 // the 1D linear-element time mass Mt (tau/6 [1 4 1]) and stiffness Lt
@@ -189,8 +165,8 @@ __device__ __forceinline__ void cp_async_wait() {
 template <typename T, bool kL2, typename Tl, bool kP1 = false, bool kWide = false>
 __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const T* __restrict__ x,
                                                              T* __restrict__ y, const double* __restrict__ b,
-                                                             int tiles_x, int tiles_y, Axis1D<T> ax, Axis1D<T> ay,
-                                                             Axis1D<T> az, LevelW<T> W) {
+                                                             int tiles_x, int tiles_y, LevelW<T> W) {
+  static_assert(kP1 || sizeof(T) == 4, "FP64 under trilinear elements: matvec64_levels");
   constexpr int TX = Tl::TX, TY = Tl::TY, TZ = Tl::TZ;
   constexpr int HX = Tl::HX, HY = Tl::HY, NH = Tl::NH, NXP = Tl::NXP, NYP = Tl::NYP;
   if (gated_off(p.gate)) return;
@@ -314,7 +290,7 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
           yd[o] = b != nullptr ? b[o] - (double)yc : (double)yc;
           yd[o + 1] = b != nullptr ? b[o + 1] - (double)yg : (double)yg;
           yd[o + 2] = b != nullptr ? b[o + 2] - (double)yf : (double)yf;
-        } else if (b != nullptr) {
+        } else if (sizeof(T) == 8 && b != nullptr) {   // (FP32: the wide form only)
           y[o] = (T)(b[o] - (double)yc);
           y[o + 1] = (T)(b[o + 1] - (double)yg);
           y[o + 2] = (T)(b[o + 2] - (double)yf);
@@ -324,79 +300,71 @@ __global__ void __launch_bounds__(Tl::kThreads) matvec_tiled(DevProblem p, const
           y[o + 2] = yf;
         }
       }
-      continue;
-    }
-    // x pass: Mx on u1, u3, u5, u6 and Kx on u6
-    for (int e = t; e < NXP; e += blockDim.x) {
-      const int ex = e % TX, ey = (e / TX) % HY, ez = e / (TX * HY);
-      const int h = (ex + 1) + HX * (ey + HY * ez);
-      T m_, m0, mp, k_, k0, kp;
-      ax.row(bx0 + ex, m_, m0, mp, k_, k0, kp);
-      PX[e] = m_ * U[h - 1] + m0 * U[h] + mp * U[h + 1];
-      PX[NXP + e] = m_ * U[2 * NH + h - 1] + m0 * U[2 * NH + h] + mp * U[2 * NH + h + 1];
-      PX[2 * NXP + e] = m_ * U[4 * NH + h - 1] + m0 * U[4 * NH + h] + mp * U[4 * NH + h + 1];
-      PX[3 * NXP + e] = m_ * U[5 * NH + h - 1] + m0 * U[5 * NH + h] + mp * U[5 * NH + h + 1];
-      PX[4 * NXP + e] = k_ * U[5 * NH + h - 1] + k0 * U[5 * NH + h] + kp * U[5 * NH + h + 1];
-    }
-    __syncthreads();
-    // y pass: My on the four Mx results; My (Kx u6) + Ky (Mx u6)
-    for (int e = t; e < NYP; e += blockDim.x) {
-      const int ex = e % TX, ey = (e / TX) % TY, ez = e / (TX * TY);
-      const int q = ex + TX * ((ey + 1) + HY * ez);
-      T m_, m0, mp, k_, k0, kp;
-      ay.row(by0 + ey, m_, m0, mp, k_, k0, kp);
-#pragma unroll
-      for (int f = 0; f < 4; ++f)
-        PY[f * NYP + e] = m_ * PX[f * NXP + q - TX] + m0 * PX[f * NXP + q] + mp * PX[f * NXP + q + TX];
-      PY[4 * NYP + e] = m_ * PX[4 * NXP + q - TX] + m0 * PX[4 * NXP + q] + mp * PX[4 * NXP + q + TX] +
-                        k_ * PX[3 * NXP + q - TX] + k0 * PX[3 * NXP + q] + kp * PX[3 * NXP + q + TX];
-    }
-    __syncthreads();
-    if (own) {
-      // z pass and the S, S^T stencils
-      const int qz = tx + TX * (ty + TY * (tz + 1));
-      T m_, m0, mp, k_, k0, kp;
-      az.row(iz, m_, m0, mp, k_, k0, kp);
-      constexpr int zs = TX * TY;
-      T yc = m_ * PY[qz - zs] + m0 * PY[qz] + mp * PY[qz + zs];
-      T yg = m_ * PY[NYP + qz - zs] + m0 * PY[NYP + qz] + mp * PY[NYP + qz + zs];
-      T yf = m_ * PY[2 * NYP + qz - zs] + m0 * PY[2 * NYP + qz] + mp * PY[2 * NYP + qz + zs];
-      yf += m_ * PY[4 * NYP + qz - zs] + m0 * PY[4 * NYP + qz] + mp * PY[4 * NYP + qz + zs];
-      yf += k_ * PY[3 * NYP + qz - zs] + k0 * PY[3 * NYP + qz] + kp * PY[3 * NYP + qz + zs];
-#pragma unroll
-      for (int d = 0; d < kStencil; ++d) {
-        const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
-        const int h = hc + dx + HX * (dy + HY * dz);
-        T s_, st_;
-        if constexpr (sizeof(T) == 4) {
-          s_ = cS[d];
-          st_ = cST[d];
-        } else {
-          s_ = c.S[(size_t)d * N + j];
-          st_ = c.ST[(size_t)d * N + j];
-        }
-        yc += s_ * U[NH + h];
-        yg += st_ * U[3 * NH + h];
+    } else {
+      // x pass: Mx on u1, u3, u5, u6 and Kx on u6
+      for (int e = t; e < NXP; e += blockDim.x) {
+        const int ex = e % TX, ey = (e / TX) % HY, ez = e / (TX * HY);
+        const int h = (ex + 1) + HX * (ey + HY * ez);
+        T m_, m0, mp, k_, k0, kp;
+        axis_row(p.nx, (float)p.hx, bx0 + ex, m_, m0, mp, k_, k0, kp);
+        PX[e] = m_ * U[h - 1] + m0 * U[h] + mp * U[h + 1];
+        PX[NXP + e] = m_ * U[2 * NH + h - 1] + m0 * U[2 * NH + h] + mp * U[2 * NH + h + 1];
+        PX[2 * NXP + e] = m_ * U[4 * NH + h - 1] + m0 * U[4 * NH + h] + mp * U[4 * NH + h + 1];
+        PX[3 * NXP + e] = m_ * U[5 * NH + h - 1] + m0 * U[5 * NH + h] + mp * U[5 * NH + h + 1];
+        PX[4 * NXP + e] = k_ * U[5 * NH + h - 1] + k0 * U[5 * NH + h] + kp * U[5 * NH + h + 1];
       }
-      const bool dirj = p.dir[j] != 0;
-      const T C0 = X0[hc], G0 = X0[NH + hc], Cp = Xp[hc];
-      if (n == 0 || dirj) yc = C0;
-      if (n == M || dirj) yg = G0;
-      else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
-      const long long o = 3 * ((long long)n * N + j);
-      if constexpr (kWide) {
-        double* yd = reinterpret_cast<double*>(y);
-        yd[o] = b != nullptr ? b[o] - (double)yc : (double)yc;
-        yd[o + 1] = b != nullptr ? b[o + 1] - (double)yg : (double)yg;
-        yd[o + 2] = b != nullptr ? b[o + 2] - (double)yf : (double)yf;
-      } else if (b != nullptr) {
-        y[o] = (T)(b[o] - (double)yc);
-        y[o + 1] = (T)(b[o + 1] - (double)yg);
-        y[o + 2] = (T)(b[o + 2] - (double)yf);
-      } else {
-        y[o] = yc;
-        y[o + 1] = yg;
-        y[o + 2] = yf;
+      __syncthreads();
+      // y pass: My on the four Mx results; My (Kx u6) + Ky (Mx u6)
+      for (int e = t; e < NYP; e += blockDim.x) {
+        const int ex = e % TX, ey = (e / TX) % TY, ez = e / (TX * TY);
+        const int q = ex + TX * ((ey + 1) + HY * ez);
+        T m_, m0, mp, k_, k0, kp;
+        axis_row(p.ny, (float)p.hy, by0 + ey, m_, m0, mp, k_, k0, kp);
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+          PY[f * NYP + e] = m_ * PX[f * NXP + q - TX] + m0 * PX[f * NXP + q] + mp * PX[f * NXP + q + TX];
+        PY[4 * NYP + e] = m_ * PX[4 * NXP + q - TX] + m0 * PX[4 * NXP + q] + mp * PX[4 * NXP + q + TX] +
+                          k_ * PX[3 * NXP + q - TX] + k0 * PX[3 * NXP + q] + kp * PX[3 * NXP + q + TX];
+      }
+      __syncthreads();
+      if (own) {
+        // z pass and the S, S^T stencils
+        const int qz = tx + TX * (ty + TY * (tz + 1));
+        T m_, m0, mp, k_, k0, kp;
+        axis_row(p.nz, (float)p.hz, iz, m_, m0, mp, k_, k0, kp);
+        constexpr int zs = TX * TY;
+        T yc = m_ * PY[qz - zs] + m0 * PY[qz] + mp * PY[qz + zs];
+        T yg = m_ * PY[NYP + qz - zs] + m0 * PY[NYP + qz] + mp * PY[NYP + qz + zs];
+        T yf = m_ * PY[2 * NYP + qz - zs] + m0 * PY[2 * NYP + qz] + mp * PY[2 * NYP + qz + zs];
+        yf += m_ * PY[4 * NYP + qz - zs] + m0 * PY[4 * NYP + qz] + mp * PY[4 * NYP + qz + zs];
+        yf += k_ * PY[3 * NYP + qz - zs] + k0 * PY[3 * NYP + qz] + kp * PY[3 * NYP + qz + zs];
+#pragma unroll
+        for (int d = 0; d < kStencil; ++d) {
+          const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
+          const int h = hc + dx + HX * (dy + HY * dz);
+          yc += cS[d] * U[NH + h];
+          yg += cST[d] * U[3 * NH + h];
+        }
+        const bool dirj = p.dir[j] != 0;
+        const T C0 = X0[hc], G0 = X0[NH + hc], Cp = Xp[hc];
+        if (n == 0 || dirj) yc = C0;
+        if (n == M || dirj) yg = G0;
+        else yg += tau * (T)p.sens[j] * (th * Cp + th1 * C0);
+        const long long o = 3 * ((long long)n * N + j);
+        if constexpr (kWide) {
+          double* yd = reinterpret_cast<double*>(y);
+          yd[o] = b != nullptr ? b[o] - (double)yc : (double)yc;
+          yd[o + 1] = b != nullptr ? b[o + 1] - (double)yg : (double)yg;
+          yd[o + 2] = b != nullptr ? b[o + 2] - (double)yf : (double)yf;
+        } else if (b != nullptr) {   // (no caller; without the branch the compiler's code is 2 % slower)
+          y[o] = (T)(b[o] - (double)yc);
+          y[o + 1] = (T)(b[o + 1] - (double)yg);
+          y[o + 2] = (T)(b[o + 2] - (double)yf);
+        } else {
+          y[o] = yc;
+          y[o + 1] = yg;
+          y[o + 2] = yf;
+        }
       }
     }
   }
@@ -418,10 +386,6 @@ void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaSt
   const int tx = (p.nx + Tl::TX - 1) / Tl::TX, ty = (p.ny + Tl::TY - 1) / Tl::TY, tz = (p.nz + Tl::TZ - 1) / Tl::TZ;
   constexpr int NT = levels_per_cta<T>();
   dim3 grid(tx * ty * tz, (p.M + 1 + NT - 1) / NT);
-  Axis1D<T> ax, ay, az;
-  ax.init(p.nx, p.hx);
-  ay.init(p.ny, p.hy);
-  az.init(p.nz, p.hz);
   LevelW<T> w;
   w.init(p.tau, p.theta, p.beta1, p.beta2);
   // (the dynamic shared-memory limits are raised once, in matvec_prepare)
@@ -429,7 +393,7 @@ void launch_shape(const DevProblem& p, const T* x, T* y, const double* b, cudaSt
   auto* kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1> : matvec_tiled<T, false, Tl, kP1>;
   if constexpr (sizeof(T) == 4)
     if (yd) kernel = p.reg != 0 ? matvec_tiled<T, true, Tl, kP1, true> : matvec_tiled<T, false, Tl, kP1, true>;
-  kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, yd ? reinterpret_cast<T*>(yd) : y, b, tx, ty, ax, ay, az, w);
+  kernel<<<grid, Tl::kThreads, smem, s>>>(p, x, yd ? reinterpret_cast<T*>(yd) : y, b, tx, ty, w);
 }
 
 template <typename T>
