@@ -921,6 +921,11 @@ struct SolveShape {
 };
 // groups per wavefront from which the largest CTA is taken
 constexpr int kFillGroups = 4;
+// smallest cluster that shares a box (choose_cluster)
+template <typename T>
+constexpr int min_cluster() {
+  return sizeof(T) == 8 ? 2 : 4;
+}
 template <typename T, bool HOLD = false>
 const void* solve_kernel(int group, bool smem_vec, bool ring, int cluster) {
   constexpr int N = narrow_group(8 * sizeof(T));
@@ -933,9 +938,10 @@ const void* solve_kernel(int group, bool smem_vec, bool ring, int cluster) {
   if constexpr (LaneFactors<T, kGroup>::kStaged)
     if (ring) return (const void*)ras_solve<T, false, true, 1, HOLD>;
   if (smem_vec) return (const void*)ras_solve<T, true, false, 1, HOLD>;
+  if constexpr (min_cluster<T>() == 2)
+    if (cluster == 2) return (const void*)ras_solve<T, false, false, 2, HOLD>;
   return cluster == 8   ? (const void*)ras_solve<T, false, false, 8, HOLD>
          : cluster == 4 ? (const void*)ras_solve<T, false, false, 4, HOLD>
-         : cluster == 2 ? (const void*)ras_solve<T, false, false, 2, HOLD>
                         : (const void*)ras_solve<T, false, false, 1, HOLD>;
 }
 // CTAs (a cluster) per box where the boxes alone leave SMs idle: the most whose clusters all
@@ -952,7 +958,7 @@ const void* solve_kernel(int group, bool smem_vec, bool ring, int cluster) {
 template <typename T>
 kkt_status choose_cluster(int nbox, double groups, int warps, size_t smem, int* out) {
   *out = 1;
-  for (int cs = 8; cs >= (sizeof(T) == 8 ? 2 : 4); cs /= 2) {
+  for (int cs = 8; cs >= min_cluster<T>(); cs /= 2) {
     if (groups < 2.5 * cs) continue;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(nbox * cs);
