@@ -1023,8 +1023,8 @@ def main():
     ap.add_argument("--levels", type=int, default=64)
     ap.add_argument("--reps", type=int, default=10)
     ap.add_argument("--prec", type=int, default=32)
-    ap.add_argument("--chunk", type=int, default=0, help="--kernel ras: points per chunk (0: the library's choice)")
-    ap.add_argument("--stages", type=int, default=0, help="--kernel ras: copy-ring buffers (0: the library's choice)")
+    ap.add_argument("--chunk", type=int, default=0, help="--kernel ras: size class of the solve (0: the library's choice)")
+    ap.add_argument("--stages", type=int, default=0, help="--kernel ras: groups a warp holds (0: the library's choice)")
     ap.add_argument("--place", type=int, default=0,
                     help="--kernel ras: local vectors 1 in shared, 2 in global memory (0: the library's choice)")
     ap.add_argument("--overlap", type=int, default=2, help="--kernel ras/matvec: subdomain overlap")

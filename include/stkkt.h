@@ -342,7 +342,7 @@ kkt_status lu_selftest_quotient(const double* v, const double* d, double* q, lon
  * ras_apply -- z = sum_ij (R^0_ij)^T M_ij^{-1} R^delta_ij r (restricted prolongation,
  *   Cai-Sarkis form cited in Sec. 3.2); all boxes in one launch.  r, z FP64,
  *   3*N*(M+1) values each; the two spans must not overlap (ERR_ARG).  Does not
- *   synchronise; a solve that gave up on a factor copy is reported by
+ *   synchronise; a solve that gave up waiting is reported by
  *   ras_status (and by gmres_solve).
  */
 kkt_status ras_apply(ras_precond* m, const double* r, double* z, void* stream);

@@ -124,7 +124,7 @@ class RAS:
         """factor_prec 64, 32 or 16 (BF16 storage); local "ilu0", "lu" (exact, FP64 only), "ilu1" (ILU(1))
         or "bilu0" (3x3 point-block ILU(0)); the last two in FP64 or FP32.
 
-        shape: None (chosen by the library) or (chunk points, ring buffers, lanes, placement) for
+        shape: None (chosen by the library) or (size class, groups held, lanes, placement) for
         ras_setup_shape, placement 1 = local vectors in shared memory, 2 = in global memory, 0 = any.
         """
         self._lib = _lib.load()
@@ -161,7 +161,8 @@ class RAS:
         return dict(nbox=nb.value, points=pts.value, factor_values=fv.value, value_bytes=vb.value)
 
     def solve_shape(self):
-        """dict(chunk_points, stages, lanes, smem_vectors) of the subdomain solve."""
+        """dict of the subdomain solve's shape: chunk_points (its size class), stages (groups a warp
+        holds), lanes, smem_vectors."""
         ch, ns, ln, sv = C.c_int(), C.c_int(), C.c_int(), C.c_int()
         check(self._lib.ras_solve_shape(self.h, C.byref(ch), C.byref(ns), C.byref(ln), C.byref(sv)),
               "ras_solve_shape")
@@ -174,7 +175,7 @@ class RAS:
         return dict(warps=v[0].value, buffers=v[1].value, cluster=v[2].value, ring=bool(v[3].value))
 
     def status(self, stream=None) -> int:
-        """The device status word (ras_status); raises KktError for 1 (zero pivot) and 2 (copy wait gave up)."""
+        """The device status word (ras_status); raises KktError for 1 (zero pivot) and 2 (a wait of a solve gave up)."""
         code = C.c_int()
         check(self._lib.ras_status(self.h, C.byref(code), _stream(stream)), "ras_status")
         return code.value

@@ -48,9 +48,10 @@ def _compile(src: str, verbose_ptxas: bool) -> str:
         return obj
     cmd = [nvcc(), "-c", src, "-o", obj] + _flags()
     if os.path.basename(src).startswith("factor"):
-        # the generated elimination code is one long block of independent
-        # loads; at -O3 the LLVM optimiser moves them so far ahead that ptxas
-        # spills registers, at -O2 it leaves the scheduling to ptxas
+        # factor64*.cu: the generated elimination code is one long block of
+        # independent loads; at -O3 the LLVM optimiser moves them so far ahead
+        # that ptxas spills registers, at -O2 it leaves the scheduling to ptxas.
+        # factor32.cu has no such code; its figures were measured with -O2 too
         cmd += ["-Xcicc", "-O2"]
     if verbose_ptxas:
         cmd += ["-Xptxas", "-v"]

@@ -28,8 +28,9 @@
 // (lexicographic) order of the box; with this stencil every lower-triangular
 // dependency of point (x, y, z, t) lies on a wavefront w' < w where
 // w = x + 2y + 4z + 8t, so all points of one wavefront are independent.  Within
-// a point the rows go C, G, f.  One CTA owns one box and steps through its
-// wavefronts with a barrier between them.
+// a point the rows go C, G, f.  A box is worked on by one CTA or a cluster: the
+// factorisations have a barrier between wavefronts, the solve a counter of
+// finished groups.
 //
 // ILU(0) (IKJ form, on the structural pattern):
 //   for each row i in order, for each k < i in pattern(i) ascending:
@@ -39,10 +40,11 @@
 // slot of a factored row stores 1/u_kk, so both the factorisation and the
 // backward sweep multiply instead of divide.
 //
-// Solve.  One CTA per box, or a cluster of 2 to 8 where few boxes leave SMs idle; a warp takes a group of 8 points of the wavefront.
-// The local vector of each box has a ghost layer of zeros one point wide in
-// every direction, so the triangular sweeps need no bounds tests: a slot whose
-// column leaves the box reads 0 and has factor value 0.
+// Solve.  One CTA per box, or a cluster of 2 to 8 where few boxes leave SMs
+// idle; a warp takes a group of points of the wavefront.  The local vector of
+// each box has a ghost layer of zeros one point wide in every direction, so the
+// triangular sweeps need no bounds tests: a slot whose column leaves the box
+// reads 0 and has factor value 0.
 
 #include <algorithm>
 #include <array>
@@ -324,6 +326,9 @@ __global__ void lane_selftest(int* status, unsigned long long limit_ns, int* ver
 // the wavefronts before its group's are done.  What does not depend on the
 // last of them -- all neighbours but those one wavefront away -- is loaded and
 // multiplied before that wait.
+//
+// A wait that runs out sets status 2, tells every CTA of the box, waits for the
+// warp's copies in flight and leaves z unwritten.
 // ---------------------------------------------------------------------------
 constexpr size_t kSmemLimit = 227 * 1024;          // dynamic shared memory of one CTA
 constexpr size_t kSolveReserve = 2048;   // what the shape interface sets aside beside the buffers it counts
@@ -450,8 +455,7 @@ struct LaneFactors<double, G> {
   __device__ __forceinline__ double rank(int r) const { return __ldcs(p + r * G); }
 };
 
-// S: type of the stored factor values; T: arithmetic and local-vector type.
-// Most warps of a CTA and CTAs per SM (ras_setup_shape's largest size class).
+// Most warps of a CTA (ras_setup_shape's largest size class).
 constexpr int kSolveWarpsMax = 16;
 
 // Lanes (bits) whose neighbour q = lane + 4 i lies one wavefront away (w - 1 in
@@ -484,6 +488,8 @@ __host__ __device__ constexpr int solve_buffer(int group, bool ring) {
 }
 constexpr int kSolveHeader = 1024;   // mbarriers (kMaxStages per warp), counter of finished groups, abort word
 
+// S: type of the stored factor values; T: arithmetic and local-vector type.
+// SMEM: the local vector in shared memory.  RING: the last wavefronts there.  G: points per group.
 // CS: CTAs of a cluster that share a box: the groups go round the warps of all of them, the
 // local vector stays in global memory (the L2 holds it), and each CTA has its own counter of
 // the box's finished groups, to which every group adds.  The bits are those of one CTA.
@@ -1558,7 +1564,7 @@ kkt_status ras_check(ras_precond* m) {
   int st = 0;
   KKT_TRY_CUDA(cudaMemcpy(&st, m->status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st == 2) {
-    set_error("ras_apply: a subdomain solve gave up waiting for its factor copy");
+    set_error("ras_apply: a subdomain solve gave up waiting for a factor copy or an earlier wavefront");
     return KKT_ERR_CUDA;
   }
   return KKT_OK;
@@ -1578,7 +1584,7 @@ extern "C" kkt_status ras_setup_shape(kkt_problem* p, const int nsub[4], int ove
   }
   if (shape[0] < 0 || shape[1] < 0 || (shape[1] != 0 && (shape[1] < 2 || shape[1] > kMaxStages)) ||
       (shape[2] != 0 && shape[2] != kLanes) || shape[3] < 0 || shape[3] > 2) {
-    set_error("ras_setup_shape: shape = {chunk points >= 0, ring buffers 0 or 2..4, lanes 0 or 4, "
+    set_error("ras_setup_shape: shape = {size class >= 0, groups held 0 or 2..4, lanes 0 or 4, "
               "vector placement 0, 1 or 2}");
     return KKT_ERR_ARG;
   }
@@ -1589,7 +1595,7 @@ extern "C" kkt_status ras_setup_batch(kkt_problem* const* probs, int nprob, cons
                                       int factor_prec, const int shape[4], ras_precond** out) {
   if (shape && (shape[0] < 0 || shape[1] < 0 || (shape[1] != 0 && (shape[1] < 2 || shape[1] > kMaxStages)) ||
                 (shape[2] != 0 && shape[2] != kLanes) || shape[3] < 0 || shape[3] > 2)) {
-    set_error("ras_setup_batch: shape = {chunk points >= 0, ring buffers 0 or 2..4, lanes 0 or 4, "
+    set_error("ras_setup_batch: shape = {size class >= 0, groups held 0 or 2..4, lanes 0 or 4, "
               "vector placement 0, 1 or 2}");
     return KKT_ERR_ARG;
   }
@@ -1645,7 +1651,7 @@ extern "C" kkt_status ras_status(ras_precond* m, int* code, void* stream) {
   KKT_TRY_CUDA(cudaStreamSynchronize(s));
   *code = st;
   if (*code == 2) {
-    set_error("ras_status: a subdomain solve gave up waiting for its factor copy");
+    set_error("ras_status: a subdomain solve gave up waiting for a factor copy or an earlier wavefront");
     return KKT_ERR_CUDA;
   }
   if (*code == 1) {
@@ -1861,7 +1867,7 @@ extern "C" kkt_status ras_apply_static(ras_precond* m, const double* r, double* 
 // set up on the given problems and timed over `reps` applies with CUDA
 // events; the fastest is returned and, with a cache file, remembered there
 // under a key of the problems' sizes, the split, the precision and the
-// device, one line per key ("key<TAB>chunk stages ms").
+// device, one line per key ("key<TAB>size class, groups held, ms").
 // ---------------------------------------------------------------------------
 namespace {
 

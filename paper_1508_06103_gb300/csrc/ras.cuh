@@ -117,7 +117,7 @@ struct ras_precond {
   GpFactor* gp = nullptr;      // local 2 (ILU(1)) or 3 (point-block ILU(0))
 };
 
-// shape: NULL, or {chunk points, ring buffers, lanes per point, vector placement
+// shape: NULL, or {size class, groups held, lanes per point, vector placement
 // (1 shared, 2 global)} of the subdomain solve, 0 = chosen automatically.
 // Several problems: every problem is split by nsub and all boxes form one list,
 // largest first (so the CTAs of a launch finish together as far as they can).
