@@ -954,13 +954,13 @@ const void* solve_kernel(int group, bool smem_vec, bool ring, int cluster) {
 // run at once and that have 2.5 groups of a wavefront each; FP32 and BF16, less bound by
 // arithmetic, 4 or 8 only.  Counting in every CTA's counter and waiting for the
 // other SMs costs more than fewer groups give.  Measured, FP64 (FP32) us a solve with 1, 2, 4, 8 CTAs a box:
-//   16 boxes, 2.1 groups a wavefront:   553   715   711  1167   ( 105  217  201  350)
-//   64 boxes, 6.8:                     1471  1419  2604         (the wait for a second wave)
-//   16 boxes, 9.2:                     1962  1655  1493  2637   ( 425  513  456  809)
-//   64 boxes, 9.0:                     3048  2626  4691
-//   16 boxes, 15.6:                    3878  2470  1974  3374   ( 827  849  635 1027)
-//   1 box, 21.9:                       5653  3708  2376  1932   (1154 1138  761  638)
-//   8 boxes, 82:                      28476 16691  9412  5708   (7447 6086 3368 2029)
+//   16 boxes, 2.3 groups a wavefront:   593   709   643  1031   ( 112     -  210  345)
+//   64 boxes, 5.4:                     1702  1642  2992  7151   ( 342, the ring)  (4: the wait for a second wave)
+//   16 boxes, 9.3:                     2434  1991  1737  3143   ( 535     -  604 1117)
+//   64 boxes, 8.4:                     2903  2385  4009  9522   ( 614, the ring)
+//   16 boxes, 16.4:                    5026  3103  2251  3544   (1080     -  782 1229)
+//   1 box, 25.2:                       5703  3803  2229  1759   (1306     -  732  592)
+//   8 boxes, 125:                     56892 31839 17992  9836   (16045    - 6644 3675)
 template <typename T>
 kkt_status choose_cluster(int nbox, double groups, int warps, size_t smem, int* out) {
   *out = 1;
@@ -990,11 +990,11 @@ struct ShapeRequest {
 };
 // Picks the best shape allowed by `req`; KKT_ERR_ARG when none is.  Boxes whose
 // wavefronts fill the largest CTA take it (one per SM, its L1 to itself); others
-// take the shape with the fewest waves of CTAs over the SMs.  Measured (before
-// the ring below) at 32^3 x 64, FP32, 256 boxes: fine boxes (15 groups a wavefront) 2.16 ms with 16 warps,
-// 2.46 with 8 (two CTAs an SM), 4.04 with 4; coarse boxes (2.5 groups) 303, 221,
-// 300 us; 192 uneven boxes (5.6 groups) 695, 1039, 1633 us.  FP64, 64 boxes of 9
-// groups: 3.01, 3.87, 6.27 ms.  Then the local vectors in
+// take the shape with the fewest waves of CTAs over the SMs.  Measured with 16, 8 (two
+// CTAs an SM) and 4 warps, FP32, before the ring below, 256 boxes of 32^3 x 64: fine boxes
+// (11 groups a wavefront) 2.16, 2.46, 4.04 ms, coarse boxes (2.5 groups) 303, 221, 300 us;
+// 192 uneven boxes (5.6 groups) 695, 1039, 1633 us.  FP64, one CTA a box: 64 boxes of 8.4
+// groups 2.91, 3.46, 5.41 ms; 256 boxes of 32^3 x 64 9.31, 8.89, 11.15.  Then the local vectors in
 // global memory, the fewest buffers, the largest CTA.  ras_autotune measures instead.
 template <typename T>
 kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int nlev, int group, double gpw, int wcap,
@@ -1055,12 +1055,12 @@ kkt_status choose_solve_shape(int nbox, long long points, long long max_pad, int
         // Boxes beyond what the SMs hold at a time, with hardly more than a group a wavefront: fewer warps
         // each, more boxes at a time.  A wave of CTAs of w warps with g groups a wavefront was measured
         // to take about 1 + 5 g / w.  us an apply with 1, 2, 3, 4 warps, FP64 (FP32; BF16):
-        //   9537 lines of 17 points:         1013 1153 1663 2034   (221 240 277 306; 214 234 273 307)
-        //   4913 lines of 33 levels:         1228 1365 1771 2222   (364 370 421 461; 341 359 415 455)
-        //   4096 boxes of 2^4 points:         426  520  691  802   (106 112 124 136;  99 108 122 136)
-        //   1296 boxes of 3^4 points:         485  623  561  733   (103 111  87 105; 101 105  83 102)
-        //   4096 boxes of 3 or 4 a side:     1276 1661 2258 2674   (381 369 364 367; 297 291 307 326)
-        //   256 boxes of 3 or 4 a side:       421  366  364  365   (171  93  68  58; 161  87  64  54)
+        //   9537 lines of 17 points:         1012 1090 1481 1818   (221 240 277 306; 214 234 273 307)
+        //   4913 lines of 33 levels:         1202 1270 1580 1976   (364 370 421 461; 341 359 415 455)
+        //   4096 boxes of 2^4 points:         424  505  636  742   (106 112 124 136;  99 108 122 136)
+        //   1296 boxes of 3^4 points:         472  615  539  701   (103 111  87 105; 101 105  83 102)
+        //   4096 boxes of 3 or 4 a side:     1263 1508 1949 2295   (381 369 364 367; 297 291 307 326)
+        //   256 boxes of 3 or 4 a side:       358  311  308  311   (171  93  68  58; 161  87  64  54)
         // The last are one wave in any case; the last but one are FP32's groups of 8, bound by their bytes.
         double cost = waves * (1 + 5 * gpw / w);
         for (int fewer = w - 1; fewer >= 1 && fewer >= gpw; --fewer) {
