@@ -438,7 +438,7 @@ void launch_tiled(const DevProblem& p, const T* x, T* y, const double* b, cudaSt
 // fill the SMs.
 // Measured against matvec_tiled: 32^3 x 64 1016 -> 650 us (11 x 11 x 3 tiles, runs of 22),
 // 5 x 4 x 3 x 6 56 -> 22.5 us (runs of one level); the error against extended precision is
-// slightly smaller, on random and on smooth fields.
+// the same to within rounding, on random and on smooth fields.
 // ---------------------------------------------------------------------------
 template <typename Tl>
 constexpr size_t mv64_smem() {
